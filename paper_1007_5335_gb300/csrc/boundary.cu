@@ -11,6 +11,7 @@
 #include "alpert_rule.h"
 #include "bessel.cuh"
 #include "mh_internal.cuh"
+#include "pair64.cuh"
 
 namespace {
 
@@ -969,59 +970,70 @@ __global__ void __launch_bounds__(256) k_dlp_fine32_grp(
     if (threadIdx.x == 0) cnt[grp] = 0u;
 }
 
-__global__ void k_dlp_fine64_blk(const double* __restrict__ xy, const int32_t* __restrict__ ptgt,
-                                 const int32_t* __restrict__ pcurve, const double* __restrict__ fg,
-                                 const double* __restrict__ wf, const int64_t* __restrict__ foff, double inv_alpha,
-                                 double pref, double* out) {
-    __shared__ double red[8];
-    const int64_t p = blockIdx.x;
+// The same in binary64: one block per (group of TG targets on curve k, slice of its fine nodes),
+// one load of a node for TG pairs, the pair term f(rho) (d . w n) from the table of pair64.cuh;
+// pref holds the factor 1/alpha^2.
+template <int TG>
+__global__ void __launch_bounds__(256) k_dlp_fine64_grp(
+    const double* __restrict__ xy, const int32_t* __restrict__ pair_tgt, const int32_t* __restrict__ grp_curve,
+    const int32_t* __restrict__ grp_pair, int slices, const double* __restrict__ fg, const double* __restrict__ wf,
+    const int64_t* __restrict__ foff, mh_pair_tab tab, double pref, double* part, unsigned* cnt, double* out) {
+    __shared__ double red[8][TG];
+    __shared__ int last;
+    const int grp = blockIdx.x / slices, sl = blockIdx.x % slices;
+    const int k = grp_curve[grp];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int64_t t = ptgt[p];
-    const int k = pcurve[p];
-    const double px = xy[2 * t], py = xy[2 * t + 1];
-    double acc = 0.0;
-    for (int64_t f = foff[k] + threadIdx.x; f < foff[k + 1]; f += blockDim.x) {
-        const double* g = fg + 6 * f;
-        acc += dl_kernel(g[0], g[1], g[2], g[3], px, py, inv_alpha) * wf[f];
+    double px[TG], py[TG], acc[TG];
+#pragma unroll
+    for (int j = 0; j < TG; ++j) {
+        const int p = grp_pair[grp * TG + j];
+        // a padding entry sits beyond every cut: its pairs come out 0
+        px[j] = p >= 0 ? xy[2 * (int64_t)pair_tgt[p]] : 1e150;
+        py[j] = p >= 0 ? xy[2 * (int64_t)pair_tgt[p] + 1] : 1e150;
+        acc[j] = 0.0;
     }
-    acc = warp_sum(acc);
-    if (lane == 0) red[warp] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int i = 0; i < nw; ++i) s += red[i];
-        atomicAdd(out + t, pref * s);
-    }
-}
-
-// Upsampled rule in binary32, one warp per (target, curve) pair, fine nodes in chunks of
-// MH_TILE with binary64 chunk centres.
-__global__ void k_dlp_fine32(const double* __restrict__ xy, const int32_t* __restrict__ ptgt,
-                             const int32_t* __restrict__ pcurve, int64_t npairs, const float4* __restrict__ fine32,
-                             const float* __restrict__ wf, const int64_t* __restrict__ foff,
-                             const int64_t* __restrict__ coff, const double2* __restrict__ cc, mh_dl32 c32,
-                             double pref, double* out) {
-    const int64_t p = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (p >= npairs) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t t = ptgt[p];
-    const int k = pcurve[p];
-    const double px = xy[2 * t], py = xy[2 * t + 1];
-    double acc = 0.0;
-    for (int64_t ch = coff[k]; ch < coff[k + 1]; ++ch) {
-        const double2 c = cc[ch];
-        const float tx = (float)(px - c.x), ty = (float)(py - c.y);
-        const int64_t f0 = foff[k] + (ch - coff[k]) * MH_TILE;
-        const int64_t f1 = min(f0 + MH_TILE, foff[k + 1]);
-        float part = 0.f;
-        for (int64_t f = f0 + lane; f < f1; f += 32) {
-            const float4 v = fine32[f];
-            part += mh_dl32_pair(v.x - tx, v.y - ty, v.z, v.w, c32) * wf[f];
+    const int64_t n = foff[k + 1] - foff[k];
+    const int64_t f1 = foff[k] + n * (sl + 1) / slices;
+    for (int64_t f = foff[k] + n * sl / slices + threadIdx.x; f < f1; f += blockDim.x) {
+        const double2* g = reinterpret_cast<const double2*>(fg + 6 * f);
+        const double2 y = g[0], nv = g[1];
+        const double w = wf[f], nx = nv.x * w, ny = nv.y * w;
+#pragma unroll
+        for (int j = 0; j < TG; ++j) {
+            const double dx = y.x - px[j], dy = y.y - py[j];
+            acc[j] = fma(mh_pair_f(fma(dx, dx, dy * dy), tab), fma(dx, nx, dy * ny), acc[j]);
         }
-        acc += (double)part;
     }
-    acc = warp_sum(acc);
-    if (lane == 0) atomicAdd(out + t, pref * acc);
+#pragma unroll
+    for (int j = 0; j < TG; ++j) {
+        acc[j] = warp_sum(acc[j]);
+        if (lane == 0) red[warp][j] = acc[j];
+    }
+    __syncthreads();
+    double s = 0.0;
+    int t = -1;
+    if (threadIdx.x < TG) {
+        for (int w = 0; w < nw; ++w) s += red[w][threadIdx.x];
+        const int p = grp_pair[grp * TG + threadIdx.x];
+        t = p >= 0 ? pair_tgt[p] : -1;
+    }
+    if (slices == 1) {
+        if (t >= 0) atomicAdd(out + t, pref * s);
+        return;
+    }
+    if (threadIdx.x < TG) part[((int64_t)grp * slices + sl) * TG + threadIdx.x] = s;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(cnt + grp, 1u) == (unsigned)(slices - 1);
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (threadIdx.x < TG) {
+        double tot = 0.0;
+        for (int q = 0; q < slices; ++q) tot += __ldcg(part + ((int64_t)grp * slices + q) * TG + threadIdx.x);
+        if (t >= 0) atomicAdd(out + t, pref * tot);
+    }
+    if (threadIdx.x == 0) cnt[grp] = 0u;
 }
 
 // ---------------- GMRES helpers (binary64 Arnoldi) ----------------
@@ -1732,41 +1744,43 @@ __global__ void __launch_bounds__(256) k_fine_weights_fft(const double* __restri
 
 // Coarse trapezoid sum over all curves not flagged fine for the target:
 //   out[t] = -(1/(2 pi alpha^2)) sum_n K(y_n, x_t) sigma_n |y'_n| h
-// Sources are staged through shared memory in tiles of the block size.
+// Sources are staged through shared memory in tiles of the block size, the weight in the normal;
+// the pair term is f(rho) (d . w n) from the table of pair64.cuh and pref holds the 1/alpha^2.
+// gridDim.y > 1 splits the source tiles between blocks (few targets would leave most SMs
+// idle): partial sums without the prefactor go to out[blockIdx.y * nt + t] for a fixed-order
+// reduction.
 template <int BS>
-__global__ void k_dlp_coarse(const double* __restrict__ xy, const uint32_t* __restrict__ fine, int64_t nt,
-                             const double* __restrict__ geo, const double* __restrict__ sigma,
-                             const int32_t* __restrict__ curve_of, const int32_t* __restrict__ nn, int64_t ns,
-                             double inv_alpha, double pref, double* out) {
-    __shared__ double sx[BS], sy[BS], snx[BS], sny[BS], sw[BS];
+__global__ void __launch_bounds__(BS) k_dlp_coarse(const double* __restrict__ xy, const uint32_t* __restrict__ fine,
+                                                   int64_t nt, const double* __restrict__ geo,
+                                                   const double* __restrict__ sigma,
+                                                   const int32_t* __restrict__ curve_of, const int32_t* __restrict__ nn,
+                                                   int64_t ns, mh_pair_tab tab, double pref, double* out) {
+    __shared__ double2 sp[BS], sn[BS];
     __shared__ int sk[BS];
     const int64_t t = blockIdx.x * (int64_t)BS + threadIdx.x;
     const bool active = t < nt;
     const double px = active ? xy[2 * t] : 0.0, py = active ? xy[2 * t + 1] : 0.0;
     const uint32_t mask = active ? fine[t] : 0xffffffffu;
     double acc = 0.0;
-    // gridDim.y > 1 splits the sources between blocks (partials without the prefactor)
     const int64_t ntile = (ns + BS - 1) / BS, per = (ntile + gridDim.y - 1) / gridDim.y;
     const int64_t sbeg = blockIdx.y * per * BS, send = min(ns, (blockIdx.y + 1) * per * BS);
     for (int64_t s0 = sbeg; s0 < send; s0 += BS) {
-        int64_t s = s0 + threadIdx.x;
+        const int64_t s = s0 + threadIdx.x;
         if (s < ns) {
             const double* g = geo + 8 * s;
-            int k = curve_of[s];
-            double sp = g[6];
-            sx[threadIdx.x] = g[0];
-            sy[threadIdx.x] = g[1];
-            snx[threadIdx.x] = g[3] / sp;
-            sny[threadIdx.x] = -g[2] / sp;
-            sw[threadIdx.x] = sigma[s] * sp * (2.0 * MH_PI / nn[k]);
+            const int k = curve_of[s];
+            const double wh = sigma[s] * (2.0 * MH_PI / nn[k]);   // n |y'| = (y2', -y1')
+            sp[threadIdx.x] = make_double2(g[0], g[1]);
+            sn[threadIdx.x] = make_double2(g[3] * wh, -g[2] * wh);
             sk[threadIdx.x] = k;
         }
         __syncthreads();
         const int cnt = (ns - s0) < BS ? (int)(ns - s0) : BS;
         if (active) {
             for (int i = 0; i < cnt; ++i) {
-                if (mask & (1u << sk[i])) continue;
-                acc += dl_kernel(sx[i], sy[i], snx[i], sny[i], px, py, inv_alpha) * sw[i];
+                if ((mask >> sk[i]) & 1u) continue;
+                const double dx = sp[i].x - px, dy = sp[i].y - py;
+                acc = fma(mh_pair_f(fma(dx, dx, dy * dy), tab), fma(dx, sn[i].x, dy * sn[i].y), acc);
             }
         }
         __syncthreads();
@@ -1777,97 +1791,6 @@ __global__ void k_dlp_coarse(const double* __restrict__ xy, const uint32_t* __re
         else
             out[blockIdx.y * nt + t] = acc;
     }
-}
-
-// Upsampled rule for (target, curve) pairs: one warp per pair.
-__global__ void k_dlp_fine(const double* __restrict__ xy, const int32_t* __restrict__ ptgt,
-                           const int32_t* __restrict__ pcurve, int64_t npairs, const double* __restrict__ fg,
-                           const double* __restrict__ wf, const int64_t* __restrict__ foff, double inv_alpha,
-                           double pref, double* out) {
-    const int64_t p = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (p >= npairs) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t t = ptgt[p];
-    const int k = pcurve[p];
-    const double px = xy[2 * t], py = xy[2 * t + 1];
-    double acc = 0.0;
-    for (int64_t f = foff[k] + lane; f < foff[k + 1]; f += 32) {
-        const double* g = fg + 6 * f;
-        acc += dl_kernel(g[0], g[1], g[2], g[3], px, py, inv_alpha) * wf[f];
-    }
-    acc = warp_sum(acc);
-    if (lane == 0) atomicAdd(out + t, pref * acc);
-}
-
-// Near-boundary correction for targets whose trapezoid sum came from the multipole
-// method: upsampled sum over curve k minus the trapezoid sum over the nodes of curve k.
-__global__ void k_dlp_fine_corr(const double* __restrict__ xy, const int32_t* __restrict__ ptgt,
-                                const int32_t* __restrict__ pcurve, int64_t npairs, const double* __restrict__ fg,
-                                const double* __restrict__ wf, const int64_t* __restrict__ foff,
-                                const double* __restrict__ geo, const double* __restrict__ sigma,
-                                const int32_t* __restrict__ nn, const int32_t* __restrict__ off, double inv_alpha,
-                                double pref, double* out) {
-    const int64_t p = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (p >= npairs) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t t = ptgt[p];
-    const int k = pcurve[p];
-    const double px = xy[2 * t], py = xy[2 * t + 1];
-    double acc = 0.0;
-    for (int64_t f = foff[k] + lane; f < foff[k + 1]; f += 32) {
-        const double* g = fg + 6 * f;
-        acc += dl_kernel(g[0], g[1], g[2], g[3], px, py, inv_alpha) * wf[f];
-    }
-    const double h = 2.0 * MH_PI / nn[k];
-    for (int64_t s = off[k] + lane; s < off[k + 1]; s += 32) {
-        const double* g = geo + 8 * s;
-        const double sp = g[6];
-        acc -= dl_kernel(g[0], g[1], g[3] / sp, -g[2] / sp, px, py, inv_alpha) * sigma[s] * sp * h;
-    }
-    acc = warp_sum(acc);
-    if (lane == 0) out[t] += pref * acc;
-}
-
-__global__ void k_dlp_fine_corr32(const double* __restrict__ xy, const int32_t* __restrict__ ptgt,
-                                  const int32_t* __restrict__ pcurve, int64_t npairs,
-                                  const float4* __restrict__ fine32, const float* __restrict__ wf,
-                                  const int64_t* __restrict__ foff, const int64_t* __restrict__ coff,
-                                  const double2* __restrict__ cc, const float4* __restrict__ src32,
-                                  const float* __restrict__ w32, const double2* __restrict__ tc,
-                                  const int32_t* __restrict__ off, mh_dl32 c32, double pref, double* out) {
-    const int64_t p = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (p >= npairs) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t t = ptgt[p];
-    const int k = pcurve[p];
-    const double px = xy[2 * t], py = xy[2 * t + 1];
-    double acc = 0.0;
-    for (int64_t ch = coff[k]; ch < coff[k + 1]; ++ch) {
-        const double2 c = cc[ch];
-        const float tx = (float)(px - c.x), ty = (float)(py - c.y);
-        const int64_t f0 = foff[k] + (ch - coff[k]) * MH_TILE;
-        const int64_t f1 = min(f0 + MH_TILE, foff[k + 1]);
-        float part = 0.f;
-        for (int64_t f = f0 + lane; f < f1; f += 32) {
-            const float4 v = fine32[f];
-            part += mh_dl32_pair(v.x - tx, v.y - ty, v.z, v.w, c32) * wf[f];
-        }
-        acc += (double)part;
-    }
-    // trapezoid nodes of curve k, offsets from their tile centres
-    for (int64_t tile = off[k] / MH_TILE; tile * MH_TILE < off[k + 1]; ++tile) {
-        const double2 c = tc[tile];
-        const float tx = (float)(px - c.x), ty = (float)(py - c.y);
-        const int64_t s0 = max((int64_t)off[k], tile * MH_TILE), s1 = min((int64_t)off[k + 1], (tile + 1) * MH_TILE);
-        float part = 0.f;
-        for (int64_t s = s0 + lane; s < s1; s += 32) {
-            const float4 v = src32[s];
-            part += mh_dl32_pair(v.x - tx, v.y - ty, v.z, v.w, c32) * w32[s];
-        }
-        acc -= (double)part;
-    }
-    acc = warp_sum(acc);
-    if (lane == 0) out[t] += pref * acc;
 }
 
 // Normal-line rule: degree-4 interpolation in the distance through the interior limit
@@ -3125,7 +3048,8 @@ mh_status gmres_info_from_dev(const gmres_dev& g, double tol, mh_gmres_info* inf
     return MH_OK;
 }
 
-mh_status dlp_classify(mh_ctx* ctx, mh_boundary* b, const double* xy_dev, int64_t n, dlp_targets* tg) {
+mh_status dlp_classify(mh_ctx* ctx, mh_boundary* b, const double* xy_dev, int64_t n, dlp_targets* tg,
+                       bool all_groups) {
     cudaStream_t st = ctx->stream;
     tg->n = n;
     dbuf<uint32_t> fine0;
@@ -3173,21 +3097,20 @@ mh_status dlp_classify(mh_ctx* ctx, mh_boundary* b, const double* xy_dev, int64_
     tg->n_pairs = (int64_t)pt.size();
     tg->n_pairs_main = 0;
     while (tg->n_pairs_main < tg->n_pairs && pt[tg->n_pairs_main] < n) tg->n_pairs_main++;
-    tg->fine_nodes_main = tg->fine_nodes_aux = tg->curve_nodes_main = 0;
+    tg->fine_nodes_main = tg->fine_nodes_aux = 0;
     for (int64_t i = 0; i < tg->n_pairs; ++i) {
         const double nk = b->n_nodes[pc[i]];
         if (i < tg->n_pairs_main) {
             tg->fine_nodes_main += UPSAMPLE * nk;
-            tg->curve_nodes_main += nk;
         } else {
             tg->fine_nodes_aux += UPSAMPLE * nk;
         }
     }
-    // groups of FINE_TG auxiliary pairs on one curve (pairs in their order within a curve)
+    // groups of FINE_TG pairs on one curve (pairs in their order within a curve)
     std::vector<int32_t> gcur, gpair;
     {
         std::vector<std::vector<int32_t>> byc(b->n_curves);
-        for (int64_t i = tg->n_pairs_main; i < tg->n_pairs; ++i) byc[pc[i]].push_back((int32_t)i);
+        for (int64_t i = all_groups ? 0 : tg->n_pairs_main; i < tg->n_pairs; ++i) byc[pc[i]].push_back((int32_t)i);
         int64_t min_chunks = INT64_MAX;
         for (int k = 0; k < b->n_curves; ++k) {
             if (byc[k].empty()) continue;
@@ -3292,13 +3215,74 @@ static mh_status prep_mixed(mh_ctx* ctx, mh_boundary* b) {
 static mh_status fine_density(mh_ctx* ctx, mh_boundary* b, const double* sc, mh_precision prec, float* wf32,
                               double* wf64);
 
+// The binary64 pair table of the boundary for alpha (recorded graphs hold it: a rebuild counts as
+// a new operator generation, and the eager step before a recording makes it).
+static mh_status pair_table(mh_ctx* ctx, mh_boundary* b, double alpha) {
+    if (b->ptab_alpha == alpha) return MH_OK;
+    if (!b->ptab.p) MH_ALLOC(ctx, b->ptab, 4 * PT_BINS);
+    k_pair_table<<<(PT_BINS + 127) / 128, 128, 0, ctx->stream>>>(mh_pair_tab_make(nullptr, alpha), alpha, b->ptab.p);
+    MH_LAUNCHED(ctx);
+    b->ptab_alpha = alpha;
+    b->op.gen += 1;
+    return MH_OK;
+}
+
+// Trapezoid sums at the points [i0, i0 + count) of the extended target set into tg->ext (mixed
+// precision: b->w32 holds this density's weights).  The sources are split over the grid so that
+// about 8 blocks per SM run whatever the number of targets, the partial sums added in a fixed order.
+static mh_status coarse_sums(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* tg, int64_t i0, int64_t count,
+                             const double* sigma, mh_precision prec) {
+    cudaStream_t st = ctx->stream;
+    const double pref = -1.0 / (2.0 * MH_PI * alpha * alpha) / (alpha * alpha);
+    const int64_t nblk = (count + MH_TILE - 1) / MH_TILE, ntile = (b->n + MH_TILE - 1) / MH_TILE;
+    const int nsplit = (int)std::max<int64_t>(1, std::min<int64_t>(ntile, (152 * 8) / nblk));
+    if (nsplit > 1 && (int64_t)tg->part.n < nsplit * count) MH_ALLOC(ctx, tg->part, nsplit * count);
+    const dim3 grid((unsigned)nblk, (unsigned)nsplit);
+    double* out = nsplit > 1 ? tg->part.p : tg->ext.p + i0;
+    if (prec == MH_PREC_MIXED)
+        k_dlp_coarse32<<<grid, MH_TILE, 0, st>>>(tg->xy.p + 2 * i0, tg->fine.p + i0, count, b->src32.p, b->w32.p,
+                                                 b->d_curve_of.p, b->tile_c.p, b->tile_r.p, b->n,
+                                                 mh_dl32_make(alpha, MH_DL_CUT32), pref, out);
+    else {
+        MH_TRY(pair_table(ctx, b, alpha));
+        k_dlp_coarse<MH_TILE><<<grid, MH_TILE, 0, st>>>(tg->xy.p + 2 * i0, tg->fine.p + i0, count, b->geo.p, sigma,
+                                                        b->d_curve_of.p, b->d_nn.p, b->n,
+                                                        mh_pair_tab_make(b->ptab.p, alpha), pref, out);
+    }
+    MH_LAUNCHED(ctx);
+    if (nsplit > 1) {
+        k_sum_partials<<<mh_grid(count, 256), 256, 0, st>>>(tg->part.p, nsplit, count, pref, tg->ext.p + i0);
+        MH_LAUNCHED(ctx);
+    }
+    return MH_OK;
+}
+
+// Upsampled sums of the set's groups, added to tg->ext; weights b->wf32 (mixed) or wf64.
+static mh_status fine_sums(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* tg, const double* wf64,
+                           mh_precision prec) {
+    cudaStream_t st = ctx->stream;
+    const double pref = -1.0 / (2.0 * MH_PI * alpha * alpha) / (alpha * alpha);
+    const unsigned grid = (unsigned)(tg->n_groups * tg->fine_slices);
+    if (prec == MH_PREC_MIXED)
+        k_dlp_fine32_grp<FINE_TG><<<grid, 256, 0, st>>>(
+            tg->xy.p, tg->pair_tgt.p, tg->grp_curve.p, tg->grp_pair.p, tg->fine_slices, b->fine32.p, b->wf32.p,
+            b->d_fine_off.p, b->d_fchunk_off.p, b->fchunk_cf.p, b->fchunk_r.p, mh_dl32_make(alpha, MH_DL_CUT32),
+            (float)(MH_DL_CUT32 * alpha), pref, tg->grp_part.p, tg->grp_cnt.p, tg->ext.p);
+    else {
+        MH_TRY(pair_table(ctx, b, alpha));
+        k_dlp_fine64_grp<FINE_TG><<<grid, 256, 0, st>>>(tg->xy.p, tg->pair_tgt.p, tg->grp_curve.p, tg->grp_pair.p,
+                                                        tg->fine_slices, b->fine_geo.p, wf64, b->d_fine_off.p,
+                                                        mh_pair_tab_make(b->ptab.p, alpha), pref, tg->grp_part.p,
+                                                        tg->grp_cnt.p, tg->ext.p);
+    }
+    MH_LAUNCHED(ctx);
+    return MH_OK;
+}
+
 mh_status dlp_evaluate(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* tg, const double* sigma,
                        double* out, mh_precision prec) {
     cudaStream_t st = ctx->stream;
     MH_TRY(bie_assemble(ctx, b, alpha));
-    const double pref = -1.0 / (2.0 * MH_PI * alpha * alpha);
-    const double pref32 = pref / (alpha * alpha);
-    const mh_dl32 c32 = mh_dl32_make(alpha, MH_DL_CUT32);
     dbuf<double>& ext = tg->ext;
     dbuf<double>& sc = tg->sc;
     dbuf<double>& wf = tg->wf;
@@ -3311,41 +3295,29 @@ mh_status dlp_evaluate(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* t
         MH_LAUNCHED(ctx);
         if (tg->n_ext) {
             prof_scope ps(ctx, "dlp_coarse", DL_FLOPS * tg->n_ext * b->n, 24.0 * (tg->n_ext + b->n));
-            k_dlp_coarse32<<<mh_grid(tg->n_ext, MH_TILE), MH_TILE, 0, st>>>(
-                tg->xy.p, tg->fine.p, tg->n_ext, b->src32.p, b->w32.p, b->d_curve_of.p, b->tile_c.p, b->tile_r.p, b->n,
-                c32, pref32, ext.p);
-            MH_LAUNCHED(ctx);
+            MH_TRY(coarse_sums(ctx, b, alpha, tg, 0, tg->n_ext, sigma, MH_PREC_MIXED));
         }
         if (tg->n_pairs) {
             k_fourier_scalar<<<(unsigned)nmodes, 128, 0, st>>>(sigma, b->d_nn.p, b->d_off.p, b->tw.p, b->n_curves,
                                                                nmodes, sc.p);
             MH_LAUNCHED(ctx);
             MH_TRY(fine_density(ctx, b, sc.p, MH_PREC_MIXED, b->wf32.p, nullptr));
-            prof_scope ps(ctx, "dlp_fine", DL_FLOPS * (tg->fine_nodes_main + tg->fine_nodes_aux), 24.0 * b->n_fine);
-            k_dlp_fine32<<<mh_grid(tg->n_pairs * 32, 256), 256, 0, st>>>(
-                tg->xy.p, tg->pair_tgt.p, tg->pair_curve.p, tg->n_pairs, b->fine32.p, b->wf32.p, b->d_fine_off.p,
-                b->d_fchunk_off.p, b->fchunk_c.p, c32, pref32, ext.p);
-            MH_LAUNCHED(ctx);
         }
     } else {
         if (tg->n_ext) {
             prof_scope ps(ctx, "dlp_coarse", DL_FLOPS * tg->n_ext * b->n, 24.0 * (tg->n_ext + b->n));
-            k_dlp_coarse<128><<<mh_grid(tg->n_ext, 128), 128, 0, st>>>(tg->xy.p, tg->fine.p, tg->n_ext, b->geo.p,
-                                                                       sigma, b->d_curve_of.p, b->d_nn.p, b->n,
-                                                                       1.0 / alpha, pref, ext.p);
-            MH_LAUNCHED(ctx);
+            MH_TRY(coarse_sums(ctx, b, alpha, tg, 0, tg->n_ext, sigma, MH_PREC_FP64));
         }
         if (tg->n_pairs) {
             k_fourier_scalar<<<(unsigned)nmodes, 128, 0, st>>>(sigma, b->d_nn.p, b->d_off.p, b->tw.p, b->n_curves,
                                                                nmodes, sc.p);
             MH_LAUNCHED(ctx);
             MH_TRY(fine_density(ctx, b, sc.p, MH_PREC_FP64, nullptr, wf.p));
-            prof_scope ps(ctx, "dlp_fine", DL_FLOPS * (tg->fine_nodes_main + tg->fine_nodes_aux), 24.0 * b->n_fine);
-            k_dlp_fine<<<mh_grid(tg->n_pairs * 32, 256), 256, 0, st>>>(tg->xy.p, tg->pair_tgt.p, tg->pair_curve.p,
-                                                                       tg->n_pairs, b->fine_geo.p, wf.p,
-                                                                       b->d_fine_off.p, 1.0 / alpha, pref, ext.p);
-            MH_LAUNCHED(ctx);
         }
+    }
+    if (tg->n_pairs) {
+        prof_scope ps(ctx, "dlp_fine", DL_FLOPS * (tg->fine_nodes_main + tg->fine_nodes_aux), 24.0 * b->n_fine);
+        MH_TRY(fine_sums(ctx, b, alpha, tg, wf.p, prec));
     }
     if (tg->n_line) {
         MH_TRY(bie_apply(ctx, b, sigma, asig.p, MH_PREC_FP64));
@@ -3433,95 +3405,27 @@ mh_status dlp_fine_weights(mh_ctx* ctx, mh_boundary* b, const double* sigma, mh_
 }
 
 mh_status dlp_evaluate_fmm_tail(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* tg, const double* sigma,
-                                const double* main_vals, double* out, mh_precision prec, bool fine_in_fmm,
-                                const double* asig_given, int part) {
-    if (part != 0 && !fine_in_fmm) return mh_fail(ctx, MH_ERR_INVALID_ARG, "a split tail needs the fine rule in the passes");
+                                const double* main_vals, double* out, mh_precision prec, const double* asig_given,
+                                int part) {
     const bool do_aux = part != 2, do_finish = part != 1;
     cudaStream_t st = ctx->stream;
-    const double pref = -1.0 / (2.0 * MH_PI * alpha * alpha);
-    const double pref32 = pref / (alpha * alpha);
-    const mh_dl32 c32 = mh_dl32_make(alpha, MH_DL_CUT32);
     const int64_t n = tg->n, naux = tg->n_ext - tg->n;
-    const int64_t np_main = tg->n_pairs_main, np_aux = tg->n_pairs - tg->n_pairs_main;
     dbuf<double>& ext = tg->ext;
-    dbuf<double>& sc = tg->sc;
-    dbuf<double>& wf = tg->wf;
     prof_scope ps_all(ctx, "dlp_evaluate");
     // ext[0, n): the given values at the targets; ext[n, n_ext): the auxiliary points, written
     // only by the auxiliary part (part 1), so that part can run beside the work that produces
     // main_vals
     if (do_finish && n) MH_CUDA(ctx, cudaMemcpyAsync(ext.p, main_vals, n * 8, cudaMemcpyDeviceToDevice, st));
-    if (do_aux) {
-        const int64_t np_do_main = fine_in_fmm ? 0 : np_main;
-        if (tg->n_pairs && !fine_in_fmm) MH_TRY(dlp_fine_weights(ctx, b, sigma, prec));
-        (void)sc;
-        (void)wf;
+    if (do_aux && naux) {
         if (prec == MH_PREC_MIXED) {
             MH_TRY(prep_mixed(ctx, b));
             k_weights32<<<mh_grid(b->n, 256), 256, 0, st>>>(sigma, b->geo.p, b->d_curve_of.p, b->d_nn.p, b->n, b->w32.p);
             MH_LAUNCHED(ctx);
-            if (naux) {
-                // few auxiliary points: split the sources over the grid, then reduce in a fixed order
-                const int64_t nblk = (naux + MH_TILE - 1) / MH_TILE;
-                const int64_t ntile = (b->n + MH_TILE - 1) / MH_TILE;
-                const int nsplit = (int)std::max<int64_t>(1, std::min<int64_t>(ntile, (152 * 8) / std::max<int64_t>(nblk, 1)));
-                if ((int64_t)tg->part.n < nsplit * naux) MH_ALLOC(ctx, tg->part, nsplit * naux);
-                k_dlp_coarse32<<<dim3((unsigned)nblk, (unsigned)nsplit), MH_TILE, 0, st>>>(
-                    tg->xy.p + 2 * n, tg->fine.p + n, naux, b->src32.p, b->w32.p, b->d_curve_of.p, b->tile_c.p, b->tile_r.p, b->n,
-                    c32, pref32, nsplit > 1 ? tg->part.p : ext.p + n);
-                MH_LAUNCHED(ctx);
-                if (nsplit > 1) {
-                    k_sum_partials<<<mh_grid(naux, 256), 256, 0, st>>>(tg->part.p, nsplit, naux, pref32, ext.p + n);
-                    MH_LAUNCHED(ctx);
-                }
-            }
-            if (tg->n_pairs) {
-                prof_scope ps(ctx, "dlp_fine", DL_FLOPS * ((fine_in_fmm ? 0 : tg->fine_nodes_main + tg->curve_nodes_main) + tg->fine_nodes_aux), 24.0 * b->n_fine);
-                if (np_do_main) {
-                    k_dlp_fine_corr32<<<mh_grid(np_do_main * 32, 256), 256, 0, st>>>(
-                        tg->xy.p, tg->pair_tgt.p, tg->pair_curve.p, np_do_main, b->fine32.p, b->wf32.p, b->d_fine_off.p,
-                        b->d_fchunk_off.p, b->fchunk_c.p, b->src32.p, b->w32.p, b->tile_c.p, b->d_off.p,
-                        c32, pref32, ext.p);
-                    MH_LAUNCHED(ctx);
-                }
-                if (np_aux) {
-                    k_dlp_fine32_grp<FINE_TG><<<(unsigned)(tg->n_groups * tg->fine_slices), 256, 0, st>>>(
-                        tg->xy.p, tg->pair_tgt.p, tg->grp_curve.p, tg->grp_pair.p, tg->fine_slices, b->fine32.p,
-                        b->wf32.p, b->d_fine_off.p, b->d_fchunk_off.p, b->fchunk_cf.p, b->fchunk_r.p, c32,
-                        (float)(MH_DL_CUT32 * alpha), pref32, tg->grp_part.p, tg->grp_cnt.p, ext.p);
-                    MH_LAUNCHED(ctx);
-                }
-            }
-        } else {
-            if (naux) {
-                const int64_t nblk = (naux + 127) / 128, ntile = (b->n + 127) / 128;
-                const int nsplit = (int)std::max<int64_t>(1, std::min<int64_t>(ntile, (152 * 8) / std::max<int64_t>(nblk, 1)));
-                if ((int64_t)tg->part.n < nsplit * naux) MH_ALLOC(ctx, tg->part, nsplit * naux);
-                k_dlp_coarse<128><<<dim3((unsigned)nblk, (unsigned)nsplit), 128, 0, st>>>(
-                    tg->xy.p + 2 * n, tg->fine.p + n, naux, b->geo.p, sigma, b->d_curve_of.p, b->d_nn.p, b->n, 1.0 / alpha,
-                    pref, nsplit > 1 ? tg->part.p : ext.p + n);
-                MH_LAUNCHED(ctx);
-                if (nsplit > 1) {
-                    k_sum_partials<<<mh_grid(naux, 256), 256, 0, st>>>(tg->part.p, nsplit, naux, pref, ext.p + n);
-                    MH_LAUNCHED(ctx);
-                }
-            }
-            if (tg->n_pairs) {
-                prof_scope ps(ctx, "dlp_fine", DL_FLOPS * ((fine_in_fmm ? 0 : tg->fine_nodes_main + tg->curve_nodes_main) + tg->fine_nodes_aux), 24.0 * b->n_fine);
-                if (np_do_main) {
-                    k_dlp_fine_corr<<<mh_grid(np_do_main * 32, 256), 256, 0, st>>>(
-                        tg->xy.p, tg->pair_tgt.p, tg->pair_curve.p, np_do_main, b->fine_geo.p, b->wf64.p,
-                        b->d_fine_off.p, b->geo.p, sigma, b->d_nn.p, b->d_off.p, 1.0 / alpha, pref, ext.p);
-                    MH_LAUNCHED(ctx);
-                }
-                if (np_aux) {
-                    k_dlp_fine64_blk<<<(unsigned)np_aux, 256, 0, st>>>(tg->xy.p, tg->pair_tgt.p + np_main,
-                                                                       tg->pair_curve.p + np_main, b->fine_geo.p,
-                                                                       b->wf64.p, b->d_fine_off.p, 1.0 / alpha, pref,
-                                                                       ext.p);
-                    MH_LAUNCHED(ctx);
-                }
-            }
+        }
+        MH_TRY(coarse_sums(ctx, b, alpha, tg, n, naux, sigma, prec));
+        if (tg->n_groups) {
+            prof_scope ps(ctx, "dlp_fine", DL_FLOPS * tg->fine_nodes_aux, 24.0 * b->n_fine);
+            MH_TRY(fine_sums(ctx, b, alpha, tg, b->wf64.p, prec));
         }
     }
     if (!do_finish) return MH_OK;
@@ -3557,7 +3461,7 @@ extern "C" mh_status mh_double_layer_apply(mh_ctx* ctx, mh_boundary* b, double a
     if (n_targets < 0) return mh_fail(ctx, MH_ERR_INVALID_ARG, "n_targets < 0");
     if (n_targets == 0) return MH_OK;   // no targets: nothing to evaluate, out_dev untouched
     dlp_targets tg;
-    MH_TRY(dlp_classify(ctx, b, targets_dev, n_targets, &tg));
+    MH_TRY(dlp_classify(ctx, b, targets_dev, n_targets, &tg, true));
     MH_TRY(dlp_evaluate(ctx, b, alpha, &tg, sigma_dev, out_dev, prec));
     MH_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     return MH_OK;

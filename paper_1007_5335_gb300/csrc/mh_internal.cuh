@@ -249,6 +249,8 @@ struct mh_boundary {
     dbuf<float> fchunk_r;                // fine chunk radii
     dbuf<float> w32, wf32, x32;          // per call: weights, fine weights, GEMV input
     dbuf<double> sc64, wf64;             // per call: density Fourier coefficients, fine weights
+    dbuf<double2> ptab;                  // binary64 pair table (pair64.cuh) for ptab_alpha
+    double ptab_alpha = -1.0;
     // matrix-free operator: the trapezoid sum by the on-surface multipole pass of a tree that
     // holds every node, the Alpert correction by binary64 chirp transforms per curve
     bool mfree = false;
@@ -287,11 +289,12 @@ struct dlp_targets {
     dbuf<int64_t> line_woff;    // [n_line + 1] offsets into line_w
     // fine pairs (ext target, curve)
     int64_t n_pairs = 0, n_pairs_main = 0;   // pairs of user targets come first
-    double fine_nodes_main = 0, fine_nodes_aux = 0, curve_nodes_main = 0;   // work counts
+    double fine_nodes_main = 0, fine_nodes_aux = 0;   // work counts
     dbuf<int32_t> pair_tgt, pair_curve;
-    // binary32 upsampled rule at the auxiliary points: groups of FINE_TG pairs on one curve
-    // (grp_pair, -1 padded), each group's fine chunks in fine_slices slices, one block per
-    // (group, slice); partial sums per (group, slice, pair) in grp_part
+    // upsampled rule at the auxiliary points (at every pair of a set classified with all_groups):
+    // groups of FINE_TG pairs on one curve (grp_pair, -1 padded), each group's fine nodes in
+    // fine_slices slices, one block per (group, slice); partial sums per (group, slice, pair) in
+    // grp_part
     int64_t n_groups = 0;
     int fine_slices = 1;
     dbuf<int32_t> grp_curve, grp_pair;
@@ -382,19 +385,19 @@ mh_status bie_apply_resid(mh_ctx* ctx, mh_boundary* b, const double* x, double* 
 const double* gmres_final_residual(mh_boundary* b, mh_precision prec, bool graph);
 // Everything a sync-free solve in precision prec needs (binary32 operator copy).
 mh_status bie_prepare(mh_ctx* ctx, mh_boundary* b, mh_precision prec);
-mh_status dlp_classify(mh_ctx* ctx, mh_boundary* b, const double* xy_dev, int64_t n, dlp_targets* tg);
+// all_groups: the upsampled rule will run at every pair (dlp_evaluate), not at the auxiliary ones only.
+mh_status dlp_classify(mh_ctx* ctx, mh_boundary* b, const double* xy_dev, int64_t n, dlp_targets* tg,
+                       bool all_groups = false);
 mh_status dlp_evaluate(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* tg,
                        const double* sigma, double* out, mh_precision prec);
-// U^h when the trapezoid sum at the user targets (main_vals, n values) comes from the
-// multipole method: adds the near-boundary corrections and the normal-line rule.
-// fine_in_fmm: main_vals already use the 16x upsampled rule on every curve (the fine
-// nodes went through the multipole method), so only the auxiliary points of the
-// normal-line rule need near-boundary work.  Requires dlp_fine_weights for this sigma.
-// part (fine_in_fmm only): 0 = everything; 1 = the sums at the auxiliary points (they need
-// sigma and its fine weights only, so they may run beside the pass that produces main_vals);
-// 2 = the rest, after part 1 (main_vals, the normal-line rule, out).
+// U^h when the upsampled sum of every curve at the user targets (main_vals, n values) comes from
+// the multipole method: adds the normal-line rule and its auxiliary points.  Requires
+// dlp_fine_weights for this sigma.
+// part: 0 = everything; 1 = the sums at the auxiliary points (they need sigma and its fine
+// weights only, so they may run beside the pass that produces main_vals); 2 = the rest, after
+// part 1 (main_vals, the normal-line rule, out).
 mh_status dlp_evaluate_fmm_tail(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* tg, const double* sigma,
-                                const double* main_vals, double* out, mh_precision prec, bool fine_in_fmm,
+                                const double* main_vals, double* out, mh_precision prec,
                                 const double* asig_given = nullptr, int part = 0);
 // Density on the 16x fine grid times |y'| h_f (binary64 in b->wf64; binary32 also in b->wf32
 // when prec is mixed).

@@ -424,7 +424,7 @@ static mh_status step_solve(mh_ctx* ctx, ProblemImpl* P, const double* f_next_de
     if (aux_fork) {
         MH_TRY(P->aux.begin(ctx, st));
         ctx->stream = P->aux.s;
-        const mh_status sa = dlp_evaluate_fmm_tail(ctx, b, P->alpha, &P->tg, sigma_dev, nullptr, nullptr, prec, true,
+        const mh_status sa = dlp_evaluate_fmm_tail(ctx, b, P->alpha, &P->tg, sigma_dev, nullptr, nullptr, prec,
                                                    nullptr, 1);
         ctx->stream = st;
         MH_TRY(sa);
@@ -445,7 +445,7 @@ static mh_status step_solve(mh_ctx* ctx, ProblemImpl* P, const double* f_next_de
         MH_LAUNCHED(ctx);
     }
     if (aux_fork) MH_CUDA(ctx, cudaStreamWaitEvent(st, P->aux.join, 0));
-    MH_TRY(dlp_evaluate_fmm_tail(ctx, b, P->alpha, &P->tg, sigma_dev, P->Uh.p, P->Uh.p, prec, true,
+    MH_TRY(dlp_evaluate_fmm_tail(ctx, b, P->alpha, &P->tg, sigma_dev, P->Uh.p, P->Uh.p, prec,
                                  P->tg.n_line ? P->tg.asig.p : nullptr, aux_fork ? 2 : 0));
     k_combine<<<mh_grid(n, 256), 256, 0, st>>>(P->Up.p, P->Uh.p, P->region.p, P->slot.p, P->d_ext_const.p,
                                                P->ext_mode, n, u_next_dev);

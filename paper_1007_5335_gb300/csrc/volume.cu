@@ -32,6 +32,7 @@
 #include <cooperative_groups.h>
 
 #include "mh_internal.cuh"
+#include "pair64.cuh"
 
 namespace {
 
@@ -1545,13 +1546,16 @@ __device__ __forceinline__ void near_finish(double acc, bool act, int qq, int i,
     if (threadIdx.x == 0) cnt[ch.leaf] = 0u;
 }
 
+// Binary64: the staged dipole carries its weight in the normal, the pair term is f(rho) (d . w n)
+// from the table of pair64.cuh; pref holds the factor 1/alpha^2.  Bound by the binary64 pipe (15
+// instructions a pair, 16 cycles each per warp and SM); the four 16-byte table loads of a pair
+// run beside them from L1 (the threads of a warp share the dipole, so their bins are close).
 __global__ void __launch_bounds__(NEAR_T) k_dip_near64(
     const double* __restrict__ nodes, const NearChunk* __restrict__ chunks, const int2* __restrict__ leaf_red,
     const int32_t* __restrict__ flat_idx, const double2* __restrict__ dxy, const double2* __restrict__ dnrm,
-    const double* __restrict__ w, int qq, double inv_alpha, double pref, double* part, unsigned* cnt,
+    const double* __restrict__ w, int qq, mh_pair_tab tab, double pref, double* part, unsigned* cnt,
     double* out) {
     __shared__ double2 sp[NEAR_T], sn[NEAR_T];
-    __shared__ double sw[NEAR_T];
     const NearChunk ch = chunks[blockIdx.x];
     const int groups = NEAR_T / qq;   // >= 4 for q <= 8
     const int i = threadIdx.x % qq, g = threadIdx.x / qq;
@@ -1564,18 +1568,16 @@ __global__ void __launch_bounds__(NEAR_T) k_dip_near64(
         __syncthreads();
         if (threadIdx.x < m) {
             const int d = flat_idx[k0 + threadIdx.x];
+            const double2 n = dnrm[d];
+            const double wd = w[d];
             sp[threadIdx.x] = dxy[d];
-            sn[threadIdx.x] = dnrm[d];
-            sw[threadIdx.x] = w[d];
+            sn[threadIdx.x] = make_double2(n.x * wd, n.y * wd);
         }
         __syncthreads();
         if (act)
             for (int e = g; e < m; e += groups) {
                 const double dx = sp[e].x - px, dy = sp[e].y - py;
-                const double r = sqrt(dx * dx + dy * dy);
-                // pairs beyond 45 alpha are below the binary64 rounding of the sum (e^{-45})
-                if (r > 0.0 && r * inv_alpha <= 45.0)
-                    acc += mh_k1(r * inv_alpha) * inv_alpha * (dx * sn[e].x + dy * sn[e].y) / r * sw[e];
+                acc = fma(mh_pair_f(fma(dx, dx, dy * dy), tab), fma(dx, sn[e].x, dy * sn[e].y), acc);
             }
     }
     near_finish<NEAR_T>(acc, act, qq, i, groups, ch, leaf_red, pref, part, cnt, out);
@@ -1650,7 +1652,8 @@ struct DipData {
     dbuf<int32_t> flat_idx;                // dipole of every flat entry
     dbuf<float4> flat32;                   // its offset from the target leaf centre + normal (binary32)
     dbuf<double2> leaf_c, dxy, dnrm;       // leaf centres; dipole positions and normals (sorted)
-    double pref = 0, inv_alpha = 0;
+    double pref = 0, inv_alpha = 0, alpha = 0;
+    dbuf<double2> ptab;                    // binary64 pair table of the near field (pair64.cuh)
     double near_pairs = 0;
     int near_t = 256;                      // threads per block of the binary32 near-field kernel
     dbuf<double> vec, temp, ops64;
@@ -1857,6 +1860,7 @@ mh_status volume_dipole_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, cons
     D->qq = qq;
     D->pref = pref;
     D->inv_alpha = k;
+    D->alpha = alpha;
     std::vector<int32_t> nleaf;
     D->W_off = 0;
     D->DM_off = nd;
@@ -1984,6 +1988,9 @@ mh_status volume_dipole_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, cons
         MH_ALLOC(ctx, D->leaf_c, nl);
         MH_ALLOC(ctx, D->dxy, std::max<int64_t>(nd, 1));
         MH_ALLOC(ctx, D->dnrm, std::max<int64_t>(nd, 1));
+        MH_ALLOC(ctx, D->ptab, 4 * PT_BINS);
+        k_pair_table<<<(PT_BINS + 127) / 128, 128, 0, st>>>(mh_pair_tab_make(nullptr, alpha), alpha, D->ptab.p);
+        MH_LAUNCHED(ctx);
         if (!ch.empty())
             MH_CUDA(ctx, cudaMemcpyAsync(D->chunks.p, ch.data(), ch.size() * sizeof(NearChunk), cudaMemcpyHostToDevice, st));
         MH_CUDA(ctx, cudaMemcpyAsync(D->leaf_red.p, lred.data(), nl * sizeof(int2), cudaMemcpyHostToDevice, st));
@@ -2123,8 +2130,9 @@ mh_status volume_dipole_apply(mh_ctx* ctx, mh_tree* t, const double* w_sorted, m
 #undef MH_NEAR32
         } else {
             k_dip_near64<<<nb, NEAR_T, 0, st>>>(t->nodes.p, D->chunks.p, D->leaf_red.p, D->flat_idx.p, D->dxy.p,
-                                                D->dnrm.p, D->vec.p + D->W_off, D->qq, D->inv_alpha, D->pref,
-                                                D->part.p, D->red_cnt.p, out);
+                                                D->dnrm.p, D->vec.p + D->W_off, D->qq,
+                                                mh_pair_tab_make(D->ptab.p, D->alpha),
+                                                D->pref * D->inv_alpha * D->inv_alpha, D->part.p, D->red_cnt.p, out);
         }
         MH_LAUNCHED(ctx);
     }
