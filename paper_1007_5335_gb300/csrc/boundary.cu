@@ -10,6 +10,7 @@
 
 #include "alpert_rule.h"
 #include "bessel.cuh"
+#include "gmres_kernels.cuh"
 #include "mh_internal.cuh"
 #include "pair64.cuh"
 
@@ -1133,182 +1134,6 @@ __global__ void k_update_x(const double* __restrict__ V, const double* __restric
     }
 }
 
-// ---- fused Arnoldi step: classical Gram-Schmidt twice over row slices of ARN_ROWS rows ----
-// Every reduction runs in a fixed order (slice partials, then the slices in index order),
-// so the iteration is deterministic.
-constexpr int ARN_ROWS = 64;
-
-// P[s k1 + i] = sum over slice s of V_i[e] w[e], i < k1 (a warp per i).  With kdev, k1 is
-// *kdev + 1 (the iteration count of a sweep kept on the device: one kernel node serves every
-// iteration of a graph loop).
-__global__ void __launch_bounds__(256) k_arn_dots(const double* __restrict__ V, const double* __restrict__ w,
-                                                  int64_t n, int k1, double* __restrict__ P,
-                                                  const int* __restrict__ gate = nullptr,
-                                                  const int* __restrict__ kdev = nullptr) {
-    if (gate && *gate) return;
-    if (kdev) k1 = *kdev + 1;
-    const int s = blockIdx.x;
-    const int64_t r0 = (int64_t)s * ARN_ROWS;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t e0 = r0 + lane, e1 = r0 + lane + 32;
-    const double w0 = e0 < n ? w[e0] : 0.0, w1 = e1 < n ? w[e1] : 0.0;
-    for (int i = warp; i < k1; i += 8) {
-        const double* v = V + (int64_t)i * n;
-        double a = 0.0;
-        if (e0 < n) a = v[e0] * w0;
-        if (e1 < n) a = fma(v[e1], w1, a);
-        a = warp_sum(a);
-        if (lane == 0) P[(int64_t)s * k1 + i] = a;
-    }
-}
-
-// h_i = sum_s Pin[s k1 + i]; w -= sum_i h_i V_i on the slice; then the partial dots of the
-// new w (Pdots) or its partial squared norm (Pnorm).  Block 0 stores h in hout.
-__global__ void __launch_bounds__(256) k_arn_update(const double* __restrict__ V, double* __restrict__ w, int64_t n,
-                                                    int k1, const double* __restrict__ Pin, int S,
-                                                    double* __restrict__ Pdots, double* __restrict__ Pnorm,
-                                                    double* __restrict__ hout, const int* __restrict__ gate = nullptr,
-                                                    const int* __restrict__ kdev = nullptr) {
-    if (gate && *gate) return;
-    if (kdev) k1 = *kdev + 1;
-    extern __shared__ double sh[];      // h[k1], then the slice of w
-    double* h = sh;
-    double* wsl = sh + k1;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int i = warp; i < k1; i += 8) {      // a warp per coefficient, lanes over the slices
-        double a = 0.0;
-        for (int q = lane; q < S; q += 32) a += Pin[(int64_t)q * k1 + i];
-        a = warp_sum(a);
-        if (lane == 0) {
-            h[i] = a;
-            if (blockIdx.x == 0) hout[i] = a;
-        }
-    }
-    __syncthreads();
-    const int s = blockIdx.x;
-    const int64_t r0 = (int64_t)s * ARN_ROWS;
-    if (threadIdx.x < ARN_ROWS) {
-        const int64_t e = r0 + threadIdx.x;
-        double a = 0.0;
-        if (e < n) {
-            a = w[e];
-            for (int i = 0; i < k1; ++i) a = fma(-h[i], V[(int64_t)i * n + e], a);
-            w[e] = a;
-        }
-        wsl[threadIdx.x] = a;
-    }
-    __syncthreads();
-    if (Pdots) {
-        const int64_t e0 = r0 + lane, e1 = r0 + lane + 32;
-        for (int i = warp; i < k1; i += 8) {
-            const double* v = V + (int64_t)i * n;
-            double a = 0.0;
-            if (e0 < n) a = v[e0] * wsl[lane];
-            if (e1 < n) a = fma(v[e1], wsl[lane + 32], a);
-            a = warp_sum(a);
-            if (lane == 0) Pdots[(int64_t)s * k1 + i] = a;
-        }
-    } else if (warp == 0) {
-        double a = fma(wsl[lane], wsl[lane], wsl[lane + 32] * wsl[lane + 32]);
-        a = warp_sum(a);
-        if (lane == 0) Pnorm[s] = a;
-    }
-}
-
-// ||w|| from the partial norms; v_{k+1} = w / ||w|| (and its binary32 copy when vnext32 is
-// given).  Block 0 forms column k of H (h1 + h2, ||w||), applies the previous Givens
-// rotations, forms rotation k, updates g and stores |g_{k+1}| in small[0].
-// Graph loops: with kdev (= &gs->k), k comes from the device and v_{k+1} goes to
-// vnext + (k + 1) n; with loop_set, block 0 sets the loop's condition to "not ended".
-__global__ void __launch_bounds__(256) k_arn_finish(const double* __restrict__ w, int64_t n,
-                                                    const double* __restrict__ Pn, int S, int k,
-                                                    const double* __restrict__ h1, const double* __restrict__ h2,
-                                                    double* H, int ldh, double* cs, double* sn, double* g,
-                                                    double* small, double* __restrict__ vnext,
-                                                    float* __restrict__ vnext32, gmres_dev* gs = nullptr,
-                                                    int m_max = 0, const int* kdev = nullptr,
-                                                    cudaGraphConditionalHandle loop = 0, int loop_set = 0) {
-    if (gs && gs->skip) return;
-    if (kdev) {
-        k = *kdev;
-        vnext += (int64_t)(k + 1) * n;
-    }
-    __shared__ double nrm;
-    if (threadIdx.x < 32) {
-        double a = 0.0;
-        for (int q = threadIdx.x; q < S; q += 32) a += Pn[q];
-        a = warp_sum(a);
-        if (threadIdx.x == 0) nrm = sqrt(a);
-    }
-    __syncthreads();
-    const double s = nrm;
-    const double inv = s > 0.0 ? 1.0 / s : 0.0;
-    const int64_t r0 = (int64_t)blockIdx.x * ARN_ROWS;
-    if (threadIdx.x < ARN_ROWS) {
-        const int64_t e = r0 + threadIdx.x;
-        if (e < n) {
-            const double v = w[e] * inv;
-            vnext[e] = v;
-            if (vnext32) vnext32[e] = (float)v;
-        }
-    }
-    // Column k is formed by block 0 when k is a launch argument; with the device-side state
-    // (gs) by the last block to arrive: every block has read gs->k and gs->skip before it
-    // counts its arrival, so the update of both cannot reach a block that has not started.
-    if (gs) {
-        __shared__ int last;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            last = atomicAdd(&gs->arrive, 1) == (int)gridDim.x - 1;
-        }
-        __syncthreads();
-        if (!last) return;
-        if (threadIdx.x == 0) gs->arrive = 0;
-    } else if (blockIdx.x != 0) {
-        return;
-    }
-    // column k and the previous rotations staged in shared memory, then one thread rotates
-    extern __shared__ double gsh[];      // col[k + 2], cs[k], sn[k]
-    double* col = gsh;
-    double* c_s = gsh + k + 2;
-    double* s_s = c_s + k;
-    for (int i = threadIdx.x; i <= k; i += blockDim.x) col[i] = h1[i] + h2[i];
-    for (int i = threadIdx.x; i < k; i += blockDim.x) {
-        c_s[i] = cs[i];
-        s_s[i] = sn[i];
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        col[k + 1] = s;
-        for (int i = 0; i < k; ++i) {
-            const double t = c_s[i] * col[i] + s_s[i] * col[i + 1];
-            col[i + 1] = -s_s[i] * col[i] + c_s[i] * col[i + 1];
-            col[i] = t;
-        }
-        const double a = col[k], b = col[k + 1];
-        const double den = hypot(a, b);
-        const double c = den > 0 ? a / den : 1.0, sv = den > 0 ? b / den : 0.0;
-        cs[k] = c;
-        sn[k] = sv;
-        col[k] = den;
-        col[k + 1] = 0.0;
-        const double gk = g[k];
-        g[k + 1] = -sv * gk;
-        g[k] = c * gk;
-        small[0] = fabs(-sv * gk);
-        if (gs) {   // sync-free schedule: iteration count and the end of this sweep's Arnoldi process
-            gs->k = k + 1;
-            gs->total += 1;
-            if (fabs(sv * gk) <= gs->target || k + 1 >= m_max || den == 0.0) gs->skip = 1;
-            if (loop_set) cudaGraphSetConditional(loop, gs->skip ? 0u : 1u);
-        }
-    }
-    __syncthreads();
-    double* hc = H + (int64_t)k * ldh;
-    for (int i = threadIdx.x; i <= k + 1; i += blockDim.x) hc[i] = col[i];
-}
-
 // r = b - r (in place on r), v0 = r / ||r|| later
 __global__ void k_sub_from(const double* __restrict__ b, double* r, int64_t n) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
@@ -1322,11 +1147,6 @@ __global__ void k_scale_into(const double* __restrict__ r, const double* __restr
     int64_t e0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (e0 == 0) g[0] = s;
     for (int64_t e = e0; e < n; e += (int64_t)gridDim.x * blockDim.x) v[e] = r[e] * inv;
-}
-
-__global__ void k_axpy(double a, const double* __restrict__ x, double* y, int64_t n) {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
-        y[e] = fma(a, x[e], y[e]);
 }
 
 // ---------------- classification of off-surface targets ----------------
@@ -2531,11 +2351,6 @@ static void resid_gemv(cudaStream_t st, mh_boundary* b, const double* x, double*
         gemv64(st, b->op.A64.p, x, y, n, gate);
 }
 
-static void gemv_resid(cudaStream_t st, mh_boundary* b, const double* x, double* y, const int* gate, bool mixed) {
-    if (resid_ff(b, mixed)) resid_split(st, b, x);
-    resid_gemv(st, b, x, y, gate, mixed);
-}
-
 static const char* resid_region(mh_boundary* b, bool mixed, const int* gate) {
     if (gate) return "bie_gemv64_gated";   // may be skipped on the device: timed apart
     return resid_ff(b, mixed) ? "bie_gemvff" : "bie_gemv64";
@@ -2548,13 +2363,13 @@ static double resid_bytes(mh_boundary* b, bool mixed) {
 }
 
 mh_status bie_apply64_gated(mh_ctx* ctx, mh_boundary* b, const double* x, double* y, const int* gate,
-                            mh_precision prec) {
+                            mh_precision prec, bool x_split) {
     // the gate only skips work whose result the caller then ignores: the matrix-free form
     // always computes
     if (b->mfree) return bie_apply_mfree(ctx, b, x, y);
     MH_TRY(need_dense(ctx, b));
     const bool mixed = prec == MH_PREC_MIXED;
-    if (resid_ff(b, mixed)) {   // the split of x is not part of the timed GEMV region
+    if (resid_ff(b, mixed) && !x_split) {   // the split of x is not part of the timed GEMV region
         resid_split(ctx->stream, b, x);
         MH_LAUNCHED(ctx);
     }
@@ -2564,13 +2379,7 @@ mh_status bie_apply64_gated(mh_ctx* ctx, mh_boundary* b, const double* x, double
     return MH_OK;
 }
 
-mh_status bie_apply_resid(mh_ctx* ctx, mh_boundary* b, const double* x, double* y, mh_precision prec) {
-    return bie_apply64_gated(ctx, b, x, y, nullptr, prec);
-}
-
-const double* gmres_final_residual(mh_boundary* b, mh_precision prec, bool graph) {
-    return (graph || prec == MH_PREC_MIXED) ? b->ws.r.p : b->ws.w.p;
-}
+const double* gmres_final_residual(mh_boundary* b) { return b->ws.r.p; }
 
 
 mh_status bie_apply(mh_ctx* ctx, mh_boundary* b, const double* x, double* y, mh_precision prec) {
@@ -2599,32 +2408,103 @@ static mh_status vec_norm(mh_ctx* ctx, const double* v, int64_t n, double* dev_o
     return MH_OK;
 }
 
-// Unrestarted GMRES on A (precision prec) for A x = b; x holds the initial guess.
-// Returns iterations used and the Givens residual estimate (absolute).
-static mh_status gmres_core(mh_ctx* ctx, mh_boundary* bd, gmres_ws& ws, const double* b, double* x, double abs_tol,
-                            int max_iter, mh_precision prec, int* iters, double* resid, const double* r0,
-                            double* beta0) {
-    const int64_t n = bd->n;
-    cudaStream_t st = ctx->stream;
-    const int ew = mh_grid(n, 256) < 152 * 4 ? mh_grid(n, 256) : 152 * 4;
-    const int ldh = max_iter + 1;
-    if (prec == MH_PREC_MIXED) MH_TRY(ensure_fp32(ctx, bd));
-    // r = b - A x (or the caller's residual of x)
-    if (r0) {
-        MH_CUDA(ctx, cudaMemcpyAsync(ws.w.p, r0, n * 8, cudaMemcpyDeviceToDevice, st));
-    } else {
-        MH_TRY(bie_apply(ctx, bd, x, ws.w.p, prec));
-        k_sub_from<<<ew, 256, 0, st>>>(b, ws.w.p, n);
-        MH_LAUNCHED(ctx);
-    }
-    double beta;
-    MH_TRY(vec_norm(ctx, ws.w.p, n, ws.small.p + 1, &beta));
-    if (beta0) *beta0 = beta;
-    *iters = 0;
-    *resid = beta;
-    if (beta <= abs_tol) return MH_OK;
-    k_scale_into<<<ew, 256, 0, st>>>(ws.w.p, ws.small.p + 1, ws.V.p, ws.g.p, n);
+// Launch of a GMRES kernel as one cluster of `blocks` thread blocks.
+template <class A>
+static mh_status launch_cluster(mh_ctx* ctx, void (*kernel)(A), int blocks, size_t smem, const A& args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim = {(unsigned)blocks, 1, 1};
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(gmres_k::GM_T);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = ctx->stream;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    MH_CUDA(ctx, cudaLaunchKernelEx(&cfg, kernel, args));
     MH_LAUNCHED(ctx);
+    return MH_OK;
+}
+
+// Blocks of the cluster for a basis of k1 vectors: 8 on short boundaries, where the barriers cost
+// more than the work, and for bases so long that 16 sets of partial sums would not fit.
+static int gm_blocks(const gmres_ws& ws, int64_t n, int k1) { return n < 1024 || k1 > 400 ? 8 : ws.cluster; }
+
+static mh_status arnoldi_step(mh_ctx* ctx, gmres_ws& ws, int64_t n, int k, int kcap, int ldh, bool mixed,
+                              gmres_dev* gs = nullptr, int m_max = 0, cudaGraphConditionalHandle loop = 0,
+                              int loop_set = 0) {
+    const int C = gm_blocks(ws, n, kcap);
+    gmres_k::step_args a = {};
+    const size_t smem = gmres_k::step_smem(n, C, kcap, &a.shared_w);
+    a.V = a.Vn = ws.V.p;
+    a.w = ws.w.p;
+    a.n = n;
+    a.k = k;
+    a.kcap = kcap;
+    a.ldh = ldh;
+    a.H = ws.H.p;
+    a.cs = ws.cs.p;
+    a.sn = ws.sn.p;
+    a.g = ws.g.p;
+    a.small = ws.small.p;
+    a.v32 = mixed ? ws.v32.p : nullptr;
+    a.gs = gs;
+    a.m_max = m_max;
+    a.loop = loop;
+    a.loop_set = loop_set;
+    return launch_cluster(ctx, gmres_k::k_arnoldi, C, smem, a);
+}
+
+// r = b - ax (or r0) into ws.r, its norm, V_0 = r / ||r||, g; see k_sweep_begin.
+static gmres_k::begin_args begin_of(gmres_ws& ws, const double* b, const double* ax, const double* r0, int64_t n,
+                                    int gsz, bool mixed, bool first) {
+    gmres_k::begin_args a = {};
+    a.b = b;
+    a.ax = ax;
+    a.r0 = r0;
+    a.r = ws.r.p;
+    a.V0 = ws.V.p;
+    a.g = ws.g.p;
+    a.scal = ws.small.p + 1;
+    a.v32 = mixed ? ws.v32.p : nullptr;
+    a.n = n;
+    a.gsz = gsz;
+    a.mixed = mixed;
+    a.first = first;
+    return a;
+}
+
+static mh_status sweep_begin(mh_ctx* ctx, gmres_ws& ws, const gmres_k::begin_args& a) {
+    return launch_cluster(ctx, gmres_k::k_sweep_begin, gm_blocks(ws, a.n, 1), 0, a);
+}
+
+// The same for the interactive solver, which reads the norms back: *rn = ||r||, *bn = ||b|| (first).
+static mh_status sweep_begin_read(mh_ctx* ctx, gmres_ws& ws, const gmres_k::begin_args& a, double* rn, double* bn) {
+    MH_TRY(sweep_begin(ctx, ws, a));
+    double v[2];
+    MH_CUDA(ctx, cudaMemcpyAsync(v, a.scal, 16, cudaMemcpyDeviceToHost, ctx->stream));
+    MH_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    *rn = v[0];
+    if (a.first) *bn = v[1];
+    return MH_OK;
+}
+
+static mh_status sweep_end(mh_ctx* ctx, mh_boundary* bd, int ldh, int k, int kcap, const gmres_dev* gs, double* x,
+                           bool split) {
+    gmres_ws& ws = bd->ws;
+    gmres_k::k_sweep_end<<<mh_grid(bd->n, 256), 256, kcap * sizeof(double), ctx->stream>>>(
+        ws.V.p, ws.H.p, ldh, ws.g.p, k, gs, bd->n, x, split ? bd->xhi32.p : nullptr, split ? bd->xlo32.p : nullptr);
+    MH_LAUNCHED(ctx);
+    return MH_OK;
+}
+
+// Arnoldi process from V_0 = r / beta (sweep_begin) until the residual estimate is <= abs_tol or
+// max_iter steps: steps taken and the estimate (absolute).
+static mh_status arnoldi_run(mh_ctx* ctx, mh_boundary* bd, double beta, double abs_tol, int max_iter, bool mixed,
+                             int* iters, double* resid) {
+    const int64_t n = bd->n;
+    gmres_ws& ws = bd->ws;
+    cudaStream_t st = ctx->stream;
     int k = 0;
     double res = beta;
     // The residual estimate is read back only at predicted convergence points: from the
@@ -2632,14 +2512,7 @@ static mh_status gmres_core(mh_ctx* ctx, mh_boundary* bd, gmres_ws& ws, const do
     // reach the tolerance (iterations between reads are queued without host round trips).
     int next_check = 1, k_prev = 0;
     double res_prev = beta;
-    const bool mixed = prec == MH_PREC_MIXED;
-    const int S = (int)((n + ARN_ROWS - 1) / ARN_ROWS);
-    if (mixed) {
-        k_to_float_vec<<<mh_grid(n, 256), 256, 0, st>>>(ws.V.p, ws.v32.p, n);
-        MH_LAUNCHED(ctx);
-    }
     for (; k < max_iter; ++k) {
-        const int k1 = k + 1;
         {   // w = A v_k
             const double* vk = ws.V.p + (int64_t)k * n;
             if (bd->mfree) {
@@ -2654,18 +2527,7 @@ static mh_status gmres_core(mh_ctx* ctx, mh_boundary* bd, gmres_ws& ws, const do
                 MH_LAUNCHED(ctx);
             }
         }
-        // classical Gram-Schmidt twice, normalisation and the Givens update (four launches)
-        const size_t shm = (size_t)(k1 + ARN_ROWS) * sizeof(double);
-        k_arn_dots<<<S, 256, 0, st>>>(ws.V.p, ws.w.p, n, k1, ws.P1.p);
-        MH_LAUNCHED(ctx);
-        k_arn_update<<<S, 256, shm, st>>>(ws.V.p, ws.w.p, n, k1, ws.P1.p, S, ws.P2.p, nullptr, ws.h1.p);
-        MH_LAUNCHED(ctx);
-        k_arn_update<<<S, 256, shm, st>>>(ws.V.p, ws.w.p, n, k1, ws.P2.p, S, nullptr, ws.Pn.p, ws.h2.p);
-        MH_LAUNCHED(ctx);
-        k_arn_finish<<<S, 256, (size_t)(3 * k + 2) * sizeof(double), st>>>(ws.w.p, n, ws.Pn.p, S, k, ws.h1.p,
-                                                                            ws.h2.p, ws.H.p, ldh, ws.cs.p, ws.sn.p,
-                                        ws.g.p, ws.small.p, ws.V.p + (int64_t)k1 * n, mixed ? ws.v32.p : nullptr);
-        MH_LAUNCHED(ctx);
+        MH_TRY(arnoldi_step(ctx, ws, n, k, k + 1, max_iter + 1, mixed));
         if (k + 1 < next_check && k + 1 < max_iter) continue;
         MH_CUDA(ctx, cudaMemcpyAsync(&res, ws.small.p, 8, cudaMemcpyDeviceToHost, st));
         MH_CUDA(ctx, cudaStreamSynchronize(st));
@@ -2683,10 +2545,6 @@ static mh_status gmres_core(mh_ctx* ctx, mh_boundary* bd, gmres_ws& ws, const do
         res_prev = res;
         next_check = k + 1 + ahead;
     }
-    k_backsolve<<<1, 1, 0, st>>>(ws.H.p, ldh, k, ws.g.p, ws.y.p);
-    MH_LAUNCHED(ctx);
-    k_update_x<<<ew, 256, 0, st>>>(ws.V.p, ws.y.p, k, n, x);
-    MH_LAUNCHED(ctx);
     *iters = k;
     *resid = res;
     return MH_OK;
@@ -2701,78 +2559,51 @@ mh_status gmres_run(mh_ctx* ctx, mh_boundary* bd, const double* b, double* x, do
         return mh_fail(ctx, MH_ERR_INVALID_ARG, "the matrix-free operator runs in binary64 only");
     if (!bd->mfree) MH_TRY(need_dense(ctx, bd));
     MH_TRY(gmres_graph_ensure(ctx, bd, max_iter));
+    const bool mixed = prec == MH_PREC_MIXED;
+    if (mixed) MH_TRY(ensure_fp32(ctx, bd));
     gmres_ws& ws = bd->ws;
-    MH_CUDA(ctx, cudaMemsetAsync(ws.g.p, 0, (max_iter + 2) * 8, ctx->stream));
-    double bnorm;
-    MH_TRY(vec_norm(ctx, b, n, ws.small.p + 2, &bnorm));
+    const bool split = !bd->mfree && resid_ff(bd, mixed);
+    double bnorm = 0.0, rn = 0.0;
     mh_gmres_info inf{0, 0, 0.0, 0, 0.0};
-    if (bnorm == 0.0) {
-        MH_CUDA(ctx, cudaMemsetAsync(x, 0, n * 8, ctx->stream));
-        MH_CUDA(ctx, cudaMemsetAsync(ws.r.p, 0, n * 8, ctx->stream));   // residual of x = 0
-        MH_CUDA(ctx, cudaMemsetAsync(ws.w.p, 0, n * 8, ctx->stream));
-        inf.converged = 1;
-        if (info) *info = inf;
-        return MH_OK;
-    }
-    if (prec == MH_PREC_FP64) {
+    // binary64: one sweep to the tolerance, then the true residual.  Mixed: sweeps of the
+    // binary32-operator process inside binary64 iterative refinement.
+    for (int sweep = 0;; ++sweep) {
+        // binary64 residual of x; at the first sweep the caller's r0 (if given) stands in
+        // for it, but convergence is only ever accepted on a residual computed here
+        bool computed = sweep > 0 || !r0;
+        if (computed) MH_TRY(bie_apply64_gated(ctx, bd, x, ws.w.p, nullptr, prec, split && sweep > 0));
+        MH_TRY(sweep_begin_read(ctx, ws,
+                                begin_of(ws, b, computed ? ws.w.p : nullptr, r0, n, max_iter + 2, mixed, sweep == 0),
+                                &rn, &bnorm));
+        if (sweep == 0) {
+            if (bnorm == 0.0) {
+                MH_CUDA(ctx, cudaMemsetAsync(x, 0, n * 8, ctx->stream));
+                MH_CUDA(ctx, cudaMemsetAsync(ws.r.p, 0, n * 8, ctx->stream));   // residual of x = 0
+                inf.converged = 1;
+                if (info) *info = inf;
+                return MH_OK;
+            }
+            if (!std::isfinite(rn)) return mh_fail(ctx, MH_ERR_NUMERIC, "GMRES residual is not finite");
+            inf.initial_rel_residual = rn / bnorm;
+        }
+        if (!computed && rn <= tol * bnorm) {
+            MH_TRY(bie_apply64_gated(ctx, bd, x, ws.w.p, nullptr, prec));
+            MH_TRY(sweep_begin_read(ctx, ws, begin_of(ws, b, ws.w.p, nullptr, n, max_iter + 2, mixed, false), &rn,
+                                    &bnorm));
+        }
+        if (rn <= tol * bnorm || inf.iterations >= max_iter || sweep >= (mixed ? 12 : 1)) break;
         int it;
         double res;
-        double beta0;
-        MH_TRY(gmres_core(ctx, bd, ws, b, x, tol * bnorm, max_iter, MH_PREC_FP64, &it, &res, r0, &beta0));
-        inf.iterations = it;
-        inf.initial_rel_residual = beta0 / bnorm;
-    } else {
-        // binary64 iterative refinement around binary32-operator GMRES
-        dbuf<double>& r = ws.r;
-        dbuf<double>& dx = ws.dx;
-        int total = 0;
-        double rn = -1.0;
-        for (int sweep = 0;; ++sweep) {
-            // binary64 residual of x; at the first sweep the caller's r0 (if given) stands in
-            // for it, but convergence is only ever accepted on a residual computed here
-            bool computed = true;
-            if (sweep == 0 && r0) {
-                MH_CUDA(ctx, cudaMemcpyAsync(r.p, r0, n * 8, cudaMemcpyDeviceToDevice, ctx->stream));
-                computed = false;
-            } else {
-                MH_TRY(bie_apply_resid(ctx, bd, x, r.p, MH_PREC_MIXED));
-                k_sub_from<<<mh_grid(n, 256), 256, 0, ctx->stream>>>(b, r.p, n);
-                MH_LAUNCHED(ctx);
-            }
-            MH_TRY(vec_norm(ctx, r.p, n, ws.small.p + 2, &rn));
-            if (sweep == 0) inf.initial_rel_residual = rn / bnorm;
-            if (!computed && rn <= tol * bnorm) {
-                MH_TRY(bie_apply_resid(ctx, bd, x, r.p, MH_PREC_MIXED));
-                k_sub_from<<<mh_grid(n, 256), 256, 0, ctx->stream>>>(b, r.p, n);
-                MH_LAUNCHED(ctx);
-                MH_TRY(vec_norm(ctx, r.p, n, ws.small.p + 2, &rn));
-            }
-            if (rn <= tol * bnorm || total >= max_iter || sweep >= 12) break;
-            MH_CUDA(ctx, cudaMemsetAsync(dx.p, 0, n * 8, ctx->stream));
-            MH_CUDA(ctx, cudaMemsetAsync(ws.g.p, 0, (max_iter + 2) * 8, ctx->stream));
-            int it;
-            double res;
-            // half the tolerance: the binary64 residual after the sweep then lands below tol
-            // instead of just above it (which would cost another sweep and binary64 GEMV)
-            MH_TRY(gmres_core(ctx, bd, ws, r.p, dx.p, std::max(0.5 * tol * bnorm, 1e-5 * rn), max_iter - total,
-                              MH_PREC_MIXED, &it, &res, r.p, nullptr));
-            total += it;
-            inf.refinements++;
-            k_axpy<<<mh_grid(n, 256), 256, 0, ctx->stream>>>(1.0, dx.p, x, n);
-            MH_LAUNCHED(ctx);
-        }
-        inf.iterations = total;
-        inf.rel_residual = rn / bnorm;   // binary64 residual of the final iterate (last sweep)
+        // mixed: half the tolerance, so that the binary64 residual after the sweep lands below tol
+        // instead of just above it (which would cost another sweep and binary64 GEMV)
+        const double target = mixed ? std::max(0.5 * tol * bnorm, 1e-5 * rn) : tol * bnorm;
+        const int left = max_iter - inf.iterations;
+        MH_TRY(arnoldi_run(ctx, bd, rn, target, left, mixed, &it, &res));
+        MH_TRY(sweep_end(ctx, bd, left + 1, it, left, nullptr, x, split));
+        inf.iterations += it;
+        if (mixed) inf.refinements++;
     }
-    if (prec == MH_PREC_FP64) {
-        // true residual in binary64
-        MH_TRY(bie_apply(ctx, bd, x, ws.w.p, MH_PREC_FP64));
-        k_sub_from<<<mh_grid(n, 256), 256, 0, ctx->stream>>>(b, ws.w.p, n);
-        MH_LAUNCHED(ctx);
-        double rn;
-        MH_TRY(vec_norm(ctx, ws.w.p, n, ws.small.p + 2, &rn));
-        inf.rel_residual = rn / bnorm;
-    }
+    inf.rel_residual = rn / bnorm;   // binary64 residual of the final iterate
     inf.converged = inf.rel_residual <= tol;
     if (info) *info = inf;
     if (!inf.converged)
@@ -2793,19 +2624,33 @@ mh_status gmres_graph_ensure(mh_ctx* ctx, mh_boundary* bd, int max_iter) {
     MH_ALLOC(ctx, ws.cs, max_iter + 1);
     MH_ALLOC(ctx, ws.sn, max_iter + 1);
     MH_ALLOC(ctx, ws.g, max_iter + 2);
-    MH_ALLOC(ctx, ws.y, max_iter + 1);
-    MH_ALLOC(ctx, ws.h1, max_iter + 2);
-    MH_ALLOC(ctx, ws.h2, max_iter + 2);
     MH_ALLOC(ctx, ws.small, 8);
     MH_ALLOC(ctx, ws.w, n);
     MH_ALLOC(ctx, ws.r, n);
-    MH_ALLOC(ctx, ws.dx, n);
-    const int64_t S = (n + ARN_ROWS - 1) / ARN_ROWS;
-    MH_ALLOC(ctx, ws.P1, S * (max_iter + 1));
-    MH_ALLOC(ctx, ws.P2, S * (max_iter + 1));
-    MH_ALLOC(ctx, ws.Pn, S);
     MH_ALLOC(ctx, ws.v32, n);
     if (!ws.body_stream) MH_CUDA(ctx, cudaStreamCreateWithFlags(&ws.body_stream, cudaStreamNonBlocking));
+    if (!ws.cluster) {
+        MH_CUDA(ctx, cudaFuncSetAttribute(gmres_k::k_arnoldi, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)gmres_k::GM_SMEM_MAX));
+        MH_CUDA(ctx, cudaFuncSetAttribute(gmres_k::k_arnoldi, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        MH_CUDA(ctx, cudaFuncSetAttribute(gmres_k::k_sweep_begin, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        ws.cluster = 16;
+        // a device partition without 16 free SMs side by side takes the portable cluster size
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim = {16, 1, 1};
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(16);
+        cfg.blockDim = dim3(gmres_k::GM_T);
+        cfg.dynamicSmemBytes = gmres_k::GM_SMEM_MAX;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int active = 0;
+        if (cudaOccupancyMaxActiveClusters(&active, gmres_k::k_arnoldi, &cfg) != cudaSuccess || active < 1) {
+            (void)cudaGetLastError();
+            ws.cluster = 8;
+        }
+    }
     ws.m = max_iter;
     ws.n = n;
     ws.gen += 1;
@@ -2822,105 +2667,14 @@ void gmres_graph_schedule(mh_precision prec, int* sweeps, int* m_max) {
     }
 }
 
-__global__ void k_gnorm(const double* __restrict__ v, int64_t n, double* out, const int* __restrict__ gate) {
-    if (gate && *gate) return;
-    double acc = 0.0;
-    for (int64_t e = threadIdx.x; e < n; e += blockDim.x) acc = fma(v[e], v[e], acc);
-    acc = block_sum<1024>(acc);
-    if (threadIdx.x == 0) *out = sqrt(acc);
-}
-
-__global__ void k_gsub(const double* __restrict__ b, double* r, int64_t n, const int* __restrict__ gate) {
-    if (gate && *gate) return;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
-        r[e] = b[e] - r[e];
-}
-
-// Start of a sweep from the residual r (norm gs->rn): accept (converged) when allowed and
-// rn <= tol ||b||, else start an Arnoldi process on r (V_0 = r / rn, g = (rn, 0, ...), inner
-// target max(tol ||b||, 1e-5 rn) in mixed precision, tol ||b|| in binary64).  final_check: the
-// last residual of the schedule, recorded only.  ||b|| = 0 gives x = 0.
-// With loop_set, the condition of the sweep's Arnoldi loop (a graph WHILE node, 0 by default at
-// every launch) is set to "start".
-__global__ void k_sweep_begin(gmres_dev* gs, double tol, int mixed, int may_accept, int final_check, int first,
-                              const double* __restrict__ r, double* V0, float* v32, double* g, int gsz, int64_t n,
-                              double* x, cudaGraphConditionalHandle loop = 0, int loop_set = 0) {
-    if (gs->done) return;
-    const double rn = gs->rn, bn = gs->bnorm;
-    if (bn == 0.0) {
-        for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-            x[e] = 0.0;
-            const_cast<double*>(r)[e] = 0.0;   // the residual of x = 0 for b = 0
-        }
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            gs->done = gs->skip = gs->converged = 1;
-            gs->rel = 0.0;
-        }
-        return;
-    }
-    const bool accept = may_accept || final_check;
-    const bool conv = accept && rn <= tol * bn;
-    const bool start = !conv && !final_check && rn > 0.0;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        if (first) gs->init_rel = rn / bn;
-        if (accept) gs->rel = rn / bn;
-        if (conv) {
-            gs->done = gs->skip = gs->converged = 1;
-        } else if (start) {
-            gs->skip = 0;
-            gs->k = 0;
-            gs->sweeps += 1;
-            gs->target = mixed ? fmax(0.5 * tol * bn, 1e-5 * rn) : tol * bn;
-        } else {
-            gs->skip = 1;
-        }
-        if (loop_set) cudaGraphSetConditional(loop, start ? 1u : 0u);
-    }
-    if (!start) return;
-    const double inv = 1.0 / rn;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-        const double v = r[e] * inv;
-        V0[e] = v;
-        if (v32) v32[e] = (float)v;
-    }
-    if (blockIdx.x == 0)
-        for (int i = threadIdx.x; i < gsz; i += blockDim.x) g[i] = i == 0 ? rn : 0.0;
-}
-
-// R y = g with the iteration count of the sweep (device); skipped once converged.
-__global__ void k_backsolve_g(const double* H, int ldh, const double* g, double* y, const gmres_dev* gs) {
-    if (gs->done) return;
-    const int k = gs->k;
-    for (int i = k - 1; i >= 0; --i) {
-        double acc = g[i];
-        for (int j = i + 1; j < k; ++j) acc -= H[(int64_t)j * ldh + i] * y[j];
-        const double d = H[(int64_t)i * ldh + i];
-        y[i] = d != 0.0 ? acc / d : 0.0;
-    }
-}
-
-// x += sum_{i < k} y_i V_i (k of the sweep, device); skipped once converged.
-__global__ void k_update_x_g(const double* __restrict__ V, const double* __restrict__ y, const gmres_dev* gs,
-                             int64_t n, double* x) {
-    if (gs->done) return;
-    const int k = gs->k;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-        double acc = x[e];
-        for (int i = 0; i < k; ++i) acc = fma(y[i], V[(int64_t)i * n + e], acc);
-        x[e] = acc;
-    }
-}
-
 // One binary32-operator Arnoldi iteration as the body of a graph WHILE node on the capturing
 // stream ctx->stream: the node is added after the stream's current dependencies, the body is
 // captured on the boundary's helper stream, and the stream continues after the node.  The body
-// reads the iteration count from gs->k; k_arn_finish ends the loop.
-static mh_status gmres_loop_node(mh_ctx* ctx, mh_boundary* bd, gmres_dev* gs, cudaGraphConditionalHandle h, int m,
-                                 int SL) {
+// reads the iteration count from gs->k; k_arnoldi ends the loop.
+static mh_status gmres_loop_node(mh_ctx* ctx, mh_boundary* bd, gmres_dev* gs, cudaGraphConditionalHandle h, int m) {
     cudaStream_t st = ctx->stream;
     gmres_ws& ws = bd->ws;
     const int64_t n = bd->n;
-    const int ldh = m + 1;
     cudaStreamCaptureStatus cs;
     cudaGraph_t g = nullptr;
     const cudaGraphNode_t* deps = nullptr;
@@ -2940,21 +2694,12 @@ static mh_status gmres_loop_node(mh_ctx* ctx, mh_boundary* bd, gmres_dev* gs, cu
     MH_CUDA(ctx, cudaStreamBeginCaptureToGraph(bs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
     ctx->stream = bs;
     gemv32(bs, bd->op.A32.p, ws.v32.p, ws.w.p, n, nullptr);
-    MH_LAUNCHED(ctx);
-    const size_t shm = (size_t)(m + ARN_ROWS) * sizeof(double);
-    k_arn_dots<<<SL, 256, 0, bs>>>(ws.V.p, ws.w.p, n, 1, ws.P1.p, nullptr, &gs->k);
-    MH_LAUNCHED(ctx);
-    k_arn_update<<<SL, 256, shm, bs>>>(ws.V.p, ws.w.p, n, 1, ws.P1.p, SL, ws.P2.p, nullptr, ws.h1.p, nullptr, &gs->k);
-    MH_LAUNCHED(ctx);
-    k_arn_update<<<SL, 256, shm, bs>>>(ws.V.p, ws.w.p, n, 1, ws.P2.p, SL, nullptr, ws.Pn.p, ws.h2.p, nullptr, &gs->k);
-    MH_LAUNCHED(ctx);
-    k_arn_finish<<<SL, 256, (size_t)(3 * m + 2) * sizeof(double), bs>>>(
-        ws.w.p, n, ws.Pn.p, SL, 0, ws.h1.p, ws.h2.p, ws.H.p, ldh, ws.cs.p, ws.sn.p, ws.g.p, ws.small.p, ws.V.p,
-        ws.v32.p, gs, m, &gs->k, h, 1);
-    MH_LAUNCHED(ctx);
+    ctx->launches++;
+    const mh_status s = arnoldi_step(ctx, ws, n, 0, m, m + 1, true, gs, m, h, 1);
     ctx->stream = st;
     cudaGraph_t out = nullptr;
     MH_CUDA(ctx, cudaStreamEndCapture(bs, &out));
+    MH_TRY(s);
     ctx->loop_nodes += 1;
     return MH_OK;
 }
@@ -2971,27 +2716,21 @@ mh_status gmres_run_graph(mh_ctx* ctx, mh_boundary* bd, const double* b, double*
     const bool mixed = prec == MH_PREC_MIXED;
     if (ws.m < m || ws.n != n || (mixed && !bd->op.A32.p) || !bd->op.A64.p)
         return mh_fail(ctx, MH_ERR_INVALID_ARG, "sync-free GMRES: workspace or operator not prepared");
-    const int ldh = m + 1;
-    const int ew = mh_grid(n, 256) < 152 * 4 ? mh_grid(n, 256) : 152 * 4;
-    const int SL = (int)((n + ARN_ROWS - 1) / ARN_ROWS);
     cudaStreamCaptureStatus cst = cudaStreamCaptureStatusNone;
     MH_CUDA(ctx, cudaStreamIsCapturing(st, &cst));
     const bool capturing = cst == cudaStreamCaptureStatusActive;
+    const bool split = resid_ff(bd, mixed);
     MH_CUDA(ctx, cudaMemsetAsync(gs, 0, sizeof(gmres_dev), st));
-    k_gnorm<<<1, 1024, 0, st>>>(b, n, &gs->bnorm, nullptr);
-    MH_LAUNCHED(ctx);
     for (int sw = 0; sw <= S; ++sw) {
         const bool supplied = sw == 0 && r0;
-        if (supplied) {
-            MH_CUDA(ctx, cudaMemcpyAsync(ws.r.p, r0, n * 8, cudaMemcpyDeviceToDevice, st));
-        } else {
-            gemv_resid(st, bd, x, ws.r.p, &gs->done, mixed);
-            MH_LAUNCHED(ctx);
-            k_gsub<<<ew, 256, 0, st>>>(b, ws.r.p, n, &gs->done);
+        if (!supplied) {
+            if (split && sw == 0) {
+                resid_split(st, bd, x);
+                MH_LAUNCHED(ctx);
+            }
+            resid_gemv(st, bd, x, ws.w.p, &gs->done, mixed);
             MH_LAUNCHED(ctx);
         }
-        k_gnorm<<<1, 1024, 0, st>>>(ws.r.p, n, &gs->rn, &gs->done);
-        MH_LAUNCHED(ctx);
         // while the stream is being captured (a batch graph), the Arnoldi process of a sweep is a
         // graph WHILE node over one iteration: only the iterations needed run
         const bool loop = mixed && capturing && sw < S;
@@ -3002,38 +2741,29 @@ mh_status gmres_run_graph(mh_ctx* ctx, mh_boundary* bd, const double* b, double*
             MH_CUDA(ctx, cudaStreamGetCaptureInfo(st, &cs, nullptr, &g, nullptr, nullptr, nullptr));
             MH_CUDA(ctx, cudaGraphConditionalHandleCreate(&h, g, 0, cudaGraphCondAssignDefault));
         }
-        k_sweep_begin<<<ew, 256, 0, st>>>(gs, tol, mixed, !supplied, sw == S, sw == 0, ws.r.p, ws.V.p,
-                                          mixed ? ws.v32.p : nullptr, ws.g.p, m + 2, n, x, h, loop ? 1 : 0);
-        MH_LAUNCHED(ctx);
+        gmres_k::begin_args a = begin_of(ws, b, supplied ? nullptr : ws.w.p, r0, n, m + 2, mixed, sw == 0);
+        a.x = x;
+        a.gs = gs;
+        a.tol = tol;
+        a.may_accept = !supplied;
+        a.final_check = sw == S;
+        a.loop = h;
+        a.loop_set = loop ? 1 : 0;
+        MH_TRY(sweep_begin(ctx, ws, a));
         if (sw == S) break;
         if (loop) {
-            MH_TRY(gmres_loop_node(ctx, bd, gs, h, m, SL));
-        } else
-        for (int k = 0; k < m; ++k) {
-            const int k1 = k + 1;
-            if (mixed)
-                gemv32(st, bd->op.A32.p, ws.v32.p, ws.w.p, n, &gs->skip);
-            else
-                gemv64(st, bd->op.A64.p, ws.V.p + (int64_t)k * n, ws.w.p, n, &gs->skip);
-            MH_LAUNCHED(ctx);
-            const size_t shm = (size_t)(k1 + ARN_ROWS) * sizeof(double);
-            k_arn_dots<<<SL, 256, 0, st>>>(ws.V.p, ws.w.p, n, k1, ws.P1.p, &gs->skip);
-            MH_LAUNCHED(ctx);
-            k_arn_update<<<SL, 256, shm, st>>>(ws.V.p, ws.w.p, n, k1, ws.P1.p, SL, ws.P2.p, nullptr, ws.h1.p,
-                                               &gs->skip);
-            MH_LAUNCHED(ctx);
-            k_arn_update<<<SL, 256, shm, st>>>(ws.V.p, ws.w.p, n, k1, ws.P2.p, SL, nullptr, ws.Pn.p, ws.h2.p,
-                                               &gs->skip);
-            MH_LAUNCHED(ctx);
-            k_arn_finish<<<SL, 256, (size_t)(3 * k + 2) * sizeof(double), st>>>(
-                ws.w.p, n, ws.Pn.p, SL, k, ws.h1.p, ws.h2.p, ws.H.p, ldh, ws.cs.p, ws.sn.p, ws.g.p, ws.small.p,
-                ws.V.p + (int64_t)k1 * n, mixed ? ws.v32.p : nullptr, gs, m);
-            MH_LAUNCHED(ctx);
+            MH_TRY(gmres_loop_node(ctx, bd, gs, h, m));
+        } else {
+            for (int k = 0; k < m; ++k) {
+                if (mixed)
+                    gemv32(st, bd->op.A32.p, ws.v32.p, ws.w.p, n, &gs->skip);
+                else
+                    gemv64(st, bd->op.A64.p, ws.V.p + (int64_t)k * n, ws.w.p, n, &gs->skip);
+                MH_LAUNCHED(ctx);
+                MH_TRY(arnoldi_step(ctx, ws, n, k, k + 1, m + 1, mixed, gs, m));
+            }
         }
-        k_backsolve_g<<<1, 1, 0, st>>>(ws.H.p, ldh, ws.g.p, ws.y.p, gs);
-        MH_LAUNCHED(ctx);
-        k_update_x_g<<<ew, 256, 0, st>>>(ws.V.p, ws.y.p, gs, n, x);
-        MH_LAUNCHED(ctx);
+        MH_TRY(sweep_end(ctx, bd, m + 1, 0, m, gs, x, split));
     }
     return MH_OK;
 }

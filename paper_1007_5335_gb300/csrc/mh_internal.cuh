@@ -175,7 +175,7 @@ mh_status tc_split_launch(mh_ctx* ctx, const float* src, int len, int64_t count,
 
 // Device-resident state of the sync-free GMRES (gmres_run_graph): every kernel of its fixed
 // schedule reads the flags at entry and returns at once when its work is not needed.
-constexpr int GMRES_LOOP_KERNELS = 5;   // kernels in the body of a graph Arnoldi loop
+constexpr int GMRES_LOOP_KERNELS = 2;   // kernels in the body of a graph Arnoldi loop
 
 struct gmres_dev {
     double bnorm, rn, target, rel, init_rel;
@@ -185,13 +185,12 @@ struct gmres_dev {
     int total;       // all Arnoldi iterations
     int sweeps;      // sweeps started (refinement passes in mixed precision)
     int converged;
-    int arrive;      // blocks of the running Arnoldi normalisation that have finished (reset by the last)
 };
 
 // GMRES workspace (kept by the boundary so that repeated solves allocate nothing).
 struct gmres_ws {
-    dbuf<double> V, H, cs, sn, g, y, h1, h2, small, w, r, dx;
-    dbuf<double> P1, P2, Pn;             // per-slice partial dot products / squared norms
+    dbuf<double> V, H, cs, sn, g, small, w, r;
+    int cluster = 0;                     // thread blocks in the cluster of an Arnoldi step (16 or 8)
     dbuf<float> v32;                     // binary32 copy of the newest Krylov vector
     cudaStream_t body_stream = nullptr;  // captures the body of a graph loop (batch graphs)
     int m = 0;
@@ -377,12 +376,11 @@ mh_status bie_apply(mh_ctx* ctx, mh_boundary* b, const double* x, double* y, mh_
 mh_status bie_mfree_setup(mh_ctx* ctx, mh_boundary* b, mh_tree* t, double alpha);
 mh_status bie_apply_mfree(mh_ctx* ctx, mh_boundary* b, const double* x, double* y);
 // y = A x in binary64, skipped when *gate != 0 (gate nullable).
+// Mixed precision: accurate to binary64 for residuals (float-float); x_split: b->xhi32, xlo32 hold x.
 mh_status bie_apply64_gated(mh_ctx* ctx, mh_boundary* b, const double* x, double* y, const int* gate,
-                            mh_precision prec);
-// y = A x accurate to binary64 for residuals: float-float in mixed precision, binary64 otherwise
-mh_status bie_apply_resid(mh_ctx* ctx, mh_boundary* b, const double* x, double* y, mh_precision prec);
+                            mh_precision prec, bool x_split = false);
 // Where the last solve left the binary64 residual rhs - A x of its result.
-const double* gmres_final_residual(mh_boundary* b, mh_precision prec, bool graph);
+const double* gmres_final_residual(mh_boundary* b);
 // Everything a sync-free solve in precision prec needs (binary32 operator copy).
 mh_status bie_prepare(mh_ctx* ctx, mh_boundary* b, mh_precision prec);
 // all_groups: the upsampled rule will run at every pair (dlp_evaluate), not at the auxiliary ones only.

@@ -403,7 +403,7 @@ static mh_status step_solve(mh_ctx* ctx, ProblemImpl* P, const double* f_next_de
     if (s == MH_OK) {
         MH_CUDA(ctx, cudaMemcpyAsync(P->rc_sigma.p, sigma_dev, ng * 8, cudaMemcpyDeviceToDevice, st));
         MH_CUDA(ctx, cudaMemcpyAsync(P->rc_b.p, P->rhs.p, ng * 8, cudaMemcpyDeviceToDevice, st));
-        MH_CUDA(ctx, cudaMemcpyAsync(P->rc_r.p, gmres_final_residual(b, prec, P->graph_mode), ng * 8,
+        MH_CUDA(ctx, cudaMemcpyAsync(P->rc_r.p, gmres_final_residual(b), ng * 8,
                                      cudaMemcpyDeviceToDevice, st));
         P->rc_valid = true;
     } else {
