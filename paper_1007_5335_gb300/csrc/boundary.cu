@@ -286,6 +286,7 @@ __global__ void k_split_lo16(const double* __restrict__ a, const float* __restri
 
 // x = xh + xl with xh = x rounded to binary32
 __global__ void k_split_vec(const double* __restrict__ x, float* __restrict__ xh, float* __restrict__ xl, int64_t n) {
+    mh_dep_wait();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i < n) {
         const float h = (float)x[i];
@@ -297,6 +298,7 @@ __global__ void k_split_vec(const double* __restrict__ x, float* __restrict__ xh
 // y = A x, one warp per row, 16-byte loads (N_Gamma is even, so rows stay aligned).
 __global__ void k_gemv64(const double* __restrict__ A, const double* __restrict__ x, double* __restrict__ y,
                          int64_t n, const int* __restrict__ gate = nullptr) {
+    mh_dep_wait();
     if (gate && *gate) return;
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -321,6 +323,7 @@ __global__ void k_gemv64(const double* __restrict__ A, const double* __restrict_
 // row length is a multiple of 4, 8-byte loads otherwise).
 __global__ void k_gemv32(const float* __restrict__ A, const float* __restrict__ x, double* __restrict__ y,
                          int64_t n, const int* __restrict__ gate = nullptr) {
+    mh_dep_wait();
     if (gate && *gate) return;
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -368,6 +371,7 @@ __global__ void k_gemv32(const float* __restrict__ A, const float* __restrict__ 
 template <int SPLIT>
 __global__ void __launch_bounds__(256) k_gemv32s(const float* __restrict__ A, const float* __restrict__ x,
                                                  double* __restrict__ y, int64_t n, const int* __restrict__ gate) {
+    mh_dep_wait();
     if (gate && *gate) return;
     __shared__ float part[8];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -375,14 +379,15 @@ __global__ void __launch_bounds__(256) k_gemv32s(const float* __restrict__ A, co
     const int q = warp % SPLIT;
     float f0 = 0.f, f1 = 0.f, f2 = 0.f, f3 = 0.f;
     if (row < n) {
+        const uint64_t pol = mh_l2_policy((row + 1) * n * 4 <= MH_L2_KEEP);
         const int64_t n4 = n >> 2;
         const int64_t c0 = q * n4 / SPLIT, c1 = (q + 1) * n4 / SPLIT;
         const float4* a4 = reinterpret_cast<const float4*>(A + row * n);
         const float4* x4 = reinterpret_cast<const float4*>(x);
         int64_t c = c0 + lane;
         for (; c + 96 < c1; c += 128) {
-            const float4 a0 = __ldcs(a4 + c), a1 = __ldcs(a4 + c + 32), a2 = __ldcs(a4 + c + 64),
-                         a3 = __ldcs(a4 + c + 96);
+            const float4 a0 = mh_ld_hint(a4 + c, pol), a1 = mh_ld_hint(a4 + c + 32, pol),
+                         a2 = mh_ld_hint(a4 + c + 64, pol), a3 = mh_ld_hint(a4 + c + 96, pol);
             const float4 x0 = __ldg(x4 + c), x1 = __ldg(x4 + c + 32), x2 = __ldg(x4 + c + 64), x3 = __ldg(x4 + c + 96);
             f0 = fmaf(a0.x, x0.x, fmaf(a0.y, x0.y, fmaf(a0.z, x0.z, fmaf(a0.w, x0.w, f0))));
             f1 = fmaf(a1.x, x1.x, fmaf(a1.y, x1.y, fmaf(a1.z, x1.z, fmaf(a1.w, x1.w, f1))));
@@ -390,7 +395,7 @@ __global__ void __launch_bounds__(256) k_gemv32s(const float* __restrict__ A, co
             f3 = fmaf(a3.x, x3.x, fmaf(a3.y, x3.y, fmaf(a3.z, x3.z, fmaf(a3.w, x3.w, f3))));
         }
         for (; c < c1; c += 32) {
-            const float4 av = __ldcs(a4 + c), xv = __ldg(x4 + c);
+            const float4 av = mh_ld_hint(a4 + c, pol), xv = __ldg(x4 + c);
             f0 = fmaf(av.x, xv.x, fmaf(av.y, xv.y, fmaf(av.z, xv.z, fmaf(av.w, xv.w, f0))));
         }
     }
@@ -429,9 +434,10 @@ __device__ __forceinline__ void ff_acc(float& sh, float& sl, float a, float al, 
 // n a multiple of 4; SPLIT warps per row, 8 / SPLIT rows per 256-thread block.
 constexpr int GC_PIECE = 3;   // float4 per lane and matrix per piece: 24 KB per block, up to 8 blocks per SM
 
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)),
-                 "l"(gmem)
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem, uint64_t policy) {
+    asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(smem)),
+                 "l"(gmem), "l"(policy)
                  : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() {
@@ -442,6 +448,7 @@ template <int SPLIT, int M>
 __global__ void __launch_bounds__(256) k_gemv_cpa(const float* __restrict__ A, const float* __restrict__ Al,
                                                   const float* __restrict__ xh, const float* __restrict__ xl,
                                                   double* __restrict__ y, int64_t n, const int* __restrict__ gate) {
+    mh_dep_wait();
     if (gate && *gate) return;
     extern __shared__ __align__(16) float4 gc_stage[];   // [warp][M][GC_PIECE * 32]
     __shared__ float part[2][8];
@@ -451,6 +458,7 @@ __global__ void __launch_bounds__(256) k_gemv_cpa(const float* __restrict__ A, c
     const int q = warp % SPLIT;
     float hi = 0.f, lo = 0.f;
     if (row < n) {
+        const uint64_t pol = mh_l2_policy((row + 1) * n * 4 <= MH_L2_KEEP), once = mh_l2_policy(false);
         const int64_t n4 = n >> 2;
         const int64_t c0 = q * n4 / SPLIT, c1 = (q + 1) * n4 / SPLIT;
         const float4* a4 = reinterpret_cast<const float4*>(A + row * n);
@@ -462,8 +470,8 @@ __global__ void __launch_bounds__(256) k_gemv_cpa(const float* __restrict__ A, c
             for (int u = 0; u < GC_PIECE; ++u) {
                 const int64_t c = p0 + lane + 32 * u;
                 if (c < c1) {
-                    cp_async16(st + lane + 32 * u, a4 + c);
-                    if (M == 2) cp_async16(st + GC_PIECE * 32 + lane + 32 * u, b4 + c);
+                    cp_async16(st + lane + 32 * u, a4 + c, pol);
+                    if (M == 2) cp_async16(st + GC_PIECE * 32 + lane + 32 * u, b4 + c, once);
                 }
             }
             cp_async_wait_all();
@@ -529,9 +537,10 @@ __global__ void __launch_bounds__(256) k_gemv_cpa(const float* __restrict__ A, c
 constexpr int GH_PIECE = 2;   // 16-byte groups of binary16 per lane per piece: 24 KB per block
 
 template <int SPLIT>
-__global__ void __launch_bounds__(256) k_gemv_cph(const float* __restrict__ A, const uint16_t* __restrict__ Ah,
+__global__ void __launch_bounds__(256, 4) k_gemv_cph(const float* __restrict__ A, const uint16_t* __restrict__ Ah,
                                                   const float* __restrict__ xh, const float* __restrict__ xl,
                                                   double* __restrict__ y, int64_t n, const int* __restrict__ gate) {
+    mh_dep_wait();
     if (gate && *gate) return;
     extern __shared__ __align__(16) float4 gc_stage[];   // [warp][3 GH_PIECE * 32]
     __shared__ float part[2][8];
@@ -544,6 +553,7 @@ __global__ void __launch_bounds__(256) k_gemv_cph(const float* __restrict__ A, c
     const int q = warp % SPLIT;
     float hi = 0.f, lo = 0.f;
     if (row < n) {
+        const uint64_t pol = mh_l2_policy((row + 1) * n * 4 <= MH_L2_KEEP), once = mh_l2_policy(false);
         const int64_t n8 = n >> 3;
         const int64_t c0 = q * n8 / SPLIT, c1 = (q + 1) * n8 / SPLIT;   // column octets of the quarter
         const float4* a4 = reinterpret_cast<const float4*>(A + row * n);
@@ -554,12 +564,12 @@ __global__ void __launch_bounds__(256) k_gemv_cph(const float* __restrict__ A, c
 #pragma unroll
             for (int v = 0; v < 2 * GH_PIECE; ++v) {
                 const int j = lane + 32 * v;
-                if (2 * p0 + j < 2 * c1) cp_async16(stA + j, a4 + 2 * p0 + j);
+                if (2 * p0 + j < 2 * c1) cp_async16(stA + j, a4 + 2 * p0 + j, pol);
             }
 #pragma unroll
             for (int u = 0; u < GH_PIECE; ++u) {
                 const int o = lane + 32 * u;
-                if (p0 + o < c1) cp_async16(stH + o, h8 + p0 + o);
+                if (p0 + o < c1) cp_async16(stH + o, h8 + p0 + o, once);
             }
             // the piece's x values are loaded while the operator copies are in flight
             float4 xu[2 * GH_PIECE], xv[2 * GH_PIECE];
@@ -613,6 +623,7 @@ __global__ void __launch_bounds__(256) k_gemv_cph(const float* __restrict__ A, c
 template <int SPLIT>
 __global__ void __launch_bounds__(256) k_gemv64s(const double* __restrict__ A, const double* __restrict__ x,
                                                  double* __restrict__ y, int64_t n, const int* __restrict__ gate) {
+    mh_dep_wait();
     if (gate && *gate) return;
     __shared__ double part[8];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -2301,10 +2312,10 @@ constexpr size_t GH_SMEM = 8 * 3 * GH_PIECE * 32 * sizeof(float4);    // 24 KB
 // computes, and small pieces leave room for 8 blocks per SM, so some compute while others load).
 static void gemv32(cudaStream_t st, const float* A, const float* x, double* y, int64_t n, const int* gate) {
     if ((n & 3) == 0)
-        k_gemv32s<GEMV_SPLIT><<<(unsigned)((n + 8 / GEMV_SPLIT - 1) / (8 / GEMV_SPLIT)), 256, 0, st>>>(A, x, y, n,
-                                                                                                     gate);
+        (void)mh_launch_dep(st, k_gemv32s<GEMV_SPLIT>, dim3((unsigned)((n + 8 / GEMV_SPLIT - 1) / (8 / GEMV_SPLIT))),
+                            dim3(256), 0, A, x, y, n, gate);
     else
-        k_gemv32<<<gemv_blocks(n), 256, 0, st>>>(A, x, y, n, gate);
+        (void)mh_launch_dep(st, k_gemv32, dim3(gemv_blocks(n)), dim3(256), 0, A, x, y, n, gate);
 }
 
 // Shared-memory opt-in of the cp.async GEMVs (once per process, outside any graph capture).
@@ -2321,10 +2332,10 @@ static mh_status gemv_cpa_prepare(mh_ctx* ctx) {
 
 static void gemv64(cudaStream_t st, const double* A, const double* x, double* y, int64_t n, const int* gate) {
     if ((n & 1) == 0)
-        k_gemv64s<GEMV_SPLIT><<<(unsigned)((n + 8 / GEMV_SPLIT - 1) / (8 / GEMV_SPLIT)), 256, 0, st>>>(A, x, y, n,
-                                                                                                     gate);
+        (void)mh_launch_dep(st, k_gemv64s<GEMV_SPLIT>, dim3((unsigned)((n + 8 / GEMV_SPLIT - 1) / (8 / GEMV_SPLIT))),
+                            dim3(256), 0, A, x, y, n, gate);
     else
-        k_gemv64<<<gemv_blocks(n), 256, 0, st>>>(A, x, y, n, gate);
+        (void)mh_launch_dep(st, k_gemv64, dim3(gemv_blocks(n)), dim3(256), 0, A, x, y, n, gate);
 }
 
 // Product with the binary64 operator for a residual: in mixed precision a float-float product
@@ -2342,11 +2353,11 @@ static void resid_gemv(cudaStream_t st, mh_boundary* b, const double* x, double*
     const int64_t n = b->n;
     const unsigned grid = (unsigned)((n + 8 / GEMV_SPLIT - 1) / (8 / GEMV_SPLIT));
     if (mixed && b->op.A16lo.p)
-        k_gemv_cph<GEMV_SPLIT><<<grid, 256, GH_SMEM, st>>>(b->op.A32.p, b->op.A16lo.p, b->xhi32.p, b->xlo32.p, y, n,
-                                                          gate);
+        (void)mh_launch_dep(st, k_gemv_cph<GEMV_SPLIT>, dim3(grid), dim3(256), GH_SMEM, b->op.A32.p, b->op.A16lo.p,
+                            b->xhi32.p, b->xlo32.p, y, n, gate);
     else if (mixed && b->op.A32lo.p)
-        k_gemv_cpa<GEMV_SPLIT, 2><<<grid, 256, GC_SMEM2, st>>>(b->op.A32.p, b->op.A32lo.p, b->xhi32.p, b->xlo32.p, y,
-                                                               n, gate);
+        (void)mh_launch_dep(st, k_gemv_cpa<GEMV_SPLIT, 2>, dim3(grid), dim3(256), GC_SMEM2, b->op.A32.p, b->op.A32lo.p,
+                            b->xhi32.p, b->xlo32.p, y, n, gate);
     else
         gemv64(st, b->op.A64.p, x, y, n, gate);
 }
@@ -2411,7 +2422,9 @@ static mh_status vec_norm(mh_ctx* ctx, const double* v, int64_t n, double* dev_o
 // Launch of a GMRES kernel as one cluster of `blocks` thread blocks.
 template <class A>
 static mh_status launch_cluster(mh_ctx* ctx, void (*kernel)(A), int blocks, size_t smem, const A& args) {
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // always behind a product (or a copy)
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim = {(unsigned)blocks, 1, 1};
     cudaLaunchConfig_t cfg = {};
@@ -2420,7 +2433,7 @@ static mh_status launch_cluster(mh_ctx* ctx, void (*kernel)(A), int blocks, size
     cfg.dynamicSmemBytes = smem;
     cfg.stream = ctx->stream;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     MH_CUDA(ctx, cudaLaunchKernelEx(&cfg, kernel, args));
     MH_LAUNCHED(ctx);
     return MH_OK;
@@ -2492,8 +2505,14 @@ static mh_status sweep_begin_read(mh_ctx* ctx, gmres_ws& ws, const gmres_k::begi
 static mh_status sweep_end(mh_ctx* ctx, mh_boundary* bd, int ldh, int k, int kcap, const gmres_dev* gs, double* x,
                            bool split) {
     gmres_ws& ws = bd->ws;
-    gmres_k::k_sweep_end<<<mh_grid(bd->n, 256), 256, kcap * sizeof(double), ctx->stream>>>(
-        ws.V.p, ws.H.p, ldh, ws.g.p, k, gs, bd->n, x, split ? bd->xhi32.p : nullptr, split ? bd->xlo32.p : nullptr);
+    const auto kern = gmres_k::k_sweep_end;
+    const dim3 grid((unsigned)mh_grid(bd->n, 256));
+    float *xh = split ? bd->xhi32.p : nullptr, *xl = split ? bd->xlo32.p : nullptr;
+    if (gs)   // behind a graph loop: an ordinary launch
+        kern<<<grid, 256, kcap * sizeof(double), ctx->stream>>>(ws.V.p, ws.H.p, ldh, ws.g.p, k, gs, bd->n, x, xh, xl);
+    else
+        (void)mh_launch_dep(ctx->stream, kern, grid, dim3(256), kcap * sizeof(double), ws.V.p, ws.H.p, ldh, ws.g.p, k,
+                            gs, bd->n, x, xh, xl);
     MH_LAUNCHED(ctx);
     return MH_OK;
 }

@@ -71,6 +71,7 @@ struct begin_args {
 __global__ void __launch_bounds__(GM_T) k_sweep_begin(begin_args a) {
     __shared__ double red[2][GM_T / 32], all[2][16], nrm[3];
     cg::cluster_group cl = cg::this_cluster();
+    mh_dep_wait();
     if (a.gs && a.gs->done) return;   // the same for every block: written after the last barrier only
     cl.barrier_arrive();              // every block of the cluster runs before the first remote store
     const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
@@ -241,6 +242,7 @@ __device__ __forceinline__ void subtract(const double* __restrict__ V, int64_t n
 }
 
 __global__ void __launch_bounds__(GM_T) k_arnoldi(step_args a) {
+    mh_dep_wait();
     if (a.gs && a.gs->skip) return;   // the same for every block: written after the last barrier only
     extern __shared__ double sm[];
     __shared__ double npart[16], inv_s;
@@ -369,6 +371,7 @@ constexpr int GE_REG = 32;
 __global__ void __launch_bounds__(256) k_sweep_end(const double* __restrict__ V, const double* __restrict__ H, int ldh,
                                                    const double* __restrict__ g, int k, const gmres_dev* gs, int64_t n,
                                                    double* x, float* __restrict__ xh, float* __restrict__ xl) {
+    mh_dep_wait();
     if (gs) {
         if (gs->done) return;
         k = gs->k;

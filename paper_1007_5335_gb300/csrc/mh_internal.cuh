@@ -106,6 +106,58 @@ struct dbuf {
 
 #define MH_ALLOC(ctx, buf, count) MH_CUDA(ctx, (buf).alloc(count))
 
+// ---- dependent launches ----
+// A kernel launched right behind another one on a stream costs about 2.2 us of drain and launch
+// latency (0.9 us inside a graph); with programmatic dependent launch it is on the SMs and waiting
+// when its predecessor ends (0.6 us; 16 blocks of 512 threads, chains of 500 launches).  The
+// rules here: a kernel launched by mh_launch_dep calls mh_dep_wait() first thing, in every thread
+// and before any return, so it touches memory only when everything before it on the stream has
+// completed, and completes only after its predecessors; mh_launch_dep is used behind a kernel of
+// the same stream (a launch behind an event wait, a copy or a graph's conditional node is an ordinary
+// one).  Kernels that are launched either way call mh_dep_wait() too (no effect in an ordinary
+// launch).  The wait comes before the trigger: at most one kernel waits behind the running one.
+__device__ __forceinline__ void mh_dep_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <class... K, class... A>
+inline cudaError_t mh_launch_dep(cudaStream_t st, void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, A... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<K>(args)...);
+}
+
+// ---- L2 residency hints ----
+// The binary32 operator is read once per Arnoldi step; at 6144 nodes it is 151 MB against 129 MB of
+// L2, so in plain order every step streams all of it from HBM.  The first MH_L2_KEEP bytes are read
+// with an evict-last hint and stay for the next step, the rest with evict-first.  k_gemv32s in a
+// chain, 6144 nodes: 24.2 us without, 20.4 with 40 MB kept, 19.0 (64), 17.5 (80), 17.0 (88), 18.2
+// (96), 23.5 (112): 72 MB leaves the rest of the step its share.
+constexpr int64_t MH_L2_KEEP = 72 << 20;
+
+__device__ __forceinline__ uint64_t mh_l2_policy(bool keep) {
+    uint64_t last, first;
+    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(last));
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(first));
+    return keep ? last : first;
+}
+__device__ __forceinline__ float4 mh_ld_hint(const float4* p, uint64_t policy) {
+    float4 v;
+    asm volatile("ld.global.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "l"(p), "l"(policy));
+    return v;
+}
+
 // A second stream with fork / join events, for work that does not depend on what the context
 // stream runs meanwhile: the multipole passes (latency chains, on a stream of the device's
 // highest priority, so that their blocks start before queued near-field blocks) beside the
