@@ -4,6 +4,7 @@
 // off-surface double-layer potential U^h (Section 2) with the near-boundary rules.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <mutex>
 
 #include <cuda_fp16.h>
@@ -2443,8 +2444,8 @@ static mh_status launch_cluster(mh_ctx* ctx, void (*kernel)(A), int blocks, size
 // more than the work, and for bases so long that 16 sets of partial sums would not fit.
 static int gm_blocks(const gmres_ws& ws, int64_t n, int k1) { return n < 1024 || k1 > 400 ? 8 : ws.cluster; }
 
-static mh_status arnoldi_step(mh_ctx* ctx, gmres_ws& ws, int64_t n, int k, int kcap, int ldh, bool mixed,
-                              gmres_dev* gs = nullptr, int m_max = 0, cudaGraphConditionalHandle loop = 0,
+static mh_status arnoldi_step(mh_ctx* ctx, gmres_ws& ws, int64_t n, int kcap, int ldh, bool mixed, gmres_dev* gs,
+                              int m_max, gmres_k::progress* prog = nullptr, cudaGraphConditionalHandle loop = 0,
                               int loop_set = 0) {
     const int C = gm_blocks(ws, n, kcap);
     gmres_k::step_args a = {};
@@ -2452,38 +2453,39 @@ static mh_status arnoldi_step(mh_ctx* ctx, gmres_ws& ws, int64_t n, int k, int k
     a.V = a.Vn = ws.V.p;
     a.w = ws.w.p;
     a.n = n;
-    a.k = k;
     a.kcap = kcap;
     a.ldh = ldh;
     a.H = ws.H.p;
     a.cs = ws.cs.p;
     a.sn = ws.sn.p;
     a.g = ws.g.p;
-    a.small = ws.small.p;
     a.v32 = mixed ? ws.v32.p : nullptr;
     a.gs = gs;
     a.m_max = m_max;
     a.loop = loop;
     a.loop_set = loop_set;
+    a.prog = prog;
     return launch_cluster(ctx, gmres_k::k_arnoldi, C, smem, a);
 }
 
-// r = b - ax (or r0) into ws.r, its norm, V_0 = r / ||r||, g; see k_sweep_begin.
-static gmres_k::begin_args begin_of(gmres_ws& ws, const double* b, const double* ax, const double* r0, int64_t n,
-                                    int gsz, bool mixed, bool first) {
+// Start of a sweep from the residual b - ax (ax = ws.w, or r0): see k_sweep_begin.
+static gmres_k::begin_args begin_of(gmres_ws& ws, const double* b, const double* r0, double* x, int64_t n, int gsz,
+                                    bool mixed, double tol, gmres_dev* gs) {
     gmres_k::begin_args a = {};
     a.b = b;
-    a.ax = ax;
+    a.ax = r0 ? nullptr : ws.w.p;
     a.r0 = r0;
     a.r = ws.r.p;
     a.V0 = ws.V.p;
     a.g = ws.g.p;
-    a.scal = ws.small.p + 1;
+    a.x = x;
     a.v32 = mixed ? ws.v32.p : nullptr;
     a.n = n;
     a.gsz = gsz;
+    a.gs = gs;
+    a.tol = tol;
     a.mixed = mixed;
-    a.first = first;
+    a.may_accept = r0 == nullptr;
     return a;
 }
 
@@ -2491,84 +2493,40 @@ static mh_status sweep_begin(mh_ctx* ctx, gmres_ws& ws, const gmres_k::begin_arg
     return launch_cluster(ctx, gmres_k::k_sweep_begin, gm_blocks(ws, a.n, 1), 0, a);
 }
 
-// The same for the interactive solver, which reads the norms back: *rn = ||r||, *bn = ||b|| (first).
-static mh_status sweep_begin_read(mh_ctx* ctx, gmres_ws& ws, const gmres_k::begin_args& a, double* rn, double* bn) {
-    MH_TRY(sweep_begin(ctx, ws, a));
-    double v[2];
-    MH_CUDA(ctx, cudaMemcpyAsync(v, a.scal, 16, cudaMemcpyDeviceToHost, ctx->stream));
-    MH_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    *rn = v[0];
-    if (a.first) *bn = v[1];
-    return MH_OK;
-}
-
-static mh_status sweep_end(mh_ctx* ctx, mh_boundary* bd, int ldh, int k, int kcap, const gmres_dev* gs, double* x,
-                           bool split) {
+// dep: directly behind a kernel (not behind a graph loop).
+static mh_status sweep_end(mh_ctx* ctx, mh_boundary* bd, int ldh, int kcap, const gmres_dev* gs, double* x, bool split,
+                           bool dep) {
     gmres_ws& ws = bd->ws;
     const auto kern = gmres_k::k_sweep_end;
     const dim3 grid((unsigned)mh_grid(bd->n, 256));
     float *xh = split ? bd->xhi32.p : nullptr, *xl = split ? bd->xlo32.p : nullptr;
-    if (gs)   // behind a graph loop: an ordinary launch
-        kern<<<grid, 256, kcap * sizeof(double), ctx->stream>>>(ws.V.p, ws.H.p, ldh, ws.g.p, k, gs, bd->n, x, xh, xl);
+    if (dep)
+        (void)mh_launch_dep(ctx->stream, kern, grid, dim3(256), kcap * sizeof(double), ws.V.p, ws.H.p, ldh, ws.g.p, gs,
+                            bd->n, x, xh, xl);
     else
-        (void)mh_launch_dep(ctx->stream, kern, grid, dim3(256), kcap * sizeof(double), ws.V.p, ws.H.p, ldh, ws.g.p, k,
-                            gs, bd->n, x, xh, xl);
+        kern<<<grid, 256, kcap * sizeof(double), ctx->stream>>>(ws.V.p, ws.H.p, ldh, ws.g.p, gs, bd->n, x, xh, xl);
     MH_LAUNCHED(ctx);
     return MH_OK;
 }
 
-// Arnoldi process from V_0 = r / beta (sweep_begin) until the residual estimate is <= abs_tol or
-// max_iter steps: steps taken and the estimate (absolute).
-static mh_status arnoldi_run(mh_ctx* ctx, mh_boundary* bd, double beta, double abs_tol, int max_iter, bool mixed,
-                             int* iters, double* resid) {
-    const int64_t n = bd->n;
-    gmres_ws& ws = bd->ws;
-    cudaStream_t st = ctx->stream;
-    int k = 0;
-    double res = beta;
-    // The residual estimate is read back only at predicted convergence points: from the
-    // decay observed between two reads, the next read is placed where the estimate should
-    // reach the tolerance (iterations between reads are queued without host round trips).
-    int next_check = 1, k_prev = 0;
-    double res_prev = beta;
-    for (; k < max_iter; ++k) {
-        {   // w = A v_k
-            const double* vk = ws.V.p + (int64_t)k * n;
-            if (bd->mfree) {
-                MH_TRY(bie_apply_mfree(ctx, bd, vk, ws.w.p));
-            } else {
-                prof_scope ps(ctx, mixed ? "bie_gemv32" : "bie_gemv64", 2.0 * n * n,
-                              mixed ? 4.0 * n * n + 12.0 * n : 8.0 * n * n + 16.0 * n);
-                if (mixed)
-                    gemv32(st, bd->op.A32.p, ws.v32.p, ws.w.p, n, nullptr);
-                else
-                    gemv64(st, bd->op.A64.p, vk, ws.w.p, n, nullptr);
-                MH_LAUNCHED(ctx);
-            }
-        }
-        MH_TRY(arnoldi_step(ctx, ws, n, k, k + 1, max_iter + 1, mixed));
-        if (k + 1 < next_check && k + 1 < max_iter) continue;
-        MH_CUDA(ctx, cudaMemcpyAsync(&res, ws.small.p, 8, cudaMemcpyDeviceToHost, st));
-        MH_CUDA(ctx, cudaStreamSynchronize(st));
-        if (!std::isfinite(res)) return mh_fail(ctx, MH_ERR_NUMERIC, "GMRES residual is not finite");
-        if (res <= abs_tol) {
-            ++k;
-            break;
-        }
-        const double rate = (res > 0 && res_prev > 0 && k + 1 > k_prev)
-                                ? std::pow(res / res_prev, 1.0 / (k + 1 - k_prev)) : 0.5;
-        int ahead = 1;
-        if (rate > 0 && rate < 0.999) ahead = (int)std::floor(std::log(abs_tol / res) / std::log(rate));
-        ahead = std::max(1, std::min(ahead, 8));
-        k_prev = k + 1;
-        res_prev = res;
-        next_check = k + 1 + ahead;
+// Waits until the counter in pinned memory has reached `value` (a kernel publishes it); returns at
+// once with an error if the stream has failed, or has run dry without publishing.
+static mh_status wait_progress(mh_ctx* ctx, const int* counter, int value) {
+    for (int spin = 0;; ++spin) {
+        if (__atomic_load_n(counter, __ATOMIC_ACQUIRE) - value >= 0) return MH_OK;
+        if (spin % 4096 != 4095) continue;
+        const cudaError_t e = cudaStreamQuery(ctx->stream);
+        if (e == cudaErrorNotReady) continue;
+        MH_CUDA(ctx, e);
+        if (__atomic_load_n(counter, __ATOMIC_ACQUIRE) - value >= 0) return MH_OK;
+        return mh_fail(ctx, MH_ERR_CUDA, "the solver's kernels ended without a result");
     }
-    *iters = k;
-    *resid = res;
-    return MH_OK;
 }
 
+// The interactive solver.  The decisions are the device's (gs): a sweep's steps are queued ahead of
+// what the host has seen, and a step queued past the end of the process returns at once.  The
+// host follows through pinned memory instead of a copy and a synchronisation per look (~10 us of
+// idle GPU each: a solve at 6144 nodes of 13 steps in two sweeps took 705 us with those looks).
 mh_status gmres_run(mh_ctx* ctx, mh_boundary* bd, const double* b, double* x, double tol, int max_iter,
                     mh_precision prec, mh_gmres_info* info, const double* r0) {
     prof_scope ps_all(ctx, "gmres");
@@ -2581,48 +2539,101 @@ mh_status gmres_run(mh_ctx* ctx, mh_boundary* bd, const double* b, double* x, do
     const bool mixed = prec == MH_PREC_MIXED;
     if (mixed) MH_TRY(ensure_fp32(ctx, bd));
     gmres_ws& ws = bd->ws;
+    cudaStream_t st = ctx->stream;
     const bool split = !bd->mfree && resid_ff(bd, mixed);
-    double bnorm = 0.0, rn = 0.0;
+    gmres_dev* gs = ws.gs.p;
+    gmres_k::progress* P = static_cast<gmres_k::progress*>(ws.prog);
+    // the counters run on from solve to solve (an earlier solve has nothing left that writes them)
+    const int steps0 = P->steps >> 1;
+    int begins = P->begins;
     mh_gmres_info inf{0, 0, 0.0, 0, 0.0};
     // binary64: one sweep to the tolerance, then the true residual.  Mixed: sweeps of the
     // binary32-operator process inside binary64 iterative refinement.
-    for (int sweep = 0;; ++sweep) {
+    bool supplied = r0 != nullptr, first = true;
+    for (int sweep = 0;;) {
         // binary64 residual of x; at the first sweep the caller's r0 (if given) stands in
         // for it, but convergence is only ever accepted on a residual computed here
-        bool computed = sweep > 0 || !r0;
-        if (computed) MH_TRY(bie_apply64_gated(ctx, bd, x, ws.w.p, nullptr, prec, split && sweep > 0));
-        MH_TRY(sweep_begin_read(ctx, ws,
-                                begin_of(ws, b, computed ? ws.w.p : nullptr, r0, n, max_iter + 2, mixed, sweep == 0),
-                                &rn, &bnorm));
-        if (sweep == 0) {
-            if (bnorm == 0.0) {
-                MH_CUDA(ctx, cudaMemsetAsync(x, 0, n * 8, ctx->stream));
-                MH_CUDA(ctx, cudaMemsetAsync(ws.r.p, 0, n * 8, ctx->stream));   // residual of x = 0
-                inf.converged = 1;
-                if (info) *info = inf;
-                return MH_OK;
+        if (!supplied) MH_TRY(bie_apply64_gated(ctx, bd, x, ws.w.p, nullptr, prec, split && sweep > 0));
+        gmres_k::begin_args a = begin_of(ws, b, supplied ? r0 : nullptr, x, n, max_iter + 2, mixed, tol, gs);
+        a.first = first;
+        a.recheck = supplied;
+        a.final_check = sweep >= (mixed ? 12 : 1) || inf.iterations >= max_iter;
+        a.prog = P;
+        a.seq = ++begins;
+        a.total0 = steps0;
+        MH_TRY(sweep_begin(ctx, ws, a));
+        const int left = max_iter - inf.iterations, base = steps0 + inf.iterations;
+        int queued = 0, seen = 0, seen_prev = 0;
+        double res_prev = 0.0;
+        // steps queued beyond the last one seen: two for the dense operator (a step past the end costs
+        // two empty launches), for the matrix-free one as many as the observed decay says are needed
+        // (with region timers none: a timed product is one that ran)
+        const bool careful = bd->mfree || ctx->profiling;
+        int ahead = careful ? 1 : 2;
+        bool begun = false, ended = a.final_check;
+        while (!ended || !begun) {
+            if (!begun && (__atomic_load_n(&P->begins, __ATOMIC_ACQUIRE) - begins >= 0 || ended || careful ||
+                           queued >= std::min(left, 2))) {
+                MH_TRY(wait_progress(ctx, &P->begins, begins));
+                begun = true;
+                res_prev = P->rn;
+                if (!P->started) break;
             }
-            if (!std::isfinite(rn)) return mh_fail(ctx, MH_ERR_NUMERIC, "GMRES residual is not finite");
-            inf.initial_rel_residual = rn / bnorm;
+            if (ended) continue;
+            if (queued < left && queued < seen + ahead) {
+                // w = A v_k
+                const double* vk = ws.V.p + (int64_t)queued * n;
+                if (bd->mfree) {
+                    MH_TRY(bie_apply_mfree(ctx, bd, vk, ws.w.p));
+                } else {
+                    prof_scope ps(ctx, mixed ? "bie_gemv32" : "bie_gemv64", 2.0 * n * n,
+                                  mixed ? 4.0 * n * n + 12.0 * n : 8.0 * n * n + 16.0 * n);
+                    if (mixed)
+                        gemv32(st, bd->op.A32.p, ws.v32.p, ws.w.p, n, &gs->skip);
+                    else
+                        gemv64(st, bd->op.A64.p, vk, ws.w.p, n, &gs->skip);
+                    MH_LAUNCHED(ctx);
+                }
+                ++queued;
+                MH_TRY(arnoldi_step(ctx, ws, n, queued, left + 1, mixed, gs, left, P));
+                continue;
+            }
+            MH_TRY(wait_progress(ctx, &P->steps, 2 * (base + seen + 1)));
+            const int word = __atomic_load_n(&P->steps, __ATOMIC_ACQUIRE);
+            seen = (word >> 1) - base;
+            ended = word & 1;
+            if (bd->mfree && !ended) {
+                const double target = tol * P->bn, res = P->res;
+                const double rate = res > 0 && res_prev > 0 ? std::pow(res / res_prev, 1.0 / (seen - seen_prev)) : 0.5;
+                ahead = 1;
+                if (rate > 0 && rate < 0.999) ahead = (int)std::floor(std::log(target / res) / std::log(rate));
+                ahead = std::max(1, std::min(ahead, 8));
+                res_prev = res;
+                seen_prev = seen;
+            }
         }
-        if (!computed && rn <= tol * bnorm) {
-            MH_TRY(bie_apply64_gated(ctx, bd, x, ws.w.p, nullptr, prec));
-            MH_TRY(sweep_begin_read(ctx, ws, begin_of(ws, b, ws.w.p, nullptr, n, max_iter + 2, mixed, false), &rn,
-                                    &bnorm));
+        if (first) {
+            if (P->bn != 0.0) inf.initial_rel_residual = P->rn / P->bn;
+            first = false;
         }
-        if (rn <= tol * bnorm || inf.iterations >= max_iter || sweep >= (mixed ? 12 : 1)) break;
-        int it;
-        double res;
-        // mixed: half the tolerance, so that the binary64 residual after the sweep lands below tol
-        // instead of just above it (which would cost another sweep and binary64 GEMV)
-        const double target = mixed ? std::max(0.5 * tol * bnorm, 1e-5 * rn) : tol * bnorm;
-        const int left = max_iter - inf.iterations;
-        MH_TRY(arnoldi_run(ctx, bd, rn, target, left, mixed, &it, &res));
-        MH_TRY(sweep_end(ctx, bd, left + 1, it, left, nullptr, x, split));
-        inf.iterations += it;
+        if (!std::isfinite(P->rn) || (P->started && !std::isfinite(P->res))) {
+            MH_CUDA(ctx, cudaStreamSynchronize(st));
+            return mh_fail(ctx, MH_ERR_NUMERIC, "GMRES residual is not finite");
+        }
+        if (!P->started) {
+            if (!P->done && supplied && P->rn <= tol * P->bn) {   // the caller's residual is within the tolerance: compute it
+                supplied = false;
+                continue;
+            }
+            break;   // accepted, or the last residual of the schedule
+        }
+        inf.iterations += seen;
         if (mixed) inf.refinements++;
+        MH_TRY(sweep_end(ctx, bd, left + 1, left, gs, x, split, true));
+        supplied = false;
+        ++sweep;
     }
-    inf.rel_residual = rn / bnorm;   // binary64 residual of the final iterate
+    inf.rel_residual = P->bn != 0.0 ? P->rn / P->bn : 0.0;   // binary64 residual of the final iterate
     inf.converged = inf.rel_residual <= tol;
     if (info) *info = inf;
     if (!inf.converged)
@@ -2643,10 +2654,14 @@ mh_status gmres_graph_ensure(mh_ctx* ctx, mh_boundary* bd, int max_iter) {
     MH_ALLOC(ctx, ws.cs, max_iter + 1);
     MH_ALLOC(ctx, ws.sn, max_iter + 1);
     MH_ALLOC(ctx, ws.g, max_iter + 2);
-    MH_ALLOC(ctx, ws.small, 8);
     MH_ALLOC(ctx, ws.w, n);
     MH_ALLOC(ctx, ws.r, n);
     MH_ALLOC(ctx, ws.v32, n);
+    if (!ws.gs.p) MH_ALLOC(ctx, ws.gs, 1);
+    if (!ws.prog) {
+        MH_CUDA(ctx, cudaMallocHost(&ws.prog, sizeof(gmres_k::progress)));
+        std::memset(ws.prog, 0, sizeof(gmres_k::progress));
+    }
     if (!ws.body_stream) MH_CUDA(ctx, cudaStreamCreateWithFlags(&ws.body_stream, cudaStreamNonBlocking));
     if (!ws.cluster) {
         MH_CUDA(ctx, cudaFuncSetAttribute(gmres_k::k_arnoldi, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2714,7 +2729,7 @@ static mh_status gmres_loop_node(mh_ctx* ctx, mh_boundary* bd, gmres_dev* gs, cu
     ctx->stream = bs;
     gemv32(bs, bd->op.A32.p, ws.v32.p, ws.w.p, n, nullptr);
     ctx->launches++;
-    const mh_status s = arnoldi_step(ctx, ws, n, 0, m, m + 1, true, gs, m, h, 1);
+    const mh_status s = arnoldi_step(ctx, ws, n, m, m + 1, true, gs, m, nullptr, h, 1);
     ctx->stream = st;
     cudaGraph_t out = nullptr;
     MH_CUDA(ctx, cudaStreamEndCapture(bs, &out));
@@ -2760,11 +2775,8 @@ mh_status gmres_run_graph(mh_ctx* ctx, mh_boundary* bd, const double* b, double*
             MH_CUDA(ctx, cudaStreamGetCaptureInfo(st, &cs, nullptr, &g, nullptr, nullptr, nullptr));
             MH_CUDA(ctx, cudaGraphConditionalHandleCreate(&h, g, 0, cudaGraphCondAssignDefault));
         }
-        gmres_k::begin_args a = begin_of(ws, b, supplied ? nullptr : ws.w.p, r0, n, m + 2, mixed, sw == 0);
-        a.x = x;
-        a.gs = gs;
-        a.tol = tol;
-        a.may_accept = !supplied;
+        gmres_k::begin_args a = begin_of(ws, b, supplied ? r0 : nullptr, x, n, m + 2, mixed, tol, gs);
+        a.first = sw == 0;
         a.final_check = sw == S;
         a.loop = h;
         a.loop_set = loop ? 1 : 0;
@@ -2779,10 +2791,10 @@ mh_status gmres_run_graph(mh_ctx* ctx, mh_boundary* bd, const double* b, double*
                 else
                     gemv64(st, bd->op.A64.p, ws.V.p + (int64_t)k * n, ws.w.p, n, &gs->skip);
                 MH_LAUNCHED(ctx);
-                MH_TRY(arnoldi_step(ctx, ws, n, k, k + 1, m + 1, mixed, gs, m));
+                MH_TRY(arnoldi_step(ctx, ws, n, k + 1, m + 1, mixed, gs, m));
             }
         }
-        MH_TRY(sweep_end(ctx, bd, m + 1, 0, m, gs, x, split));
+        MH_TRY(sweep_end(ctx, bd, m + 1, m, gs, x, split, !loop));
     }
     return MH_OK;
 }

@@ -47,36 +47,46 @@ __device__ __forceinline__ double tree_sum(double v, int m) {
 // Rows of a block's slice: a multiple of 32.
 __host__ __device__ inline int64_t gm_rows(int64_t n, int blocks) { return ((n + blocks - 1) / blocks + 31) / 32 * 32; }
 
+// What the interactive solver sees of a solve in progress: pinned host memory that the kernels
+// write (fields first, then the counter they are published by) and the host polls.
+struct progress {
+    double rn, bn, res;     // ||r||, ||b|| of the last sweep start; residual estimate of the last step
+    int begins;             // sweep starts so far ...
+    int started, done;      // ... and what the last one decided
+    int steps;              // 2 x Arnoldi steps so far (all sweeps and solves) + 1 if the last one ended its process
+};
+
 // Start of a sweep: r = b - ax (ax given) or r = r0 (r0 given, may alias r), its norm rn and, in
 // a first sweep, ||b||; then V_0 = r / rn (and its binary32 copy), g = (rn, 0, ...).
-// Without gs (interactive solver): scal[0] = rn, scal[1] = ||b|| for the host.
-// With gs (sync-free solver): accept (converged) when allowed and rn <= tol ||b||, else start an
-// Arnoldi process with the inner target max(tol ||b||, 1e-5 rn) in mixed precision (half the
+// Accept (converged) when allowed and rn <= tol ||b||, else start an Arnoldi process with the inner target max(tol ||b||, 1e-5 rn) in mixed precision (half the
 // tolerance: the binary64 residual after the sweep then lands below it instead of just above,
 // which would cost another sweep), tol ||b|| in binary64.  final_check: the last residual of the
-// schedule, recorded only.  ||b|| = 0 gives x = 0.  With loop_set, the condition of the sweep's
+// schedule, recorded only.  recheck: a supplied residual within the tolerance starts nothing (the
+// interactive solver then computes the residual).  ||b|| = 0 gives x = 0.  With loop_set, the condition of the sweep's
 // Arnoldi loop (a graph WHILE node, 0 by default at every launch) is set to "start".
 struct begin_args {
     const double *b, *ax, *r0;
-    double *r, *V0, *g, *x, *scal;
+    double *r, *V0, *g, *x;
     float* v32;
     int64_t n;
     int gsz;
     gmres_dev* gs;
     double tol;
-    int mixed, may_accept, final_check, first, loop_set;
+    int mixed, may_accept, final_check, recheck, first, loop_set;
     cudaGraphConditionalHandle loop;
+    progress* prog;
+    int seq, total0;   // (prog) the start's number, steps counted before this solve
 };
 
 __global__ void __launch_bounds__(GM_T) k_sweep_begin(begin_args a) {
     __shared__ double red[2][GM_T / 32], all[2][16], nrm[3];
     cg::cluster_group cl = cg::this_cluster();
     mh_dep_wait();
-    if (a.gs && a.gs->done) return;   // the same for every block: written after the last barrier only
+    if (!a.first && a.gs->done) return;   // the same for every block: written after the last barrier only
     cl.barrier_arrive();              // every block of the cluster runs before the first remote store
     const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const double bn_kept = a.gs && !a.first ? a.gs->bnorm : 0.0;
+    const double bn_kept = a.first ? 0.0 : a.gs->bnorm;
     const int64_t R = gm_rows(a.n, C), e0 = R * rank, e1 = min(a.n, e0 + R);
     double s = 0.0, sb = 0.0;
     for (int64_t e = e0 + threadIdx.x; e < e1; e += GM_T) {
@@ -108,20 +118,23 @@ __global__ void __launch_bounds__(GM_T) k_sweep_begin(begin_args a) {
     __syncthreads();
     const double rn = nrm[0], bn = a.first ? nrm[1] : bn_kept, inv = nrm[2];
     const bool lead = rank == 0 && threadIdx.x == 0;
-    bool start = rn > 0.0;
-    if (a.gs) {
-        if (bn == 0.0) {
-            for (int64_t e = e0 + threadIdx.x; e < e1; e += GM_T) a.x[e] = a.r[e] = 0.0;   // b = 0: x = 0, residual 0
-            if (lead) {
-                a.gs->bnorm = 0.0;
-                a.gs->done = a.gs->skip = a.gs->converged = 1;
-                a.gs->rel = 0.0;
-            }
-            return;
+    bool start = rn > 0.0, conv = false;
+    if (lead && a.first) {
+        a.gs->done = a.gs->converged = a.gs->sweeps = a.gs->k = 0;
+        a.gs->total = a.total0;
+    }
+    if (bn == 0.0) {
+        for (int64_t e = e0 + threadIdx.x; e < e1; e += GM_T) a.x[e] = a.r[e] = 0.0;   // b = 0: x = 0, residual 0
+        start = false;
+        if (lead) {
+            a.gs->bnorm = 0.0;
+            a.gs->done = a.gs->skip = a.gs->converged = 1;
+            a.gs->rel = 0.0;
         }
+    } else {
         const bool accept = a.may_accept || a.final_check;
-        const bool conv = accept && rn <= a.tol * bn;
-        start = start && !conv && !a.final_check;
+        conv = accept && rn <= a.tol * bn;
+        start = start && !conv && !a.final_check && !(a.recheck && rn <= a.tol * bn);
         if (lead) {
             if (a.first) {
                 a.gs->bnorm = bn;
@@ -140,9 +153,14 @@ __global__ void __launch_bounds__(GM_T) k_sweep_begin(begin_args a) {
             }
             if (a.loop_set) cudaGraphSetConditional(a.loop, start ? 1u : 0u);
         }
-    } else if (lead) {
-        a.scal[0] = rn;
-        a.scal[1] = bn;
+    }
+    if (lead && a.prog) {
+        a.prog->rn = rn;
+        a.prog->bn = bn;
+        a.prog->started = start;
+        a.prog->done = conv || bn == 0.0;
+        __threadfence_system();
+        *(volatile int*)&a.prog->begins = a.seq;
     }
     if (!start) return;
     for (int64_t e = e0 + threadIdx.x; e < e1; e += GM_T) {
@@ -156,21 +174,21 @@ __global__ void __launch_bounds__(GM_T) k_sweep_begin(begin_args a) {
 
 // One Arnoldi step after w = A v_k: classical Gram-Schmidt twice against V_0..V_k, v_{k+1} =
 // w / ||w|| (and its binary32 copy), column k of H rotated by the previous Givens rotations,
-// rotation k, g updated, |g_{k+1}| in small[0].
-// With gs, k and the end of the sweep's process live on the device (gs->k, gs->skip; the step
-// is skipped once it has ended), and with loop_set the condition of the graph loop is set to
+// rotation k, g updated.  k and the end of the sweep's process live on the device (gs->k,
+// gs->skip; the step is skipped once it has ended), and with loop_set the condition of the graph loop is set to
 // "not ended".  kcap >= k + 1 is the stride of the partial sums.
 struct step_args {
     const double* V;
     double* w;        // overwritten when the slices stay in global memory
     int64_t n;
-    int k, kcap, ldh;
+    int kcap, ldh;
     int shared_w;     // the slices of w fit in shared memory
-    double *H, *cs, *sn, *g, *small, *Vn;   // Vn = V (next column at (k + 1) n)
+    double *H, *cs, *sn, *g, *Vn;   // Vn = V (next column at (k + 1) n)
     float* v32;
     gmres_dev* gs;
     int m_max, loop_set;
     cudaGraphConditionalHandle loop;
+    progress* prog;
 };
 
 constexpr size_t GM_SMEM_MAX = 200 * 1024;
@@ -243,14 +261,14 @@ __device__ __forceinline__ void subtract(const double* __restrict__ V, int64_t n
 
 __global__ void __launch_bounds__(GM_T) k_arnoldi(step_args a) {
     mh_dep_wait();
-    if (a.gs && a.gs->skip) return;   // the same for every block: written after the last barrier only
+    if (a.gs->skip) return;   // the same for every block: written after the last barrier only
     extern __shared__ double sm[];
     __shared__ double npart[16], inv_s;
     cg::cluster_group cl = cg::this_cluster();
     cl.barrier_arrive();   // every block of the cluster runs before the first remote store
     const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int k = a.gs ? a.gs->k : a.k, k1 = k + 1, cap = a.kcap + 1;
+    const int k = a.gs->k, k1 = k + 1, cap = a.kcap + 1;
     const int64_t R = gm_rows(a.n, C), e0 = R * rank;
     const int cnt = (int)max((int64_t)0, min(a.n - e0, R));
     double* ws = a.shared_w ? sm + step_fixed(C, a.kcap) : a.w + e0;   // the block's slice of w
@@ -348,15 +366,19 @@ __global__ void __launch_bounds__(GM_T) k_arnoldi(step_args a) {
         a.sn[k] = sv;
         a.g[k + 1] = g1;
         a.g[k] = c * gk;
-        a.small[0] = fabs(g1);
         hc[k] = den;
         hc[k1] = 0.0;
-        if (a.gs) {
-            const bool end = fabs(g1) <= a.gs->target || k + 1 >= a.m_max || den == 0.0;
-            a.gs->k = k + 1;
-            a.gs->total += 1;
-            if (end) a.gs->skip = 1;
-            if (a.loop_set) cudaGraphSetConditional(a.loop, end ? 0u : 1u);
+        // an estimate that is not finite ends the process too
+        const bool end = !(fabs(g1) > a.gs->target) || k + 1 >= a.m_max || den == 0.0;
+        const int total = a.gs->total + 1;
+        a.gs->k = k + 1;
+        a.gs->total = total;
+        if (end) a.gs->skip = 1;
+        if (a.loop_set) cudaGraphSetConditional(a.loop, end ? 0u : 1u);
+        if (a.prog) {
+            a.prog->res = fabs(g1);
+            __threadfence_system();
+            *(volatile int*)&a.prog->steps = 2 * total + (end ? 1 : 0);
         }
     }
 }
@@ -369,13 +391,11 @@ __global__ void __launch_bounds__(GM_T) k_arnoldi(step_args a) {
 constexpr int GE_REG = 32;
 
 __global__ void __launch_bounds__(256) k_sweep_end(const double* __restrict__ V, const double* __restrict__ H, int ldh,
-                                                   const double* __restrict__ g, int k, const gmres_dev* gs, int64_t n,
+                                                   const double* __restrict__ g, const gmres_dev* gs, int64_t n,
                                                    double* x, float* __restrict__ xh, float* __restrict__ xl) {
     mh_dep_wait();
-    if (gs) {
-        if (gs->done) return;
-        k = gs->k;
-    }
+    if (gs->done) return;
+    const int k = gs->k;
     extern __shared__ double y[];   // [k]
     __shared__ double sR[GE_REG][GE_REG + 1];
     const int lane = threadIdx.x & 31;

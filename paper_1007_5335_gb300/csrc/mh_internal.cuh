@@ -241,7 +241,9 @@ struct gmres_dev {
 
 // GMRES workspace (kept by the boundary so that repeated solves allocate nothing).
 struct gmres_ws {
-    dbuf<double> V, H, cs, sn, g, small, w, r;
+    dbuf<double> V, H, cs, sn, g, w, r;
+    dbuf<gmres_dev> gs;                  // state of an interactive solve
+    void* prog = nullptr;                // what the host sees of it (pinned, gmres_k::progress)
     int cluster = 0;                     // thread blocks in the cluster of an Arnoldi step (16 or 8)
     dbuf<float> v32;                     // binary32 copy of the newest Krylov vector
     cudaStream_t body_stream = nullptr;  // captures the body of a graph loop (batch graphs)
@@ -253,6 +255,7 @@ struct gmres_ws {
     gmres_ws& operator=(const gmres_ws&) = delete;
     ~gmres_ws() {
         if (body_stream) cudaStreamDestroy(body_stream);
+        if (prog) cudaFreeHost(prog);
     }
 };
 
