@@ -43,77 +43,124 @@ struct mh_net {
     // training scratch
     dbuf<float> G, Mo, Vo, best, xb, yb, yh, act[3], dzd, dzw1, dzw2;
     dbuf<double> lpart;
+    dbuf<float> gpart;               // partial tiles of split training products, and their counters
+    dbuf<unsigned> gcnt;
     int64_t cap_rows = 0;
 };
 
 namespace {
 
-constexpr int GEMM_T = 64;   // tile edge
-constexpr int GEMM_K = 16;   // k slab
+constexpr int GEMM_T = 64;    // tile edge
+constexpr int GEMM_K = 16;    // k slab
+constexpr int GEMM_PARTS = 304;   // partial tiles of a split product (two blocks per SM)
 
 enum { EPI_NONE = 0, EPI_BIAS = 1, EPI_BIAS_TANH = 2, EPI_TANH_BACK = 3 };
 
 // C[i][j] = epi(sum_k A(i,k) B(k,j)); A(i,k) = A[i sam + k sak], B(k,j) = B[k sbk + j sbn].
 // EPI_BIAS: + bias[j]; EPI_BIAS_TANH: tanh(. + bias[j]); EPI_TANH_BACK: . * (1 - aux[i][j]^2).
+// The next slab is loaded into registers while the current one is multiplied (double-buffered
+// shared memory, one barrier a slab).  gridDim.z > 1 splits k between blocks: each writes its
+// partial tile, the last block of a tile to finish (counted per tile, reset by that block) adds
+// them in k order and applies the epilogue.  A minibatch of 64 has 4 tiles in most of its products
+// and chains of up to 192 slabs, so 4 of 152 SMs worked through ~2 us a slab: loss and gradient at
+// d = 3072, w = 256 took 788 us unsplit.
 template <typename T, int EPI>
 __global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, const T* __restrict__ A, int64_t sam, int64_t sak,
                                               const T* __restrict__ B, int64_t sbk, int64_t sbn, T* __restrict__ C,
-                                              int64_t ldc, const T* __restrict__ bias, const T* __restrict__ aux) {
-    __shared__ T As[GEMM_K][GEMM_T + 1];
-    __shared__ T Bs[GEMM_K][GEMM_T + 1];
+                                              int64_t ldc, const T* __restrict__ bias, const T* __restrict__ aux,
+                                              T* part, unsigned* cnt) {
+    mh_dep_wait();
+    __shared__ __align__(16) T As[2][GEMM_K][GEMM_T + 4];
+    __shared__ __align__(16) T Bs[2][GEMM_K][GEMM_T + 4];
+    __shared__ int last;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int i0 = blockIdx.y * GEMM_T, j0 = blockIdx.x * GEMM_T;
-    T acc[4][4];
+    const int S = gridDim.z, slabs = (K + GEMM_K - 1) / GEMM_K;
+    const int s0 = (int)((int64_t)slabs * blockIdx.z / S), s1 = (int)((int64_t)slabs * (blockIdx.z + 1) / S);
+    const bool ka = sak == 1, nb = sbn == 1;
+    T ra[4], rb[4], acc[4][4];
 #pragma unroll
     for (int r = 0; r < 4; ++r)
 #pragma unroll
         for (int c = 0; c < 4; ++c) acc[r][c] = T(0);
-    for (int k0 = 0; k0 < K; k0 += GEMM_K) {
+    auto load = [&](int slab) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int e = tid + 256 * q;
-            int ii, kk;
-            if (sak == 1) {
-                kk = e & 15;
-                ii = e >> 4;
-            } else {
-                ii = e & 63;
-                kk = e >> 6;
-            }
-            int gi = i0 + ii, gk = k0 + kk;
-            As[kk][ii] = (gi < M && gk < K) ? A[(int64_t)gi * sam + (int64_t)gk * sak] : T(0);
-            int jj;
-            if (sbn == 1) {
-                jj = e & 63;
-                kk = e >> 6;
-            } else {
-                kk = e & 15;
-                jj = e >> 4;
-            }
-            const int gj = j0 + jj;
-            gk = k0 + kk;
-            Bs[kk][jj] = (gj < N && gk < K) ? B[(int64_t)gk * sbk + (int64_t)gj * sbn] : T(0);
+            const int ii = ka ? e >> 4 : e & 63, ki = slab * GEMM_K + (ka ? e & 15 : e >> 6);
+            ra[q] = (i0 + ii < M && ki < K) ? A[(int64_t)(i0 + ii) * sam + (int64_t)ki * sak] : T(0);
+            const int jj = nb ? e & 63 : e >> 4, kj = slab * GEMM_K + (nb ? e >> 6 : e & 15);
+            rb[q] = (j0 + jj < N && kj < K) ? B[(int64_t)kj * sbk + (int64_t)(j0 + jj) * sbn] : T(0);
         }
-        __syncthreads();
+    };
+    auto store = [&](int buf) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int e = tid + 256 * q;
+            if (ka)
+                As[buf][e & 15][e >> 4] = ra[q];
+            else
+                As[buf][e >> 6][e & 63] = ra[q];
+            if (nb)
+                Bs[buf][e >> 6][e & 63] = rb[q];
+            else
+                Bs[buf][e & 15][e >> 4] = rb[q];
+        }
+    };
+    if (s0 < s1) {
+        load(s0);
+        store(0);
+    }
+    __syncthreads();
+    for (int s = s0; s < s1; ++s) {
+        const int buf = (s - s0) & 1;
+        if (s + 1 < s1) load(s + 1);
 #pragma unroll
         for (int kk = 0; kk < GEMM_K; ++kk) {
             T a[4], b[4];
 #pragma unroll
-            for (int r = 0; r < 4; ++r) a[r] = As[kk][ty + 16 * r];
+            for (int r = 0; r < 4; ++r) a[r] = As[buf][kk][4 * ty + r];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) b[c] = Bs[kk][tx + 16 * c];
+            for (int c = 0; c < 4; ++c) b[c] = Bs[buf][kk][4 * tx + c];
 #pragma unroll
             for (int r = 0; r < 4; ++r)
 #pragma unroll
                 for (int c = 0; c < 4; ++c) acc[r][c] = fma(a[r], b[c], acc[r][c]);
         }
+        if (s + 1 < s1) store(buf ^ 1);
         __syncthreads();
+    }
+    if (S > 1) {
+        const int tile = blockIdx.y * gridDim.x + blockIdx.x, tiles = gridDim.x * gridDim.y;
+        T* mine = part + ((int64_t)blockIdx.z * tiles + tile) * (GEMM_T * GEMM_T) + tid;
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) mine[256 * (4 * r + c)] = acc[r][c];
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) last = atomicAdd(cnt + tile, 1u) == (unsigned)(S - 1);
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        if (tid == 0) cnt[tile] = 0u;
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[r][c] = T(0);
+        for (int z = 0; z < S; ++z) {
+            const T* p = part + ((int64_t)z * tiles + tile) * (GEMM_T * GEMM_T) + tid;
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) acc[r][c] += __ldcg(p + 256 * (4 * r + c));
+        }
     }
 #pragma unroll
     for (int r = 0; r < 4; ++r)
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-            const int i = i0 + ty + 16 * r, j = j0 + tx + 16 * c;
+            const int i = i0 + 4 * ty + r, j = j0 + 4 * tx + c;
             if (i >= M || j >= N) continue;
             T v = acc[r][c];
             if (EPI == EPI_BIAS || EPI == EPI_BIAS_TANH) v += bias[j];
@@ -126,11 +173,19 @@ __global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, const T* __re
         }
 }
 
+// part, cnt (nullable): workspace of a split product (GEMM_PARTS tiles); k is split while the
+// tiles leave SMs without a block, down to two slabs a block.
 template <typename T, int EPI>
 void gemm(cudaStream_t st, int M, int N, int K, const T* A, int64_t sam, int64_t sak, const T* B, int64_t sbk,
-          int64_t sbn, T* C, int64_t ldc, const T* bias = nullptr, const T* aux = nullptr) {
+          int64_t sbn, T* C, int64_t ldc, const T* bias = nullptr, const T* aux = nullptr, T* part = nullptr,
+          unsigned* cnt = nullptr) {
     dim3 grid((unsigned)((N + GEMM_T - 1) / GEMM_T), (unsigned)((M + GEMM_T - 1) / GEMM_T));
-    k_gemm<T, EPI><<<grid, 256, 0, st>>>(M, N, K, A, sam, sak, B, sbk, sbn, C, ldc, bias, aux);
+    const int64_t tiles = (int64_t)grid.x * grid.y;
+    const int slabs = (K + GEMM_K - 1) / GEMM_K;
+    if (part && tiles <= GEMM_PARTS / 2)
+        grid.z = (unsigned)std::max<int64_t>(1, std::min<int64_t>(GEMM_PARTS / tiles, slabs / 2));
+    (void)mh_launch_dep(st, k_gemm<T, EPI>, grid, dim3(256), 0, M, N, K, A, sam, sak, B, sbk, sbn, C, ldc, bias, aux,
+                        part, cnt);
 }
 
 __device__ __forceinline__ double warp_sum_d(double v) {
@@ -431,6 +486,7 @@ __global__ void k_gather_rows(const float* __restrict__ X, const int32_t* __rest
 // dz = (yh - t) * inv; per-block partial sums of (yh - t)^2 (binary64) into part.
 __global__ void k_loss_dz(const float* __restrict__ yh, const float* __restrict__ t, int64_t n, float inv,
                           float* __restrict__ dz, double* __restrict__ part) {
+    mh_dep_wait();
     double s = 0.0;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
         const float df = yh[e] - t[e];
@@ -442,17 +498,28 @@ __global__ void k_loss_dz(const float* __restrict__ yh, const float* __restrict_
 }
 
 __global__ void k_sum_parts(const double* __restrict__ part, int n, double scale, double* out) {
+    mh_dep_wait();
     double s = 0.0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) s += part[i];
     s = block_sum_d(s);
     if (threadIdx.x == 0) out[0] = s * scale;
 }
 
-__global__ void k_colsum(const float* __restrict__ z, int64_t rows, int64_t cols, float* __restrict__ out) {
-    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (j >= cols) return;
+// out[j] = sum_i z[i][j] in binary64: 32 columns x 8 row shares per block, the shares added in order
+// (a thread per column took 15 us at 64 rows: a chain of binary64 additions).
+__global__ void __launch_bounds__(256) k_colsum(const float* __restrict__ z, int64_t rows, int64_t cols,
+                                                float* __restrict__ out) {
+    mh_dep_wait();
+    __shared__ double sh[8][33];
+    const int c = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const int64_t j = blockIdx.x * (int64_t)32 + c;
     double s = 0.0;
-    for (int64_t i = 0; i < rows; ++i) s += z[i * cols + j];
+    if (j < cols)
+        for (int64_t i = g; i < rows; i += 8) s += z[i * cols + j];
+    sh[g][c] = s;
+    __syncthreads();
+    if (g != 0 || j >= cols) return;
+    for (int q = 1; q < 8; ++q) s += sh[q][c];
     out[j] = (float)s;
 }
 
@@ -628,6 +695,11 @@ mh_status check_net(mh_ctx* ctx, const mh_net* net) {
 }
 
 mh_status ensure_rows(mh_ctx* ctx, mh_net* net, int64_t rows) {
+    if (!net->gcnt.p) {
+        MH_ALLOC(ctx, net->gpart, (int64_t)GEMM_PARTS * GEMM_T * GEMM_T);
+        MH_ALLOC(ctx, net->gcnt, GEMM_PARTS);
+        MH_CUDA(ctx, cudaMemsetAsync(net->gcnt.p, 0, GEMM_PARTS * sizeof(unsigned), ctx->stream));
+    }
     if (rows <= net->cap_rows) return MH_OK;
     MH_ALLOC(ctx, net->xb, rows * net->d);
     MH_ALLOC(ctx, net->yb, rows * net->d);
@@ -650,12 +722,13 @@ mh_status train_forward(mh_ctx* ctx, mh_net* net, int64_t rows) {
     int64_t ld_in = d;
     for (int l = 0; l < 3; ++l) {
         gemm<float, EPI_BIAS_TANH>(st, (int)rows, w, net->lin[l], in, ld_in, 1, P + net->oW[l], 1, net->lin[l],
-                                   net->act[l].p, w, P + net->ob[l]);
+                                   net->act[l].p, w, P + net->ob[l], (const float*)nullptr, net->gpart.p, net->gcnt.p);
         MH_LAUNCHED(ctx);
         in = net->act[l].p;
         ld_in = w;
     }
-    gemm<float, EPI_BIAS>(st, (int)rows, (int)d, w, in, w, 1, P + net->oW[3], 1, w, net->yh.p, d, P + net->ob[3]);
+    gemm<float, EPI_BIAS>(st, (int)rows, (int)d, w, in, w, 1, P + net->oW[3], 1, w, net->yh.p, d, P + net->ob[3],
+                          (const float*)nullptr, net->gpart.p, net->gcnt.p);
     MH_LAUNCHED(ctx);
     return MH_OK;
 }
@@ -665,9 +738,10 @@ mh_status train_loss(mh_ctx* ctx, mh_net* net, int64_t rows, float* dz, double* 
     const int64_t n = rows * net->d;
     const int nb = ew_grid(n);
     if ((int64_t)net->lpart.n < nb) MH_ALLOC(ctx, net->lpart, 152 * 8);
-    k_loss_dz<<<nb, 256, 0, ctx->stream>>>(net->yh.p, net->yb.p, n, (float)(1.0 / (double)n), dz, net->lpart.p);
+    (void)mh_launch_dep(ctx->stream, k_loss_dz, dim3(nb), dim3(256), 0, net->yh.p, net->yb.p, n,
+                        (float)(1.0 / (double)n), dz, net->lpart.p);
     MH_LAUNCHED(ctx);
-    k_sum_parts<<<1, 1024, 0, ctx->stream>>>(net->lpart.p, nb, 0.5 / (double)n, out);
+    (void)mh_launch_dep(ctx->stream, k_sum_parts, dim3(1), dim3(1024), 0, net->lpart.p, nb, 0.5 / (double)n, out);
     MH_LAUNCHED(ctx);
     return MH_OK;
 }
@@ -680,25 +754,28 @@ mh_status train_backward(mh_ctx* ctx, mh_net* net, int64_t rows, float* g) {
     const int64_t d = net->d;
     const int R = (int)rows;
     // layer 4
-    gemm<float, EPI_NONE>(st, (int)d, w, R, net->dzd.p, 1, d, net->act[2].p, w, 1, g + net->oW[3], w);
+    gemm<float, EPI_NONE>(st, (int)d, w, R, net->dzd.p, 1, d, net->act[2].p, w, 1, g + net->oW[3], w,
+                          (const float*)nullptr, (const float*)nullptr, net->gpart.p, net->gcnt.p);
     MH_LAUNCHED(ctx);
-    k_colsum<<<mh_grid(d, 256), 256, 0, st>>>(net->dzd.p, rows, d, g + net->ob[3]);
+    (void)mh_launch_dep(st, k_colsum, dim3(mh_grid(d, 32)), dim3(256), 0, net->dzd.p, rows, d, g + net->ob[3]);
     MH_LAUNCHED(ctx);
-    gemm<float, EPI_TANH_BACK>(st, R, w, (int)d, net->dzd.p, d, 1, P + net->oW[3], w, 1, net->dzw1.p, w, nullptr,
-                               net->act[2].p);
+    gemm<float, EPI_TANH_BACK>(st, R, w, (int)d, net->dzd.p, d, 1, P + net->oW[3], w, 1, net->dzw1.p, w,
+                               (const float*)nullptr, (const float*)net->act[2].p, net->gpart.p, net->gcnt.p);
     MH_LAUNCHED(ctx);
     float* dz = net->dzw1.p;
     float* dn = net->dzw2.p;
     for (int l = 2; l >= 0; --l) {
         const float* a_in = l > 0 ? net->act[l - 1].p : net->xb.p;
         const int64_t ld_in = l > 0 ? w : d;
-        gemm<float, EPI_NONE>(st, w, net->lin[l], R, dz, 1, w, a_in, ld_in, 1, g + net->oW[l], net->lin[l]);
+        gemm<float, EPI_NONE>(st, w, net->lin[l], R, dz, 1, w, a_in, ld_in, 1, g + net->oW[l], net->lin[l],
+                              (const float*)nullptr, (const float*)nullptr, net->gpart.p, net->gcnt.p);
         MH_LAUNCHED(ctx);
-        k_colsum<<<mh_grid(w, 256), 256, 0, st>>>(dz, rows, w, g + net->ob[l]);
+        (void)mh_launch_dep(st, k_colsum, dim3(mh_grid(w, 32)), dim3(256), 0, dz, rows, (int64_t)w, g + net->ob[l]);
         MH_LAUNCHED(ctx);
         if (l > 0) {
-            gemm<float, EPI_TANH_BACK>(st, R, w, w, dz, w, 1, P + net->oW[l], w, 1, dn, w, nullptr,
-                                       net->act[l - 1].p);
+            gemm<float, EPI_TANH_BACK>(st, R, w, w, dz, w, 1, P + net->oW[l], w, 1, dn, w,
+                                       (const float*)nullptr, (const float*)net->act[l - 1].p, net->gpart.p,
+                                       net->gcnt.p);
             MH_LAUNCHED(ctx);
             std::swap(dz, dn);
         }
