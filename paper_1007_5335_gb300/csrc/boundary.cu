@@ -19,6 +19,7 @@ namespace {
 
 constexpr int UPSAMPLE = 16;        // fine grid for targets within 10 h_s of a curve
 constexpr int FINE_TG = 4;          // auxiliary targets per block of the binary32 upsampled rule
+constexpr int64_t DLP_KEEP = 1 << 16;   // largest target set whose buffers a boundary keeps (some 50 MB)
 constexpr double NEAR_NODE = 12.0;  // project on the curve when the nearest node is within 12 h*
 constexpr double NEAR_FINE = 10.0;  // d < 10 h_s: upsampled rule
 constexpr double NEAR_LINE = 0.25;  // d < h_s/4: interpolation along the normal
@@ -156,15 +157,22 @@ __global__ void k_fine_geometry(const double* __restrict__ coef, const int32_t* 
     o[5] = 2.0 * MH_PI / NF;
 }
 
-// Warp-cooperative evaluation of a curve (position, y', y'') at an arbitrary parameter t.
+// Warp-cooperative evaluation of a curve (position, y', y'') at an arbitrary parameter t.  Lane l
+// takes the modes l, l + 32, ...: one sincos of its first angle and one of the rotation by 32 t, the
+// others by multiplication (a binary64 sincos per mode costs ~25 times that; its argument m t
+// carries the same rounding, m t eps, as the product of rotations).
 __device__ void curve_eval_warp(const double* c, int N, double t, double out[6]) {
     const int lane = threadIdx.x & 31;
     double x = 0, dx = 0, ddx = 0, y = 0, dy = 0, ddy = 0;
+    double s, co, rs, rc;
+    sincos(lane * t, &s, &co);
+    sincos(32.0 * t, &rs, &rc);
     for (int m = lane; m <= N / 2; m += 32) {
-        double s, co;
-        sincos(m * t, &s, &co);
         mode_acc(m, N, c[4 * m], c[4 * m + 1], s, co, x, dx, ddx);
         mode_acc(m, N, c[4 * m + 2], c[4 * m + 3], s, co, y, dy, ddy);
+        const double cn = fma(co, rc, -s * rs);
+        s = fma(s, rc, co * rs);
+        co = cn;
     }
     out[0] = warp_sum(x);
     out[1] = warp_sum(y);
@@ -1163,11 +1171,30 @@ __global__ void k_scale_into(const double* __restrict__ r, const double* __restr
 
 // ---------------- classification of off-surface targets ----------------
 
+// Binary32 copy of the nodes for the classification: position relative to the origin (the mean node)
+// and normal times |y'| h.
+__global__ void k_cls32(const double* __restrict__ geo, const int32_t* __restrict__ curve_of,
+                        const int32_t* __restrict__ nn, int64_t n, double ox, double oy, float4* __restrict__ out) {
+    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    const double* g = geo + 8 * j;
+    const double h = 2.0 * MH_PI / nn[curve_of[j]];
+    out[j] = make_float4((float)(g[0] - ox), (float)(g[1] - oy), (float)(g[3] * h), (float)(-g[2] * h));
+}
+
 // One warp per target.  For every curve: nearest node (smallest index on ties); if it is
 // closer than 12 h*, Newton projection on the trigonometric interpolant giving the foot
 // t*, distance d and side; otherwise the side from the trapezoid Laplace double layer of
 // unit density (1 inside the outer curve, -1 inside a hole).
+// The scans over all nodes run in binary32 (the binary64 pipe has 1/64 of that rate): one finds
+// the smallest distance, a second one re-measures in binary64 every node whose binary32 distance
+// is within its rounding of it, so the nearest node is the binary64 one; the double layer, near
+// 0 or +-1 at these distances, is formed in binary64 only when it is not near either.  Newton's
+// iteration stops with a step below 1e-9 that is also 1000 times smaller than the one before
+// (quadratic convergence: the next one is below the rounding of t).  2000 targets, 6 x 1024 nodes: 1303 us with binary64 scans and 30
+// steps of a sincos per mode.
 __global__ void k_classify(const double* __restrict__ pts, int64_t npts, const double* __restrict__ geo,
+                           const float4* __restrict__ geo32, double ox, double oy, float extent,
                            const double* __restrict__ coef, const int32_t* __restrict__ nn,
                            const int32_t* __restrict__ off, int ncurves, int32_t* region, uint32_t* fine,
                            int32_t* line_curve, double* line_data) {
@@ -1175,6 +1202,9 @@ __global__ void k_classify(const double* __restrict__ pts, int64_t npts, const d
     const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     if (t >= npts) return;
     const double px = pts[2 * t], py = pts[2 * t + 1];
+    const float fx = (float)(px - ox), fy = (float)(py - oy);
+    // rounding of a binary32 distance: coordinates, their differences, the square root
+    const float slack = 1e-6f * fmaxf(extent, fmaxf(fabsf(fx), fabsf(fy)));
     int reg = -1;
     uint32_t mask = 0;
     int lc = -1;
@@ -1184,9 +1214,27 @@ __global__ void k_classify(const double* __restrict__ pts, int64_t npts, const d
         const int N = nn[k];
         const int o = off[k];
         const double h = 2.0 * MH_PI / N;
+        float d2min = 3e38f, wind = 0.f;
+        for (int i = lane; i < N; i += 32) {
+            const float4 g = geo32[o + i];
+            const float dx = g.x - fx, dy = g.y - fy;
+            const float d2 = fmaf(dx, dx, dy * dy);
+            d2min = fminf(d2min, d2);
+            wind += __fdividef(fmaf(dx, g.z, dy * g.w), fmaxf(d2, 1e-30f));
+        }
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1) {
+            d2min = fminf(d2min, __shfl_xor_sync(0xffffffffu, d2min, s));
+            wind += __shfl_xor_sync(0xffffffffu, wind, s);
+        }
+        wind = __shfl_sync(0xffffffffu, wind, 0) * (float)(1.0 / (2.0 * MH_PI));
+        const float reach = sqrtf(d2min) * (1.f + 4e-6f) + slack, lim = reach * reach;
         double best = 1e300;
         int bi = 0x7fffffff;
         for (int i = lane; i < N; i += 32) {
+            const float4 q = geo32[o + i];
+            const float ex = q.x - fx, ey = q.y - fy;
+            if (fmaf(ex, ex, ey * ey) > lim) continue;   // a NaN takes the binary64 path too
             const double* g = geo + 8 * (int64_t)(o + i);
             double dx = g[0] - px, dy = g[1] - py;
             double d2 = dx * dx + dy * dy;
@@ -1204,12 +1252,13 @@ __global__ void k_classify(const double* __restrict__ pts, int64_t npts, const d
                 bi = oi;
             }
         }
-        const double hstar = geo[8 * (int64_t)(o + bi) + 6] * h;
         bool outside;
-        if (sqrt(best) < NEAR_NODE * hstar) {
+        if (bi >= N) {   // no finite distance (a target that is not a number): no node is nearest
+            outside = true;
+        } else if (sqrt(best) < NEAR_NODE * (geo[8 * (int64_t)(o + bi) + 6] * h)) {
             const double* c = coef + 4 * coef_base(off, k);
             double tt = bi * h;
-            double v[6];
+            double v[6], before = 1.0;
             for (int it = 0; it < 30; ++it) {
                 curve_eval_warp(c, N, tt, v);
                 double rx = v[0] - px, ry = v[1] - py;
@@ -1218,7 +1267,9 @@ __global__ void k_classify(const double* __restrict__ pts, int64_t npts, const d
                 if (hs <= 0) hs = v[2] * v[2] + v[3] * v[3];
                 double dt = gr / hs;
                 tt -= dt;
-                if (fabs(dt) < 1e-15) break;
+                const double step = fabs(dt);
+                if (step < 1e-15 || (step < 1e-9 && step < 1e-3 * before)) break;
+                before = step;
             }
             tt = fmod(tt, 2.0 * MH_PI);
             if (tt < 0) tt += 2.0 * MH_PI;
@@ -1239,14 +1290,18 @@ __global__ void k_classify(const double* __restrict__ pts, int64_t npts, const d
                 ld[2] = hs;
             }
         } else {
-            double acc = 0.0;
-            for (int i = lane; i < N; i += 32) {
-                const double* g = geo + 8 * (int64_t)(o + i);
-                double dx = g[0] - px, dy = g[1] - py;
-                double sp = g[6];
-                acc += (dx * g[3] / sp - dy * g[2] / sp) / (dx * dx + dy * dy) * sp * h;
+            double acc = wind;
+            const float a = fabsf(wind);
+            if (!(a < 0.1f || fabsf(a - 1.f) < 0.1f)) {
+                acc = 0.0;
+                for (int i = lane; i < N; i += 32) {
+                    const double* g = geo + 8 * (int64_t)(o + i);
+                    double dx = g[0] - px, dy = g[1] - py;
+                    double sp = g[6];
+                    acc += (dx * g[3] / sp - dy * g[2] / sp) / (dx * dx + dy * dy) * sp * h;
+                }
+                acc = warp_sum(acc) / (2.0 * MH_PI);
             }
-            acc = warp_sum(acc) / (2.0 * MH_PI);
             outside = (k == 0) ? (acc < 0.5) : (acc < -0.5);
         }
         if (outside && reg == -1) reg = k;
@@ -1450,100 +1505,73 @@ __global__ void __launch_bounds__(256) k_fine_density_s(const T2* __restrict__ c
     wf[g] = (T)((double)acc * fg[6 * g + 4] * fg[6 * g + 5]);
 }
 
-// The same fine-grid density by inverse FFT, for curves of N = 2^L <= FFT_MAX nodes: block
-// (s, k) forms p(t_{16 j + s}) = Re sum_{m <= N/2} C_m^{(s)} e^{2 pi i m j / N} for every j of
-// curve k by one radix-2 decimation-in-time transform of length N in shared memory (input in
-// bit-reversed order, twiddles e^{2 pi i r / N} from the curve's binary32 table staged beside
-// it), then multiplies by |y'| h_f as k_fine_density_s does.  N log2 N / 2 butterflies per
-// sub-offset instead of N (N/2 + 1) products; rounding ~log2 N units of binary32 against ~sqrt N
-// for the direct sum.
-constexpr int FFT_MAX = 2048;
-
-__global__ void __launch_bounds__(256) k_fine_density_fft(const float2* __restrict__ cp, const float2* __restrict__ tw,
-                                                          const double* __restrict__ fg, const int32_t* __restrict__ nn,
-                                                          const int32_t* __restrict__ off,
-                                                          const int64_t* __restrict__ foff, float* __restrict__ wf) {
-    extern __shared__ float2 fz[];   // [N] values, then [N] twiddles
-    const int s = blockIdx.x, k = blockIdx.y;
-    const int N = nn[k];
-    float2* z = fz;
-    float2* w = fz + N;
-    const int L = __ffs(N) - 1;   // N = 2^L
-    const float2* c = cp + coef_base(off, k) * UPSAMPLE + s;
-    for (int m = threadIdx.x; m < N; m += blockDim.x) {
-        z[__brev((unsigned)m) >> (32 - L)] = m <= N / 2 ? c[(int64_t)m * UPSAMPLE] : make_float2(0.f, 0.f);
-        w[m] = tw[off[k] + m];
-    }
-    __syncthreads();
-    for (int len = 2; len <= N; len <<= 1) {
-        const int half = len >> 1, step = N / len;
-        for (int b = threadIdx.x; b < N / 2; b += blockDim.x) {
-            const int pos = b & (half - 1), i = (b - pos) * 2 + pos;   // (group b / half) * len + pos
-            const float2 t = w[pos * step];
-            const float2 u = z[i], v = z[i + half];
-            const float2 vt = make_float2(v.x * t.x - v.y * t.y, v.x * t.y + v.y * t.x);
-            z[i] = make_float2(u.x + vt.x, u.y + vt.y);
-            z[i + half] = make_float2(u.x - vt.x, u.y - vt.y);
-        }
-        __syncthreads();
-    }
-    for (int j = threadIdx.x; j < N; j += blockDim.x) {
-        const int64_t g = foff[k] + (int64_t)UPSAMPLE * j + s;
-        wf[g] = (float)((double)z[j].x * fg[6 * g + 4] * fg[6 * g + 5]);
-    }
-}
+constexpr int FFT_MAX = 2048;   // longest curve of the transforms below
 
 // The density times |y'| h_f on the 16x grid straight from the density, for curves of
-// N = 2^L <= FFT_MAX nodes, in one launch: block (s, k) takes curve k's density to binary32,
+// N = 2^L <= FFT_MAX nodes, in one launch: block (s, k) takes curve k's density to T,
 // forms c_m = (1/N) sum_j sigma_j e^{-2 pi i m j / N} by a radix-2 forward FFT in shared memory
 // (the conjugate twiddles; each of the UPSAMPLE blocks of a curve repeats this small transform),
 // multiplies in its own sub-offset's phases, C_m^{(s)} = w_m c_m e^{2 pi i m s / (16 N)} (m <= N/2;
-// w_0 = 1, w_m = 2, the Nyquist term real with w = 1; the phases by sincospif), and finishes as
-// k_fine_density_fft does (the inverse transform, the real part times |y'| h_f into wf and its
-// binary64 image wf64).
-__global__ void __launch_bounds__(256) k_fine_weights_fft(const double* __restrict__ sigma, const float2* __restrict__ tw,
+// w_0 = 1, w_m = 2, the Nyquist term real with w = 1), and finishes with the inverse transform, the
+// real part times |y'| h_f into wf64 and, when given, wf (binary32).  Rounding ~log2 N units against ~sqrt N
+// for the direct sums.  Binary64: three launches of direct sums (spectrum, phases, synthesis over
+// N/2 modes at every fine node) took 256 us for 6 x 1024 nodes.
+__device__ __forceinline__ void sincospi_t(float x, float* s, float* c) { sincospif(x, s, c); }
+__device__ __forceinline__ void sincospi_t(double x, double* s, double* c) { sincospi(x, s, c); }
+
+template <typename T, typename T2>
+__global__ void __launch_bounds__(256) k_fine_weights_fft(const double* __restrict__ sigma, const T2* __restrict__ tw,
                                                           const double* __restrict__ fg, const int32_t* __restrict__ nn,
                                                           const int32_t* __restrict__ off,
                                                           const int64_t* __restrict__ foff, float* __restrict__ wf,
                                                           double* __restrict__ wf64) {
-    extern __shared__ float2 fz[];   // [N] values, then [N] twiddles
+    extern __shared__ __align__(16) unsigned char fft_smem[];   // [N] values, then [N] twiddles
     constexpr int PER = FFT_MAX / 256;   // values per thread when the spectrum is reordered
     const int s = blockIdx.x, k = blockIdx.y;
     const int N = nn[k];
-    float2* z = fz;
-    float2* w = fz + N;
+    T2* z = reinterpret_cast<T2*>(fft_smem);
+    T2* w = z + N;
     const int L = __ffs(N) - 1;   // N = 2^L
     for (int m = threadIdx.x; m < N; m += blockDim.x) {
-        z[__brev((unsigned)m) >> (32 - L)] = make_float2((float)sigma[off[k] + m], 0.f);
+        T2 v;
+        v.x = (T)sigma[off[k] + m];
+        v.y = T(0);
+        z[__brev((unsigned)m) >> (32 - L)] = v;
         w[m] = tw[off[k] + m];
     }
     __syncthreads();
-    // forward transform (decimation in time, conjugate twiddles): z[m] = N c_m
-    for (int len = 2; len <= N; len <<= 1) {
-        const int half = len >> 1, step = N / len;
-        for (int b = threadIdx.x; b < N / 2; b += blockDim.x) {
-            const int pos = b & (half - 1), i = (b - pos) * 2 + pos;
-            const float2 t = w[pos * step];
-            const float2 u = z[i], v = z[i + half];
-            const float2 vt = make_float2(v.x * t.x + v.y * t.y, v.y * t.x - v.x * t.y);
-            z[i] = make_float2(u.x + vt.x, u.y + vt.y);
-            z[i + half] = make_float2(u.x - vt.x, u.y - vt.y);
+    // decimation in time; sg = -1: conjugate twiddles (forward, z[m] = N c_m), +1: inverse
+    auto transform = [&](T sg) {
+        for (int len = 2; len <= N; len <<= 1) {
+            const int half = len >> 1, step = N / len;
+            for (int b = threadIdx.x; b < N / 2; b += blockDim.x) {
+                const int pos = b & (half - 1), i = (b - pos) * 2 + pos;
+                const T2 t = w[pos * step], u = z[i], v = z[i + half];
+                const T ti = sg * t.y;
+                const T vx = fma(v.x, t.x, -v.y * ti), vy = fma(v.x, ti, v.y * t.x);
+                z[i].x = u.x + vx;
+                z[i].y = u.y + vy;
+                z[i + half].x = u.x - vx;
+                z[i + half].y = u.y - vy;
+            }
+            __syncthreads();
         }
-        __syncthreads();
-    }
+    };
+    transform(T(-1));
     // this sub-offset's coefficients, then back into bit-reversed order for the inverse
-    float2 cm[PER];
-    const float invN = 1.f / (float)N;   // a power of two: exact
+    T2 cm[PER];
+    const T invN = T(1) / (T)N;   // a power of two: exact
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
         const int m = threadIdx.x + 256 * q;
-        cm[q] = make_float2(0.f, 0.f);
+        cm[q].x = cm[q].y = T(0);
         if (m < N && 2 * m <= N) {
-            const float re = z[m].x * invN, im = 2 * m == N ? 0.f : z[m].y * invN;
-            const float wm = (m == 0 || 2 * m == N) ? 1.f : 2.f;
-            float sn, cs;
-            sincospif((float)(2 * m * s) / (float)(UPSAMPLE * N), &sn, &cs);
-            cm[q] = make_float2(wm * (re * cs - im * sn), wm * (re * sn + im * cs));
+            const T re = z[m].x * invN, im = 2 * m == N ? T(0) : z[m].y * invN;
+            const T wm = (m == 0 || 2 * m == N) ? T(1) : T(2);
+            T sn, cs;
+            sincospi_t((T)(2 * m * s) / (T)(UPSAMPLE * N), &sn, &cs);
+            cm[q].x = wm * (re * cs - im * sn);
+            cm[q].y = wm * (re * sn + im * cs);
         }
     }
     __syncthreads();
@@ -1553,24 +1581,12 @@ __global__ void __launch_bounds__(256) k_fine_weights_fft(const double* __restri
         if (m < N) z[__brev((unsigned)m) >> (32 - L)] = cm[q];
     }
     __syncthreads();
-    // inverse transform: z[j] = sum_m C_m e^{2 pi i m j / N}
-    for (int len = 2; len <= N; len <<= 1) {
-        const int half = len >> 1, step = N / len;
-        for (int b = threadIdx.x; b < N / 2; b += blockDim.x) {
-            const int pos = b & (half - 1), i = (b - pos) * 2 + pos;
-            const float2 t = w[pos * step];
-            const float2 u = z[i], v = z[i + half];
-            const float2 vt = make_float2(v.x * t.x - v.y * t.y, v.x * t.y + v.y * t.x);
-            z[i] = make_float2(u.x + vt.x, u.y + vt.y);
-            z[i + half] = make_float2(u.x - vt.x, u.y - vt.y);
-        }
-        __syncthreads();
-    }
+    transform(T(1));
     for (int j = threadIdx.x; j < N; j += blockDim.x) {
         const int64_t g = foff[k] + (int64_t)UPSAMPLE * j + s;
-        const float v = (float)((double)z[j].x * fg[6 * g + 4] * fg[6 * g + 5]);
-        wf[g] = v;
-        wf64[g] = (double)v;   // the binary64 image the dipole weights are taken from
+        const double v = (double)z[j].x * fg[6 * g + 4] * fg[6 * g + 5];
+        if (wf) wf[g] = (float)v;
+        wf64[g] = sizeof(T) == 4 ? (double)(float)v : v;   // binary32: the image the dipole weights are taken from
     }
 }
 
@@ -2053,6 +2069,24 @@ extern "C" mh_status mh_boundary_create(mh_ctx* ctx, int n_curves, const int32_t
     BCHK(b->d_fine_off.alloc(n_curves + 1));
     BCHK(b->fine_geo.alloc(6 * b->n_fine));
     BCHK(cudaMemcpyAsync(b->d_fine_off.p, b->fine_off.data(), (n_curves + 1) * 8, cudaMemcpyHostToDevice, st));
+    BCHK(cudaFuncSetAttribute(k_fine_weights_fft<double, double2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              2 * FFT_MAX * (int)sizeof(double2)));
+    {
+        double lo[2] = {1e300, 1e300}, hi[2] = {-1e300, -1e300}, sum[2] = {0.0, 0.0};
+        for (int64_t i = 0; i < tot; ++i)
+            for (int c = 0; c < 2; ++c) {
+                lo[c] = std::min(lo[c], xy_host[2 * i + c]);
+                hi[c] = std::max(hi[c], xy_host[2 * i + c]);
+                sum[c] += xy_host[2 * i + c];
+            }
+        b->cls_ox = sum[0] / tot;
+        b->cls_oy = sum[1] / tot;
+        b->cls_extent = (float)std::max(hi[0] - lo[0], hi[1] - lo[1]);
+    }
+    BCHK(b->geo32.alloc(tot));
+    k_cls32<<<mh_grid(tot, 128), 128, 0, st>>>(b->geo.p, b->d_curve_of.p, b->d_nn.p, tot, b->cls_ox, b->cls_oy,
+                                               b->geo32.p);
+    ctx->launches++;
     BCHK(b->tw.alloc(tot));
     BCHK(b->half.alloc(tot));
     k_twiddles<<<mh_grid(tot, 128), 128, 0, st>>>(b->d_nn.p, b->d_off.p, b->d_curve_of.p, tot, b->tw.p, b->half.p);
@@ -2813,16 +2847,17 @@ mh_status dlp_classify(mh_ctx* ctx, mh_boundary* b, const double* xy_dev, int64_
                        bool all_groups) {
     cudaStream_t st = ctx->stream;
     tg->n = n;
-    dbuf<uint32_t> fine0;
-    dbuf<int32_t> lcurve;
-    dbuf<double> ldata;
-    MH_ALLOC(ctx, tg->region, n);
-    MH_ALLOC(ctx, fine0, n);
-    MH_ALLOC(ctx, lcurve, n);
-    MH_ALLOC(ctx, ldata, 4 * n);
+    dbuf<uint32_t>& fine0 = tg->fine0;
+    dbuf<int32_t>& lcurve = tg->lcurve;
+    dbuf<double>& ldata = tg->ldata;
+    MH_RESERVE(ctx, tg->region, n);
+    MH_RESERVE(ctx, fine0, n);
+    MH_RESERVE(ctx, lcurve, n);
+    MH_RESERVE(ctx, ldata, 4 * n);
     if (n > 0) {
-        k_classify<<<mh_grid(n * 32, 256), 256, 0, st>>>(xy_dev, n, b->geo.p, b->coef.p, b->d_nn.p, b->d_off.p,
-                                                         b->n_curves, tg->region.p, fine0.p, lcurve.p, ldata.p);
+        k_classify<<<mh_grid(n * 32, 256), 256, 0, st>>>(xy_dev, n, b->geo.p, b->geo32.p, b->cls_ox, b->cls_oy,
+                                                         b->cls_extent, b->coef.p, b->d_nn.p, b->d_off.p, b->n_curves,
+                                                         tg->region.p, fine0.p, lcurve.p, ldata.p);
         MH_LAUNCHED(ctx);
     }
     // host-side compaction of the (few) line targets and fine pairs
@@ -2888,22 +2923,22 @@ mh_status dlp_classify(mh_ctx* ctx, mh_boundary* b, const double* xy_dev, int64_
                                                                             (152 * 8 + tg->n_groups - 1) / tg->n_groups))
                               : 1;
     }
-    MH_ALLOC(ctx, tg->grp_curve, std::max<int64_t>(tg->n_groups, 1));
-    MH_ALLOC(ctx, tg->grp_pair, std::max<int64_t>(tg->n_groups * FINE_TG, 1));
-    MH_ALLOC(ctx, tg->grp_part, std::max<int64_t>(tg->fine_slices > 1 ? tg->n_groups * tg->fine_slices * FINE_TG : 0, 1));
-    MH_ALLOC(ctx, tg->grp_cnt, std::max<int64_t>(tg->n_groups, 1));
+    MH_RESERVE(ctx, tg->grp_curve, std::max<int64_t>(tg->n_groups, 1));
+    MH_RESERVE(ctx, tg->grp_pair, std::max<int64_t>(tg->n_groups * FINE_TG, 1));
+    MH_RESERVE(ctx, tg->grp_part, std::max<int64_t>(tg->fine_slices > 1 ? tg->n_groups * tg->fine_slices * FINE_TG : 0, 1));
+    MH_RESERVE(ctx, tg->grp_cnt, std::max<int64_t>(tg->n_groups, 1));
     MH_CUDA(ctx, cudaMemsetAsync(tg->grp_cnt.p, 0, std::max<int64_t>(tg->n_groups, 1) * sizeof(unsigned), st));
     if (tg->n_groups) {
         MH_CUDA(ctx, cudaMemcpyAsync(tg->grp_curve.p, gcur.data(), gcur.size() * 4, cudaMemcpyHostToDevice, st));
         MH_CUDA(ctx, cudaMemcpyAsync(tg->grp_pair.p, gpair.data(), gpair.size() * 4, cudaMemcpyHostToDevice, st));
     }
-    MH_ALLOC(ctx, tg->xy, 2 * tg->n_ext);
-    MH_ALLOC(ctx, tg->fine, tg->n_ext);
-    MH_ALLOC(ctx, tg->line_tgt, tg->n_line);
-    MH_ALLOC(ctx, tg->line_curve, tg->n_line);
-    MH_ALLOC(ctx, tg->line_data, 4 * tg->n_line);
-    MH_ALLOC(ctx, tg->pair_tgt, tg->n_pairs);
-    MH_ALLOC(ctx, tg->pair_curve, tg->n_pairs);
+    MH_RESERVE(ctx, tg->xy, 2 * tg->n_ext);
+    MH_RESERVE(ctx, tg->fine, tg->n_ext);
+    MH_RESERVE(ctx, tg->line_tgt, tg->n_line);
+    MH_RESERVE(ctx, tg->line_curve, tg->n_line);
+    MH_RESERVE(ctx, tg->line_data, 4 * tg->n_line);
+    MH_RESERVE(ctx, tg->pair_tgt, tg->n_pairs);
+    MH_RESERVE(ctx, tg->pair_curve, tg->n_pairs);
     if (n > 0) MH_CUDA(ctx, cudaMemcpyAsync(tg->xy.p, xy_dev, 2 * n * 8, cudaMemcpyDeviceToDevice, st));
     if (tg->n_ext) MH_CUDA(ctx, cudaMemcpyAsync(tg->fine.p, fext.data(), tg->n_ext * 4, cudaMemcpyHostToDevice, st));
     if (tg->n_line) {
@@ -2917,8 +2952,8 @@ mh_status dlp_classify(mh_ctx* ctx, mh_boundary* b, const double* xy_dev, int64_
         // trigonometric interpolation weights of every line target (fixed with the target)
         std::vector<int64_t> woff(tg->n_line + 1, 0);
         for (int64_t t = 0; t < tg->n_line; ++t) woff[t + 1] = woff[t] + b->n_nodes[lcur[t]];
-        MH_ALLOC(ctx, tg->line_woff, tg->n_line + 1);
-        MH_ALLOC(ctx, tg->line_w, std::max<int64_t>(woff[tg->n_line], 1));
+        MH_RESERVE(ctx, tg->line_woff, tg->n_line + 1);
+        MH_RESERVE(ctx, tg->line_w, std::max<int64_t>(woff[tg->n_line], 1));
         MH_CUDA(ctx, cudaMemcpyAsync(tg->line_woff.p, woff.data(), (tg->n_line + 1) * 8, cudaMemcpyHostToDevice, st));
         k_line_weights<<<mh_grid(tg->n_line * 32, 256), 256, 0, st>>>(tg->line_curve.p, tg->line_data.p, tg->n_line,
                                                                       b->d_nn.p, b->d_off.p, b->half.p,
@@ -2929,10 +2964,8 @@ mh_status dlp_classify(mh_ctx* ctx, mh_boundary* b, const double* xy_dev, int64_
         MH_CUDA(ctx, cudaMemcpyAsync(tg->pair_tgt.p, pt.data(), tg->n_pairs * 4, cudaMemcpyHostToDevice, st));
         MH_CUDA(ctx, cudaMemcpyAsync(tg->pair_curve.p, pc.data(), tg->n_pairs * 4, cudaMemcpyHostToDevice, st));
     }
-    MH_ALLOC(ctx, tg->ext, std::max<int64_t>(tg->n_ext, 1));
-    MH_ALLOC(ctx, tg->sc, 2 * (b->n / 2 + b->n_curves));
-    MH_ALLOC(ctx, tg->wf, b->n_fine);
-    MH_ALLOC(ctx, tg->asig, b->n);
+    MH_RESERVE(ctx, tg->ext, std::max<int64_t>(tg->n_ext, 1));
+    MH_RESERVE(ctx, tg->asig, b->n);
     MH_CUDA(ctx, cudaStreamSynchronize(st));
     return MH_OK;
 }
@@ -2972,9 +3005,6 @@ static mh_status prep_mixed(mh_ctx* ctx, mh_boundary* b) {
     MH_CUDA(ctx, cudaStreamSynchronize(st));
     return MH_OK;
 }
-
-static mh_status fine_density(mh_ctx* ctx, mh_boundary* b, const double* sc, mh_precision prec, float* wf32,
-                              double* wf64);
 
 // The binary64 pair table of the boundary for alpha (recorded graphs hold it: a rebuild counts as
 // a new operator generation, and the eager step before a recording makes it).
@@ -3045,40 +3075,21 @@ mh_status dlp_evaluate(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* t
     cudaStream_t st = ctx->stream;
     MH_TRY(bie_assemble(ctx, b, alpha));
     dbuf<double>& ext = tg->ext;
-    dbuf<double>& sc = tg->sc;
-    dbuf<double>& wf = tg->wf;
     dbuf<double>& asig = tg->asig;
     prof_scope ps_all(ctx, "dlp_evaluate");
-    const int64_t nmodes = b->n / 2 + b->n_curves;
     if (prec == MH_PREC_MIXED) {
         MH_TRY(prep_mixed(ctx, b));
         k_weights32<<<mh_grid(b->n, 256), 256, 0, st>>>(sigma, b->geo.p, b->d_curve_of.p, b->d_nn.p, b->n, b->w32.p);
         MH_LAUNCHED(ctx);
-        if (tg->n_ext) {
-            prof_scope ps(ctx, "dlp_coarse", DL_FLOPS * tg->n_ext * b->n, 24.0 * (tg->n_ext + b->n));
-            MH_TRY(coarse_sums(ctx, b, alpha, tg, 0, tg->n_ext, sigma, MH_PREC_MIXED));
-        }
-        if (tg->n_pairs) {
-            k_fourier_scalar<<<(unsigned)nmodes, 128, 0, st>>>(sigma, b->d_nn.p, b->d_off.p, b->tw.p, b->n_curves,
-                                                               nmodes, sc.p);
-            MH_LAUNCHED(ctx);
-            MH_TRY(fine_density(ctx, b, sc.p, MH_PREC_MIXED, b->wf32.p, nullptr));
-        }
-    } else {
-        if (tg->n_ext) {
-            prof_scope ps(ctx, "dlp_coarse", DL_FLOPS * tg->n_ext * b->n, 24.0 * (tg->n_ext + b->n));
-            MH_TRY(coarse_sums(ctx, b, alpha, tg, 0, tg->n_ext, sigma, MH_PREC_FP64));
-        }
-        if (tg->n_pairs) {
-            k_fourier_scalar<<<(unsigned)nmodes, 128, 0, st>>>(sigma, b->d_nn.p, b->d_off.p, b->tw.p, b->n_curves,
-                                                               nmodes, sc.p);
-            MH_LAUNCHED(ctx);
-            MH_TRY(fine_density(ctx, b, sc.p, MH_PREC_FP64, nullptr, wf.p));
-        }
+    }
+    if (tg->n_ext) {
+        prof_scope ps(ctx, "dlp_coarse", DL_FLOPS * tg->n_ext * b->n, 24.0 * (tg->n_ext + b->n));
+        MH_TRY(coarse_sums(ctx, b, alpha, tg, 0, tg->n_ext, sigma, prec));
     }
     if (tg->n_pairs) {
+        MH_TRY(dlp_fine_weights(ctx, b, sigma, prec, true));
         prof_scope ps(ctx, "dlp_fine", DL_FLOPS * (tg->fine_nodes_main + tg->fine_nodes_aux), 24.0 * b->n_fine);
-        MH_TRY(fine_sums(ctx, b, alpha, tg, wf.p, prec));
+        MH_TRY(fine_sums(ctx, b, alpha, tg, b->wf64.p, prec));
     }
     if (tg->n_line) {
         MH_TRY(bie_apply(ctx, b, sigma, asig.p, MH_PREC_FP64));
@@ -3110,14 +3121,8 @@ static mh_status fine_density(mh_ctx* ctx, mh_boundary* b, const double* sc, mh_
         k_fine_coef<float2><<<mh_grid(nmodes * UPSAMPLE, 256), 256, 0, st>>>(sc, b->d_nn.p, b->d_off.p, b->n_curves,
                                                                              nmodes, b->fcp32.p);
         MH_LAUNCHED(ctx);
-        bool pow2 = max_n <= FFT_MAX;
-        for (int nk : b->n_nodes) pow2 = pow2 && nk >= 2 && (nk & (nk - 1)) == 0;
-        if (pow2)
-            k_fine_density_fft<<<dim3(UPSAMPLE, (unsigned)b->n_curves), 256, 2 * max_n * sizeof(float2), st>>>(
-                b->fcp32.p, b->tw32.p, b->fine_geo.p, b->d_nn.p, b->d_off.p, b->d_fine_off.p, wf32);
-        else
-            k_fine_density_s<float, float2><<<grid, 256, max_n * sizeof(float2), st>>>(
-                b->fcp32.p, b->tw32.p, b->fine_geo.p, b->d_nn.p, b->d_off.p, b->d_fine_off.p, wf32);
+        k_fine_density_s<float, float2><<<grid, 256, max_n * sizeof(float2), st>>>(
+            b->fcp32.p, b->tw32.p, b->fine_geo.p, b->d_nn.p, b->d_off.p, b->d_fine_off.p, wf32);
     } else {
         if (!b->fcp64.p) MH_ALLOC(ctx, b->fcp64, nmodes * UPSAMPLE);
         k_fine_coef<double2><<<mh_grid(nmodes * UPSAMPLE, 256), 256, 0, st>>>(sc, b->d_nn.p, b->d_off.p, b->n_curves,
@@ -3130,37 +3135,44 @@ static mh_status fine_density(mh_ctx* ctx, mh_boundary* b, const double* sc, mh_
     return MH_OK;
 }
 
-mh_status dlp_fine_weights(mh_ctx* ctx, mh_boundary* b, const double* sigma, mh_precision prec) {
+mh_status dlp_fine_weights(mh_ctx* ctx, mh_boundary* b, const double* sigma, mh_precision prec, bool spectrum64) {
     cudaStream_t st = ctx->stream;
     const int64_t nmodes = b->n / 2 + b->n_curves;
     if (!b->sc64.p) {
         MH_ALLOC(ctx, b->sc64, 2 * nmodes);
         MH_ALLOC(ctx, b->wf64, b->n_fine);
     }
+    const bool mixed = prec == MH_PREC_MIXED;
+    if (mixed) MH_TRY(prep_mixed(ctx, b));
     const int max_n = *std::max_element(b->n_nodes.begin(), b->n_nodes.end());
     bool pow2 = max_n <= FFT_MAX;
     for (int nk : b->n_nodes) pow2 = pow2 && nk >= 2 && (nk & (nk - 1)) == 0;
-    if (prec == MH_PREC_MIXED && pow2) {
-        // binary32 FFTs both ways in one launch
-        MH_TRY(prep_mixed(ctx, b));
-        k_fine_weights_fft<<<dim3(UPSAMPLE, (unsigned)b->n_curves), 256, 2 * max_n * sizeof(float2), st>>>(
-            sigma, b->tw32.p, b->fine_geo.p, b->d_nn.p, b->d_off.p, b->d_fine_off.p, b->wf32.p, b->wf64.p);
+    if (pow2) {   // FFTs both ways in one launch
+        const dim3 grid(UPSAMPLE, (unsigned)b->n_curves);
+        if (mixed && !spectrum64)
+            k_fine_weights_fft<float, float2><<<grid, 256, 2 * max_n * sizeof(float2), st>>>(
+                sigma, b->tw32.p, b->fine_geo.p, b->d_nn.p, b->d_off.p, b->d_fine_off.p, b->wf32.p, b->wf64.p);
+        else
+            k_fine_weights_fft<double, double2><<<grid, 256, 2 * max_n * sizeof(double2), st>>>(
+                sigma, b->tw.p, b->fine_geo.p, b->d_nn.p, b->d_off.p, b->d_fine_off.p, mixed ? b->wf32.p : nullptr,
+                b->wf64.p);
         MH_LAUNCHED(ctx);
-    } else if (prec == MH_PREC_MIXED) {
-        MH_TRY(prep_mixed(ctx, b));
+        return MH_OK;
+    }
+    if (mixed && !spectrum64) {
         k_to_float_vec<<<mh_grid(b->n, 256), 256, 0, st>>>(sigma, b->x32.p, b->n);
         MH_LAUNCHED(ctx);
         k_fourier_scalar32<<<(unsigned)nmodes, 128, 0, st>>>(b->x32.p, b->d_nn.p, b->d_off.p, b->tw32.p, b->n_curves,
                                                              nmodes, b->sc64.p);
-        MH_LAUNCHED(ctx);
-        MH_TRY(fine_density(ctx, b, b->sc64.p, MH_PREC_MIXED, b->wf32.p, nullptr));
-        k_f2d<<<mh_grid(b->n_fine, 256), 256, 0, st>>>(b->wf32.p, b->wf64.p, b->n_fine);
-        MH_LAUNCHED(ctx);
     } else {
         k_fourier_scalar<<<(unsigned)nmodes, 128, 0, st>>>(sigma, b->d_nn.p, b->d_off.p, b->tw.p, b->n_curves,
                                                            nmodes, b->sc64.p);
+    }
+    MH_LAUNCHED(ctx);
+    MH_TRY(fine_density(ctx, b, b->sc64.p, prec, b->wf32.p, b->wf64.p));
+    if (mixed) {
+        k_f2d<<<mh_grid(b->n_fine, 256), 256, 0, st>>>(b->wf32.p, b->wf64.p, b->n_fine);
         MH_LAUNCHED(ctx);
-        MH_TRY(fine_density(ctx, b, b->sc64.p, MH_PREC_FP64, nullptr, b->wf64.p));
     }
     return MH_OK;
 }
@@ -3221,11 +3233,14 @@ extern "C" mh_status mh_double_layer_apply(mh_ctx* ctx, mh_boundary* b, double a
     }
     if (n_targets < 0) return mh_fail(ctx, MH_ERR_INVALID_ARG, "n_targets < 0");
     if (n_targets == 0) return MH_OK;   // no targets: nothing to evaluate, out_dev untouched
-    dlp_targets tg;
-    MH_TRY(dlp_classify(ctx, b, targets_dev, n_targets, &tg, true));
-    MH_TRY(dlp_evaluate(ctx, b, alpha, &tg, sigma_dev, out_dev, prec));
-    MH_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    return MH_OK;
+    // the target set's buffers stay with the boundary for the next call (some twenty allocations and
+    // frees cost ~0.3 ms), unless this call was a large one
+    if (!b->eval) b->eval.reset(new dlp_targets());
+    mh_status s = dlp_classify(ctx, b, targets_dev, n_targets, b->eval.get(), true);
+    if (s == MH_OK) s = dlp_evaluate(ctx, b, alpha, b->eval.get(), sigma_dev, out_dev, prec);
+    if (s == MH_OK) MH_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    if (s != MH_OK || n_targets > DLP_KEEP) b->eval.reset();
+    return s;
 }
 
 extern "C" mh_status mh_gmres_solve(mh_ctx* ctx, mh_boundary* b, double alpha, const double* rhs_dev,

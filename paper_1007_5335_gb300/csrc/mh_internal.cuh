@@ -8,6 +8,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <map>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -102,8 +103,10 @@ struct dbuf {
         g_mh_alloc_calls.fetch_add(1, std::memory_order_relaxed);
         return cudaMalloc((void**)&p, count * sizeof(T));
     }
+    cudaError_t reserve(size_t count) { return count <= n ? cudaSuccess : alloc(count); }
 };
 
+#define MH_RESERVE(ctx, buf, count) MH_CUDA(ctx, (buf).reserve(count))
 #define MH_ALLOC(ctx, buf, count) MH_CUDA(ctx, (buf).alloc(count))
 
 // ---- dependent launches ----
@@ -271,6 +274,40 @@ struct bie_operator {
     dbuf<uint16_t> A16lo;
 };
 
+// Classified target set for off-surface evaluation.
+struct dlp_targets {
+    int64_t n = 0;          // user targets
+    int64_t n_ext = 0;      // user targets + auxiliary points of the normal-line rule
+    dbuf<double> xy;        // [n_ext][2]
+    dbuf<uint32_t> fine0;   // classification results before compaction (masks, nearest curves, foot data)
+    dbuf<int32_t> lcurve;
+    dbuf<double> ldata;
+    dbuf<uint32_t> fine;    // [n_ext] bit k: use the upsampled rule on curve k
+    dbuf<int32_t> region;   // [n] -1 inside Omega, k exterior side of curve k
+    // normal-line rule: per line target
+    int64_t n_line = 0;
+    dbuf<int32_t> line_tgt;     // target index
+    dbuf<int32_t> line_curve;   // curve
+    dbuf<double> line_data;     // [n_line][4]: t*, d, h_s, unused
+    dbuf<double> line_w;        // trigonometric interpolation weights at t*, N_k per line target
+    dbuf<int64_t> line_woff;    // [n_line + 1] offsets into line_w
+    // fine pairs (ext target, curve)
+    int64_t n_pairs = 0, n_pairs_main = 0;   // pairs of user targets come first
+    double fine_nodes_main = 0, fine_nodes_aux = 0;   // work counts
+    dbuf<int32_t> pair_tgt, pair_curve;
+    // upsampled rule at the auxiliary points (at every pair of a set classified with all_groups):
+    // groups of FINE_TG pairs on one curve (grp_pair, -1 padded), each group's fine nodes in
+    // fine_slices slices, one block per (group, slice); partial sums per (group, slice, pair) in
+    // grp_part
+    int64_t n_groups = 0;
+    int fine_slices = 1;
+    dbuf<int32_t> grp_curve, grp_pair;
+    dbuf<double> grp_part;
+    dbuf<unsigned> grp_cnt;
+    // evaluation workspaces (allocated once by dlp_classify)
+    dbuf<double> ext, asig, part;
+};
+
 struct mh_boundary {
     int n_curves = 0;
     int64_t n = 0;                       // N_Gamma
@@ -280,6 +317,9 @@ struct mh_boundary {
     dbuf<int32_t> d_curve_of;            // curve index of every node
     dbuf<double> xy;                     // [n][2]
     dbuf<double> geo;                    // [n][8]: x y x' y' x'' y'' |y'| kdiag
+    dbuf<float4> geo32;                  // binary32 nodes for the classification: x, y from the origin, normal |y'| h
+    double cls_ox = 0, cls_oy = 0;       // the origin (mean node)
+    float cls_extent = 0;                // largest side of the nodes' bounding box
     dbuf<double> coef;                   // per curve Fourier coefficients: [off*2 ...] see boundary.cu
     dbuf<double2> tw, half;              // per node (cos, sin)(2 pi r / N) and (cos, sin)(pi r / N)
     // fine (16x) grid per curve: positions, normals, speed*h_fine
@@ -316,6 +356,7 @@ struct mh_boundary {
     dbuf<int64_t> mf_moff;               // per curve: offset of its M_k-entry blocks (twiddles at moff/2)
     dbuf<int32_t> mf_M;                  // per curve: transform length M_k (power of two >= 2 N_k - 1)
     int mf_mmax = 0;
+    std::unique_ptr<dlp_targets> eval;   // buffers of mh_double_layer_apply's last target set
     dbuf<double2> mf_spec;               // per call: spectra c_m, m <= N_k/2
     dbuf<double> mf_S;                   // per call: [2 l][n] interpolated density at the Alpert nodes
     dbuf<double> mf_w, mf_u;             // per call: dipole strengths, multipole-pass output
@@ -326,37 +367,6 @@ struct mh_boundary {
 };
 
 #define MH_TILE 128
-
-// Classified target set for off-surface evaluation.
-struct dlp_targets {
-    int64_t n = 0;          // user targets
-    int64_t n_ext = 0;      // user targets + auxiliary points of the normal-line rule
-    dbuf<double> xy;        // [n_ext][2]
-    dbuf<uint32_t> fine;    // [n_ext] bit k: use the upsampled rule on curve k
-    dbuf<int32_t> region;   // [n] -1 inside Omega, k exterior side of curve k
-    // normal-line rule: per line target
-    int64_t n_line = 0;
-    dbuf<int32_t> line_tgt;     // target index
-    dbuf<int32_t> line_curve;   // curve
-    dbuf<double> line_data;     // [n_line][4]: t*, d, h_s, unused
-    dbuf<double> line_w;        // trigonometric interpolation weights at t*, N_k per line target
-    dbuf<int64_t> line_woff;    // [n_line + 1] offsets into line_w
-    // fine pairs (ext target, curve)
-    int64_t n_pairs = 0, n_pairs_main = 0;   // pairs of user targets come first
-    double fine_nodes_main = 0, fine_nodes_aux = 0;   // work counts
-    dbuf<int32_t> pair_tgt, pair_curve;
-    // upsampled rule at the auxiliary points (at every pair of a set classified with all_groups):
-    // groups of FINE_TG pairs on one curve (grp_pair, -1 padded), each group's fine nodes in
-    // fine_slices slices, one block per (group, slice); partial sums per (group, slice, pair) in
-    // grp_part
-    int64_t n_groups = 0;
-    int fine_slices = 1;
-    dbuf<int32_t> grp_curve, grp_pair;
-    dbuf<double> grp_part;
-    dbuf<unsigned> grp_cnt;
-    // evaluation workspaces (allocated once by dlp_classify)
-    dbuf<double> ext, sc, wf, asig, part;
-};
 
 struct mh_tree {
     double box[3];
@@ -453,8 +463,9 @@ mh_status dlp_evaluate_fmm_tail(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_t
                                 const double* main_vals, double* out, mh_precision prec,
                                 const double* asig_given = nullptr, int part = 0);
 // Density on the 16x fine grid times |y'| h_f (binary64 in b->wf64; binary32 also in b->wf32
-// when prec is mixed).
-mh_status dlp_fine_weights(mh_ctx* ctx, mh_boundary* b, const double* sigma, mh_precision prec);
+// when prec is mixed); spectrum64: mixed weights rounded from a binary64 spectrum, not a binary32 one.
+mh_status dlp_fine_weights(mh_ctx* ctx, mh_boundary* b, const double* sigma, mh_precision prec,
+                           bool spectrum64 = false);
 // r0 (nullable): the binary64 residual rhs - A x of the initial guess, computed by the caller.
 mh_status gmres_run(mh_ctx* ctx, mh_boundary* b, const double* rhs, double* x, double tol, int max_iter,
                     mh_precision prec, mh_gmres_info* info, const double* r0 = nullptr);
