@@ -3010,7 +3010,7 @@ static mh_status prep_mixed(mh_ctx* ctx, mh_boundary* b) {
 // a new operator generation, and the eager step before a recording makes it).
 static mh_status pair_table(mh_ctx* ctx, mh_boundary* b, double alpha) {
     if (b->ptab_alpha == alpha) return MH_OK;
-    if (!b->ptab.p) MH_ALLOC(ctx, b->ptab, 4 * PT_BINS);
+    if (!b->ptab.p) MH_ALLOC(ctx, b->ptab, PT_WORDS * PT_BINS);
     k_pair_table<<<(PT_BINS + 127) / 128, 128, 0, ctx->stream>>>(mh_pair_tab_make(nullptr, alpha), alpha, b->ptab.p);
     MH_LAUNCHED(ctx);
     b->ptab_alpha = alpha;

@@ -8,29 +8,39 @@
 // every octave of rho is cut into equal bins (their number from the leading mantissa bits), each
 // bin holds the 7 Taylor coefficients about its centre,
 //   d^j/drho^j f = (-1/(2 alpha^2))^j K_{1+j}(z) / z^{1+j}
-// (the derivative rule of z^{-n} K_n(z)).  A pair then takes 15 binary64 instructions: offsets
-// 2, rho 2, t 1, Horner 6, dot product 2, accumulate 1, and no square root or division.
-//   bins     128 an octave from rho = 2^-14 alpha^2 for 20 octaves (t/rho <= 1/256: the eighth
+// (the derivative rule of z^{-n} K_n(z)).
+//   bins     128 an octave from rho = 2^-14 alpha^2 for 20 octaves (|t/rho| <= 1/256: the eighth
 //            term is below 256^-7 = 1.4e-17 of f), 512 an octave for the six above, where f falls
 //            like e^{-z} (z = 45: (z/2048)^7/7! = 4e-16); octaves start at a power of two, so
 //            the two ranges reach past 2025 alpha^2 = (45 alpha)^2 whatever alpha is.
-//   lookup   the bin is the top bits of rho's binary64 pattern, its centre the same bits with
-//            half a bin added (integer pipe); 64 bytes per bin, four 16-byte loads from L1.
+//   lookup   the bin is the top bits of rho's binary64 pattern; the bits below them, shifted up, are
+//            the place in the bin, tau in [-1/2, 1/2) in units of its width (integer pipe, and one
+//            subtraction).
+//   terms    tau^0..3 in binary64; tau^4..6 together are below 256^-4 = 2.4e-10 of f, so their factor
+//            of tau^4 is formed in binary32 (1.4e-17 of f) and widened by its bits.
+// 48 bytes per bin (four doubles, three floats, padding), three 16-byte loads from L1.
+// A pair then takes 12 binary64 instructions: offsets 2, rho 2, tau 1, Horner 4, dot product 2,
+// accumulate 1, and no comparison, conversion, square root or division.
 // Pairs nearer than the table (r < alpha/128) take K1 directly.
 // Measured, starfish heat step in binary64 (5.6e7 near pairs, 4.2e7 upsampled, 1.5e7 trapezoid):
-// 19.84 ms a step with K1 per pair, 5.03 ms with the table; u differs by 6e-17 (relative L2).
+// 19.84 ms a step with K1 per pair, 5.03 ms with seven binary64 coefficients (15 instructions; near
+// field 14.8 -> 1.66 ms), 0.37 ms a step less with three of them in binary32.
 #pragma once
+
+#include <cstdint>
+#include <cstring>
 
 #include "bessel.cuh"
 
 constexpr int PT_OCT = 20, PT_BITS = 7, PT_OCT_FAR = 6, PT_BITS_FAR = 9;
-constexpr int PT_BINS = (PT_OCT << PT_BITS) + (PT_OCT_FAR << PT_BITS_FAR);   // 5632 bins, 352 KB
+constexpr int PT_BINS = (PT_OCT << PT_BITS) + (PT_OCT_FAR << PT_BITS_FAR);   // 5632 bins, 264 KB
+constexpr int PT_WORDS = 3;   // double2 per bin
 
 struct mh_pair_tab {
-    const double2* c = nullptr;   // [PT_BINS][4]: coefficients 0..6, one entry of padding
+    const double2* c = nullptr;   // [PT_BINS][PT_WORDS]
     int hi0 = 0, hi1 = 0;         // high words of the first bin of the two ranges
+    int hi_cut = 0;               // high word of (45 alpha)^2: farther pairs are 0 (e^{-45} of the unit-distance value)
     double inv_alpha = 0.0;
-    double cut = 0.0;             // (45 alpha)^2: farther pairs are 0 (e^{-45} of the unit-distance value)
 };
 
 inline mh_pair_tab mh_pair_tab_make(const double2* c, double alpha) {
@@ -39,8 +49,11 @@ inline mh_pair_tab mh_pair_tab_make(const double2* c, double alpha) {
     const int e0 = std::ilogb(alpha * alpha) - 14;   // first octave: [2^e0, 2^(e0+1))
     T.hi0 = (e0 + 1023) << 20;
     T.hi1 = (e0 + PT_OCT + 1023) << 20;
+    const double cut = 2025.0 * alpha * alpha;
+    uint64_t bits;
+    std::memcpy(&bits, &cut, 8);
+    T.hi_cut = (int)(bits >> 32);
     T.inv_alpha = 1.0 / alpha;
-    T.cut = 2025.0 * alpha * alpha;
     return T;
 }
 
@@ -51,23 +64,25 @@ static __device__ __noinline__ double mh_pair_near(double rho, double inv_alpha)
     return mh_k1(z) / z;
 }
 
-// f(rho) = K1(z)/z, z = sqrt(rho)/alpha; 0 beyond the cut.
+// f(rho) = K1(z)/z, z = sqrt(rho)/alpha; 0 beyond the cut; not a number stays one.
 __device__ __forceinline__ double mh_pair_f(double rho, const mh_pair_tab& T) {
-    if (!(rho <= T.cut)) return rho > T.cut ? 0.0 : rho;   // beyond the cut; not a number stays one
-    const int hi = __double2hiint(rho);
+    const int hi = __double2hiint(rho), lo = __double2loint(rho);
+    if (hi > T.hi_cut) return rho != rho ? rho : 0.0;
     if (hi < T.hi0) return mh_pair_near(rho, T.inv_alpha);
     const bool far = hi >= T.hi1;
-    const int sh = far ? 20 - PT_BITS_FAR : 20 - PT_BITS;
-    const int bin = ((hi - (far ? T.hi1 : T.hi0)) >> sh) + (far ? PT_OCT << PT_BITS : 0);
-    const double t = rho - __hiloint2double((hi >> sh << sh) | (1 << (sh - 1)), 0);
-    const double2* c = T.c + 4 * bin;
-    const double2 a = __ldg(c), b = __ldg(c + 1), d = __ldg(c + 2), e = __ldg(c + 3);
-    double v = fma(e.x, t, d.y);
-    v = fma(v, t, d.x);
-    v = fma(v, t, b.y);
-    v = fma(v, t, b.x);
-    v = fma(v, t, a.y);
-    return fma(v, t, a.x);
+    const int bits = far ? PT_BITS_FAR : PT_BITS;
+    const int bin = ((hi - (far ? T.hi1 : T.hi0)) >> (20 - bits)) + (far ? PT_OCT << PT_BITS : 0);
+    const double2* c = T.c + PT_WORDS * bin;
+    const double2 a = __ldg(c), b = __ldg(c + 1);
+    const float4 q = __ldg(reinterpret_cast<const float4*>(c + 2));
+    // the mantissa below the bin bits as a number in [1, 2)
+    const int mh = (__funnelshift_l(lo, hi, bits) & 0xfffff) | 0x3ff00000;
+    const double tau = __hiloint2double(mh, lo << bits) - 1.5;
+    const float tf = __int_as_float((mh & 0xfffff) << 3 | 0x3f800000) - 1.5f;
+    // (double)w by its bits (w = 0 or far below the smallest normal number comes out as some 1e-38)
+    const unsigned w = __float_as_uint(fmaf(fmaf(q.z, tf, q.y), tf, q.x));
+    const double h = __hiloint2double((int)((w & 0x80000000u) | (((w >> 3) & 0x0fffffffu) + (896u << 20))), (int)(w << 29));
+    return fma(fma(fma(fma(h, tau, b.y), tau, b.x), tau, a.y), tau, a.x);
 }
 
 // Table entries for one alpha: a thread per bin, K_n by the (stable) forward recurrence.
@@ -77,16 +92,19 @@ static __global__ void k_pair_table(mh_pair_tab T, double alpha, double2* __rest
     const bool far = bin >= (PT_OCT << PT_BITS);
     const int sh = far ? 20 - PT_BITS_FAR : 20 - PT_BITS;
     const int i = far ? bin - (PT_OCT << PT_BITS) : bin;
-    const double rho = __hiloint2double((far ? T.hi1 : T.hi0) + (i << sh) + (1 << (sh - 1)), 0);
-    const double z = sqrt(rho) / alpha, d = -0.5 / (alpha * alpha);
-    double km = mh_k0(z), k = mh_k1(z), scale = 1.0 / z, c[8];
-    c[7] = 0.0;
-    for (int j = 0; j < 7; ++j) {   // c_j = (-1/(2 alpha^2))^j / j! K_{1+j}(z) / z^{1+j}
+    const int first = (far ? T.hi1 : T.hi0) + (i << sh);
+    const double lo = __hiloint2double(first, 0), width = 2.0 * (__hiloint2double(first + (1 << (sh - 1)), 0) - lo);
+    const double rho = lo + 0.5 * width;
+    const double z = sqrt(rho) / alpha, d = -0.5 * width / (alpha * alpha);
+    double km = mh_k0(z), k = mh_k1(z), scale = 1.0 / z, c[7];
+    for (int j = 0; j < 7; ++j) {   // c_j = (-width/(2 alpha^2))^j / j! K_{1+j}(z) / z^{1+j}
         c[j] = scale * k;
         const double kn = km + (2.0 * (j + 1) / z) * k;
         km = k;
         k = kn;
         scale *= d / (z * (j + 1));
     }
-    for (int q = 0; q < 4; ++q) out[4 * bin + q] = make_double2(c[2 * q], c[2 * q + 1]);
+    out[PT_WORDS * bin] = make_double2(c[0], c[1]);
+    out[PT_WORDS * bin + 1] = make_double2(c[2], c[3]);
+    *reinterpret_cast<float4*>(out + PT_WORDS * bin + 2) = make_float4((float)c[4], (float)c[5], (float)c[6], 0.f);
 }

@@ -381,106 +381,90 @@ __global__ void k_apply(const TOP* __restrict__ ops, const int64_t* __restrict__
     }
 }
 
-// ---- M2M / L2L chains without grid-wide barriers ----
-// The level chains are latency chains (a few small matvecs per tree level).  Both kernels
-// follow the data dependences instead of the levels:
-//  * upward (M2M): one block per internal box whose children are all leaves.  A block forms
-//    its box's multipole, then counts its arrival at the box's parent; the last child to
-//    arrive carries on with the parent (arrival counters reset by that block), so the
-//    critical path is the depth of the tree, not a barrier per level.
-//    M[parent] = sum over the children c = 0..3 of T_c M[child_c]: thread (c, r) forms row r
+// ---- M2M / L2L, one launch per tree level ----
+// The levels are a latency chain of small matvecs.  Every level has one set of four operators
+// (child positions), the same for all its boxes, so a block copies them to shared memory before it
+// waits for the level before (dependent launch: it is resident by then) and its critical path is
+// the children's expansions, the products and the store.
+//  * up (M2M): M[box] = sum over the children c = 0..3 of T_c M[child_c]: thread (c, r) forms row r
 //    of T_c M[child_c] (products in column order), the four are added in the order c = 0..3.
-//  * downward (L2L): one block per internal box with leaf children.  The block recomputes,
-//    in shared memory, the local expansions of the box's ancestors from the top internal
-//    level down (L[child] = L_m2l[child] + T'_c L[parent], the same operations in the same
-//    order as a level-by-level sweep), then adds T'_c L[box] to each leaf child.  Only leaf
-//    expansions are written: they are the only ones read afterwards.
+//  * down (L2L): L[child_c] += T'_c L[box], thread (c, r) forms row r.
 // Operators are stored transposed per (level, child position): ops[((l * 4 + c) * P + col) * P
-// + row], so the threads of a warp read consecutive words.
-template <typename T>
-__device__ __forceinline__ T chain_fma(T a, T b, T c);
-template <>
-__device__ __forceinline__ float chain_fma<float>(float a, float b, float c) { return fmaf(a, b, c); }
-template <>
-__device__ __forceinline__ double chain_fma<double>(double a, double b, double c) { return fma(a, b, c); }
+// + row], so the threads of a warp read consecutive words.  A dataflow form (one launch, a box's
+// last child carries on with the parent) spent ~4.5 us a level, most of it on operator loads from
+// L2: 28 us up and 22 us down for the starfish tree in binary32.  Against it: matrix-free solve at
+// 12,288 nodes (14 products) 6.13 -> 5.72 ms, mixed volume potential (255 k nodes) 186 -> 180 us,
+// binary64 volume potential 569 -> 568 us (bound by the binary64 contractions beside it).
+__device__ __forceinline__ void chain_stage(void* smem, const void* gmem, int bytes) {   // multiple of 16
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem);
+    for (int e = 16 * threadIdx.x; e < bytes; e += 16 * blockDim.x)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + e), "l"((const char*)gmem + e) : "memory");
+}
 
-// Row r of an operator times x: A points at row r of the transposed operator (A[cc * P] is
-// entry (r, cc)), x is in shared memory; products added in column order.
-template <typename TOP>
-__device__ __forceinline__ TOP chain_dot(const TOP* __restrict__ A, int P, const TOP* x) {
-    TOP acc = 0;
-    for (int cc = 0; cc < P; ++cc) acc = chain_fma<TOP>(A[(int64_t)cc * P], x[cc], acc);
+__device__ __forceinline__ void chain_staged() {
+    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+}
+
+template <typename T>
+__device__ __forceinline__ T chain_dot(const T* A, int P, const T* x) {
+    T acc = 0;
+#pragma unroll 4
+    for (int cc = 0; cc < P; ++cc) acc = fma(A[cc * P], x[cc], acc);
     return acc;
 }
 
-template <typename TOP>
-__global__ void k_chain_up(const TOP* __restrict__ ops, int P, const int32_t* __restrict__ ready,
-                           const int32_t* __restrict__ box, const int4* __restrict__ child,
-                           const int32_t* __restrict__ lvl, const int32_t* __restrict__ next,
-                           const int32_t* __restrict__ need, unsigned* cnt, int64_t base, TOP* vec) {
+template <typename T>
+__global__ void k_level_up(const T* __restrict__ ops, int P, const int32_t* __restrict__ box,
+                           const int4* __restrict__ child, int n, T* m) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    TOP* x = reinterpret_cast<TOP*>(smem_raw);   // 4 x P child expansions
-    TOP* part = x + 4 * P;                        // 4 x P products
-    __shared__ int go;
+    T* sA = reinterpret_cast<T*>(smem_raw);   // 4 operators
+    T* x = sA + 4 * P * P;                    // 4 x P child expansions
+    T* part = x + 4 * P;                      // 4 x P products
+    chain_stage(sA, ops, 4 * P * P * (int)sizeof(T));   // set-up data: may precede the wait
+    mh_dep_wait();
+    chain_staged();
     const int c = threadIdx.x / P, r = threadIdx.x - c * P;
-    const bool act = c < 4;
-    int t = ready[blockIdx.x];
-    for (;;) {
-        const int4 ch4 = child[t];
-        const int chc = c == 0 ? ch4.x : c == 1 ? ch4.y : c == 2 ? ch4.z : ch4.w;
-        // children may have been written by other blocks of this launch: read through L2
-        if (act) x[c * P + r] = chc >= 0 ? __ldcg(vec + base + (int64_t)chc * P + r) : TOP(0);
+    for (int b = blockIdx.x; b < n; b += gridDim.x) {
+        const int4 ch4 = child[b];
+        const int ch = c == 0 ? ch4.x : c == 1 ? ch4.y : c == 2 ? ch4.z : ch4.w;
+        if (c < 4) x[c * P + r] = ch >= 0 ? m[(int64_t)ch * P + r] : T(0);
         __syncthreads();
-        TOP acc = 0;
-        if (act && chc >= 0) acc = chain_dot<TOP>(ops + (int64_t)(lvl[t] * 4 + c) * P * P + r, P, x + c * P);
-        if (act) part[c * P + r] = acc;
+        if (c < 4) part[c * P + r] = ch >= 0 ? chain_dot<T>(sA + c * P * P + r, P, x + c * P) : T(0);
         __syncthreads();
         if (threadIdx.x < P) {
-            TOP s = part[r] + part[P + r];
+            T s = part[r] + part[P + r];
             s += part[2 * P + r];
             s += part[3 * P + r];
-            vec[base + (int64_t)box[t] * P + r] = s;
-            __threadfence();
+            m[(int64_t)box[b] * P + r] = s;
         }
-        const int q = next[t];
-        if (q < 0) return;
-        __syncthreads();
-        if (threadIdx.x == 0) go = atomicAdd(cnt + q, 1u) == (unsigned)(need[q] - 1);
-        __syncthreads();
-        if (!go) return;
-        if (threadIdx.x == 0) cnt[q] = 0u;
-        __threadfence();
-        t = q;
     }
 }
 
-template <typename TOP>
-__global__ void k_chain_down(const TOP* __restrict__ ops, int P, const int32_t* __restrict__ poff,
-                             const int32_t* __restrict__ pbox, const int32_t* __restrict__ pop,
-                             const int4* __restrict__ leaf, const int32_t* __restrict__ lop, int64_t base,
-                             TOP* vec) {
+template <typename T>
+__global__ void k_level_down(const T* __restrict__ ops, int P, const int32_t* __restrict__ box,
+                             const int4* __restrict__ child, int n, T* loc) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    TOP* x = reinterpret_cast<TOP*>(smem_raw);   // the running ancestor expansion
+    T* sA = reinterpret_cast<T*>(smem_raw);   // 4 operators
+    T* x = sA + 4 * P * P;                    // the box's expansion, two buffers
+    chain_stage(sA, ops, 4 * P * P * (int)sizeof(T));   // set-up data: may precede the wait
+    mh_dep_wait();
+    chain_staged();
     const int c = threadIdx.x / P, r = threadIdx.x - c * P;
-    const int k0 = poff[blockIdx.x], k1 = poff[blockIdx.x + 1];
-    const int64_t PP = (int64_t)P * P;
-    if (threadIdx.x < P) x[r] = vec[base + (int64_t)pbox[k0] * P + r];
-    for (int k = k0 + 1; k < k1; ++k) {
-        __syncthreads();
-        TOP acc = 0;
-        if (threadIdx.x < P) acc = chain_dot<TOP>(ops + (int64_t)pop[k] * PP + r, P, x);
-        __syncthreads();
-        if (threadIdx.x < P) x[r] = vec[base + (int64_t)pbox[k] * P + r] + acc;
-    }
-    __syncthreads();
-    if (c < 4) {
-        const int4 l4 = leaf[blockIdx.x];
-        const int lc = c == 0 ? l4.x : c == 1 ? l4.y : c == 2 ? l4.z : l4.w;
-        if (lc >= 0) vec[base + (int64_t)lc * P + r] += chain_dot<TOP>(ops + (lop[blockIdx.x] + c) * PP + r, P, x);
+    int buf = 0;
+    for (int b = blockIdx.x; b < n; b += gridDim.x, buf ^= 1) {
+        const int4 ch4 = child[b];
+        const int ch = c == 0 ? ch4.x : c == 1 ? ch4.y : c == 2 ? ch4.z : ch4.w;
+        if (threadIdx.x < P) x[buf * P + r] = loc[(int64_t)box[b] * P + r];
+        const T own = c < 4 && ch >= 0 ? loc[(int64_t)ch * P + r] : T(0);
+        __syncthreads();   // the other buffer is read until every thread is here again
+        if (c < 4 && ch >= 0) loc[(int64_t)ch * P + r] = own + chain_dot<T>(sA + c * P * P + r, P, x + buf * P);
     }
 }
 
 inline int chain_threads(int P) { return (4 * P + 31) / 32 * 32; }
+constexpr int CHAIN_SMEM_MAX = 224 * 1024;   // p = 40 (P = 81) in binary64 takes 215,136 bytes
+inline size_t chain_smem(int P, size_t word) { return (4 * (size_t)P * P + 8 * (size_t)P) * word; }
 
 // Per destination (one warp each): dst[r] = (acc ? dst[r] : 0) + the sum of its tasks' products,
 // in task order.  Binary64 products are summed in binary64; binary32 products in float-float
@@ -602,19 +586,13 @@ struct OpPool {
     }
 };
 
-// M2M / L2L of every level 2 <= l < L in parent-centric form (shared by the volume and the
-// double-layer passes: same tree, same operators at the same pool offsets).
-// Device description of the M2M / L2L chains (k_chain_up / k_chain_down).
-struct DfChain {
-    int64_t n_int = 0;                   // internal boxes of levels >= 2 (upward tasks)
-    int64_t n_ready = 0;                 // of which all children are leaves
-    int64_t n_down = 0;                  // internal boxes with leaf children (downward blocks)
+// M2M / L2L of every level 2 <= l < L in parent-centric form (k_level_up / k_level_down): the
+// internal boxes with their children, by level.
+struct LevelChain {
+    std::vector<int32_t> first;          // first task of level l (tasks of a level are contiguous), L + 1 entries
     double flops = 0, bytes = 0;         // one sweep (either direction), algorithmic
-    dbuf<int32_t> up_box, up_lvl, up_next, up_need, up_ready;
-    dbuf<int4> up_child;
-    dbuf<unsigned> up_cnt;
-    dbuf<int32_t> dn_off, dn_box, dn_op, dn_lop;
-    dbuf<int4> dn_leaf;
+    dbuf<int32_t> box;
+    dbuf<int4> child;
     dbuf<float> m2m32, l2l32;            // transposed operators, [level][position][col][row]
     dbuf<double> m2m64, l2l64;
 };
@@ -643,8 +621,9 @@ struct VolData {
     std::unique_ptr<Phase> near;                      // U list: near tables on the node values
     dbuf<double> temp_near;                           // its products (it may run beside the others)
     bool near_cover = true;                           // every leaf has a U-list task
+    bool local_cover = true;                          // every box of level >= 2 has an M2L or P2L task
     SideStream side;
-    std::unique_ptr<DfChain> chain;                   // M2M / L2L chains
+    std::unique_ptr<LevelChain> chain;                   // M2M / L2L chains
     int64_t temp_len = 0;
     int64_t n_near_tables = 0;
     TcImages tc;                                      // tensor-core images (mixed precision)
@@ -935,25 +914,27 @@ mh_status run_phase_on(mh_ctx* ctx, const TOP* ops, const int64_t* op_off, const
 }
 
 template <typename TOP>
-mh_status run_chain(mh_ctx* ctx, const DfChain* ch, int P, int64_t m_base, int64_t l_base, TOP* vec,
+mh_status run_chain(mh_ctx* ctx, const LevelChain* ch, int P, int64_t m_base, int64_t l_base, TOP* vec,
                     bool upward, const char* region) {
     // the level chains are timed in their own region: "<pass>_chain"
-    if (!ch || ch->n_int == 0) return MH_OK;
+    if (!ch || ch->first.empty() || ch->first.back() == 0) return MH_OK;
     prof_scope ps(ctx, region, ch->flops, ch->bytes);
     const bool f32 = sizeof(TOP) == 4;
     const TOP* ops = reinterpret_cast<const TOP*>(upward ? (f32 ? (const void*)ch->m2m32.p : (const void*)ch->m2m64.p)
                                                          : (f32 ? (const void*)ch->l2l32.p : (const void*)ch->l2l64.p));
-    const int nt = chain_threads(P);
-    if (upward) {
-        k_chain_up<TOP><<<(unsigned)ch->n_ready, nt, 8 * P * sizeof(TOP), ctx->stream>>>(
-            ops, P, ch->up_ready.p, ch->up_box.p, ch->up_child.p, ch->up_lvl.p, ch->up_next.p, ch->up_need.p,
-            ch->up_cnt.p, m_base, vec);
-    } else {
-        if (ch->n_down == 0) return MH_OK;
-        k_chain_down<TOP><<<(unsigned)ch->n_down, nt, P * sizeof(TOP), ctx->stream>>>(
-            ops, P, ch->dn_off.p, ch->dn_box.p, ch->dn_op.p, ch->dn_leaf.p, ch->dn_lop.p, l_base, vec);
+    const int L = (int)ch->first.size() - 1;
+    for (int q = 2; q < L; ++q) {
+        const int l = upward ? L + 1 - q : q;   // up: L - 1 .. 2, down: 2 .. L - 1
+        const int n = ch->first[l + 1] - ch->first[l];
+        if (n == 0) continue;
+        // at most the blocks that are resident together (27 KB of operators in binary32, 54 KB in
+        // binary64 at P = 41): a block's operators serve all its boxes
+        (void)mh_launch_dep(ctx->stream, upward ? k_level_up<TOP> : k_level_down<TOP>,
+                            dim3(std::min(n, 152 * (f32 ? 6 : 4))),
+                            dim3(chain_threads(P)), chain_smem(P, sizeof(TOP)), ops + (int64_t)l * 4 * P * P, P,
+                            ch->box.p + ch->first[l], ch->child.p + ch->first[l], n, vec + (upward ? m_base : l_base));
+        MH_LAUNCHED(ctx);
     }
-    MH_LAUNCHED(ctx);
     return MH_OK;
 }
 
@@ -989,144 +970,86 @@ mh_status fetch_tree(mh_ctx* ctx, const mh_tree* t, HostTree* h) {
     return MH_OK;
 }
 
-// Build every operator and pass of the multipole method for (tree, alpha, p).
-// M2M / L2L chains (k_chain_up / k_chain_down) of tree t: the internal boxes of levels
-// 2 <= l < L with their children.  With `active`, only active boxes take part (an inactive
-// child counts as absent).
+// M2M / L2L of tree t: the internal boxes of levels 2 <= l < L with their children.  With
+// `active`, only active boxes take part (an inactive child counts as absent).
 mh_status build_chain(mh_ctx* ctx, const mh_tree* t, const HostTree& h, int P, const OpPool& pool,
                       const std::vector<std::array<int, 4>>& op_m2m, const std::vector<std::array<int, 4>>& op_l2l,
-                      const std::vector<char>* active, std::unique_ptr<DfChain>* out) {
+                      const std::vector<char>* active, std::unique_ptr<LevelChain>* out) {
     const int64_t nb = t->n_boxes;
     const int L = t->max_level;
-    auto lev = [&](int b) { return h.boxes[3 * b]; };
-    {
-        std::vector<int32_t> child(4 * nb);
-        MH_CUDA(ctx, cudaMemcpyAsync(child.data(), t->box_child.p, 4 * nb * 4, cudaMemcpyDeviceToHost, ctx->stream));
-        MH_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-        std::unique_ptr<DfChain> ch(new DfChain());
-        std::vector<int32_t> idx(nb, -1), parent(nb, -1), quad(nb, -1);
-        if (active)   // children outside the active set are left out (zero expansions, no use)
-            for (int64_t b = 0; b < nb; ++b)
-                for (int c = 0; c < 4; ++c)
-                    if (child[4 * b + c] >= 0 && !(*active)[child[4 * b + c]]) child[4 * b + c] = -1;
-        for (int64_t b = 0; b < nb; ++b)
-            for (int c = 0; c < 4; ++c)
-                if (child[4 * b + c] >= 0) {
-                    parent[child[4 * b + c]] = (int32_t)b;
-                    quad[child[4 * b + c]] = c;
-                }
-        std::vector<int32_t> ubox, ulvl, unext, uneed, uready;
-        std::vector<int4> uchild;
-        std::vector<int64_t> npar(L + 1, 0), nchild(L + 1, 0);
-        for (int64_t b = 0; b < nb; ++b) {
-            const int l = lev((int)b);
-            if (h.box_leaf[b] >= 0 || l < 2 || l >= L || (active && !(*active)[b])) continue;
-            int cnt = 0;
-            for (int c = 0; c < 4; ++c) cnt += child[4 * b + c] >= 0;
-            if (!cnt) continue;
-            idx[b] = (int32_t)ubox.size();
-            ubox.push_back((int32_t)b);
-            ulvl.push_back(l);
-            uchild.push_back(make_int4(child[4 * b], child[4 * b + 1], child[4 * b + 2], child[4 * b + 3]));
-            npar[l] += 1;
-            nchild[l] += cnt;
+    cudaStream_t cs = ctx->stream;
+    std::vector<int32_t> child(4 * nb);
+    MH_CUDA(ctx, cudaMemcpyAsync(child.data(), t->box_child.p, 4 * nb * 4, cudaMemcpyDeviceToHost, cs));
+    MH_CUDA(ctx, cudaStreamSynchronize(cs));
+    std::unique_ptr<LevelChain> ch(new LevelChain());
+    std::vector<int32_t> box;
+    std::vector<int4> kids;
+    ch->first.assign(L + 1, 0);
+    std::vector<char> used(L + 1, 0);
+    // boxes are ordered by level, so the tasks of a level are contiguous
+    for (int64_t b = 0; b < nb; ++b) {
+        const int l = h.boxes[3 * b];
+        if (h.box_leaf[b] >= 0 || l < 2 || l >= L || (active && !(*active)[b])) continue;
+        int k[4], cnt = 0;
+        for (int c = 0; c < 4; ++c) {
+            k[c] = child[4 * b + c];
+            if (k[c] >= 0 && active && !(*active)[k[c]]) k[c] = -1;   // zero expansions, no use
+            cnt += k[c] >= 0;
         }
-        for (int l = 2; l < L; ++l)
-            if (npar[l]) {
-                ch->flops += 2.0 * P * P * nchild[l];
-                ch->bytes += 8.0 * (4.0 * P * P + 2.0 * P * (nchild[l] + npar[l]));
-            }
-        const int64_t ni = (int64_t)ubox.size();
-        ch->n_int = ni;
-        unext.assign(ni, -1);
-        uneed.assign(ni, 0);
-        // downward blocks: internal boxes with leaf children, each with its internal ancestors
-        std::vector<int32_t> doff{0}, dbox, dop, dlop;
-        std::vector<int4> dleaf;
-        for (int64_t i = 0; i < ni; ++i) {
-            const int b = ubox[i];
-            if (parent[b] >= 0 && idx[parent[b]] >= 0) unext[i] = idx[parent[b]];
-            int leaves[4] = {-1, -1, -1, -1};
-            bool any_leaf = false;
-            for (int c = 0; c < 4; ++c) {
-                const int cb = child[4 * b + c];
-                if (cb < 0) continue;
-                if (idx[cb] >= 0)
-                    uneed[i] += 1;
-                else if (h.box_leaf[cb] >= 0) {
-                    leaves[c] = cb;
-                    any_leaf = true;
-                }
-            }
-            if (uneed[i] == 0) uready.push_back((int32_t)i);
-            if (!any_leaf) continue;
-            std::vector<int32_t> path{b};
-            while (parent[path.back()] >= 0 && idx[parent[path.back()]] >= 0) path.push_back(parent[path.back()]);
-            for (size_t k = path.size(); k-- > 0;) {
-                const int e = path[k];
-                dbox.push_back(e);
-                dop.push_back(k + 1 == path.size() ? -1 : lev(parent[e]) * 4 + quad[e]);
-            }
-            doff.push_back((int32_t)dbox.size());
-            dleaf.push_back(make_int4(leaves[0], leaves[1], leaves[2], leaves[3]));
-            dlop.push_back(ulvl[i] * 4);
-        }
-        ch->n_ready = (int64_t)uready.size();
-        ch->n_down = (int64_t)dleaf.size();
-        // operators, transposed per (level, child position)
-        const size_t PP = (size_t)P * P;
-        std::vector<double> tm((size_t)L * 4 * PP, 0.0), tl((size_t)L * 4 * PP, 0.0);
-        for (int l = 2; l < L; ++l) {
-            if (!npar[l]) continue;
-            for (int c = 0; c < 4; ++c) {
-                const double* om = pool.data.data() + pool.off[op_m2m[l][c]];
-                const double* ol = pool.data.data() + pool.off[op_l2l[l][c]];
-                for (int r = 0; r < P; ++r)
-                    for (int cc = 0; cc < P; ++cc) {
-                        tm[(l * 4 + c) * PP + (size_t)cc * P + r] = om[(size_t)r * P + cc];
-                        tl[(l * 4 + c) * PP + (size_t)cc * P + r] = ol[(size_t)r * P + cc];
-                    }
-            }
-        }
-        std::vector<float> tm32(tm.begin(), tm.end()), tl32(tl.begin(), tl.end());
-        cudaStream_t cs = ctx->stream;
-        auto up_i = [&](dbuf<int32_t>& d, const std::vector<int32_t>& v) -> mh_status {
-            MH_ALLOC(ctx, d, std::max<size_t>(v.size(), 1));
-            if (!v.empty()) MH_CUDA(ctx, cudaMemcpyAsync(d.p, v.data(), v.size() * 4, cudaMemcpyHostToDevice, cs));
-            return MH_OK;
-        };
-        auto up_4 = [&](dbuf<int4>& d, const std::vector<int4>& v) -> mh_status {
-            MH_ALLOC(ctx, d, std::max<size_t>(v.size(), 1));
-            if (!v.empty()) MH_CUDA(ctx, cudaMemcpyAsync(d.p, v.data(), v.size() * 16, cudaMemcpyHostToDevice, cs));
-            return MH_OK;
-        };
-        MH_TRY(up_i(ch->up_box, ubox));
-        MH_TRY(up_i(ch->up_lvl, ulvl));
-        MH_TRY(up_i(ch->up_next, unext));
-        MH_TRY(up_i(ch->up_need, uneed));
-        MH_TRY(up_i(ch->up_ready, uready));
-        MH_TRY(up_4(ch->up_child, uchild));
-        MH_TRY(up_i(ch->dn_off, doff));
-        MH_TRY(up_i(ch->dn_box, dbox));
-        MH_TRY(up_i(ch->dn_op, dop));
-        MH_TRY(up_i(ch->dn_lop, dlop));
-        MH_TRY(up_4(ch->dn_leaf, dleaf));
-        MH_ALLOC(ctx, ch->up_cnt, std::max<int64_t>(ni, 1));
-        MH_CUDA(ctx, cudaMemsetAsync(ch->up_cnt.p, 0, std::max<int64_t>(ni, 1) * sizeof(unsigned), cs));
-        MH_ALLOC(ctx, ch->m2m32, tm32.size());
-        MH_ALLOC(ctx, ch->l2l32, tl32.size());
-        MH_ALLOC(ctx, ch->m2m64, tm.size());
-        MH_ALLOC(ctx, ch->l2l64, tl.size());
-        MH_CUDA(ctx, cudaMemcpyAsync(ch->m2m32.p, tm32.data(), tm32.size() * 4, cudaMemcpyHostToDevice, cs));
-        MH_CUDA(ctx, cudaMemcpyAsync(ch->l2l32.p, tl32.data(), tl32.size() * 4, cudaMemcpyHostToDevice, cs));
-        MH_CUDA(ctx, cudaMemcpyAsync(ch->m2m64.p, tm.data(), tm.size() * 8, cudaMemcpyHostToDevice, cs));
-        MH_CUDA(ctx, cudaMemcpyAsync(ch->l2l64.p, tl.data(), tl.size() * 8, cudaMemcpyHostToDevice, cs));
-        MH_CUDA(ctx, cudaStreamSynchronize(cs));
-        *out = std::move(ch);
+        if (!cnt) continue;
+        box.push_back((int32_t)b);
+        kids.push_back(make_int4(k[0], k[1], k[2], k[3]));
+        ch->first[l + 1] += 1;
+        used[l] = 1;
+        ch->flops += 2.0 * P * P * cnt;
+        ch->bytes += 8.0 * 2.0 * P * (cnt + 1);
     }
+    for (int l = 0; l < L; ++l) {
+        ch->first[l + 1] += ch->first[l];
+        if (used[l]) ch->bytes += 8.0 * 4.0 * P * P;
+    }
+    // operators, transposed per (level, child position)
+    const size_t PP = (size_t)P * P;
+    std::vector<double> tm((size_t)std::max(L, 1) * 4 * PP, 0.0), tl((size_t)std::max(L, 1) * 4 * PP, 0.0);
+    for (int l = 2; l < L; ++l) {
+        if (!used[l]) continue;
+        for (int c = 0; c < 4; ++c) {
+            const double* om = pool.data.data() + pool.off[op_m2m[l][c]];
+            const double* ol = pool.data.data() + pool.off[op_l2l[l][c]];
+            for (int r = 0; r < P; ++r)
+                for (int cc = 0; cc < P; ++cc) {
+                    tm[(l * 4 + c) * PP + (size_t)cc * P + r] = om[(size_t)r * P + cc];
+                    tl[(l * 4 + c) * PP + (size_t)cc * P + r] = ol[(size_t)r * P + cc];
+                }
+        }
+    }
+    std::vector<float> tm32(tm.begin(), tm.end()), tl32(tl.begin(), tl.end());
+    MH_ALLOC(ctx, ch->box, std::max<size_t>(box.size(), 1));
+    MH_ALLOC(ctx, ch->child, std::max<size_t>(kids.size(), 1));
+    if (!box.empty()) {
+        MH_CUDA(ctx, cudaMemcpyAsync(ch->box.p, box.data(), box.size() * 4, cudaMemcpyHostToDevice, cs));
+        MH_CUDA(ctx, cudaMemcpyAsync(ch->child.p, kids.data(), kids.size() * 16, cudaMemcpyHostToDevice, cs));
+    }
+    MH_ALLOC(ctx, ch->m2m32, tm32.size());
+    MH_ALLOC(ctx, ch->l2l32, tl32.size());
+    MH_ALLOC(ctx, ch->m2m64, tm.size());
+    MH_ALLOC(ctx, ch->l2l64, tl.size());
+    MH_CUDA(ctx, cudaMemcpyAsync(ch->m2m32.p, tm32.data(), tm32.size() * 4, cudaMemcpyHostToDevice, cs));
+    MH_CUDA(ctx, cudaMemcpyAsync(ch->l2l32.p, tl32.data(), tl32.size() * 4, cudaMemcpyHostToDevice, cs));
+    MH_CUDA(ctx, cudaMemcpyAsync(ch->m2m64.p, tm.data(), tm.size() * 8, cudaMemcpyHostToDevice, cs));
+    MH_CUDA(ctx, cudaMemcpyAsync(ch->l2l64.p, tl.data(), tl.size() * 8, cudaMemcpyHostToDevice, cs));
+    MH_CUDA(ctx, cudaStreamSynchronize(cs));
+    MH_CUDA(ctx, cudaFuncSetAttribute(k_level_up<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, CHAIN_SMEM_MAX));
+    MH_CUDA(ctx, cudaFuncSetAttribute(k_level_down<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, CHAIN_SMEM_MAX));
+    MH_CUDA(ctx, cudaFuncSetAttribute(k_level_up<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, CHAIN_SMEM_MAX));
+    MH_CUDA(ctx, cudaFuncSetAttribute(k_level_down<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, CHAIN_SMEM_MAX));
+    if (chain_smem(P, 8) > CHAIN_SMEM_MAX)
+        return mh_fail(ctx, MH_ERR_INVALID_ARG, "multipole order too large for the level kernels");
+    *out = std::move(ch);
     return MH_OK;
 }
 
+// Build every operator and pass of the multipole method for (tree, alpha, p).
 mh_status volume_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, VolData* V) {
     const int q = t->q, qq = q * q, P = 2 * p + 1, L = t->max_level;
     const double k = 1.0 / alpha, pref = 1.0 / (2.0 * MH_PI * alpha * alpha);
@@ -1441,6 +1364,11 @@ mh_status volume_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, VolData* V)
     MH_TRY(build_phase(ctx, t_p2m, P, false, V->op_C, V->p2m.get(), &need, &rg));
     V->m2l.reset(new Phase());
     MH_TRY(build_phase(ctx, t_m2l, P, false, V->op_C, V->m2l.get(), &need, &rg));
+    {
+        std::vector<char> has(nb, 0);
+        for (const Task& tk : t_m2l) has[(tk.dst - V->L_off) / P] = 1;
+        for (int64_t b = 0; b < nb; ++b) V->local_cover = V->local_cover && (lev((int)b) < 2 || has[b]);
+    }
     // U^h = near (U list, written first) + far (L2P, M2P: added once the passes are done)
     {
         std::vector<char> has(t->n_leaves, 0);
@@ -1547,8 +1475,8 @@ __device__ __forceinline__ void near_finish(double acc, bool act, int qq, int i,
 }
 
 // Binary64: the staged dipole carries its weight in the normal, the pair term is f(rho) (d . w n)
-// from the table of pair64.cuh; pref holds the factor 1/alpha^2.  Bound by the binary64 pipe (15
-// instructions a pair, 16 cycles each per warp and SM); the four 16-byte table loads of a pair
+// from the table of pair64.cuh; pref holds the factor 1/alpha^2.  Bound by the binary64 pipe (12
+// instructions a pair, 16 cycles each per warp and SM); the three 16-byte table loads of a pair
 // run beside them from L1 (the threads of a warp share the dipole, so their bins are close).
 __global__ void __launch_bounds__(NEAR_T) k_dip_near64(
     const double* __restrict__ nodes, const NearChunk* __restrict__ chunks, const int2* __restrict__ leaf_red,
@@ -1661,7 +1589,7 @@ struct DipData {
     dbuf<int64_t> d_op_off;
     dbuf<int32_t> d_op_C;
     std::unique_ptr<Phase> p2m, m2l, out;
-    std::unique_ptr<DfChain> chain_up;     // M2M over the boxes that hold dipoles
+    std::unique_ptr<LevelChain> chain_up;     // M2M over the boxes that hold dipoles
     SideStream side;                       // the near field runs there beside the passes
     TcImages tc;                           // tensor-core images (mixed precision)
 };
@@ -1988,7 +1916,7 @@ mh_status volume_dipole_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, cons
         MH_ALLOC(ctx, D->leaf_c, nl);
         MH_ALLOC(ctx, D->dxy, std::max<int64_t>(nd, 1));
         MH_ALLOC(ctx, D->dnrm, std::max<int64_t>(nd, 1));
-        MH_ALLOC(ctx, D->ptab, 4 * PT_BINS);
+        MH_ALLOC(ctx, D->ptab, PT_WORDS * PT_BINS);
         k_pair_table<<<(PT_BINS + 127) / 128, 128, 0, st>>>(mh_pair_tab_make(nullptr, alpha), alpha, D->ptab.p);
         MH_LAUNCHED(ctx);
         if (!ch.empty())
@@ -2168,7 +2096,7 @@ struct BieData {
     dbuf<int32_t> perm;   // sorted position -> node
     dbuf<int32_t> slot;   // node -> output slot (from T_off)
     std::unique_ptr<Phase> p2m, m2l, out;
-    std::unique_ptr<DfChain> chain;   // M2M / L2L over the active boxes (own arrival counters)
+    std::unique_ptr<LevelChain> chain;   // M2M / L2L over the active boxes
 };
 
 // Angular part of an expansion row in the real form: v0 at n = 0, then 2 v_n cos(n th) and
@@ -2398,6 +2326,8 @@ static mh_status volume_passes(mh_ctx* ctx, VolData* V, const TOP* ops) {
     MH_TRY(run_phase(ctx, V, ops, V->p2m.get()));
     MH_TRY(run_chain<TOP>(ctx, V->chain.get(), V->P, V->M_off, V->L_off, pool, true, "volume_chain"));
     if (sizeof(TOP) == 4) MH_TRY(tc_split(ctx, V->tc, 1, V->vec32.p));   // multipoles final
+    if (!V->local_cover)   // the downward chain adds into the locals: those without an M2L task start at zero
+        MH_CUDA(ctx, cudaMemsetAsync(pool + V->L_off, 0, (V->vec_len - V->L_off) * sizeof(TOP), ctx->stream));
     MH_TRY(run_phase(ctx, V, ops, V->m2l.get()));
     MH_TRY(run_chain<TOP>(ctx, V->chain.get(), V->P, V->M_off, V->L_off, pool, false, "volume_chain"));
     if (sizeof(TOP) == 4) MH_TRY(tc_split(ctx, V->tc, 2, V->vec32.p));   // locals final
