@@ -1745,7 +1745,7 @@ __global__ void k_dlp_line(const int32_t* __restrict__ line_tgt, const int32_t* 
 // form).  All binary64.
 
 // Alpert node weights of row j (the first half of k_assemble_alpert, kept per row):
-// cp[j][p] = (1/pi) h w_m |y'(t)| K(y(t), x_j) at t = t_j + s x_m h, s = +1 (p < l) or -1.
+// cp[p][j] = (1/pi) h w_m |y'(t)| K(y(t), x_j) at t = t_j + s x_m h, s = +1 (p < l) or -1.
 __global__ void k_alpert_weights(const double* __restrict__ geo, const double* __restrict__ coef,
                                  const int32_t* __restrict__ curve_of, const int32_t* __restrict__ nn,
                                  const int32_t* __restrict__ off, double inv_alpha, AlpertRule R,
@@ -1766,7 +1766,7 @@ __global__ void k_alpert_weights(const double* __restrict__ geo, const double* _
         if ((threadIdx.x & 31) == 0) {
             const double spd = sqrt(v[2] * v[2] + v[3] * v[3]);
             const double K = dl_kernel(v[0], v[1], v[3] / spd, -v[2] / spd, gj[0], gj[1], inv_alpha);
-            cp[j * 2 * R.l + p] = (1.0 / MH_PI) * h * R.w[m] * spd * K;
+            cp[(int64_t)p * gridDim.x + j] = (1.0 / MH_PI) * h * R.w[m] * spd * K;
         }
     }
 }
@@ -1778,15 +1778,15 @@ __device__ __forceinline__ int mf_win_node(int jj, int t, int N) {
     return ii < 0 ? ii + N : ii;
 }
 
-// Window weights of row j: win[j][t] = (1/pi) K(y_i, x_j) |y'_i| h for the 2(a - 1) own-curve
+// Window weights of row j: win[t][j] = (1/pi) K(y_i, x_j) |y'_i| h for the 2(a - 1) own-curve
 // nodes i with 0 < |i - j| < a (the trapezoid entries the Alpert rule replaces).
 __global__ void k_mf_window_weights(const double* __restrict__ geo, const int32_t* __restrict__ curve_of,
                                     const int32_t* __restrict__ nn, const int32_t* __restrict__ off, int64_t n,
                                     double inv_alpha, int nw, double* __restrict__ win) {
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (e >= n * nw) return;
-    const int64_t j = e / nw;
-    const int t = (int)(e - j * nw);
+    const int64_t j = e % n;
+    const int t = (int)(e / n);
     const int k = curve_of[j], N = nn[k], o = off[k];
     const double* gj = geo + 8 * j;
     const double* gi = geo + 8 * (int64_t)(o + mf_win_node((int)(j - o), t, N));
@@ -1965,6 +1965,7 @@ __global__ void __launch_bounds__(MF_THREADS) k_mf_shift(const double2* __restri
 __global__ void k_mf_weights(const double* __restrict__ sigma, const double* __restrict__ geo,
                              const int32_t* __restrict__ curve_of, const int32_t* __restrict__ nn, int64_t n,
                              double* __restrict__ w) {
+    mh_dep_wait();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i < n) w[i] = sigma[i] * geo[8 * i + 6] * (2.0 * MH_PI / nn[curve_of[i]]);
 }
@@ -1972,29 +1973,30 @@ __global__ void k_mf_weights(const double* __restrict__ sigma, const double* __r
 // y_j = sigma_j - 2 alpha^2 u_j - (1/pi) W_j + C_j (a > 0), or with the diagonal limit
 // (1/pi) kappa-term h sigma_j in place of W_j and C_j (a = 0).  u_j is the multipole-pass output
 // -(1/(2 pi alpha^2)) sum_{i != j} w_i K(y_i, x_j), so -2 alpha^2 u_j = (1/pi) T_j; the window
-// terms come from the weights of k_mf_window_weights.  One warp per node: the lanes take the
-// 2(a - 1) window terms and the 2l Alpert terms, summed by a fixed-order warp reduction.
-__global__ void k_mf_combine(const double* __restrict__ sigma, const double* __restrict__ u,
-                             const double* __restrict__ geo, const int32_t* __restrict__ curve_of,
-                             const int32_t* __restrict__ nn, const int32_t* __restrict__ off, int64_t n,
-                             double alpha, int a, int l2, const double* __restrict__ win,
-                             const double* __restrict__ cp, const double* __restrict__ S, double* __restrict__ y) {
-    const int64_t j = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (j >= n) return;   // the whole warp
+// terms come from the weights of k_mf_window_weights.  A thread per node, every weight array read
+// along the nodes (a warp per node with a warp reduction took 13 us at 12,288 nodes, two thirds of
+// its binary64 instructions in the reduction).
+__global__ void __launch_bounds__(64) k_mf_combine(
+    const double* __restrict__ sigma, const double* __restrict__ u, const double* __restrict__ geo,
+    const int32_t* __restrict__ curve_of, const int32_t* __restrict__ nn, const int32_t* __restrict__ off, int64_t n,
+    double alpha, int a, int l2, const double* __restrict__ win, const double* __restrict__ cp,
+    const double* __restrict__ S, double* __restrict__ y) {
+    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (j >= n) return;
     const int k = curve_of[j], N = nn[k], o = off[k];
     const int jj = (int)(j - o);
-    double v = 0.0;
+    double v0 = 0.0, v1 = 0.0;
     if (a > 0) {
         const int nw = 2 * (a - 1);
-        for (int t = lane; t < nw; t += 32) v -= win[j * nw + t] * sigma[o + mf_win_node(jj, t, N)];
-    } else if (lane == 0) {
+#pragma unroll 2
+        for (int t = 0; t < nw; ++t) v0 = fma(-win[(int64_t)t * n + j], sigma[o + mf_win_node(jj, t, N)], v0);
+#pragma unroll 4
+        for (int p = 0; p < l2; ++p) v1 = fma(cp[(int64_t)p * n + j], S[(int64_t)p * n + j], v1);
+    } else {
         const double* gj = geo + 8 * j;
-        v = (1.0 / MH_PI) * gj[7] * gj[6] * (2.0 * MH_PI / N) * sigma[j];
+        v0 = (1.0 / MH_PI) * gj[7] * gj[6] * (2.0 * MH_PI / N) * sigma[j];
     }
-    for (int p = lane; p < l2; p += 32) v += cp[j * l2 + p] * S[(int64_t)p * n + j];
-    v = warp_sum(v);
-    if (lane == 0) y[j] = sigma[j] - 2.0 * alpha * alpha * u[j] + v;
+    y[j] = sigma[j] - 2.0 * alpha * alpha * u[j] + (v0 + v1);
 }
 
 // ============================ host side ============================
@@ -2246,7 +2248,7 @@ mh_status bie_apply_mfree(mh_ctx* ctx, mh_boundary* b, const double* x, double* 
     MH_LAUNCHED(ctx);
     MH_TRY(volume_bie_apply(ctx, b->mf_tree, b->mf_w.p, b->mf_u.p));
     if (fork) MH_CUDA(ctx, cudaStreamWaitEvent(st, b->mf_side.join, 0));
-    k_mf_combine<<<mh_grid(n * 32, 256), 256, 0, st>>>(x, b->mf_u.p, b->geo.p, b->d_curve_of.p, b->d_nn.p, b->d_off.p,
+    k_mf_combine<<<mh_grid(n, 64), 64, 0, st>>>(x, b->mf_u.p, b->geo.p, b->d_curve_of.p, b->d_nn.p, b->d_off.p,
                                                        n, b->mf_alpha, a, l2, b->mf_win.p, b->mf_cp.p, b->mf_S.p, y);
     MH_LAUNCHED(ctx);
     return MH_OK;

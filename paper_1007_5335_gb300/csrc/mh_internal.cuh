@@ -350,8 +350,8 @@ struct mh_boundary {
     bool mfree = false;
     mh_tree* mf_tree = nullptr;          // not owned (the problem's tree)
     double mf_alpha = -1.0;
-    dbuf<double> mf_cp;                  // [n][2 l] Alpert node weights (kernel x rule weight x h / pi)
-    dbuf<double> mf_win;                 // [n][2 (a - 1)] own-curve window weights (kernel x |y'| h / pi)
+    dbuf<double> mf_cp;                  // [2 l][n] Alpert node weights (kernel x rule weight x h / pi)
+    dbuf<double> mf_win;                 // [2 (a - 1)][n] own-curve window weights (kernel x |y'| h / pi)
     dbuf<double2> mf_chirp, mf_bh, mf_tw;   // per curve: e^{i pi n^2/N}, transformed chirp filter, twiddles
     dbuf<int64_t> mf_moff;               // per curve: offset of its M_k-entry blocks (twiddles at moff/2)
     dbuf<int32_t> mf_M;                  // per curve: transform length M_k (power of two >= 2 N_k - 1)

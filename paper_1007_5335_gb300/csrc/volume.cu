@@ -27,6 +27,7 @@
 #include <map>
 #include <memory>
 #include <tuple>
+#include <type_traits>
 
 #include "bessel.cuh"
 #include <cooperative_groups.h>
@@ -276,6 +277,7 @@ __global__ void k_apply(const TOP* __restrict__ ops, const int64_t* __restrict__
                         const int32_t* __restrict__ chunk_t0, const int64_t* __restrict__ task_src,
                         const TOP* src, int R, TOP* __restrict__ temp, const int64_t* __restrict__ task_dst,
                         int accumulate, TD* dst) {
+    mh_dep_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     TOP* sA = reinterpret_cast<TOP*>(smem_raw);
     const int ch = blockIdx.x;
@@ -474,6 +476,7 @@ template <typename TT, typename TD>
 __global__ void k_reduce(const TT* __restrict__ temp, int R, const int64_t* __restrict__ dst_off,
                          const int32_t* __restrict__ dst_ptr, const int32_t* __restrict__ dst_task, int64_t n_dst,
                          int accumulate, TD* dst) {
+    mh_dep_wait();
     const int64_t d = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (d >= n_dst) return;
@@ -499,6 +502,177 @@ __global__ void k_reduce(const TT* __restrict__ temp, int R, const int64_t* __re
                 y[r] = (TD)(accumulate ? (float)y[r] + (hi + lo) : hi + lo);
         }
     }
+}
+
+// ---- one output vector from many single columns ----
+// y = sum_c a_c x[src_c] with R-vectors a_c of its own: the dipole P2M of a leaf, the dipole P2L
+// of a box, the whole output of 16 boundary nodes of the matrix-free operator.  Every entry of the
+// operator is used once, so the work is the stream of the a_c, and in binary64 the products.  The
+// columns are stored as they are read (a_c contiguous): thread (g, r) of a block takes row r
+// of every G-th column, the G partial sums meet in shared memory at the end.  As contraction tasks with
+// one source vector each (a warp per row, lanes over the columns) a row of 64 columns cost 2 products
+// and 6 instructions of reduction, and the products of an output went through memory and a second
+// kernel: matrix-free solve at 12,288 nodes (14 products) 5.72 ms.
+// Outputs of more than COL_CHUNK columns are cut; the last block of an output to finish adds the
+// parts in order.
+constexpr int COL_CHUNK = 256;
+
+struct ColChunk {
+    int32_t out;        // output
+    int32_t slot;       // partial-sum slot, -1 for an output in one chunk
+    int64_t c0, c1;     // columns
+};
+
+__device__ __forceinline__ void col_add(double& s, double& lo, double a, double x) { s = fma(a, x, s); }
+__device__ __forceinline__ void col_add(float& s, float& lo, float a, float x) {   // float-float sum
+    const float v = a * x, t = s + v, bb = t - s;
+    lo += (s - (t - bb)) + (v - bb);
+    s = t;
+}
+
+// Row r of output o goes to dst[at[o] + r] (added when accumulate is set) or, with `row`, to
+// dst[row[o R + r]] (row < 0: none).
+template <typename T>
+__global__ void __launch_bounds__(256) k_cols(const T* __restrict__ ops, const int32_t* __restrict__ src,
+                                              const ColChunk* __restrict__ chunks, const int2* __restrict__ out_red,
+                                              const int64_t* __restrict__ at, const int32_t* __restrict__ row, int R,
+                                              const T* vec, T* part, unsigned* cnt, int accumulate, T* dst) {
+    mh_dep_wait();
+    __shared__ T red[256];
+    __shared__ int last;
+    const ColChunk ch = chunks[blockIdx.x];
+    const int G = 256 / R, r = threadIdx.x % R, g = threadIdx.x / R;
+    T s0 = 0, l0 = 0, s1 = 0, l1 = 0;
+    if (g < G) {
+        int64_t c = ch.c0 + g;
+        for (; c + 3 * G < ch.c1; c += 4 * G) {
+            T a[4], x[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                a[u] = ops[(c + u * G) * R + r];
+                x[u] = vec[src[c + u * G]];
+            }
+            col_add(s0, l0, a[0], x[0]);
+            col_add(s1, l1, a[1], x[1]);
+            col_add(s0, l0, a[2], x[2]);
+            col_add(s1, l1, a[3], x[3]);
+        }
+        for (; c < ch.c1; c += G) col_add(s0, l0, ops[c * R + r], vec[src[c]]);
+    }
+    red[threadIdx.x] = (s0 + s1) + (l0 + l1);
+    __syncthreads();
+    T t = 0;
+    if (threadIdx.x < R)
+        for (int q = 0; q < G; ++q) t += red[q * R + r];
+    if (ch.slot >= 0) {
+        const int2 o = out_red[ch.out];   // {first slot, chunks}
+        if (threadIdx.x < R) part[(int64_t)ch.slot * R + r] = t;
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(cnt + ch.out, 1u) == (unsigned)(o.y - 1);
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        t = 0;
+        if (threadIdx.x < R)
+            for (int q = 0; q < o.y; ++q) t += __ldcg(part + (int64_t)(o.x + q) * R + r);
+        if (threadIdx.x == 0) cnt[ch.out] = 0u;
+    }
+    if (threadIdx.x >= R) return;
+    if (row) {
+        const int32_t i = row[(int64_t)ch.out * R + r];
+        if (i >= 0) dst[i] = t;
+    } else {
+        T* y = dst + at[ch.out] + r;
+        *y = accumulate ? *y + t : t;
+    }
+}
+
+// Host side: outputs are opened in turn and columns added to the open one.
+struct ColBuild {
+    int R = 0;
+    std::vector<double> a;
+    std::vector<int32_t> src, row;
+    std::vector<int64_t> at, first{0};
+    explicit ColBuild(int rows) : R(rows) {}
+    void open(int64_t dst) { at.push_back(dst); }
+    // nc columns of the R x nc row-major matrix m, sources src0, src0 + 1, ...
+    void add(int nc, const std::vector<double>& m, int64_t src0) {
+        for (int c = 0; c < nc; ++c) {
+            for (int r = 0; r < R; ++r) a.push_back(m[(size_t)r * nc + c]);
+            src.push_back((int32_t)(src0 + c));
+        }
+    }
+    void close() { first.push_back((int64_t)src.size()); }
+};
+
+struct ColSet {
+    int R = 0;
+    int64_t n = 0;              // outputs
+    int64_t n_chunks = 0;
+    double flops = 0, bytes = 0;
+    dbuf<double> ops64, part;   // part: sized in binary64 words, room for either type
+    dbuf<float> ops32;
+    dbuf<int32_t> src, row;
+    dbuf<ColChunk> chunks;
+    dbuf<int2> out_red;
+    dbuf<int64_t> at;
+    dbuf<unsigned> cnt;
+};
+
+mh_status build_cols(mh_ctx* ctx, const ColBuild& b, bool both, ColSet* S) {
+    S->R = b.R;
+    S->n = (int64_t)b.first.size() - 1;
+    if (S->n == 0) return MH_OK;
+    std::vector<ColChunk> ch;
+    std::vector<int2> red(S->n, make_int2(0, 1));
+    int32_t slots = 0;
+    for (int64_t i = 0; i < S->n; ++i) {
+        const int64_t c0 = b.first[i], nc = b.first[i + 1] - c0, k = std::max<int64_t>(1, (nc + COL_CHUNK - 1) / COL_CHUNK);
+        red[i] = make_int2(k > 1 ? slots : 0, (int)k);
+        for (int64_t q = 0; q < k; ++q)
+            ch.push_back(ColChunk{(int32_t)i, k > 1 ? slots + (int32_t)q : -1, c0 + nc * q / k, c0 + nc * (q + 1) / k});
+        if (k > 1) slots += (int32_t)k;
+    }
+    std::stable_sort(ch.begin(), ch.end(),
+                     [](const ColChunk& x, const ColChunk& y) { return x.c1 - x.c0 > y.c1 - y.c0; });
+    S->n_chunks = (int64_t)ch.size();
+    S->flops = 2.0 * b.R * (double)b.src.size();
+    S->bytes = 8.0 * (b.R + 1) * (double)b.src.size() + 8.0 * b.R * S->n;
+    cudaStream_t st = ctx->stream;
+    auto up = [&](auto& d, const auto& v) -> mh_status {
+        MH_ALLOC(ctx, d, std::max<size_t>(v.size(), 1));
+        if (!v.empty()) MH_CUDA(ctx, cudaMemcpyAsync(d.p, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice, st));
+        return MH_OK;
+    };
+    MH_TRY(up(S->ops64, b.a));
+    if (both) {
+        std::vector<float> f(b.a.begin(), b.a.end());
+        MH_TRY(up(S->ops32, f));
+        MH_CUDA(ctx, cudaStreamSynchronize(st));
+    }
+    MH_TRY(up(S->src, b.src));
+    MH_TRY(up(S->chunks, ch));
+    MH_TRY(up(S->out_red, red));
+    MH_TRY(up(S->at, b.at));
+    if (!b.row.empty()) MH_TRY(up(S->row, b.row));
+    MH_ALLOC(ctx, S->part, std::max<int64_t>((int64_t)slots * b.R, 1));
+    MH_ALLOC(ctx, S->cnt, S->n);
+    MH_CUDA(ctx, cudaMemsetAsync(S->cnt.p, 0, S->n * sizeof(unsigned), st));
+    MH_CUDA(ctx, cudaStreamSynchronize(st));
+    return MH_OK;
+}
+
+template <typename T>
+mh_status run_cols(mh_ctx* ctx, const ColSet& S, const T* vec, T* dst, bool accumulate, const char* region) {
+    if (S.n_chunks == 0) return MH_OK;
+    prof_scope ps(ctx, region, S.flops, S.bytes);
+    const T* ops = sizeof(T) == 4 ? reinterpret_cast<const T*>(S.ops32.p) : reinterpret_cast<const T*>(S.ops64.p);
+    (void)mh_launch_dep(ctx->stream, k_cols<T>, dim3((unsigned)S.n_chunks), dim3(256), 0, ops, S.src.p, S.chunks.p,
+                        S.out_red.p, S.at.p, S.row.p, S.R, vec, reinterpret_cast<T*>(S.part.p), S.cnt.p,
+                        accumulate ? 1 : 0, dst);
+    MH_LAUNCHED(ctx);
+    return MH_OK;
 }
 
 // ---------------- host structures ----------------
@@ -847,7 +1021,7 @@ inline float* typed_pool<float>(dbuf<double>&, dbuf<float>& v32) { return v32.p;
 template <typename TOP>
 mh_status run_phase_on(mh_ctx* ctx, const TOP* ops, const int64_t* op_off, const int32_t* op_C, TOP* pool,
                        double* out, double* temp, const Phase* ph, const char* region,
-                       const TcImages* tc = nullptr) {
+                       const TcImages* tc = nullptr, bool dep = false) {
     if (ph->n_tasks == 0) return MH_OK;
     const int smem = (int)(ph->smem / sizeof(double) * sizeof(TOP));
     // binary32 with images: the leading operators on the tensor cores, the rest on the CUDA cores
@@ -885,30 +1059,31 @@ mh_status run_phase_on(mh_ctx* ctx, const TOP* ops, const int64_t* op_off, const
                       ph->tc_flops, ph->tc_bytes);
         MH_TRY(tc_contract_launch(ctx, a));
     }
+    // the first launch is a dependent one when the caller says that a kernel precedes it directly
+    auto apply = [&](auto* dst) -> mh_status {
+        using TD = std::remove_pointer_t<decltype(dst)>;
+        if (ncc) {
+            const auto kern = k_apply<TOP, TD>;
+            const int32_t *op = ph->chunk_op.p + c0, *t0 = ph->chunk_t0.p + c0;
+            if (dep || on_tc)
+                (void)mh_launch_dep(ctx->stream, kern, dim3(ncc), dim3(256), smem, ops, op_off, op_C, op, t0, ph->task_src.p,
+                                    pool, ph->R, tmp, tdst, acc, dst);
+            else
+                kern<<<ncc, 256, smem, ctx->stream>>>(ops, op_off, op_C, op, t0, ph->task_src.p, pool, ph->R, tmp, tdst,
+                                                      acc, dst);
+            MH_LAUNCHED(ctx);
+        }
+        if (!ph->direct) {
+            (void)mh_launch_dep(ctx->stream, k_reduce<TOP, TD>, dim3(rg), dim3(256), 0, tmp, ph->R, ph->dst_off.p,
+                                ph->dst_ptr.p, ph->dst_task.p, ph->n_dst, acc, dst);
+            MH_LAUNCHED(ctx);
+        }
+        return MH_OK;
+    };
     if (ph->dst_out) {
-        if (ncc) {
-            k_apply<TOP, double><<<ncc, 256, smem, ctx->stream>>>(ops, op_off, op_C, ph->chunk_op.p + c0,
-                                                                  ph->chunk_t0.p + c0, ph->task_src.p, pool, ph->R,
-                                                                  tmp, tdst, acc, out);
-            MH_LAUNCHED(ctx);
-        }
-        if (!ph->direct) {
-            k_reduce<TOP, double><<<rg, 256, 0, ctx->stream>>>(tmp, ph->R, ph->dst_off.p, ph->dst_ptr.p,
-                                                               ph->dst_task.p, ph->n_dst, acc, out);
-            MH_LAUNCHED(ctx);
-        }
+        MH_TRY(apply(out));
     } else {
-        if (ncc) {
-            k_apply<TOP, TOP><<<ncc, 256, smem, ctx->stream>>>(ops, op_off, op_C, ph->chunk_op.p + c0,
-                                                               ph->chunk_t0.p + c0, ph->task_src.p, pool, ph->R, tmp,
-                                                               tdst, acc, pool);
-            MH_LAUNCHED(ctx);
-        }
-        if (!ph->direct) {
-            k_reduce<TOP, TOP><<<rg, 256, 0, ctx->stream>>>(tmp, ph->R, ph->dst_off.p, ph->dst_ptr.p,
-                                                            ph->dst_task.p, ph->n_dst, acc, pool);
-            MH_LAUNCHED(ctx);
-        }
+        MH_TRY(apply(pool));
     }
     return MH_OK;
 }
@@ -1588,7 +1763,8 @@ struct DipData {
     dbuf<float> ops32, vec32;              // vec32: binary32 mirror of vec (weights, expansions)
     dbuf<int64_t> d_op_off;
     dbuf<int32_t> d_op_C;
-    std::unique_ptr<Phase> p2m, m2l, out;
+    ColSet p2m, p2l;                       // dipole P2M of the leaves, dipole P2L over the X lists
+    std::unique_ptr<Phase> m2l, out;
     std::unique_ptr<LevelChain> chain_up;     // M2M over the boxes that hold dipoles
     SideStream side;                       // the near field runs there beside the passes
     TcImages tc;                           // tensor-core images (mixed precision)
@@ -1698,10 +1874,10 @@ std::vector<char> dipole_active_boxes(const HostTree& h, const std::vector<int64
 // tasks are made only from active sources (the other multipoles are zero, so leaving them out
 // changes no sum), and with `dst_active_only` (the targets are the dipoles themselves) M2L and
 // P2L tasks only into active boxes (the other locals are never evaluated).
-void dipole_source_tasks(const DipGeo& G, const VolData* V, OpPool& pool, int p, double k, double pref,
+void dipole_source_tasks(const DipGeo& G, const VolData* V, int p, double k, double pref,
                          const double* dxy, const double* dnrm, const std::vector<int64_t>& seg0,
                          const std::vector<int64_t>& segn, int64_t W_off, int64_t DM_off, int64_t DL_off,
-                         std::vector<Task>& t_p2m, std::vector<Task>& t_m2l,
+                         ColBuild& p2m, ColBuild& p2l, std::vector<Task>& t_m2l,
                          const std::vector<char>* active = nullptr, bool dst_active_only = false) {
     const HostTree& h = *G.h;
     const int P = 2 * p + 1;
@@ -1727,7 +1903,9 @@ void dipole_source_tasks(const DipGeo& G, const VolData* V, OpPool& pool, int p,
                     dip_set_row(buf.data(), nc, j, n, pref * Dn / G.Is[l][n]);
                 }
             }
-            dip_add_split(pool, P, nc, buf, W_off + seg0[leaf], DM_off + b * P, t_p2m);
+            p2m.open(DM_off + b * P);
+            p2m.add(nc, buf, W_off + seg0[leaf]);
+            p2m.close();
         }
         if (active && dst_active_only && !(*active)[b]) continue;
         for (int j = h.off[1][b]; j < h.off[1][b + 1]; ++j) {
@@ -1737,6 +1915,7 @@ void dipole_source_tasks(const DipGeo& G, const VolData* V, OpPool& pool, int p,
             t_m2l.push_back(Task{V->m2l_key.at(key), DM_off + (int64_t)s2 * P, DL_off + b * P});
         }
         // X list: dipole P2L
+        bool any = false;
         for (int j = h.off[3][b]; j < h.off[3][b + 1]; ++j) {
             const int c = h.item[3][j];
             const int lc = h.box_leaf[c];
@@ -1755,8 +1934,11 @@ void dipole_source_tasks(const DipGeo& G, const VolData* V, OpPool& pool, int p,
                     dip_set_row(buf.data(), nc, jj, m, G.Is[l][m] * pref * Dm);
                 }
             }
-            dip_add_split(pool, P, nc, buf, W_off + seg0[lc], DL_off + b * P, t_m2l);
+            if (!any) p2l.open(DL_off + b * P);
+            any = true;
+            p2l.add(nc, buf, W_off + seg0[lc]);
         }
+        if (any) p2l.close();
     }
 }
 
@@ -1796,12 +1978,15 @@ mh_status volume_dipole_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, cons
     D->DU_off = D->DL_off + nb * P;
     D->vec_len = D->DU_off + nl * qq;
     OpPool pool = V->pool_host;
-    std::vector<Task> t_p2m, t_m2l, t_out;
+    std::vector<Task> t_m2l, t_out;
+    ColBuild p2m(P), p2l(P);
     // multipoles are non-zero only in boxes that hold dipoles: M2L from those alone, and the
     // upward chain over those alone (the downward chain serves every leaf: targets everywhere)
     const std::vector<char> active = dipole_active_boxes(h, segn);
-    dipole_source_tasks(G, V, pool, p, k, pref, dxy, dnrm, seg0, segn, D->W_off, D->DM_off, D->DL_off, t_p2m, t_m2l,
+    dipole_source_tasks(G, V, p, k, pref, dxy, dnrm, seg0, segn, D->W_off, D->DM_off, D->DL_off, p2m, p2l, t_m2l,
                         &active, false);
+    MH_TRY(build_cols(ctx, p2m, true, &D->p2m));
+    MH_TRY(build_cols(ctx, p2l, true, &D->p2l));
     MH_TRY(build_chain(ctx, t, h, P, V->pool_host, V->op_m2m, V->op_l2l, &active, &D->chain_up));
     std::vector<double> buf;
     for (int64_t b = 0; b < nb; ++b) {
@@ -1950,12 +2135,9 @@ mh_status volume_dipole_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, cons
     MH_CUDA(ctx, cudaMemcpyAsync(D->d_op_off.p, pool.off.data(), pool.off.size() * 8, cudaMemcpyHostToDevice, st));
     MH_CUDA(ctx, cudaMemcpyAsync(D->d_op_C.p, pool.C.data(), pool.C.size() * 4, cudaMemcpyHostToDevice, st));
     std::vector<int> opC(pool.C.begin(), pool.C.end());
-    // split ranges of the tensor-core sources: dipole multipoles (DM), locals (DL); the dipole
-    // P2M / P2L operators (one task each, on the weights) stay on the CUDA cores
+    // split ranges of the tensor-core sources: dipole multipoles (DM), locals (DL)
     const std::vector<TcImages::Range> rg = {{D->DM_off, P, nb, 0, 0}, {D->DL_off, P, nb, 0, 0}};
     int64_t need = 1;
-    D->p2m.reset(new Phase());
-    MH_TRY(build_phase(ctx, t_p2m, P, false, opC, D->p2m.get(), &need, &rg));
     D->m2l.reset(new Phase());
     MH_TRY(build_phase(ctx, t_m2l, P, false, opC, D->m2l.get(), &need, &rg));
     D->out.reset(new Phase());
@@ -1964,7 +2146,7 @@ mh_status volume_dipole_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, cons
     {
         std::vector<int64_t> off(pool.off.begin(), pool.off.end());
         std::vector<int32_t> rr(pool.R.begin(), pool.R.end()), cc(pool.C.begin(), pool.C.end());
-        MH_TRY(build_tc_images(ctx, pool.data.data(), off, rr, cc, {D->p2m.get(), D->m2l.get(), D->out.get()}, rg,
+        MH_TRY(build_tc_images(ctx, pool.data.data(), off, rr, cc, {D->m2l.get(), D->out.get()}, rg,
                                &D->tc));
     }
     MH_ALLOC(ctx, D->vec, D->vec_len);
@@ -1987,13 +2169,14 @@ static mh_status dipole_passes(mh_ctx* ctx, VolData* V, DipData* D, const TOP* o
         return run_phase_on<TOP>(ctx, ops, D->d_op_off.p, D->d_op_C.p, pool, D->vec.p, D->temp.p, ph,
                                  "dlp_fmm_contract", &D->tc);
     };
-    MH_TRY(run(D->p2m.get()));
+    MH_TRY(run_cols<TOP>(ctx, D->p2m, pool, pool, false, "dlp_fmm_contract"));
     MH_TRY(run_chain<TOP>(ctx, D->chain_up.get(), V->P, D->DM_off, D->DL_off, pool, true, "dlp_fmm_chain"));
     if (sizeof(TOP) == 4) MH_TRY(tc_split(ctx, D->tc, 0, D->vec32.p));   // multipoles final
     // boxes whose V and X lists hold no dipoles get no M2L / P2L task: their locals are zeroed
     // here, since the downward chain adds into the leaves' locals
     MH_CUDA(ctx, cudaMemsetAsync(pool + D->DL_off, 0, (D->DU_off - D->DL_off) * sizeof(TOP), ctx->stream));
     MH_TRY(run(D->m2l.get()));
+    MH_TRY(run_cols<TOP>(ctx, D->p2l, pool, pool, true, "dlp_fmm_contract"));
     MH_TRY(run_chain<TOP>(ctx, V->chain.get(), V->P, D->DM_off, D->DL_off, pool, false, "dlp_fmm_chain"));
     if (sizeof(TOP) == 4) MH_TRY(tc_split(ctx, D->tc, 1, D->vec32.p));   // locals final
     return MH_OK;
@@ -2088,14 +2271,14 @@ constexpr int BIE_RT = 16;   // targets per output group (rows of every output o
 
 struct BieData {
     int64_t nd = 0, n_groups = 0;
-    int64_t W_off = 0, DM_off = 0, DL_off = 0, T_off = 0, vec_len = 0;
+    int64_t W_off = 0, DM_off = 0, DL_off = 0, vec_len = 0;
     double flops = 0, near_pairs = 0;
     dbuf<double> vec, temp, ops64;
     dbuf<int64_t> d_op_off;
     dbuf<int32_t> d_op_C;
     dbuf<int32_t> perm;   // sorted position -> node
-    dbuf<int32_t> slot;   // node -> output slot (from T_off)
-    std::unique_ptr<Phase> p2m, m2l, out;
+    ColSet p2m, p2l, out;
+    std::unique_ptr<Phase> m2l;
     std::unique_ptr<LevelChain> chain;   // M2M / L2L over the active boxes
 };
 
@@ -2111,14 +2294,9 @@ void bie_row(double* row, int p, const double* v, double th) {
 
 __global__ void k_bie_gather_w(const double* __restrict__ w, const int32_t* __restrict__ perm, int64_t n,
                                double* __restrict__ ws) {
+    mh_dep_wait();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i < n) ws[i] = w[perm[i]];
-}
-
-__global__ void k_bie_scatter_u(const double* __restrict__ t, const int32_t* __restrict__ slot, int64_t n,
-                                double* __restrict__ u) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) u[i] = t[slot[i]];
 }
 
 }  // namespace
@@ -2157,15 +2335,14 @@ mh_status volume_bie_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, const d
     B->W_off = 0;
     B->DM_off = nd;
     B->DL_off = B->DM_off + nb * P;
-    B->T_off = B->DL_off + nb * P;
-    B->vec_len = B->T_off + B->n_groups * BIE_RT;
+    B->vec_len = B->DL_off + nb * P;
     OpPool pool = V->pool_host;
-    std::vector<Task> t_p2m, t_m2l, t_out;
+    std::vector<Task> t_m2l;
+    ColBuild p2m(P), p2l(P), out(BIE_RT);
     const std::vector<char> active = dipole_active_boxes(h, segn);
-    dipole_source_tasks(G, V, pool, p, k, pref, sxy.data(), snrm.data(), seg0, segn, B->W_off, B->DM_off, B->DL_off,
-                        t_p2m, t_m2l, &active, true);
+    dipole_source_tasks(G, V, p, k, pref, sxy.data(), snrm.data(), seg0, segn, B->W_off, B->DM_off, B->DL_off, p2m, p2l,
+                        t_m2l, &active, true);
     MH_TRY(build_chain(ctx, t, h, P, V->pool_host, V->op_m2m, V->op_l2l, &active, &B->chain));
-    std::vector<int32_t> slot(nd);
     std::vector<double> buf, v(p + 2), Kb(p + 3);
     int64_t gi = 0;
     for (int64_t b = 0; b < nb; ++b) {
@@ -2175,12 +2352,12 @@ mh_status volume_bie_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, const d
         const std::complex<double> cb = G.centre((int)b);
         for (int64_t g0 = 0; g0 < segn[lf]; g0 += BIE_RT, ++gi) {
             const int cnt = (int)std::min<int64_t>(BIE_RT, segn[lf] - g0);
-            const int64_t dst = B->T_off + gi * BIE_RT;
+            out.open(0);
             auto tgt = [&](int i) {
                 const int64_t j = seg0[lf] + g0 + i;
                 return std::complex<double>(sxy[2 * j], sxy[2 * j + 1]);
             };
-            for (int i = 0; i < cnt; ++i) slot[perm[seg0[lf] + g0 + i]] = (int32_t)(gi * BIE_RT + i);
+            for (int i = 0; i < BIE_RT; ++i) out.row.push_back(i < cnt ? perm[seg0[lf] + g0 + i] : -1);
             // L2P at the targets
             if (l >= 2) {
                 buf.assign((size_t)BIE_RT * P, 0.0);
@@ -2189,7 +2366,7 @@ mh_status volume_bie_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, const d
                     for (int n = 0; n <= p; ++n) v[n] = h_in(n, k * std::abs(z)) / G.Is[l][n];
                     bie_row(&buf[(size_t)i * P], p, v.data(), std::arg(z));
                 }
-                t_out.push_back(Task{pool.add(BIE_RT, P, buf.data()), B->DL_off + b * P, dst});
+                out.add(P, buf, B->DL_off + b * P);
                 B->flops += 2.0 * BIE_RT * P;
             }
             // W list: M2P at the targets
@@ -2204,7 +2381,7 @@ mh_status volume_bie_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, const d
                     for (int n = 0; n <= p; ++n) v[n] = G.Is[lc][n] * Kb[n];
                     bie_row(&buf[(size_t)i * P], p, v.data(), std::arg(z));
                 }
-                t_out.push_back(Task{pool.add(BIE_RT, P, buf.data()), B->DM_off + (int64_t)c * P, dst});
+                out.add(P, buf, B->DM_off + (int64_t)c * P);
                 B->flops += 2.0 * BIE_RT * P;
             }
             // U list: direct dipole blocks (the leaf itself included; r = 0 is the target's own node)
@@ -2224,10 +2401,11 @@ mh_status volume_bie_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, const d
                                 -pref * h_k1(r * k) * k * (dx * snrm[2 * d] + dy * snrm[2 * d + 1]) / r;
                     }
                 }
-                dip_add_split(pool, BIE_RT, nc, buf, B->W_off + seg0[lc], dst, t_out);
+                out.add(nc, buf, B->W_off + seg0[lc]);
                 B->near_pairs += (double)cnt * nc;
                 B->flops += 2.0 * BIE_RT * nc;
             }
+            out.close();
         }
     }
     cudaStream_t st = ctx->stream;
@@ -2240,22 +2418,18 @@ mh_status volume_bie_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, const d
     MH_CUDA(ctx, cudaMemcpyAsync(B->d_op_C.p, pool.C.data(), pool.C.size() * 4, cudaMemcpyHostToDevice, st));
     std::vector<int> opC(pool.C.begin(), pool.C.end());
     int64_t need = 1;
-    B->p2m.reset(new Phase());
-    MH_TRY(build_phase(ctx, t_p2m, P, false, opC, B->p2m.get(), &need));
+    MH_TRY(build_cols(ctx, p2m, false, &B->p2m));
+    MH_TRY(build_cols(ctx, p2l, false, &B->p2l));
+    MH_TRY(build_cols(ctx, out, false, &B->out));
     B->m2l.reset(new Phase());
     MH_TRY(build_phase(ctx, t_m2l, P, false, opC, B->m2l.get(), &need));
-    B->out.reset(new Phase());
-    MH_TRY(build_phase(ctx, t_out, BIE_RT, false, opC, B->out.get(), &need));
-    B->out->dst_out = true;
-    B->flops += B->p2m->flops + B->m2l->flops;
+    B->flops += B->p2m.flops + B->p2l.flops + B->m2l->flops;
     MH_ALLOC(ctx, B->vec, B->vec_len);
     MH_ALLOC(ctx, B->temp, need);
     MH_CUDA(ctx, cudaMemsetAsync(B->vec.p, 0, B->vec_len * 8, st));
     MH_ALLOC(ctx, B->perm, std::max<int64_t>(nd, 1));
-    MH_ALLOC(ctx, B->slot, std::max<int64_t>(nd, 1));
     if (nd) {
         MH_CUDA(ctx, cudaMemcpyAsync(B->perm.p, perm.data(), nd * 4, cudaMemcpyHostToDevice, st));
-        MH_CUDA(ctx, cudaMemcpyAsync(B->slot.p, slot.data(), nd * 4, cudaMemcpyHostToDevice, st));
     }
     MH_CUDA(ctx, cudaStreamSynchronize(st));
     V->bie = std::move(B);
@@ -2278,20 +2452,19 @@ mh_status volume_bie_apply(mh_ctx* ctx, mh_tree* t, const double* w, double* u) 
     prof_scope ps(ctx, "bie_fmm", B->flops, 0.0);
     cudaStream_t st = ctx->stream;
     const unsigned g = (unsigned)mh_grid(B->nd, 256);
-    k_bie_gather_w<<<g, 256, 0, st>>>(w, B->perm.p, B->nd, B->vec.p + B->W_off);
+    (void)mh_launch_dep(st, k_bie_gather_w, dim3(g), dim3(256), 0, w, B->perm.p, B->nd, B->vec.p + B->W_off);
     MH_LAUNCHED(ctx);
     auto run = [&](const Phase* ph) {
         return run_phase_on<double>(ctx, B->ops64.p, B->d_op_off.p, B->d_op_C.p, B->vec.p, B->vec.p, B->temp.p, ph,
                                     "bie_fmm_contract");
     };
-    MH_TRY(run(B->p2m.get()));
+    MH_TRY(run_cols<double>(ctx, B->p2m, B->vec.p, B->vec.p, false, "bie_fmm_contract"));
     MH_TRY(run_chain<double>(ctx, B->chain.get(), V->P, B->DM_off, B->DL_off, B->vec.p, true, "bie_fmm_chain"));
-    MH_CUDA(ctx, cudaMemsetAsync(B->vec.p + B->DL_off, 0, (B->T_off - B->DL_off) * 8, st));
+    MH_CUDA(ctx, cudaMemsetAsync(B->vec.p + B->DL_off, 0, (B->vec_len - B->DL_off) * 8, st));
     MH_TRY(run(B->m2l.get()));
+    MH_TRY(run_cols<double>(ctx, B->p2l, B->vec.p, B->vec.p, true, "bie_fmm_contract"));
     MH_TRY(run_chain<double>(ctx, B->chain.get(), V->P, B->DM_off, B->DL_off, B->vec.p, false, "bie_fmm_chain"));
-    MH_TRY(run(B->out.get()));
-    k_bie_scatter_u<<<g, 256, 0, st>>>(B->vec.p + B->T_off, B->slot.p, B->nd, u);
-    MH_LAUNCHED(ctx);
+    MH_TRY(run_cols<double>(ctx, B->out, B->vec.p, u, false, "bie_fmm_contract"));
     return MH_OK;
 }
 
