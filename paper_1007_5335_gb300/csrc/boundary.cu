@@ -748,6 +748,7 @@ __global__ void k_prep_fine32(const double* __restrict__ fg, const int64_t* __re
 
 __global__ void k_weights32(const double* __restrict__ sigma, const double* __restrict__ geo,
                             const int32_t* __restrict__ curve_of, const int32_t* __restrict__ nn, int64_t n, float* w) {
+    mh_dep_wait();
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (s < n) w[s] = (float)(sigma[s] * geo[8 * s + 6] * (2.0 * MH_PI / nn[curve_of[s]]));
 }
@@ -768,6 +769,7 @@ __global__ void __launch_bounds__(MH_TILE) k_dlp_coarse32(const double* __restri
                                                           const int32_t* __restrict__ curve_of,
                                                           const double2* __restrict__ tc, const float* __restrict__ tr,
                                                           int64_t ns, mh_dl32 c32, double pref, double* out) {
+    mh_dep_wait();
     __shared__ float4 s4[MH_TILE];
     __shared__ int sk[MH_TILE];
     const float two_a = 2.0001f * c32.a;
@@ -830,12 +832,22 @@ __global__ void __launch_bounds__(MH_TILE) k_dlp_coarse32(const double* __restri
     }
 }
 
-__global__ void k_sum_partials(const double* __restrict__ part, int nsplit, int64_t nt, double pref, double* out) {
-    int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= nt) return;
+// Eight lanes per target, each a share of the splits (a thread per target was a chain of up to 48
+// binary64 additions: 11 us).
+__global__ void k_sum_partials(const double* part, int nsplit, int64_t nt, double pref, double* out) {
+    mh_dep_wait();
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t t = (e >> 8) * 32 + (e & 31);   // a warp reads 32 targets of one share
+    const int g = (int)(e >> 5) & 7;
+    __shared__ double sh[8][33];
     double s = 0.0;
-    for (int j = 0; j < nsplit; ++j) s += part[j * nt + t];
-    out[t] = pref * s;
+    if (t < nt)
+        for (int j = g; j < nsplit; j += 8) s += part[j * nt + t];
+    sh[g][e & 31] = s;
+    __syncthreads();
+    if (g != 0 || t >= nt) return;
+    const int l = (int)(e & 31);
+    out[t] = pref * (((s + sh[1][l]) + (sh[2][l] + sh[3][l])) + ((sh[4][l] + sh[5][l]) + (sh[6][l] + sh[7][l])));
 }
 
 // One warp's pairs of a fine chunk (MH_TILE nodes from f0, m of them present) against TG targets
@@ -897,6 +909,7 @@ __global__ void __launch_bounds__(256) k_dlp_fine32_grp(
     const int64_t* __restrict__ foff, const int64_t* __restrict__ coff, const float4* __restrict__ ccf,
     const float* __restrict__ crad, mh_dl32 c32, float cut_r, double pref, double* part, unsigned* cnt,
     double* out) {
+    mh_dep_wait();
     __shared__ double red[8][TG];
     const float two_a = 2.0001f * c32.a;   // beyond: z > 2 with a margin for the rounding of d2
     __shared__ int last;
@@ -999,6 +1012,7 @@ __global__ void __launch_bounds__(256) k_dlp_fine64_grp(
     const double* __restrict__ xy, const int32_t* __restrict__ pair_tgt, const int32_t* __restrict__ grp_curve,
     const int32_t* __restrict__ grp_pair, int slices, const double* __restrict__ fg, const double* __restrict__ wf,
     const int64_t* __restrict__ foff, mh_pair_tab tab, double pref, double* part, unsigned* cnt, double* out) {
+    mh_dep_wait();
     __shared__ double red[8][TG];
     __shared__ int last;
     const int grp = blockIdx.x / slices, sl = blockIdx.x % slices;
@@ -1525,6 +1539,7 @@ __global__ void __launch_bounds__(256) k_fine_weights_fft(const double* __restri
                                                           const int32_t* __restrict__ off,
                                                           const int64_t* __restrict__ foff, float* __restrict__ wf,
                                                           double* __restrict__ wf64) {
+    mh_dep_wait();
     extern __shared__ __align__(16) unsigned char fft_smem[];   // [N] values, then [N] twiddles
     constexpr int PER = FFT_MAX / 256;   // values per thread when the spectrum is reordered
     const int s = blockIdx.x, k = blockIdx.y;
@@ -1603,6 +1618,7 @@ __global__ void __launch_bounds__(BS) k_dlp_coarse(const double* __restrict__ xy
                                                    const double* __restrict__ sigma,
                                                    const int32_t* __restrict__ curve_of, const int32_t* __restrict__ nn,
                                                    int64_t ns, mh_pair_tab tab, double pref, double* out) {
+    mh_dep_wait();
     __shared__ double2 sp[BS], sn[BS];
     __shared__ int sk[BS];
     const int64_t t = blockIdx.x * (int64_t)BS + threadIdx.x;
@@ -1655,10 +1671,18 @@ __global__ void __launch_bounds__(BS) k_dlp_coarse(const double* __restrict__ xy
 // argument and the half-angle difference of t* and t_j loses it to cancellation.
 __global__ void k_line_weights(const int32_t* __restrict__ line_curve, const double* __restrict__ line_data,
                                int64_t nline, const int32_t* __restrict__ nn, const int32_t* __restrict__ off,
-                               const double2* __restrict__ half, const int64_t* __restrict__ woff, double* w) {
+                               const double2* __restrict__ half, const int64_t* __restrict__ woff, double* w,
+                               double* lag) {
     const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     if (t >= nline) return;
     const int lane = threadIdx.x & 31;
+    if (lane < 5) {   // degree-4 weights in the distance: nodes 0, h_s/4, ..., h_s
+        const double q = line_data[4 * t + 1] / (NEAR_LINE * line_data[4 * t + 2]);
+        double wi = 1.0;
+        for (int j = 0; j < 5; ++j)
+            if (j != lane) wi *= (q - j) / (lane - j);
+        lag[5 * t + lane] = wi;
+    }
     const int k = line_curve[t];
     const int N = nn[k];
     const double ts = line_data[4 * t];   // in [0, 2 pi)
@@ -1687,11 +1711,15 @@ __global__ void k_line_weights(const int32_t* __restrict__ line_curve, const dou
     }
 }
 
+// A sigma is given as asig or, with r, as asig - r (a solver's right-hand side and final residual).
+// out[tgt] = U^h or, with idx, out[idx[tgt]] = base[idx[tgt]] + U^h.
 __global__ void k_dlp_line(const int32_t* __restrict__ line_tgt, const int32_t* __restrict__ line_curve,
-                           const double* __restrict__ line_data, int64_t nline, const double* __restrict__ asig,
+                           const double* __restrict__ lag, int64_t nline, const double* asig, const double* r,
                            const int32_t* __restrict__ nn, const int32_t* __restrict__ off,
                            const double* __restrict__ lw, const int64_t* __restrict__ woff, int64_t n_user,
-                           double alpha, double* out) {
+                           double limit, const double* ext, const double* base, const int32_t* __restrict__ idx,
+                           double* out) {
+    mh_dep_wait();
     const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     if (t >= nline) return;
     const int lane = threadIdx.x & 31;
@@ -1699,27 +1727,29 @@ __global__ void k_dlp_line(const int32_t* __restrict__ line_tgt, const int32_t* 
     const int N = nn[k];
     const double* a = asig + off[k];
     const double* w = lw + woff[t];
-    double acc = 0.0;
-    for (int i = lane; i < N; i += 32) acc += w[i] * a[i];
-    acc = warp_sum(acc);
+    double a0 = 0.0, a1 = 0.0;
+    if (r) {
+        const double* rr = r + off[k];
+        int i = lane;
+        for (; i + 32 < N; i += 64) {
+            a0 = fma(w[i], a[i] - rr[i], a0);
+            a1 = fma(w[i + 32], a[i + 32] - rr[i + 32], a1);
+        }
+        if (i < N) a0 = fma(w[i], a[i] - rr[i], a0);
+    } else {
+        for (int i = lane; i < N; i += 32) a0 = fma(w[i], a[i], a0);
+    }
+    const double acc = warp_sum(a0 + a1);
+    double v = 0.0;   // limit = -1 / (2 alpha^2)
+    if (lane < 5) v = lag[5 * t + lane] * (lane == 0 ? limit * acc : ext[n_user + 4 * t + lane - 1]);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     if (lane == 0) {
-        double vals[5], dist[5];
-        vals[0] = -acc / (2.0 * alpha * alpha);
-        dist[0] = 0.0;
-        double hs = line_data[4 * t + 2];
-        for (int m = 1; m <= 4; ++m) {
-            dist[m] = m * NEAR_LINE * hs;
-            vals[m] = out[n_user + 4 * t + (m - 1)];
-        }
-        double d = line_data[4 * t + 1];
-        double r = 0.0;
-        for (int i = 0; i < 5; ++i) {
-            double wi = 1.0;
-            for (int j = 0; j < 5; ++j)
-                if (j != i) wi *= (d - dist[j]) / (dist[i] - dist[j]);
-            r += wi * vals[i];
-        }
-        out[line_tgt[t]] = r;
+        const int i = line_tgt[t];
+        if (idx)
+            out[idx[i]] = base[idx[i]] + v;
+        else
+            out[i] = v;
     }
 }
 
@@ -2383,7 +2413,7 @@ static void gemv64(cudaStream_t st, const double* A, const double* x, double* y,
 static bool resid_ff(const mh_boundary* b, bool mixed) { return mixed && (b->op.A16lo.p || b->op.A32lo.p); }
 
 static void resid_split(cudaStream_t st, mh_boundary* b, const double* x) {
-    k_split_vec<<<mh_grid(b->n, 256), 256, 0, st>>>(x, b->xhi32.p, b->xlo32.p, b->n);
+    (void)mh_launch_dep(st, k_split_vec, dim3(mh_grid(b->n, 256)), dim3(256), 0, x, b->xhi32.p, b->xlo32.p, b->n);
 }
 
 static void resid_gemv(cudaStream_t st, mh_boundary* b, const double* x, double* y, const int* gate, bool mixed) {
@@ -2955,11 +2985,12 @@ mh_status dlp_classify(mh_ctx* ctx, mh_boundary* b, const double* xy_dev, int64_
         std::vector<int64_t> woff(tg->n_line + 1, 0);
         for (int64_t t = 0; t < tg->n_line; ++t) woff[t + 1] = woff[t] + b->n_nodes[lcur[t]];
         MH_RESERVE(ctx, tg->line_woff, tg->n_line + 1);
+        MH_RESERVE(ctx, tg->line_l, 5 * tg->n_line);
         MH_RESERVE(ctx, tg->line_w, std::max<int64_t>(woff[tg->n_line], 1));
         MH_CUDA(ctx, cudaMemcpyAsync(tg->line_woff.p, woff.data(), (tg->n_line + 1) * 8, cudaMemcpyHostToDevice, st));
         k_line_weights<<<mh_grid(tg->n_line * 32, 256), 256, 0, st>>>(tg->line_curve.p, tg->line_data.p, tg->n_line,
                                                                       b->d_nn.p, b->d_off.p, b->half.p,
-                                                                      tg->line_woff.p, tg->line_w.p);
+                                                                      tg->line_woff.p, tg->line_w.p, tg->line_l.p);
         MH_LAUNCHED(ctx);
     }
     if (tg->n_pairs) {
@@ -3024,7 +3055,7 @@ static mh_status pair_table(mh_ctx* ctx, mh_boundary* b, double alpha) {
 // precision: b->w32 holds this density's weights).  The sources are split over the grid so that
 // about 8 blocks per SM run whatever the number of targets, the partial sums added in a fixed order.
 static mh_status coarse_sums(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* tg, int64_t i0, int64_t count,
-                             const double* sigma, mh_precision prec) {
+                             const double* sigma, mh_precision prec, bool dep) {
     cudaStream_t st = ctx->stream;
     const double pref = -1.0 / (2.0 * MH_PI * alpha * alpha) / (alpha * alpha);
     const int64_t nblk = (count + MH_TILE - 1) / MH_TILE, ntile = (b->n + MH_TILE - 1) / MH_TILE;
@@ -3033,18 +3064,24 @@ static mh_status coarse_sums(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targ
     const dim3 grid((unsigned)nblk, (unsigned)nsplit);
     double* out = nsplit > 1 ? tg->part.p : tg->ext.p + i0;
     if (prec == MH_PREC_MIXED)
-        k_dlp_coarse32<<<grid, MH_TILE, 0, st>>>(tg->xy.p + 2 * i0, tg->fine.p + i0, count, b->src32.p, b->w32.p,
-                                                 b->d_curve_of.p, b->tile_c.p, b->tile_r.p, b->n,
-                                                 mh_dl32_make(alpha, MH_DL_CUT32), pref, out);
+        (void)mh_launch_dep(st, k_dlp_coarse32, grid, dim3(MH_TILE), 0, tg->xy.p + 2 * i0, tg->fine.p + i0, count,
+                            b->src32.p, b->w32.p, b->d_curve_of.p, b->tile_c.p, b->tile_r.p, b->n,
+                            mh_dl32_make(alpha, MH_DL_CUT32), pref, out);
     else {
         MH_TRY(pair_table(ctx, b, alpha));
-        k_dlp_coarse<MH_TILE><<<grid, MH_TILE, 0, st>>>(tg->xy.p + 2 * i0, tg->fine.p + i0, count, b->geo.p, sigma,
-                                                        b->d_curve_of.p, b->d_nn.p, b->n,
-                                                        mh_pair_tab_make(b->ptab.p, alpha), pref, out);
+        const mh_pair_tab tab = mh_pair_tab_make(b->ptab.p, alpha);
+        const auto kern = k_dlp_coarse<MH_TILE>;
+        if (dep)
+            (void)mh_launch_dep(st, kern, grid, dim3(MH_TILE), 0, tg->xy.p + 2 * i0, tg->fine.p + i0, count, b->geo.p,
+                                sigma, b->d_curve_of.p, b->d_nn.p, b->n, tab, pref, out);
+        else
+            kern<<<grid, MH_TILE, 0, st>>>(tg->xy.p + 2 * i0, tg->fine.p + i0, count, b->geo.p, sigma, b->d_curve_of.p,
+                                           b->d_nn.p, b->n, tab, pref, out);
     }
     MH_LAUNCHED(ctx);
     if (nsplit > 1) {
-        k_sum_partials<<<mh_grid(count, 256), 256, 0, st>>>(tg->part.p, nsplit, count, pref, tg->ext.p + i0);
+        (void)mh_launch_dep(st, k_sum_partials, dim3(mh_grid(count, 32)), dim3(256), 0, tg->part.p, nsplit, count, pref,
+                            tg->ext.p + i0);
         MH_LAUNCHED(ctx);
     }
     return MH_OK;
@@ -3057,16 +3094,15 @@ static mh_status fine_sums(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_target
     const double pref = -1.0 / (2.0 * MH_PI * alpha * alpha) / (alpha * alpha);
     const unsigned grid = (unsigned)(tg->n_groups * tg->fine_slices);
     if (prec == MH_PREC_MIXED)
-        k_dlp_fine32_grp<FINE_TG><<<grid, 256, 0, st>>>(
-            tg->xy.p, tg->pair_tgt.p, tg->grp_curve.p, tg->grp_pair.p, tg->fine_slices, b->fine32.p, b->wf32.p,
-            b->d_fine_off.p, b->d_fchunk_off.p, b->fchunk_cf.p, b->fchunk_r.p, mh_dl32_make(alpha, MH_DL_CUT32),
-            (float)(MH_DL_CUT32 * alpha), pref, tg->grp_part.p, tg->grp_cnt.p, tg->ext.p);
+        (void)mh_launch_dep(st, k_dlp_fine32_grp<FINE_TG>, dim3(grid), dim3(256), 0, tg->xy.p, tg->pair_tgt.p,
+                            tg->grp_curve.p, tg->grp_pair.p, tg->fine_slices, b->fine32.p, b->wf32.p, b->d_fine_off.p,
+                            b->d_fchunk_off.p, b->fchunk_cf.p, b->fchunk_r.p, mh_dl32_make(alpha, MH_DL_CUT32),
+                            (float)(MH_DL_CUT32 * alpha), pref, tg->grp_part.p, tg->grp_cnt.p, tg->ext.p);
     else {
         MH_TRY(pair_table(ctx, b, alpha));
-        k_dlp_fine64_grp<FINE_TG><<<grid, 256, 0, st>>>(tg->xy.p, tg->pair_tgt.p, tg->grp_curve.p, tg->grp_pair.p,
-                                                        tg->fine_slices, b->fine_geo.p, wf64, b->d_fine_off.p,
-                                                        mh_pair_tab_make(b->ptab.p, alpha), pref, tg->grp_part.p,
-                                                        tg->grp_cnt.p, tg->ext.p);
+        (void)mh_launch_dep(st, k_dlp_fine64_grp<FINE_TG>, dim3(grid), dim3(256), 0, tg->xy.p, tg->pair_tgt.p,
+                            tg->grp_curve.p, tg->grp_pair.p, tg->fine_slices, b->fine_geo.p, wf64, b->d_fine_off.p,
+                            mh_pair_tab_make(b->ptab.p, alpha), pref, tg->grp_part.p, tg->grp_cnt.p, tg->ext.p);
     }
     MH_LAUNCHED(ctx);
     return MH_OK;
@@ -3086,7 +3122,7 @@ mh_status dlp_evaluate(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* t
     }
     if (tg->n_ext) {
         prof_scope ps(ctx, "dlp_coarse", DL_FLOPS * tg->n_ext * b->n, 24.0 * (tg->n_ext + b->n));
-        MH_TRY(coarse_sums(ctx, b, alpha, tg, 0, tg->n_ext, sigma, prec));
+        MH_TRY(coarse_sums(ctx, b, alpha, tg, 0, tg->n_ext, sigma, prec, true));
     }
     if (tg->n_pairs) {
         MH_TRY(dlp_fine_weights(ctx, b, sigma, prec, true));
@@ -3095,10 +3131,9 @@ mh_status dlp_evaluate(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* t
     }
     if (tg->n_line) {
         MH_TRY(bie_apply(ctx, b, sigma, asig.p, MH_PREC_FP64));
-        k_dlp_line<<<mh_grid(tg->n_line * 32, 256), 256, 0, st>>>(tg->line_tgt.p, tg->line_curve.p, tg->line_data.p,
-                                                                  tg->n_line, asig.p, b->d_nn.p, b->d_off.p,
-                                                                  tg->line_w.p, tg->line_woff.p, tg->n, alpha,
-                                                                  ext.p);
+        (void)mh_launch_dep(st, k_dlp_line, dim3(mh_grid(tg->n_line * 32, 256)), dim3(256), 0, tg->line_tgt.p,
+                            tg->line_curve.p, tg->line_l.p, tg->n_line, asig.p, nullptr, b->d_nn.p, b->d_off.p,
+                            tg->line_w.p, tg->line_woff.p, tg->n, -0.5 / (alpha * alpha), ext.p, nullptr, nullptr, ext.p);
         MH_LAUNCHED(ctx);
     }
     if (tg->n) MH_CUDA(ctx, cudaMemcpyAsync(out, ext.p, tg->n * 8, cudaMemcpyDeviceToDevice, st));
@@ -3152,12 +3187,12 @@ mh_status dlp_fine_weights(mh_ctx* ctx, mh_boundary* b, const double* sigma, mh_
     if (pow2) {   // FFTs both ways in one launch
         const dim3 grid(UPSAMPLE, (unsigned)b->n_curves);
         if (mixed && !spectrum64)
-            k_fine_weights_fft<float, float2><<<grid, 256, 2 * max_n * sizeof(float2), st>>>(
-                sigma, b->tw32.p, b->fine_geo.p, b->d_nn.p, b->d_off.p, b->d_fine_off.p, b->wf32.p, b->wf64.p);
+            (void)mh_launch_dep(st, k_fine_weights_fft<float, float2>, grid, dim3(256), 2 * max_n * sizeof(float2), sigma,
+                                b->tw32.p, b->fine_geo.p, b->d_nn.p, b->d_off.p, b->d_fine_off.p, b->wf32.p, b->wf64.p);
         else
-            k_fine_weights_fft<double, double2><<<grid, 256, 2 * max_n * sizeof(double2), st>>>(
-                sigma, b->tw.p, b->fine_geo.p, b->d_nn.p, b->d_off.p, b->d_fine_off.p, mixed ? b->wf32.p : nullptr,
-                b->wf64.p);
+            (void)mh_launch_dep(st, k_fine_weights_fft<double, double2>, grid, dim3(256), 2 * max_n * sizeof(double2),
+                                sigma, b->tw.p, b->fine_geo.p, b->d_nn.p, b->d_off.p, b->d_fine_off.p,
+                                mixed ? b->wf32.p : nullptr, b->wf64.p);
         MH_LAUNCHED(ctx);
         return MH_OK;
     }
@@ -3179,46 +3214,33 @@ mh_status dlp_fine_weights(mh_ctx* ctx, mh_boundary* b, const double* sigma, mh_
     return MH_OK;
 }
 
-mh_status dlp_evaluate_fmm_tail(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* tg, const double* sigma,
-                                const double* main_vals, double* out, mh_precision prec, const double* asig_given,
-                                int part) {
-    const bool do_aux = part != 2, do_finish = part != 1;
+mh_status dlp_aux_sums(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* tg, const double* sigma,
+                       mh_precision prec) {
     cudaStream_t st = ctx->stream;
     const int64_t n = tg->n, naux = tg->n_ext - tg->n;
-    dbuf<double>& ext = tg->ext;
+    if (naux == 0) return MH_OK;
     prof_scope ps_all(ctx, "dlp_evaluate");
-    // ext[0, n): the given values at the targets; ext[n, n_ext): the auxiliary points, written
-    // only by the auxiliary part (part 1), so that part can run beside the work that produces
-    // main_vals
-    if (do_finish && n) MH_CUDA(ctx, cudaMemcpyAsync(ext.p, main_vals, n * 8, cudaMemcpyDeviceToDevice, st));
-    if (do_aux && naux) {
-        if (prec == MH_PREC_MIXED) {
-            MH_TRY(prep_mixed(ctx, b));
-            k_weights32<<<mh_grid(b->n, 256), 256, 0, st>>>(sigma, b->geo.p, b->d_curve_of.p, b->d_nn.p, b->n, b->w32.p);
-            MH_LAUNCHED(ctx);
-        }
-        MH_TRY(coarse_sums(ctx, b, alpha, tg, n, naux, sigma, prec));
-        if (tg->n_groups) {
-            prof_scope ps(ctx, "dlp_fine", DL_FLOPS * tg->fine_nodes_aux, 24.0 * b->n_fine);
-            MH_TRY(fine_sums(ctx, b, alpha, tg, b->wf64.p, prec));
-        }
-    }
-    if (!do_finish) return MH_OK;
-    if (tg->n_line) {
-        // the interior limit needs A sigma; a caller that holds the residual r = rhs - A sigma
-        // of this density passes A sigma = rhs - r instead of a product with the operator
-        const double* asig = asig_given;
-        if (!asig) {
-            MH_TRY(bie_apply(ctx, b, sigma, tg->asig.p, prec));
-            asig = tg->asig.p;
-        }
-        k_dlp_line<<<mh_grid(tg->n_line * 32, 256), 256, 0, st>>>(tg->line_tgt.p, tg->line_curve.p, tg->line_data.p,
-                                                                  tg->n_line, asig, b->d_nn.p, b->d_off.p,
-                                                                  tg->line_w.p, tg->line_woff.p, tg->n, alpha,
-                                                                  ext.p);
+    if (prec == MH_PREC_MIXED) {
+        MH_TRY(prep_mixed(ctx, b));
+        k_weights32<<<mh_grid(b->n, 256), 256, 0, st>>>(sigma, b->geo.p, b->d_curve_of.p, b->d_nn.p, b->n, b->w32.p);
         MH_LAUNCHED(ctx);
     }
-    if (n) MH_CUDA(ctx, cudaMemcpyAsync(out, ext.p, n * 8, cudaMemcpyDeviceToDevice, st));
+    // binary64: the first launch here, behind the side stream's event wait
+    MH_TRY(coarse_sums(ctx, b, alpha, tg, n, naux, sigma, prec, prec == MH_PREC_MIXED));
+    if (tg->n_groups) {
+        prof_scope ps(ctx, "dlp_fine", DL_FLOPS * tg->fine_nodes_aux, 24.0 * b->n_fine);
+        MH_TRY(fine_sums(ctx, b, alpha, tg, b->wf64.p, prec));
+    }
+    return MH_OK;
+}
+
+mh_status dlp_line_finish(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* tg, const double* rhs,
+                          const double* r, const double* base, const int32_t* idx, double* out) {
+    if (tg->n_line == 0) return MH_OK;
+    (void)mh_launch_dep(ctx->stream, k_dlp_line, dim3(mh_grid(tg->n_line * 32, 256)), dim3(256), 0, tg->line_tgt.p,
+                        tg->line_curve.p, tg->line_l.p, tg->n_line, rhs, r, b->d_nn.p, b->d_off.p, tg->line_w.p,
+                        tg->line_woff.p, tg->n, -0.5 / (alpha * alpha), tg->ext.p, base, idx, out);
+    MH_LAUNCHED(ctx);
     return MH_OK;
 }
 

@@ -304,6 +304,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_contract_tc(
     const int32_t* __restrict__ chunk_op, const int32_t* __restrict__ chunk_t0, int n_chunks,
     const uint16_t* __restrict__ spl, int64_t plane, const int64_t* __restrict__ tc_src, int R, int npad, int kmax,
     int nst, float* __restrict__ temp, const int64_t* __restrict__ task_dst, int accumulate, TD* dst, int* err) {
+    mh_dep_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     // 1024-byte aligned base (the dynamic allocation is padded by 1 KB for this)
     unsigned char* base = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
@@ -577,14 +578,32 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_contract_tc(
 
 // Split `count` consecutive binary32 vectors of length len (src) into the three bfloat16
 // planes (plane elements apart) at dst, each vector padded with zeros to S entries.
-__global__ void k_split_pool(const float* __restrict__ src, int len, int64_t count, int S,
+__global__ void k_split_pool(const float* src, int len, int64_t count, int S,
                              uint16_t* __restrict__ planes, int64_t plane, int64_t dst) {
+    mh_dep_wait();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= count * S) return;
     const int64_t v = i / S;
     const int e = (int)(i - v * S);
     __nv_bfloat16 p0, p1, p2;
     split3(e < len ? src[v * len + e] : 0.f, p0, p1, p2);
+    planes[dst + i] = __bfloat16_as_ushort(p0);
+    planes[plane + dst + i] = __bfloat16_as_ushort(p1);
+    planes[2 * plane + dst + i] = __bfloat16_as_ushort(p2);
+}
+
+// The same from binary64 values, which also go to dst32 in binary32 (the pool's node values).
+__global__ void k_split_values(const double* src, int len, int64_t count, int S, float* __restrict__ dst32,
+                               uint16_t* __restrict__ planes, int64_t plane, int64_t dst) {
+    mh_dep_wait();
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= count * S) return;
+    const int64_t v = i / S;
+    const int e = (int)(i - v * S);
+    const float x = e < len ? (float)src[v * len + e] : 0.f;
+    if (e < len) dst32[v * len + e] = x;
+    __nv_bfloat16 p0, p1, p2;
+    split3(x, p0, p1, p2);
     planes[dst + i] = __bfloat16_as_ushort(p0);
     planes[plane + dst + i] = __bfloat16_as_ushort(p1);
     planes[2 * plane + dst + i] = __bfloat16_as_ushort(p2);
@@ -679,16 +698,21 @@ mh_status tc_contract_launch(mh_ctx* ctx, const tc_launch& a) {
     const size_t smem = tc_smem_bytes(nst, a.npad, a.kmax, a.R);
     if (smem > d.cap) return mh_fail(ctx, MH_ERR_INVALID_ARG, "tensor-core contraction needs %zu B of shared memory", smem);
     const unsigned grid = (unsigned)std::min<int64_t>(a.n_chunks, d.sms);
+    auto launch = [&](auto kern, auto* dst) {
+        const auto* img = reinterpret_cast<const __nv_bfloat16*>(a.img);
+        if (a.dep)
+            (void)mh_launch_dep(ctx->stream, kern, dim3(grid), dim3(TC_THREADS), smem, img, a.img_off, a.kpad, a.chunk_op,
+                                a.chunk_t0, (int)a.n_chunks, a.spl, a.plane, a.tc_src, a.R, a.npad, a.kmax, nst, a.temp,
+                                a.task_dst, a.accumulate, dst, a.err);
+        else
+            kern<<<grid, TC_THREADS, smem, ctx->stream>>>(img, a.img_off, a.kpad, a.chunk_op, a.chunk_t0, (int)a.n_chunks,
+                                                          a.spl, a.plane, a.tc_src, a.R, a.npad, a.kmax, nst, a.temp,
+                                                          a.task_dst, a.accumulate, dst, a.err);
+    };
     if (a.dst_double)
-        k_contract_tc<double><<<grid, TC_THREADS, smem, ctx->stream>>>(
-            reinterpret_cast<const __nv_bfloat16*>(a.img), a.img_off, a.kpad, a.chunk_op, a.chunk_t0,
-            (int)a.n_chunks, a.spl, a.plane, a.tc_src, a.R, a.npad, a.kmax, nst, a.temp, a.task_dst, a.accumulate,
-            static_cast<double*>(a.dst), a.err);
+        launch(k_contract_tc<double>, static_cast<double*>(a.dst));
     else
-        k_contract_tc<float><<<grid, TC_THREADS, smem, ctx->stream>>>(
-            reinterpret_cast<const __nv_bfloat16*>(a.img), a.img_off, a.kpad, a.chunk_op, a.chunk_t0,
-            (int)a.n_chunks, a.spl, a.plane, a.tc_src, a.R, a.npad, a.kmax, nst, a.temp, a.task_dst, a.accumulate,
-            static_cast<float*>(a.dst), a.err);
+        launch(k_contract_tc<float>, static_cast<float*>(a.dst));
     MH_LAUNCHED(ctx);
     return MH_OK;
 }
@@ -696,7 +720,17 @@ mh_status tc_contract_launch(mh_ctx* ctx, const tc_launch& a) {
 mh_status tc_split_launch(mh_ctx* ctx, const float* src, int len, int64_t count, int S, uint16_t* planes, int64_t plane,
                           int64_t dst) {
     if (count <= 0) return MH_OK;
-    k_split_pool<<<(unsigned)mh_grid(count * S, 256), 256, 0, ctx->stream>>>(src, len, count, S, planes, plane, dst);
+    (void)mh_launch_dep(ctx->stream, k_split_pool, dim3(mh_grid(count * S, 256)), dim3(256), 0, src, len, count, S, planes,
+                        plane, dst);
+    MH_LAUNCHED(ctx);
+    return MH_OK;
+}
+
+mh_status tc_split_values(mh_ctx* ctx, const double* src, int len, int64_t count, int S, float* dst32, uint16_t* planes,
+                          int64_t plane, int64_t dst) {
+    if (count <= 0) return MH_OK;
+    (void)mh_launch_dep(ctx->stream, k_split_values, dim3(mh_grid(count * S, 256)), dim3(256), 0, src, len, count, S, dst32,
+                        planes, plane, dst);
     MH_LAUNCHED(ctx);
     return MH_OK;
 }

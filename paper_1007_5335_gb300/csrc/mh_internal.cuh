@@ -217,6 +217,7 @@ struct tc_launch {
     void* dst = nullptr;
     bool dst_double = false;
     int* err = nullptr;                  // set when a bounded wait gave up
+    bool dep = false;                    // launched directly behind a kernel (mh_launch_dep)
 };
 int tc_pad_rows(int R);
 int tc_pad_cols(int C);
@@ -227,6 +228,9 @@ mh_status tc_contract_launch(mh_ctx* ctx, const tc_launch& a);
 // (rows padded with zeros to S entries).
 mh_status tc_split_launch(mh_ctx* ctx, const float* src, int len, int64_t count, int S, uint16_t* planes, int64_t plane,
                           int64_t dst);
+// The same from binary64 vectors at src, which are also written to dst32 in binary32.
+mh_status tc_split_values(mh_ctx* ctx, const double* src, int len, int64_t count, int S, float* dst32, uint16_t* planes,
+                          int64_t plane, int64_t dst);
 
 // Device-resident state of the sync-free GMRES (gmres_run_graph): every kernel of its fixed
 // schedule reads the flags at entry and returns at once when its work is not needed.
@@ -289,6 +293,7 @@ struct dlp_targets {
     dbuf<int32_t> line_tgt;     // target index
     dbuf<int32_t> line_curve;   // curve
     dbuf<double> line_data;     // [n_line][4]: t*, d, h_s, unused
+    dbuf<double> line_l;        // [n_line][5]: interpolation weights in the distance (limit, 4 auxiliary points)
     dbuf<double> line_w;        // trigonometric interpolation weights at t*, N_k per line target
     dbuf<int64_t> line_woff;    // [n_line + 1] offsets into line_w
     // fine pairs (ext target, curve)
@@ -400,7 +405,7 @@ struct mh_problem {
     dbuf<int32_t> inside_idx;            // indices of nodes inside Omega
     int64_t n_inside = 0;
     dbuf<int32_t> bnd_leaf;              // leaf of every boundary node
-    dbuf<double> B, Up, Ug, rhs, Uh;     // work arrays
+    dbuf<double> B, Up, rhs;             // work arrays
     SideStream aux;                      // the normal-line auxiliary sums beside the double layer's pass
     // GMRES start (mh_problem_set_warm_start)
     int warm_mode = 0;
@@ -453,15 +458,14 @@ mh_status dlp_classify(mh_ctx* ctx, mh_boundary* b, const double* xy_dev, int64_
                        bool all_groups = false);
 mh_status dlp_evaluate(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* tg,
                        const double* sigma, double* out, mh_precision prec);
-// U^h when the upsampled sum of every curve at the user targets (main_vals, n values) comes from
-// the multipole method: adds the normal-line rule and its auxiliary points.  Requires
-// dlp_fine_weights for this sigma.
-// part: 0 = everything; 1 = the sums at the auxiliary points (they need sigma and its fine
-// weights only, so they may run beside the pass that produces main_vals); 2 = the rest, after
-// part 1 (main_vals, the normal-line rule, out).
-mh_status dlp_evaluate_fmm_tail(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* tg, const double* sigma,
-                                const double* main_vals, double* out, mh_precision prec,
-                                const double* asig_given = nullptr, int part = 0);
+// Sums at the auxiliary points of the normal-line rule into tg->ext (they need sigma and its fine
+// weights only, so they may run beside the pass that evaluates the other targets).
+mh_status dlp_aux_sums(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* tg, const double* sigma,
+                       mh_precision prec);
+// The normal-line rule at the set's line targets, after dlp_aux_sums: out[idx[t]] = base[idx[t]] + U^h,
+// with A sigma = rhs - r.
+mh_status dlp_line_finish(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* tg, const double* rhs,
+                          const double* r, const double* base, const int32_t* idx, double* out);
 // Density on the 16x fine grid times |y'| h_f (binary64 in b->wf64; binary32 also in b->wf32
 // when prec is mixed); spectrum64: mixed weights rounded from a binary64 spectrum, not a binary32 one.
 mh_status dlp_fine_weights(mh_ctx* ctx, mh_boundary* b, const double* sigma, mh_precision prec,
@@ -493,7 +497,9 @@ int volume_near_tile(const mh_tree* t);
 // double layer through the multipole method (dipoles sorted by leaf)
 mh_status volume_dipole_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, const double* dxy, const double* dnrm,
                               const int32_t* dleaf, int64_t nd, bool near_blocks);
-mh_status volume_dipole_apply(mh_ctx* ctx, mh_tree* t, const double* w_sorted, mh_precision prec, const double** u);
+// Strengths w[perm[j]] for dipole j; *u: U^h at every volume node (valid until the next call on the tree).
+mh_status volume_dipole_apply(mh_ctx* ctx, mh_tree* t, const double* w, const int32_t* perm, mh_precision prec,
+                              const double** u);
 // On-surface double layer through the multipole method (binary64): set-up for the boundary
 // nodes (host arrays in node order: positions, unit normals, leaf of every node), then
 // u_i = -(1/(2 pi alpha^2)) sum_{d != i} w_d (1/alpha) K1(r/alpha) (y_d - x_i).nu_d / r at every
@@ -503,8 +509,9 @@ mh_status volume_bie_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, const d
 bool volume_bie_ready(const mh_tree* t);
 mh_status volume_bie_apply(mh_ctx* ctx, mh_tree* t, const double* w, double* u);
 mh_status tree_locate(mh_ctx* ctx, const mh_tree* t, const double* xy_dev, int64_t n, int32_t* leaf_out);
+// Leaf interpolation U of node values at n points with known leaves; with f, c (f - U) instead of U.
 mh_status tree_interpolate(mh_ctx* ctx, const mh_tree* t, const double* vals, const double* xy_dev,
-                           const int32_t* leaf, int64_t n, double* out);
+                           const int32_t* leaf, int64_t n, const double* f, double c, double* out);
 
 inline int mh_grid(int64_t n, int block) {
     int64_t g = (n + block - 1) / block;

@@ -66,36 +66,46 @@ __global__ void k_form_B_gear(const double* __restrict__ u, const double* __rest
 }
 
 // same[0] stays set (nonzero) only if a == b element by element.
-__global__ void k_rc_compare(const double* __restrict__ a, const double* __restrict__ b, int64_t n, int* same) {
+__global__ void k_rc_compare(const double* a, const double* b, int64_t n, int* same) {
+    mh_dep_wait();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         if (a[i] != b[i]) *same = 0;
 }
 
 // r = rhs - rhs_prev + r_prev when the density is the one the previous step ended with
 // (rhs_prev - A sigma = r_prev), else r = rhs - Ax (Ax computed for that case).
-__global__ void k_rc_resid(const double* __restrict__ rhs, const double* __restrict__ ax,
-                           const double* __restrict__ rhs_prev, const double* __restrict__ r_prev,
-                           const int* __restrict__ same, int64_t n, double* r) {
+__global__ void k_rc_resid(const double* rhs, const double* ax, const double* rhs_prev, const double* r_prev,
+                           const int* same, int64_t n, double* r) {
+    mh_dep_wait();
     const bool s = *same != 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         r[i] = s ? (rhs[i] - rhs_prev[i]) + r_prev[i] : rhs[i] - ax[i];
 }
 
-__global__ void k_rhs(const double* __restrict__ f, const double* __restrict__ ug, double c, int64_t n, double* rhs) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) rhs[i] = c * (f[i] - ug[i]);
-}
-
-__global__ void k_combine(const double* __restrict__ up, const double* __restrict__ uh,
-                          const int32_t* __restrict__ region, const int32_t* __restrict__ slot,
+// Inside Omega u = U^p + U^h, outside the extension.
+__global__ void k_combine(const double* up, const double* uh, const int32_t* __restrict__ region,
                           const double* __restrict__ ext_const, int ext_mode, int64_t n, double* out) {
+    mh_dep_wait();
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int r = region[i];
     if (r < 0)
-        out[i] = up[i] + uh[slot[i]];
+        out[i] = up[i] + uh[i];
     else
         out[i] = ext_mode == MH_EXT_CONST ? ext_const[r] : up[i];
+}
+
+// What the next step needs to skip its first binary64 operator product: the density, the
+// right-hand side and the residual this step ended with; *same = 1 for its comparison.
+__global__ void k_keep(const double* sigma, const double* rhs, const double* r, int64_t n, double* __restrict__ ks,
+                       double* __restrict__ kb, double* __restrict__ kr, int* same) {
+    mh_dep_wait();
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i == 0) *same = 1;
+    if (i >= n) return;
+    ks[i] = sigma[i];
+    kb[i] = rhs[i];
+    kr[i] = r[i];
 }
 
 __global__ void k_gather_xy(const double* __restrict__ xy, const int32_t* __restrict__ idx, int64_t n, double* out) {
@@ -107,21 +117,8 @@ __global__ void k_gather_xy(const double* __restrict__ xy, const int32_t* __rest
 
 }  // namespace
 
-__global__ void k_dip_weights(const double* __restrict__ wf, const int32_t* __restrict__ perm, int64_t n,
-                              double* w) {
-    int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (j < n) w[j] = wf[perm[j]];
-}
-
-__global__ void k_gather(const double* __restrict__ src, const int32_t* __restrict__ idx, int64_t n, double* out) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) out[i] = src[idx[i]];
-}
-
 struct ProblemImpl : mh_problem {
-    dbuf<int32_t> slot;       // position of an inside node in the inside list, else -1
-    dbuf<int32_t> perm;       // boundary nodes sorted by leaf: sorted position -> node
-    dbuf<double> w_sorted;    // dipole strengths in that order
+    dbuf<int32_t> perm;       // dipoles (fine boundary nodes) sorted by leaf: sorted position -> fine node
 };
 
 extern "C" mh_status mh_problem_create(mh_ctx* ctx, mh_tree* tree, mh_boundary* bnd, double dt, int scheme, int p,
@@ -156,18 +153,13 @@ extern "C" mh_status mh_problem_create(mh_ctx* ctx, mh_tree* tree, mh_boundary* 
         MH_TRY(dlp_classify(ctx, bnd, tree->nodes.p, n, &all));
         MH_ALLOC(ctx, P->region, n);
         MH_CUDA(ctx, cudaMemcpyAsync(P->region.p, all.region.p, n * 4, cudaMemcpyDeviceToDevice, st));
-        std::vector<int32_t> reg(n), slot(n, -1), idx;
+        std::vector<int32_t> reg(n), idx;
         MH_CUDA(ctx, cudaMemcpyAsync(reg.data(), all.region.p, n * 4, cudaMemcpyDeviceToHost, st));
         MH_CUDA(ctx, cudaStreamSynchronize(st));
         for (int64_t i = 0; i < n; ++i)
-            if (reg[i] < 0) {
-                slot[i] = (int32_t)idx.size();
-                idx.push_back((int32_t)i);
-            }
+            if (reg[i] < 0) idx.push_back((int32_t)i);
         P->n_inside = (int64_t)idx.size();
         MH_ALLOC(ctx, P->inside_idx, std::max<int64_t>(P->n_inside, 1));
-        MH_ALLOC(ctx, P->slot, n);
-        MH_CUDA(ctx, cudaMemcpyAsync(P->slot.p, slot.data(), n * 4, cudaMemcpyHostToDevice, st));
         dbuf<double> xin;
         MH_ALLOC(ctx, xin, std::max<int64_t>(2 * P->n_inside, 2));
         if (P->n_inside) {
@@ -228,12 +220,10 @@ extern "C" mh_status mh_problem_create(mh_ctx* ctx, mh_tree* tree, mh_boundary* 
         }
         MH_TRY(volume_dipole_setup(ctx, tree, P->alpha, p, dxy.data(), dnrm.data(), dleaf.data(), nf, false));
         MH_ALLOC(ctx, P->perm, nf);
-        MH_ALLOC(ctx, P->w_sorted, nf);
         MH_CUDA(ctx, cudaMemcpyAsync(P->perm.p, perm.data(), nf * 4, cudaMemcpyHostToDevice, st));
     }
     MH_ALLOC(ctx, P->B, n);
     MH_ALLOC(ctx, P->Up, n);
-    MH_ALLOC(ctx, P->Ug, bnd->n);
     MH_ALLOC(ctx, P->rhs, bnd->n);
     MH_CUDA(ctx, cudaMemsetAsync(P->rhs.p, 0, bnd->n * 8, st));
     MH_ALLOC(ctx, P->rc_sigma, bnd->n);
@@ -241,9 +231,9 @@ extern "C" mh_status mh_problem_create(mh_ctx* ctx, mh_tree* tree, mh_boundary* 
     MH_ALLOC(ctx, P->rc_r, bnd->n);
     MH_ALLOC(ctx, P->r_start, bnd->n);
     MH_ALLOC(ctx, P->rc_same, 1);
+    MH_CUDA(ctx, cudaMemsetAsync(P->rc_same.p, 0, sizeof(int), st));
     MH_CUDA(ctx, cudaMemsetAsync(P->rc_b.p, 0, bnd->n * 8, st));
     MH_CUDA(ctx, cudaMemsetAsync(P->rc_r.p, 0, bnd->n * 8, st));
-    MH_ALLOC(ctx, P->Uh, std::max<int64_t>(P->n_inside, 1));
     // operators: boundary (alpha) and volume (alpha, p) -- built once here
     MH_TRY(bie_assemble(ctx, bnd, P->alpha));
     MH_CUDA(ctx, cudaMemsetAsync(P->B.p, 0, n * 8, st));
@@ -337,26 +327,17 @@ static mh_status start_residual(mh_ctx* ctx, ProblemImpl* P, const double* sigma
     const int64_t n = b->n;
     MH_TRY(bie_assemble(ctx, b, P->alpha));
     const int grid = mh_grid(n, 256) < 152 * 4 ? mh_grid(n, 256) : 152 * 4;
-    if (P->rc_valid) {
-        MH_CUDA(ctx, cudaMemsetAsync(P->rc_same.p, 1, sizeof(int), st));
-        k_rc_compare<<<grid, 256, 0, st>>>(sigma, P->rc_sigma.p, n, P->rc_same.p);
+    if (P->rc_valid) {   // k_keep has set rc_same
+        (void)mh_launch_dep(st, k_rc_compare, dim3(grid), dim3(256), 0, sigma, P->rc_sigma.p, n, P->rc_same.p);
         MH_LAUNCHED(ctx);
         MH_TRY(bie_apply64_gated(ctx, b, sigma, r, P->rc_same.p, prec));
-        k_rc_resid<<<grid, 256, 0, st>>>(P->rhs.p, r, P->rc_b.p, P->rc_r.p, P->rc_same.p, n, r);
-        MH_LAUNCHED(ctx);
     } else {
         MH_TRY(bie_apply64_gated(ctx, b, sigma, r, nullptr, prec));
         MH_CUDA(ctx, cudaMemsetAsync(P->rc_same.p, 0, sizeof(int), st));
-        k_rc_resid<<<grid, 256, 0, st>>>(P->rhs.p, r, P->rc_b.p, P->rc_r.p, P->rc_same.p, n, r);
-        MH_LAUNCHED(ctx);
     }
+    (void)mh_launch_dep(st, k_rc_resid, dim3(grid), dim3(256), 0, P->rhs.p, r, P->rc_b.p, P->rc_r.p, P->rc_same.p, n, r);
+    MH_LAUNCHED(ctx);
     return MH_OK;
-}
-
-__global__ void k_rhs_minus_r(const double* __restrict__ rhs, const double* __restrict__ r, int64_t n,
-                              double* __restrict__ out) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) out[i] = rhs[i] - r[i];
 }
 
 // Everything after the right-hand side B (P->B) has been formed.
@@ -367,9 +348,8 @@ static mh_status step_solve(mh_ctx* ctx, ProblemImpl* P, const double* f_next_de
     mh_boundary* b = P->bnd;
     const int64_t n = t->n_nodes, ng = b->n;
     MH_TRY(volume_apply(ctx, t, P->alpha, P->p, P->B.p, P->Up.p, prec));
-    MH_TRY(tree_interpolate(ctx, t, P->Up.p, b->xy.p, P->bnd_leaf.p, ng, P->Ug.p));
-    k_rhs<<<mh_grid(ng, 256), 256, 0, st>>>(f_next_dev, P->Ug.p, -2.0 * P->alpha * P->alpha, ng, P->rhs.p);
-    MH_LAUNCHED(ctx);
+    // rhs = -2 alpha^2 (f - U^p) on Gamma
+    MH_TRY(tree_interpolate(ctx, t, P->Up.p, b->xy.p, P->bnd_leaf.p, ng, f_next_dev, -2.0 * P->alpha * P->alpha, P->rhs.p));
     mh_gmres_info gi{};
     // GMRES start (mh_problem_set_warm_start); r0 = its binary64 residual when computed here
     const double* r0 = nullptr;
@@ -401,10 +381,9 @@ static mh_status step_solve(mh_ctx* ctx, ProblemImpl* P, const double* f_next_de
     mh_status s = P->graph_mode ? MH_OK : gmres_run(ctx, b, P->rhs.p, sigma_dev, gmres_tol, 100, prec, &gi, r0);
     // keep what the next step needs to skip its first binary64 operator product
     if (s == MH_OK) {
-        MH_CUDA(ctx, cudaMemcpyAsync(P->rc_sigma.p, sigma_dev, ng * 8, cudaMemcpyDeviceToDevice, st));
-        MH_CUDA(ctx, cudaMemcpyAsync(P->rc_b.p, P->rhs.p, ng * 8, cudaMemcpyDeviceToDevice, st));
-        MH_CUDA(ctx, cudaMemcpyAsync(P->rc_r.p, gmres_final_residual(b), ng * 8,
-                                     cudaMemcpyDeviceToDevice, st));
+        (void)mh_launch_dep(st, k_keep, dim3(mh_grid(ng, 256)), dim3(256), 0, sigma_dev, P->rhs.p,
+                            gmres_final_residual(b), ng, P->rc_sigma.p, P->rc_b.p, P->rc_r.p, P->rc_same.p);
+        MH_LAUNCHED(ctx);
         P->rc_valid = true;
     } else {
         P->rc_valid = false;
@@ -424,33 +403,19 @@ static mh_status step_solve(mh_ctx* ctx, ProblemImpl* P, const double* f_next_de
     if (aux_fork) {
         MH_TRY(P->aux.begin(ctx, st));
         ctx->stream = P->aux.s;
-        const mh_status sa = dlp_evaluate_fmm_tail(ctx, b, P->alpha, &P->tg, sigma_dev, nullptr, nullptr, prec,
-                                                   nullptr, 1);
-        ctx->stream = st;
-        MH_TRY(sa);
-        MH_TRY(P->aux.end(ctx));
     }
-    k_dip_weights<<<mh_grid(b->n_fine, 256), 256, 0, st>>>(b->wf64.p, P->perm.p, b->n_fine, P->w_sorted.p);
-    MH_LAUNCHED(ctx);
+    const mh_status sa = dlp_aux_sums(ctx, b, P->alpha, &P->tg, sigma_dev, prec);
+    ctx->stream = st;
+    MH_TRY(sa);
+    if (aux_fork) MH_TRY(P->aux.end(ctx));
     const double* du = nullptr;
-    MH_TRY(volume_dipole_apply(ctx, t, P->w_sorted.p, prec, &du));
-    if (P->n_inside) {
-        k_gather<<<mh_grid(P->n_inside, 256), 256, 0, st>>>(du, P->inside_idx.p, P->n_inside, P->Uh.p);
-        MH_LAUNCHED(ctx);
-    }
-    // A sigma for the normal-line rule from the solver's final residual r = rhs - A sigma
-    // (binary64, or float-float on the binary32 operator and its low part): rhs - r, no operator product
-    if (P->tg.n_line) {
-        k_rhs_minus_r<<<mh_grid(ng, 256), 256, 0, st>>>(P->rhs.p, P->rc_r.p, ng, P->tg.asig.p);
-        MH_LAUNCHED(ctx);
-    }
+    MH_TRY(volume_dipole_apply(ctx, t, b->wf64.p, P->perm.p, prec, &du));
     if (aux_fork) MH_CUDA(ctx, cudaStreamWaitEvent(st, P->aux.join, 0));
-    MH_TRY(dlp_evaluate_fmm_tail(ctx, b, P->alpha, &P->tg, sigma_dev, P->Uh.p, P->Uh.p, prec,
-                                 P->tg.n_line ? P->tg.asig.p : nullptr, aux_fork ? 2 : 0));
-    k_combine<<<mh_grid(n, 256), 256, 0, st>>>(P->Up.p, P->Uh.p, P->region.p, P->slot.p, P->d_ext_const.p,
-                                               P->ext_mode, n, u_next_dev);
+    k_combine<<<mh_grid(n, 256), 256, 0, st>>>(P->Up.p, du, P->region.p, P->d_ext_const.p, P->ext_mode, n, u_next_dev);
     MH_LAUNCHED(ctx);
-    return MH_OK;
+    // the nodes of the normal-line rule last; A sigma from the solver's final residual r = rhs - A sigma
+    // (binary64, or float-float on the binary32 operator and its low part): no operator product
+    return dlp_line_finish(ctx, b, P->alpha, &P->tg, P->rhs.p, P->rc_r.p, P->Up.p, P->inside_idx.p, u_next_dev);
 }
 
 extern "C" mh_status heat_step(mh_ctx* ctx, mh_problem* prob, const double* u_dev, const double* F_dev,

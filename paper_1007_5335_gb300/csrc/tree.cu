@@ -452,10 +452,14 @@ __global__ void k_locate(Maps M, const int32_t* __restrict__ box_leaf, double x0
 template <int Q>
 __global__ void k_interp(const int32_t* __restrict__ boxes, const int32_t* __restrict__ leaf_box, double x0, double y0,
                          double W, const double* __restrict__ xi, const double* __restrict__ bw,
-                         const double* __restrict__ vals, const double* __restrict__ xy, const int32_t* __restrict__ leaf,
-                         int64_t n, double* out) {
+                         const double* vals, const double* __restrict__ xy, const int32_t* __restrict__ leaf,
+                         int64_t n, const double* f, double c, double* out) {
+    // the weights depend on the geometry alone: formed before the wait for the values
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    if (i >= n) {
+        mh_dep_wait();
+        return;
+    }
     const int lf = leaf[i];
     const int b = leaf_box[lf];
     const int l = boxes[3 * b];
@@ -485,6 +489,7 @@ __global__ void k_interp(const int32_t* __restrict__ boxes, const int32_t* __res
         px *= dxv[a];
         py *= dyv[a];
     }
+    mh_dep_wait();
     const double* v = vals + (int64_t)lf * Q * Q;
     double acc = 0.0;
 #pragma unroll
@@ -494,7 +499,7 @@ __global__ void k_interp(const int32_t* __restrict__ boxes, const int32_t* __res
         for (int c = 0; c < Q; ++c) row = fma(v[a * Q + c], lx[c], row);
         acc = fma(ly[a], row, acc);
     }
-    out[i] = acc;
+    out[i] = f ? c * (f[i] - acc) : acc;
 }
 
 struct TreeExtra {
@@ -848,12 +853,12 @@ mh_status tree_locate(mh_ctx* ctx, const mh_tree* t, const double* xy_dev, int64
 }
 
 mh_status tree_interpolate(mh_ctx* ctx, const mh_tree* t, const double* vals, const double* xy_dev,
-                           const int32_t* leaf, int64_t n, double* out) {
+                           const int32_t* leaf, int64_t n, const double* f, double c, double* out) {
     if (n == 0) return MH_OK;
     const TreeExtra* E = extra_of(t);
 #define MH_INTERP(QV)                                                                                     \
-    k_interp<QV><<<mh_grid(n, 128), 128, 0, ctx->stream>>>(t->boxes.p, t->leaf_box.p, t->box[0], t->box[1],  \
-                                                            t->box[2], E->xi.p, E->bw.p, vals, xy_dev, leaf, n, out)
+    (void)mh_launch_dep(ctx->stream, k_interp<QV>, dim3(mh_grid(n, 128)), dim3(128), 0, t->boxes.p, t->leaf_box.p,    \
+                        t->box[0], t->box[1], t->box[2], E->xi.p, E->bw.p, vals, xy_dev, leaf, n, f, c, out)
     switch (t->q) {
         case 2: MH_INTERP(2); break;
         case 3: MH_INTERP(3); break;

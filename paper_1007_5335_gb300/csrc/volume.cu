@@ -664,13 +664,19 @@ mh_status build_cols(mh_ctx* ctx, const ColBuild& b, bool both, ColSet* S) {
 }
 
 template <typename T>
-mh_status run_cols(mh_ctx* ctx, const ColSet& S, const T* vec, T* dst, bool accumulate, const char* region) {
+mh_status run_cols(mh_ctx* ctx, const ColSet& S, const T* vec, T* dst, bool accumulate, const char* region,
+                   bool dep = true) {
     if (S.n_chunks == 0) return MH_OK;
     prof_scope ps(ctx, region, S.flops, S.bytes);
     const T* ops = sizeof(T) == 4 ? reinterpret_cast<const T*>(S.ops32.p) : reinterpret_cast<const T*>(S.ops64.p);
-    (void)mh_launch_dep(ctx->stream, k_cols<T>, dim3((unsigned)S.n_chunks), dim3(256), 0, ops, S.src.p, S.chunks.p,
-                        S.out_red.p, S.at.p, S.row.p, S.R, vec, reinterpret_cast<T*>(S.part.p), S.cnt.p,
-                        accumulate ? 1 : 0, dst);
+    const dim3 grid((unsigned)S.n_chunks);
+    T* part = reinterpret_cast<T*>(S.part.p);
+    if (dep)
+        (void)mh_launch_dep(ctx->stream, k_cols<T>, grid, dim3(256), 0, ops, S.src.p, S.chunks.p, S.out_red.p, S.at.p,
+                            S.row.p, S.R, vec, part, S.cnt.p, accumulate ? 1 : 0, dst);
+    else   // behind an event wait or a copy
+        k_cols<T><<<grid, 256, 0, ctx->stream>>>(ops, S.src.p, S.chunks.p, S.out_red.p, S.at.p, S.row.p, S.R, vec, part,
+                                                 S.cnt.p, accumulate ? 1 : 0, dst);
     MH_LAUNCHED(ctx);
     return MH_OK;
 }
@@ -1054,6 +1060,7 @@ mh_status run_phase_on(mh_ctx* ctx, const TOP* ops, const int64_t* op_off, const
         a.dst = ph->dst_out ? static_cast<void*>(out) : static_cast<void*>(pool);
         a.dst_double = ph->dst_out;
         a.err = tc->err.p;
+        a.dep = dep;
         // the tensor-core launch alone is also timed in "<region>_tc"
         prof_scope pt(ctx, std::strcmp(region, "volume_contract") == 0 ? "volume_contract_tc" : "dlp_fmm_contract_tc",
                       ph->tc_flops, ph->tc_bytes);
@@ -1114,9 +1121,9 @@ mh_status run_chain(mh_ctx* ctx, const LevelChain* ch, int P, int64_t m_base, in
 }
 
 template <typename TOP>
-mh_status run_phase(mh_ctx* ctx, VolData* V, const TOP* ops, const Phase* ph) {
-    return run_phase_on<TOP>(ctx, ops, V->d_op_off.p, V->d_op_C.p, typed_pool<TOP>(V->vec, V->vec32), V->vec.p,
-                             V->temp.p, ph, "volume_contract", &V->tc);
+mh_status run_phase(mh_ctx* ctx, VolData* V, const TOP* ops, const Phase* ph, double* out, bool dep) {
+    return run_phase_on<TOP>(ctx, ops, V->d_op_off.p, V->d_op_C.p, typed_pool<TOP>(V->vec, V->vec32), out, V->temp.p, ph,
+                             "volume_contract", &V->tc, dep);
 }
 
 struct HostTree {
@@ -1658,6 +1665,7 @@ __global__ void __launch_bounds__(NEAR_T) k_dip_near64(
     const int32_t* __restrict__ flat_idx, const double2* __restrict__ dxy, const double2* __restrict__ dnrm,
     const double* __restrict__ w, int qq, mh_pair_tab tab, double pref, double* part, unsigned* cnt,
     double* out) {
+    mh_dep_wait();
     __shared__ double2 sp[NEAR_T], sn[NEAR_T];
     const NearChunk ch = chunks[blockIdx.x];
     const int groups = NEAR_T / qq;   // >= 4 for q <= 8
@@ -1695,6 +1703,7 @@ __global__ void __launch_bounds__(NT) k_dip_near32(
     const double* __restrict__ nodes, const NearChunk* __restrict__ chunks, const int2* __restrict__ leaf_red,
     const double2* __restrict__ leaf_c, const int32_t* __restrict__ flat_idx, const float4* __restrict__ flat32,
     const float* __restrict__ w, int qq, mh_dl32 c32, double pref, double* part, unsigned* cnt, double* out) {
+    mh_dep_wait();
     __shared__ float4 s4[NT];
     const NearChunk ch = chunks[blockIdx.x];
     const int groups = NT / qq;
@@ -1734,6 +1743,13 @@ __global__ void __launch_bounds__(NT) k_dip_near32(
         }
     }
     near_finish<NT>((double)ah + (double)al, act, qq, i, groups, ch, leaf_red, pref, part, cnt, out);
+}
+
+template <typename T>
+__global__ void k_dip_weights(const double* __restrict__ w, const int32_t* __restrict__ perm, int64_t n, T* ws) {
+    mh_dep_wait();
+    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (j < n) ws[j] = (T)w[perm[j]];
 }
 
 __global__ void k_d2f(const double* __restrict__ a, float* __restrict__ b, int64_t n) {
@@ -2163,13 +2179,13 @@ mh_status volume_dipole_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, cons
 }
 
 template <typename TOP>
-static mh_status dipole_passes(mh_ctx* ctx, VolData* V, DipData* D, const TOP* ops) {
+static mh_status dipole_passes(mh_ctx* ctx, VolData* V, DipData* D, const TOP* ops, bool dep) {
     TOP* pool = typed_pool<TOP>(D->vec, D->vec32);
     auto run = [&](const Phase* ph) {
         return run_phase_on<TOP>(ctx, ops, D->d_op_off.p, D->d_op_C.p, pool, D->vec.p, D->temp.p, ph,
                                  "dlp_fmm_contract", &D->tc);
     };
-    MH_TRY(run_cols<TOP>(ctx, D->p2m, pool, pool, false, "dlp_fmm_contract"));
+    MH_TRY(run_cols<TOP>(ctx, D->p2m, pool, pool, false, "dlp_fmm_contract", dep));
     MH_TRY(run_chain<TOP>(ctx, D->chain_up.get(), V->P, D->DM_off, D->DL_off, pool, true, "dlp_fmm_chain"));
     if (sizeof(TOP) == 4) MH_TRY(tc_split(ctx, D->tc, 0, D->vec32.p));   // multipoles final
     // boxes whose V and X lists hold no dipoles get no M2L / P2L task: their locals are zeroed
@@ -2190,7 +2206,8 @@ static mh_status dipole_out(mh_ctx* ctx, DipData* D, const TOP* ops) {
 
 // w_sorted: dipole strengths in the leaf-sorted order given to volume_dipole_setup.
 // Returns a device pointer to U^h at every volume node (leaf-major), valid until the next call.
-mh_status volume_dipole_apply(mh_ctx* ctx, mh_tree* t, const double* w_sorted, mh_precision prec, const double** u) {
+mh_status volume_dipole_apply(mh_ctx* ctx, mh_tree* t, const double* w, const int32_t* perm, mh_precision prec,
+                              const double** u) {
     VolData* V = static_cast<VolData*>(t->vol);
     if (!V || !V->dip) return mh_fail(ctx, MH_ERR_INVALID_ARG, "dipole multipole pass not set up");
     DipData* D = V->dip.get();
@@ -2198,13 +2215,13 @@ mh_status volume_dipole_apply(mh_ctx* ctx, mh_tree* t, const double* w_sorted, m
     cudaStream_t st = ctx->stream;
     const bool mixed = prec == MH_PREC_MIXED;
     if (!D->near_blocks) MH_CUDA(ctx, cudaMemsetAsync(D->vec.p + D->DU_off, 0, t->n_leaves * D->qq * 8, st));
-    if (mixed) {
-        // weights in binary32 once: the contractions and the near-field kernel read them
-        k_d2f<<<mh_grid(D->nd, 256), 256, 0, st>>>(w_sorted, D->vec32.p + D->W_off, D->nd);
-        MH_LAUNCHED(ctx);
-    } else {
-        MH_CUDA(ctx, cudaMemcpyAsync(D->vec.p + D->W_off, w_sorted, D->nd * 8, cudaMemcpyDeviceToDevice, st));
-    }
+    // strengths in dipole order, in the precision that the contractions and the near field read
+    const unsigned gw = (unsigned)mh_grid(D->nd, 256);
+    if (mixed)
+        k_dip_weights<float><<<gw, 256, 0, st>>>(w, perm, D->nd, D->vec32.p + D->W_off);
+    else
+        k_dip_weights<double><<<gw, 256, 0, st>>>(w, perm, D->nd, D->vec.p + D->W_off);
+    MH_LAUNCHED(ctx);
     // The near field reads the weights and adds into U^h only; the passes read the weights and
     // touch only the expansions until their output phase adds the far field to U^h.  Without
     // region timers the passes run on the side stream while the near field runs on the context
@@ -2215,8 +2232,8 @@ mh_status volume_dipole_apply(mh_ctx* ctx, mh_tree* t, const double* w_sorted, m
     if (fork) {
         MH_TRY(D->side.begin(ctx, st));
         ctx->stream = D->side.s;
-        const mh_status s = mixed ? dipole_passes<float>(ctx, V, D, D->ops32.p)
-                                  : dipole_passes<double>(ctx, V, D, D->ops64.p);
+        const mh_status s = mixed ? dipole_passes<float>(ctx, V, D, D->ops32.p, false)
+                                  : dipole_passes<double>(ctx, V, D, D->ops64.p, false);
         ctx->stream = st;
         MH_TRY(s);
         MH_TRY(D->side.end(ctx));
@@ -2230,8 +2247,8 @@ mh_status volume_dipole_apply(mh_ctx* ctx, mh_tree* t, const double* w_sorted, m
             const mh_dl32 c32 = mh_dl32_make(1.0 / D->inv_alpha, 30.0);
             const double pref32 = D->pref * D->inv_alpha * D->inv_alpha;
 #define MH_NEAR32(NTV)                                                                                         \
-    k_dip_near32<NTV><<<nb, NTV, 0, st>>>(t->nodes.p, D->chunks.p, D->leaf_red.p, D->leaf_c.p, D->flat_idx.p,  \
-                                          D->flat32.p, w32, D->qq, c32, pref32, D->part.p, D->red_cnt.p, out)
+    (void)mh_launch_dep(st, k_dip_near32<NTV>, dim3(nb), dim3(NTV), 0, t->nodes.p, D->chunks.p, D->leaf_red.p, \
+                        D->leaf_c.p, D->flat_idx.p, D->flat32.p, w32, D->qq, c32, pref32, D->part.p, D->red_cnt.p, out)
             if (D->near_t == 128)
                 MH_NEAR32(128);
             else if (D->near_t == 512)
@@ -2240,17 +2257,17 @@ mh_status volume_dipole_apply(mh_ctx* ctx, mh_tree* t, const double* w_sorted, m
                 MH_NEAR32(256);
 #undef MH_NEAR32
         } else {
-            k_dip_near64<<<nb, NEAR_T, 0, st>>>(t->nodes.p, D->chunks.p, D->leaf_red.p, D->flat_idx.p, D->dxy.p,
-                                                D->dnrm.p, D->vec.p + D->W_off, D->qq,
-                                                mh_pair_tab_make(D->ptab.p, D->alpha),
-                                                D->pref * D->inv_alpha * D->inv_alpha, D->part.p, D->red_cnt.p, out);
+            (void)mh_launch_dep(st, k_dip_near64, dim3(nb), dim3(NEAR_T), 0, t->nodes.p, D->chunks.p, D->leaf_red.p,
+                                D->flat_idx.p, D->dxy.p, D->dnrm.p, D->vec.p + D->W_off, D->qq,
+                                mh_pair_tab_make(D->ptab.p, D->alpha), D->pref * D->inv_alpha * D->inv_alpha, D->part.p,
+                                D->red_cnt.p, out);
         }
         MH_LAUNCHED(ctx);
     }
     if (fork)
         MH_CUDA(ctx, cudaStreamWaitEvent(st, D->side.join, 0));
     else
-        MH_TRY(mixed ? dipole_passes<float>(ctx, V, D, D->ops32.p) : dipole_passes<double>(ctx, V, D, D->ops64.p));
+        MH_TRY(mixed ? dipole_passes<float>(ctx, V, D, D->ops32.p, true) : dipole_passes<double>(ctx, V, D, D->ops64.p, true));
     MH_TRY(mixed ? dipole_out<float>(ctx, D, D->ops32.p) : dipole_out<double>(ctx, D, D->ops64.p));
     *u = D->vec.p + D->DU_off;
     return MH_OK;
@@ -2488,79 +2505,72 @@ void volume_free(mh_tree* t) {
     t->vol = nullptr;
 }
 
-// The near tables read only the node values and write U^h; the passes touch only the
-// expansions until the output phase adds L2P and M2P to U^h.  Without region timers the passes
+// The near tables read only the node values and write the potential; the passes touch only the
+// expansions until the output phase adds L2P and M2P to it.  Without region timers the passes
 // run on the side stream while the near phase runs on the context stream, joined before the
 // output phase; with the timers everything runs in order on the context stream.  Both forms
-// write U^h as near, then add far.
+// write near, then add far, straight into the caller's array.
 template <typename TOP>
-static mh_status volume_passes(mh_ctx* ctx, VolData* V, const TOP* ops) {
+static mh_status volume_passes(mh_ctx* ctx, VolData* V, const TOP* ops, bool dep) {
     TOP* pool = typed_pool<TOP>(V->vec, V->vec32);
-    MH_TRY(run_phase(ctx, V, ops, V->p2m.get()));
+    MH_TRY(run_phase(ctx, V, ops, V->p2m.get(), nullptr, dep));
     MH_TRY(run_chain<TOP>(ctx, V->chain.get(), V->P, V->M_off, V->L_off, pool, true, "volume_chain"));
     if (sizeof(TOP) == 4) MH_TRY(tc_split(ctx, V->tc, 1, V->vec32.p));   // multipoles final
     if (!V->local_cover)   // the downward chain adds into the locals: those without an M2L task start at zero
         MH_CUDA(ctx, cudaMemsetAsync(pool + V->L_off, 0, (V->vec_len - V->L_off) * sizeof(TOP), ctx->stream));
-    MH_TRY(run_phase(ctx, V, ops, V->m2l.get()));
+    MH_TRY(run_phase(ctx, V, ops, V->m2l.get(), nullptr, V->local_cover));
     MH_TRY(run_chain<TOP>(ctx, V->chain.get(), V->P, V->M_off, V->L_off, pool, false, "volume_chain"));
     if (sizeof(TOP) == 4) MH_TRY(tc_split(ctx, V->tc, 2, V->vec32.p));   // locals final
     return MH_OK;
 }
 
 template <typename TOP>
-static mh_status volume_run(mh_ctx* ctx, mh_tree* t, VolData* V, const TOP* ops) {
+static mh_status volume_run(mh_ctx* ctx, mh_tree* t, VolData* V, const TOP* ops, double* up) {
     TOP* pool = typed_pool<TOP>(V->vec, V->vec32);
     cudaStream_t main = ctx->stream;
-    if (!V->near_cover)
-        MH_CUDA(ctx, cudaMemsetAsync(V->vec.p + V->U_off, 0, t->n_leaves * V->qq * 8, main));
+    double* out = up - V->U_off;   // output offsets count from the pool's start
+    if (!V->near_cover) MH_CUDA(ctx, cudaMemsetAsync(up, 0, t->n_leaves * V->qq * 8, main));
     const bool near = V->near->n_tasks > 0;
     const bool fork = near && !ctx->profiling && V->side.s;
     if (fork) {
         MH_TRY(V->side.begin(ctx, main));
         ctx->stream = V->side.s;
-        const mh_status s = volume_passes<TOP>(ctx, V, ops);
+        const mh_status s = volume_passes<TOP>(ctx, V, ops, false);
         ctx->stream = main;
         MH_TRY(s);
         MH_TRY(V->side.end(ctx));
     }
     if (near)
-        MH_TRY(run_phase_on<TOP>(ctx, ops, V->d_op_off.p, V->d_op_C.p, pool, V->vec.p, V->temp_near.p,
-                                 V->near.get(), "volume_contract", &V->tc));
+        MH_TRY(run_phase_on<TOP>(ctx, ops, V->d_op_off.p, V->d_op_C.p, pool, out, V->temp_near.p, V->near.get(),
+                                 "volume_contract", &V->tc, sizeof(TOP) == 4 && V->near_cover));
     if (fork)
         MH_CUDA(ctx, cudaStreamWaitEvent(main, V->side.join, 0));
     else
-        MH_TRY(volume_passes<TOP>(ctx, V, ops));
-    MH_TRY(run_phase(ctx, V, ops, V->out.get()));
+        MH_TRY(volume_passes<TOP>(ctx, V, ops, false));
+    MH_TRY(run_phase(ctx, V, ops, V->out.get(), out, false));
     return MH_OK;
 }
 
 mh_status volume_apply(mh_ctx* ctx, mh_tree* t, double alpha, int p, const double* b, double* up,
                        mh_precision prec) {
+    MH_TRY(volume_ensure(ctx, t, alpha, p));
     VolData* V = static_cast<VolData*>(t->vol);
-    if (!V || V->alpha != alpha || V->p != p) {
-        delete V;
-        V = new VolData();
-        t->vol = V;
-        mh_status s = volume_setup(ctx, t, alpha, p, V);
-        if (s != MH_OK) {
-            delete V;
-            t->vol = nullptr;
-            return s;
-        }
-    }
     const int64_t nn = t->n_nodes;
     prof_scope ps(ctx, "volume_apply");
     if (prec == MH_PREC_MIXED) {
         // node values in binary32 once: every contraction then gathers binary32
-        k_d2f<<<mh_grid(nn, 256), 256, 0, ctx->stream>>>(b, V->vec32.p + V->B_off, nn);
-        MH_LAUNCHED(ctx);
-        MH_TRY(tc_split(ctx, V->tc, 0, V->vec32.p));   // node values final
-        MH_TRY(volume_run<float>(ctx, t, V, V->ops32.p));
+        if (V->tc.ready && ctx->tensor_cores && !V->tc.ranges.empty()) {
+            const TcImages::Range& r = V->tc.ranges[0];
+            MH_TRY(tc_split_values(ctx, b, r.len, r.count, r.S, V->vec32.p + V->B_off, V->tc.planes.p, V->tc.plane, r.dst));
+        } else {
+            k_d2f<<<mh_grid(nn, 256), 256, 0, ctx->stream>>>(b, V->vec32.p + V->B_off, nn);
+            MH_LAUNCHED(ctx);
+        }
+        MH_TRY(volume_run<float>(ctx, t, V, V->ops32.p, up));
     } else {
         MH_CUDA(ctx, cudaMemcpyAsync(V->vec.p + V->B_off, b, nn * 8, cudaMemcpyDeviceToDevice, ctx->stream));
-        MH_TRY(volume_run<double>(ctx, t, V, V->ops64.p));
+        MH_TRY(volume_run<double>(ctx, t, V, V->ops64.p, up));
     }
-    MH_CUDA(ctx, cudaMemcpyAsync(up, V->vec.p + V->U_off, nn * 8, cudaMemcpyDeviceToDevice, ctx->stream));
     return MH_OK;
 }
 
