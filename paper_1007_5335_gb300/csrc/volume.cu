@@ -23,11 +23,13 @@
 #include <array>
 #include <cmath>
 #include <complex>
+#include <cstdint>
 #include <cstring>
 #include <map>
 #include <memory>
 #include <tuple>
 #include <type_traits>
+#include <vector>
 
 #include "bessel.cuh"
 #include <cooperative_groups.h>
@@ -263,6 +265,8 @@ __device__ __forceinline__ void stage_rows(TD* dst, const TS* __restrict__ src, 
             if (e0 + u * stride < n) dst[oo[u]] = (TD)v[u];
     }
 }
+
+#include "orbit.cuh"
 
 // Batched contraction: each block applies one operator (R x C, row-major) to up to CHUNK
 // source vectors gathered from the pool `src` (the operators' precision: node values and
@@ -757,14 +761,247 @@ struct OpPool {
     std::vector<double> data;
     std::vector<int64_t> off;
     std::vector<int32_t> R, C;
+    // reflection orbits: the operator is the image under reflections g of operator rep, its offset is left
+    // alone by the reflections stab (rep = -1: no symmetry, as for a block of dipoles)
+    struct Sym {
+        int rep = -1, g = 0, stab = 0;
+        bool col_nodes = false;
+    };
+    std::vector<Sym> sym;
+    std::map<std::tuple<int, int, int, int, int>, int> reps;   // (kind, level, source level, |x|, |y|) -> first of the orbit
+    std::vector<int> rep_g;                               // reflections of a representative's own offset
     int add(int r, int c, const double* v) {
-        off.push_back((int64_t)data.size());
+        const int id = add_shape((int64_t)data.size(), r, c);
+        data.insert(data.end(), v, v + (size_t)r * c);
+        return id;
+    }
+    int add_shape(int64_t at, int r, int c) {
+        off.push_back(at);
         R.push_back(r);
         C.push_back(c);
-        data.insert(data.end(), v, v + (size_t)r * c);
+        sym.emplace_back();
+        rep_g.push_back(0);
         return (int)off.size() - 1;
     }
+    // kind: 0 P2M, 1 L2P, 2 M2L, 3 P2L, 4 M2P, 5 near table; (x, y): source centre - target centre in any unit
+    int mirror(int id, int kind, int level, int source_level, int x, int y) {
+        const int g = (x < 0 ? 1 : 0) | (y < 0 ? 2 : 0);
+        const int rep = reps.emplace(std::make_tuple(kind, level, source_level, std::abs(x), std::abs(y)), id).first->second;
+        if (rep == id) rep_g[id] = g;
+        Sym& s = sym[id];
+        s.rep = rep;
+        s.g = g ^ rep_g[rep];
+        s.stab = (x == 0 ? 1 : 0) | (y == 0 ? 2 : 0);
+        s.col_nodes = kind == 0 || kind == 3 || kind == 5;
+        return id;
+    }
 };
+
+// The binary64 form of a phase: its tasks by reflection orbits (k_orbit).
+struct OrbPhase {
+    int R = 0, groups = 1, smem = 0;
+    bool row_nodes = false, accumulate = false, direct = false;
+    int64_t n_tasks = 0, n_dst = 0, n_chunks = 0;
+    double flops = 0, bytes = 0;
+    OrbDims dims;
+    dbuf<double> ops;
+    dbuf<OrbOp> op;
+    dbuf<OrbSrc> src;
+    dbuf<int32_t> chunk_op, chunk_t0, dst_ptr, dst_task, perm;
+    dbuf<int64_t> task_dst, dst_off;
+};
+
+// (destination, task) pairs sorted by destination -> destinations, their first entries, the tasks.
+void group_by_destination(const std::vector<std::pair<int64_t, int32_t>>& bydst, std::vector<int64_t>* doff,
+                          std::vector<int32_t>* dptr, std::vector<int32_t>* dtask) {
+    dtask->reserve(bydst.size());
+    for (const auto& d : bydst) {
+        if (doff->empty() || doff->back() != d.first) {
+            doff->push_back(d.first);
+            dptr->push_back((int32_t)dtask->size());
+        }
+        dtask->push_back(d.second);
+    }
+    dptr->push_back((int32_t)dtask->size());
+}
+
+OrbDims orb_dims(const OrbSpace& nodes, const OrbSpace& exps) {
+    OrbDims d;
+    for (int c = 0; c < 5; ++c) {
+        d.nodes[c] = nodes.first[c];
+        d.exp[c] = exps.first[c];
+    }
+    return d;
+}
+
+// ops: every operator of the pool (host, row-major at pool.off).  Sources and destinations of
+// node values are in class order.
+mh_status build_orbits(mh_ctx* ctx, const std::vector<Task>& tasks, int R, bool row_nodes, bool accumulate,
+                       const OpPool& pool, const double* ops, int q, int p, OrbPhase* ph, int64_t* temp_need) {
+    const OrbSpace nodes = orb_nodes(q), exps = orb_expansions(p);
+    ph->R = R;
+    ph->row_nodes = row_nodes;
+    ph->accumulate = accumulate;
+    ph->dims = orb_dims(nodes, exps);
+    struct Item {
+        int stab, rep, g;
+        int64_t dst, src;
+    };
+    std::vector<Item> items;
+    items.reserve(tasks.size());
+    for (const Task& t : tasks) {
+        const OpPool::Sym& s = pool.sym[t.op];
+        items.push_back(Item{s.stab, s.rep, s.g, t.dst, t.src});
+    }
+    // by operator (the dear ones, without a reflection of their own, first), destination, image
+    std::sort(items.begin(), items.end(), [](const Item& x, const Item& y) {
+        return std::tie(x.stab, x.rep, x.dst, x.g) < std::tie(y.stab, y.rep, y.dst, y.g);
+    });
+    // operators in class order; shared memory and thread groups by the largest of the phase
+    std::vector<double> data;
+    std::vector<OrbOp> op;
+    std::map<int, int> op_id;
+    int maxC = 1, groups = 8, smem = 0;
+    for (const Item& it : items) {
+        if (op_id.count(it.rep)) continue;
+        const OpPool::Sym& s = pool.sym[it.rep];
+        const int C = pool.C[it.rep];
+        const std::vector<double> m = orb_operator(ops + pool.off[it.rep], R, C, row_nodes ? nodes : exps,
+                                                   s.col_nodes ? nodes : exps, q);
+        op_id[it.rep] = (int)op.size();
+        op.push_back(OrbOp{(int64_t)data.size(), C, s.stab, s.col_nodes ? 1 : 0, 0});
+        data.insert(data.end(), m.begin(), m.end());
+        maxC = std::max(maxC, C);
+        groups = std::min(groups, orb_groups(R, C, s.stab == 3 ? 1 : s.stab ? 2 : 4));
+    }
+    if (groups == 0)
+        return mh_fail(ctx, MH_ERR_INVALID_ARG, "contraction operator too large for shared memory (%d x %d)", R, maxC);
+    for (const OrbOp& o : op)
+        smem = std::max(smem, (int)orb_smem(R, o.C, groups, o.stab == 3 ? 1 : o.stab ? 2 : 4));
+    ph->groups = groups;
+    ph->smem = smem;
+    // tasks (orbits)
+    std::vector<OrbSrc> src;
+    std::vector<int64_t> dst;
+    std::vector<std::pair<int, size_t>> runs;   // operator, first task
+    for (const Item& it : items) {
+        const bool next = runs.empty() || runs.back().first != it.rep;
+        if (next) runs.emplace_back(it.rep, src.size());
+        if (next || dst.back() != it.dst || src.back().at[it.g] >= 0) {
+            src.push_back(OrbSrc{{-1, -1, -1, -1}});
+            dst.push_back(it.dst);
+        }
+        src.back().at[it.g] = it.src;
+    }
+    // Chunks of nearly equal numbers of tasks per operator: ORB_TT for every group, but fewer where that would
+    // leave less than 4 chunks for an SM (full chunks everywhere: matrix-free solve 3298 us against 3130, step with
+    // curves of 64 nodes 377 against 352, binary64 volume potential 394 against 357)
+    const int64_t per = ((int64_t)src.size() + 4 * 152 * groups - 1) / (4 * 152 * groups);
+    const int64_t cap = groups * std::min<int64_t>(ORB_TT, std::max<int64_t>(per, 1));
+    std::vector<int32_t> cop, ct0;
+    for (size_t k = 0; k < runs.size(); ++k) {
+        const int rep = runs[k].first;
+        const size_t first = runs[k].second;
+        const int64_t n = (int64_t)((k + 1 < runs.size() ? runs[k + 1].second : src.size()) - first);
+        const int64_t nc = (n + cap - 1) / cap;
+        const OrbOp& o = op[op_id[rep]];
+        for (int64_t c = 0; c < nc; ++c) {
+            cop.push_back(op_id[rep]);
+            ct0.push_back((int32_t)(first + n * c / nc));
+        }
+        const double images = o.stab == 3 ? 1 : o.stab ? 2 : 4;
+        ph->flops += n * (2.0 * R * o.C * images / 4 + (images > 1 ? 2.0 * images * o.C : 0.0));
+        ph->bytes += n * (8.0 * o.C * images + 16.0 * R) + 8.0 * R * o.C * nc;
+    }
+    ct0.push_back((int32_t)src.size());
+    ph->n_tasks = (int64_t)src.size();
+    ph->n_chunks = (int64_t)cop.size();
+    std::vector<std::pair<int64_t, int32_t>> bydst(dst.size());
+    for (size_t i = 0; i < dst.size(); ++i) bydst[i] = {dst[i], (int32_t)i};
+    std::sort(bydst.begin(), bydst.end());
+    std::vector<int64_t> doff;
+    std::vector<int32_t> dptr, dtask;
+    group_by_destination(bydst, &doff, &dptr, &dtask);
+    ph->n_dst = (int64_t)doff.size();
+    ph->direct = ph->n_dst == ph->n_tasks && ph->n_tasks > 0;   // (sources and destinations are different ranges)
+    cudaStream_t st = ctx->stream;
+    auto up = [&](auto& b, const auto& v) -> mh_status {
+        MH_ALLOC(ctx, b, std::max<size_t>(v.size(), 1));
+        if (!v.empty())
+            MH_CUDA(ctx, cudaMemcpyAsync(b.p, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice, st));
+        return MH_OK;
+    };
+    MH_TRY(up(ph->ops, data));
+    MH_TRY(up(ph->op, op));
+    MH_TRY(up(ph->src, src));
+    MH_TRY(up(ph->chunk_op, cop));
+    MH_TRY(up(ph->chunk_t0, ct0));
+    MH_TRY(up(ph->perm, exps.perm));
+    if (ph->direct) {
+        MH_TRY(up(ph->task_dst, dst));
+    } else {
+        MH_TRY(up(ph->dst_ptr, dptr));
+        MH_TRY(up(ph->dst_task, dtask));
+        MH_TRY(up(ph->dst_off, doff));
+        *temp_need = std::max<int64_t>(*temp_need, ph->n_tasks * R);
+    }
+    MH_CUDA(ctx, cudaStreamSynchronize(st));
+    MH_CUDA(ctx, cudaFuncSetAttribute(k_orbit, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    return MH_OK;
+}
+
+// src: pool the offsets count from; dst likewise.
+mh_status run_orbits(mh_ctx* ctx, const OrbPhase* ph, const double* src, double* dst, double* temp, const char* region,
+                     bool dep) {
+    if (ph->n_tasks == 0) return MH_OK;
+    prof_scope ps(ctx, region, ph->flops, ph->bytes + 8.0 * ph->R * ph->n_dst * (ph->accumulate ? 2 : 1));
+    const int acc = ph->accumulate ? 1 : 0, rn = ph->row_nodes ? 1 : 0;
+    const dim3 grid((unsigned)ph->n_chunks), block(ORB_THREADS);
+    const int64_t* tdst = ph->direct ? ph->task_dst.p : nullptr;
+    if (dep)
+        (void)mh_launch_dep(ctx->stream, k_orbit, grid, block, ph->smem, ph->ops.p, ph->op.p, ph->chunk_op.p, ph->chunk_t0.p,
+                            ph->src.p, ph->perm.p, ph->dims, ph->R, rn, ph->groups, src, temp, tdst, acc, dst);
+    else
+        k_orbit<<<grid, block, ph->smem, ctx->stream>>>(ph->ops.p, ph->op.p, ph->chunk_op.p, ph->chunk_t0.p, ph->src.p,
+                                                        ph->perm.p, ph->dims, ph->R, rn, ph->groups, src, temp, tdst, acc,
+                                                        dst);
+    MH_LAUNCHED(ctx);
+    if (!ph->direct) {
+        (void)mh_launch_dep(ctx->stream, k_reduce<double, double>, dim3((unsigned)mh_grid(ph->n_dst * 32, 256)), dim3(256), 0,
+                            temp, ph->R, ph->dst_off.p, ph->dst_ptr.p, ph->dst_task.p, ph->n_dst, acc, dst);
+        MH_LAUNCHED(ctx);
+    }
+    return MH_OK;
+}
+
+// Node values from their even and odd components; dep: directly behind a kernel of the same stream.
+mh_status run_back(mh_ctx* ctx, const double* w, const int32_t* at, int q, int64_t n, bool accumulate, double* u, bool dep) {
+    const dim3 grid((unsigned)mh_grid(n, 256)), block(256);
+    const int acc = accumulate ? 1 : 0;
+    if (dep)
+        (void)mh_launch_dep(ctx->stream, k_orb_back, grid, block, 0, w, at, q, n, acc, u);
+    else
+        k_orb_back<<<grid, block, 0, ctx->stream>>>(w, at, q, n, acc, u);
+    MH_LAUNCHED(ctx);
+    return MH_OK;
+}
+
+// Tables of the node transforms (k_orb_forward, k_orb_back).
+mh_status build_node_tables(mh_ctx* ctx, int q, dbuf<int32_t>* fwd, dbuf<int32_t>* back) {
+    const OrbSpace S = orb_nodes(q);
+    const int qq = q * q;
+    std::vector<int32_t> f(qq), b(4 * qq, 0);
+    for (int k = 0; k < qq; ++k) {
+        f[k] = S.a[k] | S.b[k] << 8 | S.cls[k] << 16;
+        b[S.cls[k] * qq + S.b[k] * q + S.a[k]] = k;
+    }
+    MH_ALLOC(ctx, *fwd, qq);
+    MH_ALLOC(ctx, *back, 4 * qq);
+    MH_CUDA(ctx, cudaMemcpyAsync(fwd->p, f.data(), qq * 4, cudaMemcpyHostToDevice, ctx->stream));
+    MH_CUDA(ctx, cudaMemcpyAsync(back->p, b.data(), 4 * qq * 4, cudaMemcpyHostToDevice, ctx->stream));
+    MH_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    return MH_OK;
+}
 
 // M2M / L2L of every level 2 <= l < L in parent-centric form (k_level_up / k_level_down): the
 // internal boxes with their children, by level.
@@ -798,6 +1035,8 @@ struct VolData {
     dbuf<int32_t> d_op_C;
     std::vector<int> op_C;
     std::unique_ptr<Phase> p2m, m2l, out;
+    OrbPhase p2m64, m2l64, out64, near64;             // their binary64 forms, on node values in class order
+    dbuf<int32_t> node_fwd, node_back;
     std::unique_ptr<Phase> near;                      // U list: near tables on the node values
     dbuf<double> temp_near;                           // its products (it may run beside the others)
     bool near_cover = true;                           // every leaf has a U-list task
@@ -817,11 +1056,11 @@ mh_status build_phase(mh_ctx* ctx, std::vector<Task>& tasks, int R, bool accumul
     ph->accumulate = accumulate;
     ph->n_tasks = (int64_t)tasks.size();
     // operators of the tensor-core form: >= TC_MIN_TASKS tasks and at most 64 x 64
-    std::map<int, int64_t> per_op;
+    std::vector<int64_t> per_op(op_C.size(), 0);
     for (const Task& t : tasks) per_op[t.op] += 1;
-    std::map<int, bool> on_tc;
-    for (auto& kv : per_op)
-        on_tc[kv.first] = ranges && R <= 64 && kv.second >= TC_MIN_TASKS && op_C[kv.first] <= 64;
+    std::vector<char> on_tc(op_C.size(), 0);
+    for (size_t o = 0; o < op_C.size(); ++o)
+        on_tc[o] = ranges && R <= 64 && per_op[o] >= TC_MIN_TASKS && op_C[o] <= 64;
     if (ranges)
         for (const Task& t : tasks) {
             if (!on_tc[t.op]) continue;
@@ -896,15 +1135,12 @@ mh_status build_phase(mh_ctx* ctx, std::vector<Task>& tasks, int R, bool accumul
     // destinations: tasks grouped by destination in generation order
     std::vector<int64_t> rank(tasks.size());
     for (size_t s = 0; s < order.size(); ++s) rank[order[s]] = (int64_t)s;
-    std::map<int64_t, std::vector<int32_t>> bydst;
-    for (size_t i = 0; i < tasks.size(); ++i) bydst[tasks[i].dst].push_back((int32_t)rank[i]);
+    std::vector<std::pair<int64_t, int32_t>> bydst(tasks.size());
+    for (size_t i = 0; i < tasks.size(); ++i) bydst[i] = {tasks[i].dst, (int32_t)rank[i]};
+    std::stable_sort(bydst.begin(), bydst.end(), [](const auto& x, const auto& y) { return x.first < y.first; });
     std::vector<int64_t> doff;
-    std::vector<int32_t> dptr{0}, dtask;
-    for (auto& kv : bydst) {
-        doff.push_back(kv.first);
-        dtask.insert(dtask.end(), kv.second.begin(), kv.second.end());
-        dptr.push_back((int32_t)dtask.size());
-    }
+    std::vector<int32_t> dptr, dtask;
+    group_by_destination(bydst, &doff, &dptr, &dtask);
     ph->n_dst = (int64_t)doff.size();
     // direct mode: a single task per destination and source / destination ranges apart
     if (ph->n_dst == ph->n_tasks && ph->n_tasks > 0) {
@@ -1120,10 +1356,15 @@ mh_status run_chain(mh_ctx* ctx, const LevelChain* ch, int P, int64_t m_base, in
     return MH_OK;
 }
 
+// A phase of the volume pass: binary32 on the tensor cores, binary64 by reflection orbits.
+// out: binary64 potentials (binary32 form) of the output phases.
 template <typename TOP>
-mh_status run_phase(mh_ctx* ctx, VolData* V, const TOP* ops, const Phase* ph, double* out, bool dep) {
-    return run_phase_on<TOP>(ctx, ops, V->d_op_off.p, V->d_op_C.p, typed_pool<TOP>(V->vec, V->vec32), out, V->temp.p, ph,
-                             "volume_contract", &V->tc, dep);
+mh_status run_phase(mh_ctx* ctx, VolData* V, const Phase* ph, const OrbPhase* ph64, double* out, double* temp, bool dep) {
+    if constexpr (sizeof(TOP) == 8)
+        return run_orbits(ctx, ph64, V->vec.p, V->vec.p, temp, "volume_contract", dep);
+    else
+        return run_phase_on<float>(ctx, V->ops32.p, V->d_op_off.p, V->d_op_C.p, V->vec32.p, out, temp, ph, "volume_contract",
+                                   &V->tc, dep);
 }
 
 struct HostTree {
@@ -1301,7 +1542,7 @@ mh_status volume_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, VolData* V)
                     }
                 }
             }
-        op_p2m[l] = pool.add(P, qq, buf.data());
+        op_p2m[l] = pool.mirror(pool.add(P, qq, buf.data()), 0, l, l, 0, 0);
         buf.assign((size_t)qq * P, 0.0);
         for (int i = 0; i < qq; ++i) {
             const double X = 0.5 * w * qx[i % q], Y = 0.5 * w * qx[i / q];
@@ -1316,7 +1557,7 @@ mh_status volume_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, VolData* V)
                 }
             }
         }
-        op_l2p[l] = pool.add(qq, P, buf.data());
+        op_l2p[l] = pool.mirror(pool.add(qq, P, buf.data()), 1, l, l, 0, 0);
     }
     // ---- M2M and L2L (child c at level l+1, parent at l) ----
     std::vector<std::array<int, 4>> op_m2m(L + 1), op_l2l(L + 1);
@@ -1346,7 +1587,7 @@ mh_status volume_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, VolData* V)
     // ---- configuration-keyed operators discovered from the lists ----
     std::map<std::tuple<int, int, int, int>, int> near_key, m2l_key, m2p_key, p2l_key;
     std::vector<NearCfg> near_cfg;
-    std::vector<int> near_level;
+    std::vector<std::array<int, 4>> near_off;   // target level, source level, offset of the centres
     std::vector<Task> t_out, t_m2l, t_p2m, t_near;
     // relative centre offset (source minus target) from integer coordinates
     auto rel = [&](int tb, int sb) {
@@ -1375,7 +1616,9 @@ mh_status volume_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, VolData* V)
                     near_key[key] = id;
                     const std::complex<double> r = rel((int)b, c);
                     near_cfg.push_back(NearCfg{r.real(), r.imag(), width(lc), width(l)});
-                    near_level.push_back(l);
+                    // centres in half widths of the finer box
+                    const int e = (1 << (f - lc)) - (1 << (f - l));
+                    near_off.push_back({l, lc, 2 * ox + e, 2 * oy + e});
                 } else {
                     id = it->second;
                 }
@@ -1407,7 +1650,9 @@ mh_status volume_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, VolData* V)
                             }
                         }
                     }
-                    id = pool.add(qq, P, buf.data());
+                    // centres in half widths of the source box (one level down)
+                    id = pool.mirror(pool.add(qq, P, buf.data()), 4, l, l + 1, 2 * std::get<1>(key) - 1,
+                                     2 * std::get<2>(key) - 1);
                     m2p_key[key] = id;
                 } else {
                     id = it->second;
@@ -1435,7 +1680,7 @@ mh_status volume_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, VolData* V)
                               return Is[l][m] * sg * Kb[std::abs(jj)] * std::polar(1.0, jj * Ph) * Is[l][std::abs(n)];
                           },
                           buf.data());
-                id = pool.add(P, P, buf.data());
+                id = pool.mirror(pool.add(P, P, buf.data()), 2, l, l, std::get<1>(key), std::get<2>(key));
                 m2l_key[key] = id;
             } else {
                 id = it->second;
@@ -1473,7 +1718,9 @@ mh_status volume_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, VolData* V)
                             }
                         }
                     }
-                id = pool.add(P, qq, buf.data());
+                // centres in half widths of the target box (one level down)
+                id = pool.mirror(pool.add(P, qq, buf.data()), 3, l, l - 1, 2 * std::get<1>(key) + 1,
+                                 2 * std::get<2>(key) + 1);
                 p2l_key[key] = id;
             } else {
                 id = it->second;
@@ -1496,9 +1743,8 @@ mh_status volume_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, VolData* V)
     const int64_t near_base = (int64_t)pool.data.size();
     const int first_near_op = (int)pool.off.size();
     for (int i = 0; i < nnear; ++i) {
-        pool.off.push_back(near_base + (int64_t)i * qq * qq);
-        pool.R.push_back(qq);
-        pool.C.push_back(qq);
+        const std::array<int, 4>& o = near_off[i];
+        pool.mirror(pool.add_shape(near_base + (int64_t)i * qq * qq, qq, qq), 5, o[0], o[1], o[2], o[3]);
     }
     for (auto& tk : t_near) tk.op = first_near_op + (-1 - tk.op);
     const int64_t total = near_base + (int64_t)nnear * qq * qq;
@@ -1564,6 +1810,11 @@ mh_status volume_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, VolData* V)
     V->out.reset(new Phase());
     MH_TRY(build_phase(ctx, t_out, qq, true, V->op_C, V->out.get(), &need, &rg));
     V->out->dst_out = true;
+    MH_TRY(build_orbits(ctx, t_p2m, P, false, false, pool, all.data(), q, p, &V->p2m64, &need));
+    MH_TRY(build_orbits(ctx, t_m2l, P, false, false, pool, all.data(), q, p, &V->m2l64, &need));
+    MH_TRY(build_orbits(ctx, t_near, qq, true, false, pool, all.data(), q, p, &V->near64, &need_near));
+    MH_TRY(build_orbits(ctx, t_out, qq, true, true, pool, all.data(), q, p, &V->out64, &need));
+    MH_TRY(build_node_tables(ctx, q, &V->node_fwd, &V->node_back));
     {
         std::vector<int64_t> off(pool.off.begin(), pool.off.end());
         std::vector<int32_t> rr(pool.R.begin(), pool.R.end()), cc(pool.C.begin(), pool.C.end());
@@ -1781,6 +2032,8 @@ struct DipData {
     dbuf<int32_t> d_op_C;
     ColSet p2m, p2l;                       // dipole P2M of the leaves, dipole P2L over the X lists
     std::unique_ptr<Phase> m2l, out;
+    OrbPhase m2l64, out64;                 // binary64 forms (out64: without dense near blocks)
+    dbuf<double> far;                      // far field at the nodes in class order (binary64)
     std::unique_ptr<LevelChain> chain_up;     // M2M over the boxes that hold dipoles
     SideStream side;                       // the near field runs there beside the passes
     TcImages tc;                           // tensor-core images (mixed precision)
@@ -2159,6 +2412,12 @@ mh_status volume_dipole_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, cons
     D->out.reset(new Phase());
     MH_TRY(build_phase(ctx, t_out, qq, !near_blocks, opC, D->out.get(), &need, &rg));
     D->out->dst_out = true;
+    MH_TRY(build_orbits(ctx, t_m2l, P, false, false, pool, pool.data.data(), q, p, &D->m2l64, &need));
+    if (!near_blocks) {
+        MH_TRY(build_orbits(ctx, t_out, qq, true, false, pool, pool.data.data(), q, p, &D->out64, &need));
+        MH_ALLOC(ctx, D->far, nl * qq);   // leaves without an output task stay at zero
+        MH_CUDA(ctx, cudaMemsetAsync(D->far.p, 0, nl * qq * 8, st));
+    }
     {
         std::vector<int64_t> off(pool.off.begin(), pool.off.end());
         std::vector<int32_t> rr(pool.R.begin(), pool.R.end()), cc(pool.C.begin(), pool.C.end());
@@ -2182,8 +2441,11 @@ template <typename TOP>
 static mh_status dipole_passes(mh_ctx* ctx, VolData* V, DipData* D, const TOP* ops, bool dep) {
     TOP* pool = typed_pool<TOP>(D->vec, D->vec32);
     auto run = [&](const Phase* ph) {
-        return run_phase_on<TOP>(ctx, ops, D->d_op_off.p, D->d_op_C.p, pool, D->vec.p, D->temp.p, ph,
-                                 "dlp_fmm_contract", &D->tc);
+        if constexpr (sizeof(TOP) == 8)
+            return run_orbits(ctx, &D->m2l64, D->vec.p, D->vec.p, D->temp.p, "dlp_fmm_contract", false);
+        else
+            return run_phase_on<TOP>(ctx, ops, D->d_op_off.p, D->d_op_C.p, pool, D->vec.p, D->temp.p, ph,
+                                     "dlp_fmm_contract", &D->tc);
     };
     MH_TRY(run_cols<TOP>(ctx, D->p2m, pool, pool, false, "dlp_fmm_contract", dep));
     MH_TRY(run_chain<TOP>(ctx, D->chain_up.get(), V->P, D->DM_off, D->DL_off, pool, true, "dlp_fmm_chain"));
@@ -2198,8 +2460,16 @@ static mh_status dipole_passes(mh_ctx* ctx, VolData* V, DipData* D, const TOP* o
     return MH_OK;
 }
 
+// Binary64 without dense near blocks: every operator of the output phase has the reflections, the far
+// field is formed as even and odd components and added to U^h as it is transformed back.
 template <typename TOP>
-static mh_status dipole_out(mh_ctx* ctx, DipData* D, const TOP* ops) {
+static mh_status dipole_out(mh_ctx* ctx, mh_tree* t, VolData* V, DipData* D, const TOP* ops) {
+    if (sizeof(TOP) == 8 && !D->near_blocks) {
+        const int64_t nn = t->n_leaves * D->qq;
+        double* far = D->far.p - D->DU_off;
+        MH_TRY(run_orbits(ctx, &D->out64, D->vec.p, far, D->temp.p, "dlp_fmm_contract", false));
+        return run_back(ctx, D->far.p, V->node_back.p, t->q, nn, true, D->vec.p + D->DU_off, D->out64.n_tasks > 0);
+    }
     return run_phase_on<TOP>(ctx, ops, D->d_op_off.p, D->d_op_C.p, typed_pool<TOP>(D->vec, D->vec32), D->vec.p,
                              D->temp.p, D->out.get(), "dlp_fmm_contract", &D->tc);
 }
@@ -2268,7 +2538,7 @@ mh_status volume_dipole_apply(mh_ctx* ctx, mh_tree* t, const double* w, const in
         MH_CUDA(ctx, cudaStreamWaitEvent(st, D->side.join, 0));
     else
         MH_TRY(mixed ? dipole_passes<float>(ctx, V, D, D->ops32.p, true) : dipole_passes<double>(ctx, V, D, D->ops64.p, true));
-    MH_TRY(mixed ? dipole_out<float>(ctx, D, D->ops32.p) : dipole_out<double>(ctx, D, D->ops64.p));
+    MH_TRY(mixed ? dipole_out<float>(ctx, t, V, D, D->ops32.p) : dipole_out<double>(ctx, t, V, D, D->ops64.p));
     *u = D->vec.p + D->DU_off;
     return MH_OK;
 }
@@ -2290,12 +2560,10 @@ struct BieData {
     int64_t nd = 0, n_groups = 0;
     int64_t W_off = 0, DM_off = 0, DL_off = 0, vec_len = 0;
     double flops = 0, near_pairs = 0;
-    dbuf<double> vec, temp, ops64;
-    dbuf<int64_t> d_op_off;
-    dbuf<int32_t> d_op_C;
+    dbuf<double> vec, temp;
     dbuf<int32_t> perm;   // sorted position -> node
     ColSet p2m, p2l, out;
-    std::unique_ptr<Phase> m2l;
+    OrbPhase m2l;
     std::unique_ptr<LevelChain> chain;   // M2M / L2L over the active boxes
 };
 
@@ -2353,7 +2621,7 @@ mh_status volume_bie_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, const d
     B->DM_off = nd;
     B->DL_off = B->DM_off + nb * P;
     B->vec_len = B->DL_off + nb * P;
-    OpPool pool = V->pool_host;
+    const OpPool& pool = V->pool_host;
     std::vector<Task> t_m2l;
     ColBuild p2m(P), p2l(P), out(BIE_RT);
     const std::vector<char> active = dipole_active_boxes(h, segn);
@@ -2426,21 +2694,12 @@ mh_status volume_bie_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, const d
         }
     }
     cudaStream_t st = ctx->stream;
-    const int64_t total = (int64_t)pool.data.size();
-    MH_ALLOC(ctx, B->ops64, total);
-    MH_CUDA(ctx, cudaMemcpyAsync(B->ops64.p, pool.data.data(), total * 8, cudaMemcpyHostToDevice, st));
-    MH_ALLOC(ctx, B->d_op_off, pool.off.size());
-    MH_ALLOC(ctx, B->d_op_C, pool.C.size());
-    MH_CUDA(ctx, cudaMemcpyAsync(B->d_op_off.p, pool.off.data(), pool.off.size() * 8, cudaMemcpyHostToDevice, st));
-    MH_CUDA(ctx, cudaMemcpyAsync(B->d_op_C.p, pool.C.data(), pool.C.size() * 4, cudaMemcpyHostToDevice, st));
-    std::vector<int> opC(pool.C.begin(), pool.C.end());
     int64_t need = 1;
     MH_TRY(build_cols(ctx, p2m, false, &B->p2m));
     MH_TRY(build_cols(ctx, p2l, false, &B->p2l));
     MH_TRY(build_cols(ctx, out, false, &B->out));
-    B->m2l.reset(new Phase());
-    MH_TRY(build_phase(ctx, t_m2l, P, false, opC, B->m2l.get(), &need));
-    B->flops += B->p2m.flops + B->p2l.flops + B->m2l->flops;
+    MH_TRY(build_orbits(ctx, t_m2l, P, false, false, pool, pool.data.data(), t->q, p, &B->m2l, &need));
+    B->flops += B->p2m.flops + B->p2l.flops + B->m2l.flops;
     MH_ALLOC(ctx, B->vec, B->vec_len);
     MH_ALLOC(ctx, B->temp, need);
     MH_CUDA(ctx, cudaMemsetAsync(B->vec.p, 0, B->vec_len * 8, st));
@@ -2471,14 +2730,10 @@ mh_status volume_bie_apply(mh_ctx* ctx, mh_tree* t, const double* w, double* u) 
     const unsigned g = (unsigned)mh_grid(B->nd, 256);
     (void)mh_launch_dep(st, k_bie_gather_w, dim3(g), dim3(256), 0, w, B->perm.p, B->nd, B->vec.p + B->W_off);
     MH_LAUNCHED(ctx);
-    auto run = [&](const Phase* ph) {
-        return run_phase_on<double>(ctx, B->ops64.p, B->d_op_off.p, B->d_op_C.p, B->vec.p, B->vec.p, B->temp.p, ph,
-                                    "bie_fmm_contract");
-    };
     MH_TRY(run_cols<double>(ctx, B->p2m, B->vec.p, B->vec.p, false, "bie_fmm_contract"));
     MH_TRY(run_chain<double>(ctx, B->chain.get(), V->P, B->DM_off, B->DL_off, B->vec.p, true, "bie_fmm_chain"));
     MH_CUDA(ctx, cudaMemsetAsync(B->vec.p + B->DL_off, 0, (B->vec_len - B->DL_off) * 8, st));
-    MH_TRY(run(B->m2l.get()));
+    MH_TRY(run_orbits(ctx, &B->m2l, B->vec.p, B->vec.p, B->temp.p, "bie_fmm_contract", false));
     MH_TRY(run_cols<double>(ctx, B->p2l, B->vec.p, B->vec.p, true, "bie_fmm_contract"));
     MH_TRY(run_chain<double>(ctx, B->chain.get(), V->P, B->DM_off, B->DL_off, B->vec.p, false, "bie_fmm_chain"));
     MH_TRY(run_cols<double>(ctx, B->out, B->vec.p, u, false, "bie_fmm_contract"));
@@ -2509,46 +2764,46 @@ void volume_free(mh_tree* t) {
 // expansions until the output phase adds L2P and M2P to it.  Without region timers the passes
 // run on the side stream while the near phase runs on the context stream, joined before the
 // output phase; with the timers everything runs in order on the context stream.  Both forms
-// write near, then add far, straight into the caller's array.
+// write near, then add far: in binary32 straight into the caller's array, in binary64 into the
+// pool (even and odd components), transformed back into the array.
 template <typename TOP>
-static mh_status volume_passes(mh_ctx* ctx, VolData* V, const TOP* ops, bool dep) {
+static mh_status volume_passes(mh_ctx* ctx, VolData* V, bool dep) {
     TOP* pool = typed_pool<TOP>(V->vec, V->vec32);
-    MH_TRY(run_phase(ctx, V, ops, V->p2m.get(), nullptr, dep));
+    MH_TRY(run_phase<TOP>(ctx, V, V->p2m.get(), &V->p2m64, nullptr, V->temp.p, dep));
     MH_TRY(run_chain<TOP>(ctx, V->chain.get(), V->P, V->M_off, V->L_off, pool, true, "volume_chain"));
     if (sizeof(TOP) == 4) MH_TRY(tc_split(ctx, V->tc, 1, V->vec32.p));   // multipoles final
     if (!V->local_cover)   // the downward chain adds into the locals: those without an M2L task start at zero
         MH_CUDA(ctx, cudaMemsetAsync(pool + V->L_off, 0, (V->vec_len - V->L_off) * sizeof(TOP), ctx->stream));
-    MH_TRY(run_phase(ctx, V, ops, V->m2l.get(), nullptr, V->local_cover));
+    MH_TRY(run_phase<TOP>(ctx, V, V->m2l.get(), &V->m2l64, nullptr, V->temp.p, V->local_cover));
     MH_TRY(run_chain<TOP>(ctx, V->chain.get(), V->P, V->M_off, V->L_off, pool, false, "volume_chain"));
     if (sizeof(TOP) == 4) MH_TRY(tc_split(ctx, V->tc, 2, V->vec32.p));   // locals final
     return MH_OK;
 }
 
 template <typename TOP>
-static mh_status volume_run(mh_ctx* ctx, mh_tree* t, VolData* V, const TOP* ops, double* up) {
-    TOP* pool = typed_pool<TOP>(V->vec, V->vec32);
+static mh_status volume_run(mh_ctx* ctx, mh_tree* t, VolData* V, double* up) {
     cudaStream_t main = ctx->stream;
+    const bool f64 = sizeof(TOP) == 8;
+    const int64_t nn = t->n_leaves * V->qq;
     double* out = up - V->U_off;   // output offsets count from the pool's start
-    if (!V->near_cover) MH_CUDA(ctx, cudaMemsetAsync(up, 0, t->n_leaves * V->qq * 8, main));
+    if (!V->near_cover) MH_CUDA(ctx, cudaMemsetAsync(f64 ? V->vec.p + V->U_off : up, 0, nn * 8, main));
     const bool near = V->near->n_tasks > 0;
     const bool fork = near && !ctx->profiling && V->side.s;
     if (fork) {
         MH_TRY(V->side.begin(ctx, main));
         ctx->stream = V->side.s;
-        const mh_status s = volume_passes<TOP>(ctx, V, ops, false);
+        const mh_status s = volume_passes<TOP>(ctx, V, false);
         ctx->stream = main;
         MH_TRY(s);
         MH_TRY(V->side.end(ctx));
     }
-    if (near)
-        MH_TRY(run_phase_on<TOP>(ctx, ops, V->d_op_off.p, V->d_op_C.p, pool, out, V->temp_near.p, V->near.get(),
-                                 "volume_contract", &V->tc, sizeof(TOP) == 4 && V->near_cover));
+    if (near) MH_TRY(run_phase<TOP>(ctx, V, V->near.get(), &V->near64, out, V->temp_near.p, V->near_cover));
     if (fork)
         MH_CUDA(ctx, cudaStreamWaitEvent(main, V->side.join, 0));
     else
-        MH_TRY(volume_passes<TOP>(ctx, V, ops, false));
-    MH_TRY(run_phase(ctx, V, ops, V->out.get(), out, false));
-    return MH_OK;
+        MH_TRY(volume_passes<TOP>(ctx, V, false));
+    MH_TRY(run_phase<TOP>(ctx, V, V->out.get(), &V->out64, out, V->temp.p, false));
+    return f64 ? run_back(ctx, V->vec.p + V->U_off, V->node_back.p, t->q, nn, false, up, V->out64.n_tasks > 0) : MH_OK;
 }
 
 mh_status volume_apply(mh_ctx* ctx, mh_tree* t, double alpha, int p, const double* b, double* up,
@@ -2566,10 +2821,11 @@ mh_status volume_apply(mh_ctx* ctx, mh_tree* t, double alpha, int p, const doubl
             k_d2f<<<mh_grid(nn, 256), 256, 0, ctx->stream>>>(b, V->vec32.p + V->B_off, nn);
             MH_LAUNCHED(ctx);
         }
-        MH_TRY(volume_run<float>(ctx, t, V, V->ops32.p, up));
+        MH_TRY(volume_run<float>(ctx, t, V, up));
     } else {
-        MH_CUDA(ctx, cudaMemcpyAsync(V->vec.p + V->B_off, b, nn * 8, cudaMemcpyDeviceToDevice, ctx->stream));
-        MH_TRY(volume_run<double>(ctx, t, V, V->ops64.p, up));
+        k_orb_forward<<<mh_grid(nn, 256), 256, 0, ctx->stream>>>(b, V->node_fwd.p, t->q, nn, V->vec.p + V->B_off);
+        MH_LAUNCHED(ctx);
+        MH_TRY(volume_run<double>(ctx, t, V, up));
     }
     return MH_OK;
 }
