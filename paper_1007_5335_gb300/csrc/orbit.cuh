@@ -186,10 +186,11 @@ __global__ void __launch_bounds__(ORB_THREADS) k_orbit(
     mh_dep_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int first[2][5];
-    if (threadIdx.x < 5) {
-        first[0][threadIdx.x] = dims.exp[threadIdx.x];
-        first[1][threadIdx.x] = dims.nodes[threadIdx.x];
-    }
+    if (threadIdx.x == 0)
+        for (int k = 0; k < 5; ++k) {
+            first[0][k] = dims.exp[k];
+            first[1][k] = dims.nodes[k];
+        }
     const OrbOp op = op_of[chunk_op[blockIdx.x]];
     const int t0 = chunk_t0[blockIdx.x], nt = chunk_t0[blockIdx.x + 1] - t0;
     const int C = op.C, ld = orb_ld(C);

@@ -388,19 +388,20 @@ __global__ void k_apply(const TOP* __restrict__ ops, const int64_t* __restrict__
 }
 
 // ---- M2M / L2L, one launch per tree level ----
-// The levels are a latency chain of small matvecs.  Every level has one set of four operators
-// (child positions), the same for all its boxes, so a block copies them to shared memory before it
-// waits for the level before (dependent launch: it is resident by then) and its critical path is
-// the children's expansions, the products and the store.
-//  * up (M2M): M[box] = sum over the children c = 0..3 of T_c M[child_c]: thread (c, r) forms row r
-//    of T_c M[child_c] (products in column order), the four are added in the order c = 0..3.
-//  * down (L2L): L[child_c] += T'_c L[box], thread (c, r) forms row r.
-// Operators are stored transposed per (level, child position): ops[((l * 4 + c) * P + col) * P
-// + row], so the threads of a warp read consecutive words.  A dataflow form (one launch, a box's
-// last child carries on with the parent) spent ~4.5 us a level, most of it on operator loads from
-// L2: 28 us up and 22 us down for the starfish tree in binary32.  Against it: matrix-free solve at
-// 12,288 nodes (14 products) 6.13 -> 5.72 ms, mixed volume potential (255 k nodes) 186 -> 180 us,
-// binary64 volume potential 569 -> 568 us (bound by the binary64 contractions beside it).
+// The levels are a latency chain of small matvecs.  The four children of a box are mirror images, so a level
+// has one operator T (of child 0, class order): in the components of orbit.cuh
+//  * up (M2M): M[box]_i = sum over the characters c of sum_j T_ij X_{c, j}, X_c the character sums of the
+//    four children, j in class c(i)^c: thread (c, i) forms one term, the four are added in the order c = 0..3.
+//  * down (L2L): W_{c, i} = sum_j T'_ij L[box]_j, L[child_g]_i += sum_c (-1)^(c.g) W_{c, i}.
+// About P / 4 products a thread in a row instead of P, a quarter of the multiply-adds and of the operator
+// bytes.  A block copies the operator to shared memory before it waits for the level before (dependent
+// launch: it is resident by then), so its critical path is the children's expansions, the
+// products and the store.  T is stored by columns (ops[l * stride + col * P + row]): the threads of
+// a warp read consecutive words.
+// A dataflow form (one launch, a box's last child carries on with the parent) spent ~4.5 us a level,
+// most of it on operator loads from L2.
+__host__ __device__ inline int chain_stride(int P) { return (P * P + 3) / 4 * 4; }   // words of an operator: 16-byte copies
+
 __device__ __forceinline__ void chain_stage(void* smem, const void* gmem, int bytes) {   // multiple of 16
     const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem);
     for (int e = 16 * threadIdx.x; e < bytes; e += 16 * blockDim.x)
@@ -412,65 +413,88 @@ __device__ __forceinline__ void chain_staged() {
     __syncthreads();
 }
 
+// Row r of the operator against the columns of class c(r)^c.
 template <typename T>
-__device__ __forceinline__ T chain_dot(const T* A, int P, const T* x) {
+__device__ __forceinline__ T chain_dot(const T* A, int P, int r, int c, const int* first, const T* x) {
+    const int k = ((r >= first[1]) + (r >= first[2]) + (r >= first[3])) ^ c;
     T acc = 0;
 #pragma unroll 4
-    for (int cc = 0; cc < P; ++cc) acc = fma(A[cc * P], x[cc], acc);
+    for (int j = first[k]; j < first[k + 1]; ++j) acc = fma(A[j * P + r], x[j], acc);
     return acc;
 }
 
+// a + (-1)^(c.1) b + (-1)^(c.2) d + (-1)^(c.3) e
 template <typename T>
-__global__ void k_level_up(const T* __restrict__ ops, int P, const int32_t* __restrict__ box,
-                           const int4* __restrict__ child, int n, T* m) {
+__device__ __forceinline__ T chain_signs(int c, T a, T b, T d, T e) {
+    const T s = (c & 1) ? a - b : a + b, t = (c & 1) ? d - e : d + e;
+    return (c & 2) ? s - t : s + t;
+}
+
+template <typename T>
+__global__ void k_level_up(const T* __restrict__ ops, int P, OrbDims dims, const int32_t* __restrict__ perm,
+                           const int32_t* __restrict__ box, const int4* __restrict__ child, int n, T* m) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* sA = reinterpret_cast<T*>(smem_raw);   // 4 operators
-    T* x = sA + 4 * P * P;                    // 4 x P child expansions
+    __shared__ int first[5];
+    T* sA = reinterpret_cast<T*>(smem_raw);
+    T* x = sA + chain_stride(P);              // 4 x P character sums
     T* part = x + 4 * P;                      // 4 x P products
-    chain_stage(sA, ops, 4 * P * P * (int)sizeof(T));   // set-up data: may precede the wait
+    chain_stage(sA, ops, chain_stride(P) * (int)sizeof(T));   // set-up data: may precede the wait
+    if (threadIdx.x == 0)
+        for (int k = 0; k < 5; ++k) first[k] = dims.exp[k];
+    const int c = threadIdx.x / P, r = threadIdx.x - c * P;
+    const int pr = perm[r];
     mh_dep_wait();
     chain_staged();
-    const int c = threadIdx.x / P, r = threadIdx.x - c * P;
     for (int b = blockIdx.x; b < n; b += gridDim.x) {
-        const int4 ch4 = child[b];
-        const int ch = c == 0 ? ch4.x : c == 1 ? ch4.y : c == 2 ? ch4.z : ch4.w;
-        if (c < 4) x[c * P + r] = ch >= 0 ? m[(int64_t)ch * P + r] : T(0);
+        if (c < 4) {
+            const int4 ch = child[b];
+            const T v0 = ch.x >= 0 ? m[(int64_t)ch.x * P + pr] : T(0), v1 = ch.y >= 0 ? m[(int64_t)ch.y * P + pr] : T(0);
+            const T v2 = ch.z >= 0 ? m[(int64_t)ch.z * P + pr] : T(0), v3 = ch.w >= 0 ? m[(int64_t)ch.w * P + pr] : T(0);
+            x[c * P + r] = chain_signs(c, v0, v1, v2, v3);
+        }
         __syncthreads();
-        if (c < 4) part[c * P + r] = ch >= 0 ? chain_dot<T>(sA + c * P * P + r, P, x + c * P) : T(0);
+        if (c < 4) part[c * P + r] = chain_dot<T>(sA, P, r, c, first, x + c * P);
         __syncthreads();
         if (threadIdx.x < P) {
             T s = part[r] + part[P + r];
             s += part[2 * P + r];
             s += part[3 * P + r];
-            m[(int64_t)box[b] * P + r] = s;
+            m[(int64_t)box[b] * P + pr] = s;
         }
     }
 }
 
 template <typename T>
-__global__ void k_level_down(const T* __restrict__ ops, int P, const int32_t* __restrict__ box,
-                             const int4* __restrict__ child, int n, T* loc) {
+__global__ void k_level_down(const T* __restrict__ ops, int P, OrbDims dims, const int32_t* __restrict__ perm,
+                             const int32_t* __restrict__ box, const int4* __restrict__ child, int n, T* loc) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* sA = reinterpret_cast<T*>(smem_raw);   // 4 operators
-    T* x = sA + 4 * P * P;                    // the box's expansion, two buffers
-    chain_stage(sA, ops, 4 * P * P * (int)sizeof(T));   // set-up data: may precede the wait
+    __shared__ int first[5];
+    T* sA = reinterpret_cast<T*>(smem_raw);
+    T* x = sA + chain_stride(P);              // the box's expansion
+    T* part = x + 4 * P;                      // 4 x P products
+    chain_stage(sA, ops, chain_stride(P) * (int)sizeof(T));   // set-up data: may precede the wait
+    if (threadIdx.x == 0)
+        for (int k = 0; k < 5; ++k) first[k] = dims.exp[k];
+    const int c = threadIdx.x / P, r = threadIdx.x - c * P;
+    const int pr = perm[r];
     mh_dep_wait();
     chain_staged();
-    const int c = threadIdx.x / P, r = threadIdx.x - c * P;
-    int buf = 0;
-    for (int b = blockIdx.x; b < n; b += gridDim.x, buf ^= 1) {
+    for (int b = blockIdx.x; b < n; b += gridDim.x) {
         const int4 ch4 = child[b];
         const int ch = c == 0 ? ch4.x : c == 1 ? ch4.y : c == 2 ? ch4.z : ch4.w;
-        if (threadIdx.x < P) x[buf * P + r] = loc[(int64_t)box[b] * P + r];
-        const T own = c < 4 && ch >= 0 ? loc[(int64_t)ch * P + r] : T(0);
-        __syncthreads();   // the other buffer is read until every thread is here again
-        if (c < 4 && ch >= 0) loc[(int64_t)ch * P + r] = own + chain_dot<T>(sA + c * P * P + r, P, x + buf * P);
+        if (threadIdx.x < P) x[r] = loc[(int64_t)box[b] * P + pr];
+        const T own = c < 4 && ch >= 0 ? loc[(int64_t)ch * P + pr] : T(0);
+        __syncthreads();
+        if (c < 4) part[c * P + r] = chain_dot<T>(sA, P, r, c, first, x);
+        __syncthreads();
+        if (c < 4 && ch >= 0)
+            loc[(int64_t)ch * P + pr] = own + chain_signs(c, part[r], part[P + r], part[2 * P + r], part[3 * P + r]);
     }
 }
 
 inline int chain_threads(int P) { return (4 * P + 31) / 32 * 32; }
-constexpr int CHAIN_SMEM_MAX = 224 * 1024;   // p = 40 (P = 81) in binary64 takes 215,136 bytes
-inline size_t chain_smem(int P, size_t word) { return (4 * (size_t)P * P + 8 * (size_t)P) * word; }
+inline size_t chain_smem(int P, size_t word) { return (chain_stride(P) + 8 * (size_t)P) * word; }
+constexpr int CHAIN_SMEM_MAX = 64 * 1024;   // p = 40 (P = 81) in binary64 takes 57,696 bytes
 
 // Per destination (one warp each): dst[r] = (acc ? dst[r] : 0) + the sum of its tasks' products,
 // in task order.  Binary64 products are summed in binary64; binary32 products in float-float
@@ -1010,7 +1034,9 @@ struct LevelChain {
     double flops = 0, bytes = 0;         // one sweep (either direction), algorithmic
     dbuf<int32_t> box;
     dbuf<int4> child;
-    dbuf<float> m2m32, l2l32;            // transposed operators, [level][position][col][row]
+    OrbDims dims;                        // classes of the components, and their coefficients
+    dbuf<int32_t> perm;
+    dbuf<float> m2m32, l2l32;            // operators of child 0, [level][col][row], class order
     dbuf<double> m2m64, l2l64;
 };
 
@@ -1345,12 +1371,12 @@ mh_status run_chain(mh_ctx* ctx, const LevelChain* ch, int P, int64_t m_base, in
         const int l = upward ? L + 1 - q : q;   // up: L - 1 .. 2, down: 2 .. L - 1
         const int n = ch->first[l + 1] - ch->first[l];
         if (n == 0) continue;
-        // at most the blocks that are resident together (27 KB of operators in binary32, 54 KB in
-        // binary64 at P = 41): a block's operators serve all its boxes
-        (void)mh_launch_dep(ctx->stream, upward ? k_level_up<TOP> : k_level_down<TOP>,
-                            dim3(std::min(n, 152 * (f32 ? 6 : 4))),
-                            dim3(chain_threads(P)), chain_smem(P, sizeof(TOP)), ops + (int64_t)l * 4 * P * P, P,
-                            ch->box.p + ch->first[l], ch->child.p + ch->first[l], n, vec + (upward ? m_base : l_base));
+        // at most the blocks that are resident together (9 KB of shared memory in binary32, 16 KB in
+        // binary64, 192 threads at P = 41): a block's operator serves all its boxes
+        (void)mh_launch_dep(ctx->stream, upward ? k_level_up<TOP> : k_level_down<TOP>, dim3(std::min(n, 152 * 8)),
+                            dim3(chain_threads(P)), chain_smem(P, sizeof(TOP)), ops + (int64_t)l * chain_stride(P), P, ch->dims,
+                            ch->perm.p, ch->box.p + ch->first[l], ch->child.p + ch->first[l], n,
+                            vec + (upward ? m_base : l_base));
         MH_LAUNCHED(ctx);
     }
     return MH_OK;
@@ -1424,28 +1450,30 @@ mh_status build_chain(mh_ctx* ctx, const mh_tree* t, const HostTree& h, int P, c
         kids.push_back(make_int4(k[0], k[1], k[2], k[3]));
         ch->first[l + 1] += 1;
         used[l] = 1;
-        ch->flops += 2.0 * P * P * cnt;
+        ch->flops += 2.0 * P * P + 12.0 * P;
         ch->bytes += 8.0 * 2.0 * P * (cnt + 1);
     }
     for (int l = 0; l < L; ++l) {
         ch->first[l + 1] += ch->first[l];
-        if (used[l]) ch->bytes += 8.0 * 4.0 * P * P;
+        if (used[l]) ch->bytes += 8.0 * P * P;
     }
-    // operators, transposed per (level, child position)
-    const size_t PP = (size_t)P * P;
-    std::vector<double> tm((size_t)std::max(L, 1) * 4 * PP, 0.0), tl((size_t)std::max(L, 1) * 4 * PP, 0.0);
+    // operators of child 0 in class order, by columns
+    const OrbSpace es = orb_expansions((P - 1) / 2);
+    const size_t S = chain_stride(P);
+    std::vector<double> tm((size_t)std::max(L, 1) * S, 0.0), tl((size_t)std::max(L, 1) * S, 0.0);
     for (int l = 2; l < L; ++l) {
         if (!used[l]) continue;
-        for (int c = 0; c < 4; ++c) {
-            const double* om = pool.data.data() + pool.off[op_m2m[l][c]];
-            const double* ol = pool.data.data() + pool.off[op_l2l[l][c]];
-            for (int r = 0; r < P; ++r)
-                for (int cc = 0; cc < P; ++cc) {
-                    tm[(l * 4 + c) * PP + (size_t)cc * P + r] = om[(size_t)r * P + cc];
-                    tl[(l * 4 + c) * PP + (size_t)cc * P + r] = ol[(size_t)r * P + cc];
-                }
-        }
+        const std::vector<double> om = orb_operator(pool.data.data() + pool.off[op_m2m[l][0]], P, P, es, es, 0);
+        const std::vector<double> ol = orb_operator(pool.data.data() + pool.off[op_l2l[l][0]], P, P, es, es, 0);
+        for (int r = 0; r < P; ++r)
+            for (int cc = 0; cc < P; ++cc) {
+                tm[l * S + (size_t)cc * P + r] = om[(size_t)r * P + cc];
+                tl[l * S + (size_t)cc * P + r] = ol[(size_t)r * P + cc];
+            }
     }
+    ch->dims = orb_dims(es, es);
+    MH_ALLOC(ctx, ch->perm, es.perm.size());
+    MH_CUDA(ctx, cudaMemcpyAsync(ch->perm.p, es.perm.data(), es.perm.size() * 4, cudaMemcpyHostToDevice, cs));
     std::vector<float> tm32(tm.begin(), tm.end()), tl32(tl.begin(), tl.end());
     MH_ALLOC(ctx, ch->box, std::max<size_t>(box.size(), 1));
     MH_ALLOC(ctx, ch->child, std::max<size_t>(kids.size(), 1));
