@@ -1991,15 +1991,6 @@ __global__ void __launch_bounds__(MF_THREADS) k_mf_shift(const double2* __restri
         S[(int64_t)p * n + off[k] + j] = direct ? z[j].x : cmul(cconj(b[j]), cconj(z[j])).x * sc;
 }
 
-// Dipole strengths w_i = sigma_i |y'_i| h_k.
-__global__ void k_mf_weights(const double* __restrict__ sigma, const double* __restrict__ geo,
-                             const int32_t* __restrict__ curve_of, const int32_t* __restrict__ nn, int64_t n,
-                             double* __restrict__ w) {
-    mh_dep_wait();
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) w[i] = sigma[i] * geo[8 * i + 6] * (2.0 * MH_PI / nn[curve_of[i]]);
-}
-
 // y_j = sigma_j - 2 alpha^2 u_j - (1/pi) W_j + C_j (a > 0), or with the diagonal limit
 // (1/pi) kappa-term h sigma_j in place of W_j and C_j (a = 0).  u_j is the multipole-pass output
 // -(1/(2 pi alpha^2)) sum_{i != j} w_i K(y_i, x_j), so -2 alpha^2 u_j = (1/pi) T_j; the window
@@ -2199,7 +2190,6 @@ mh_status bie_mfree_setup(mh_ctx* ctx, mh_boundary* b, mh_tree* t, double alpha)
     MH_ALLOC(ctx, b->mf_bh, moff[nc]);
     MH_ALLOC(ctx, b->mf_tw, moff[nc] / 2);
     MH_ALLOC(ctx, b->mf_spec, n / 2 + nc);   // N_k/2 + 1 modes per curve
-    MH_ALLOC(ctx, b->mf_w, n);
     MH_ALLOC(ctx, b->mf_u, n);
     const size_t smem = 24 * (size_t)mmax;
     MH_CUDA(ctx, cudaFuncSetAttribute(k_mf_chirp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -2258,11 +2248,12 @@ mh_status bie_apply_mfree(mh_ctx* ctx, mh_boundary* b, const double* x, double* 
     if (a > 0) {
         upload_alpert(a, &R);
         l2 = 2 * R.l;
-        cudaStream_t as = st;
-        if (fork) {
-            MH_TRY(b->mf_side.begin(ctx, st));
-            as = b->mf_side.s;
-        }
+        if (fork) MH_TRY(b->mf_side.begin(ctx, st));
+    }
+    // the multipole pass is the longer chain: it is queued first
+    MH_TRY(volume_bie_apply(ctx, b->mf_tree, x, b->geo.p, b->d_curve_of.p, b->d_nn.p, b->mf_u.p));
+    if (a > 0) {
+        cudaStream_t as = fork ? b->mf_side.s : st;
         const size_t smem = 24 * (size_t)b->mf_mmax;
         k_mf_spectrum<<<(unsigned)b->n_curves, MF_THREADS, smem, as>>>(x, b->d_nn.p, b->d_off.p, b->mf_moff.p, b->mf_M.p,
                                                                         b->mf_chirp.p, b->mf_bh.p, b->mf_tw.p,
@@ -2274,9 +2265,6 @@ mh_status bie_apply_mfree(mh_ctx* ctx, mh_boundary* b, const double* x, double* 
         MH_LAUNCHED(ctx);
         if (fork) MH_TRY(b->mf_side.end(ctx));
     }
-    k_mf_weights<<<mh_grid(n, 256), 256, 0, st>>>(x, b->geo.p, b->d_curve_of.p, b->d_nn.p, n, b->mf_w.p);
-    MH_LAUNCHED(ctx);
-    MH_TRY(volume_bie_apply(ctx, b->mf_tree, b->mf_w.p, b->mf_u.p));
     if (fork) MH_CUDA(ctx, cudaStreamWaitEvent(st, b->mf_side.join, 0));
     k_mf_combine<<<mh_grid(n, 64), 64, 0, st>>>(x, b->mf_u.p, b->geo.p, b->d_curve_of.p, b->d_nn.p, b->d_off.p,
                                                        n, b->mf_alpha, a, l2, b->mf_win.p, b->mf_cp.p, b->mf_S.p, y);

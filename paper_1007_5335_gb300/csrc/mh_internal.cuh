@@ -364,7 +364,7 @@ struct mh_boundary {
     std::unique_ptr<dlp_targets> eval;   // buffers of mh_double_layer_apply's last target set
     dbuf<double2> mf_spec;               // per call: spectra c_m, m <= N_k/2
     dbuf<double> mf_S;                   // per call: [2 l][n] interpolated density at the Alpert nodes
-    dbuf<double> mf_w, mf_u;             // per call: dipole strengths, multipole-pass output
+    dbuf<double> mf_u;                   // per call: multipole-pass output
     SideStream mf_side;                  // the Alpert transforms run there beside the multipole pass
     dbuf<double> warm_dir, warm_w, warm_scal;   // warm-start direction, its image, scalars
     dbuf<float2> fcp32;                  // fine-grid coefficients by sub-offset (binary32)
@@ -507,7 +507,8 @@ mh_status volume_dipole_apply(mh_ctx* ctx, mh_tree* t, const double* w, const in
 mh_status volume_bie_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, const double* xy, const double* nrm,
                            const int32_t* leaf, int64_t nd);
 bool volume_bie_ready(const mh_tree* t);
-mh_status volume_bie_apply(mh_ctx* ctx, mh_tree* t, const double* w, double* u);
+mh_status volume_bie_apply(mh_ctx* ctx, mh_tree* t, const double* sigma, const double* geo, const int32_t* curve_of,
+                           const int32_t* nn, double* u);
 mh_status tree_locate(mh_ctx* ctx, const mh_tree* t, const double* xy_dev, int64_t n, int32_t* leaf_out);
 // Leaf interpolation U of node values at n points with known leaves; with f, c (f - U) instead of U.
 mh_status tree_interpolate(mh_ctx* ctx, const mh_tree* t, const double* vals, const double* xy_dev,

@@ -540,10 +540,13 @@ __global__ void k_reduce(const TT* __restrict__ temp, int R, const int64_t* __re
 // of every G-th column, the G partial sums meet in shared memory at the end.  As contraction tasks with
 // one source vector each (a warp per row, lanes over the columns) a row of 64 columns cost 2 products
 // and 6 instructions of reduction, and the products of an output went through memory and a second
-// kernel: matrix-free solve at 12,288 nodes (14 products) 5.72 ms.
-// Outputs of more than COL_CHUNK columns are cut; the last block of an output to finish adds the
-// parts in order.
-constexpr int COL_CHUNK = 256;
+// kernel: matrix-free solve at 12,288 nodes (14 products) 5.72 -> 3.43 ms.
+// Outputs of many columns are cut; the last block of an output to finish adds the parts in order.  A chunk
+// ends in R serial sums of its groups, so it should be long, and the chip wants 12 blocks an SM: between
+// 32 and 1024 columns by the total (build_cols).  256 columns everywhere left the P2M of those 12,288 nodes 146
+// blocks, 21 us a product: the solve 2957 -> 2553 us with the chunks, the operator loaded before the wait, the
+// locals zeroed with the strengths and the pass queued before the Alpert transforms.
+constexpr int COL_CHUNK_MIN = 32, COL_CHUNK_MAX = 1024;
 
 struct ColChunk {
     int32_t out;        // output
@@ -551,45 +554,72 @@ struct ColChunk {
     int64_t c0, c1;     // columns
 };
 
-__device__ __forceinline__ void col_add(double& s, double& lo, double a, double x) { s = fma(a, x, s); }
-__device__ __forceinline__ void col_add(float& s, float& lo, float a, float x) {   // float-float sum
-    const float v = a * x, t = s + v, bb = t - s;
-    lo += (s - (t - bb)) + (v - bb);
-    s = t;
-}
+// Running sum: plain in binary64, float-float (the rounding errors in lo) in binary32.
+template <typename T>
+struct ColSum {
+    T s = 0, lo = 0;
+    __device__ __forceinline__ void add(T a, T x) {
+        if constexpr (sizeof(T) == 8) {
+            s = fma(a, x, s);
+        } else {
+            const T v = a * x, t = s + v, bb = t - s;
+            lo += (s - (t - bb)) + (v - bb);
+            s = t;
+        }
+    }
+};
 
 // Row r of output o goes to dst[at[o] + r] (added when accumulate is set) or, with `row`, to
-// dst[row[o R + r]] (row < 0: none).
+// dst[row[o R + r]] (row < 0: none).  The operator is set-up data: its first columns are loaded before the
+// wait for the vector, the next ones while a batch is summed.
 template <typename T>
 __global__ void __launch_bounds__(256) k_cols(const T* __restrict__ ops, const int32_t* __restrict__ src,
                                               const ColChunk* __restrict__ chunks, const int2* __restrict__ out_red,
                                               const int64_t* __restrict__ at, const int32_t* __restrict__ row, int R,
                                               const T* vec, T* part, unsigned* cnt, int accumulate, T* dst) {
-    mh_dep_wait();
+    constexpr int U = 4;
     __shared__ T red[256];
     __shared__ int last;
     const ColChunk ch = chunks[blockIdx.x];
     const int G = 256 / R, r = threadIdx.x % R, g = threadIdx.x / R;
-    T s0 = 0, l0 = 0, s1 = 0, l1 = 0;
-    if (g < G) {
-        int64_t c = ch.c0 + g;
-        for (; c + 3 * G < ch.c1; c += 4 * G) {
-            T a[4], x[4];
+    int64_t c = ch.c0 + g;
+    const int64_t end = g < G ? ch.c1 : 0;
+    T a[U];
+    int32_t at_x[U];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                a[u] = ops[(c + u * G) * R + r];
-                x[u] = vec[src[c + u * G]];
-            }
-            col_add(s0, l0, a[0], x[0]);
-            col_add(s1, l1, a[1], x[1]);
-            col_add(s0, l0, a[2], x[2]);
-            col_add(s1, l1, a[3], x[3]);
+    for (int u = 0; u < U; ++u)
+        if (c + u * G < end) {
+            a[u] = ops[(c + u * G) * R + r];
+            at_x[u] = src[c + u * G];
         }
-        for (; c < ch.c1; c += G) col_add(s0, l0, ops[c * R + r], vec[src[c]]);
+    mh_dep_wait();
+    ColSum<T> s0, s1;
+    while (c < end) {
+        T x[U], b[U];
+        int m = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (c + u * G < end) {
+                x[u] = vec[at_x[u]];
+                b[u] = a[u];
+                m = u + 1;
+            }
+        c += U * G;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (c + u * G < end) {
+                a[u] = ops[(c + u * G) * R + r];
+                at_x[u] = src[c + u * G];
+            }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (u < m) ((u & 1) ? s1 : s0).add(b[u], x[u]);
     }
-    red[threadIdx.x] = (s0 + s1) + (l0 + l1);
+    T t = s0.s + s1.s;
+    if constexpr (sizeof(T) == 4) t += s0.lo + s1.lo;
+    red[threadIdx.x] = t;
     __syncthreads();
-    T t = 0;
+    t = 0;
     if (threadIdx.x < R)
         for (int q = 0; q < G; ++q) t += red[q * R + r];
     if (ch.slot >= 0) {
@@ -655,8 +685,9 @@ mh_status build_cols(mh_ctx* ctx, const ColBuild& b, bool both, ColSet* S) {
     std::vector<ColChunk> ch;
     std::vector<int2> red(S->n, make_int2(0, 1));
     int32_t slots = 0;
+    const int64_t cap = std::min<int64_t>(COL_CHUNK_MAX, std::max<int64_t>(COL_CHUNK_MIN, (int64_t)b.src.size() / (12 * 152)));
     for (int64_t i = 0; i < S->n; ++i) {
-        const int64_t c0 = b.first[i], nc = b.first[i + 1] - c0, k = std::max<int64_t>(1, (nc + COL_CHUNK - 1) / COL_CHUNK);
+        const int64_t c0 = b.first[i], nc = b.first[i + 1] - c0, k = std::max<int64_t>(1, (nc + cap - 1) / cap);
         red[i] = make_int2(k > 1 ? slots : 0, (int)k);
         for (int64_t q = 0; q < k; ++q)
             ch.push_back(ColChunk{(int32_t)i, k > 1 ? slots + (int32_t)q : -1, c0 + nc * q / k, c0 + nc * (q + 1) / k});
@@ -2024,11 +2055,15 @@ __global__ void __launch_bounds__(NT) k_dip_near32(
     near_finish<NT>((double)ah + (double)al, act, qq, i, groups, ch, leaf_red, pref, part, cnt, out);
 }
 
+// zero: the locals of the pass (boxes whose V and X lists hold no dipoles get no M2L / P2L task, and the
+// downward chain adds into the leaves' locals).
 template <typename T>
-__global__ void k_dip_weights(const double* __restrict__ w, const int32_t* __restrict__ perm, int64_t n, T* ws) {
+__global__ void k_dip_weights(const double* __restrict__ w, const int32_t* __restrict__ perm, int64_t n, T* ws, T* zero,
+                              int64_t n_zero) {
     mh_dep_wait();
-    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
     if (j < n) ws[j] = (T)w[perm[j]];
+    for (int64_t e = j; e < n_zero; e += stride) zero[e] = T(0);
 }
 
 __global__ void k_d2f(const double* __restrict__ a, float* __restrict__ b, int64_t n) {
@@ -2468,20 +2503,15 @@ mh_status volume_dipole_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, cons
 template <typename TOP>
 static mh_status dipole_passes(mh_ctx* ctx, VolData* V, DipData* D, const TOP* ops, bool dep) {
     TOP* pool = typed_pool<TOP>(D->vec, D->vec32);
-    auto run = [&](const Phase* ph) {
-        if constexpr (sizeof(TOP) == 8)
-            return run_orbits(ctx, &D->m2l64, D->vec.p, D->vec.p, D->temp.p, "dlp_fmm_contract", false);
-        else
-            return run_phase_on<TOP>(ctx, ops, D->d_op_off.p, D->d_op_C.p, pool, D->vec.p, D->temp.p, ph,
-                                     "dlp_fmm_contract", &D->tc);
-    };
+    const bool behind = D->p2m.n_chunks > 0;   // the M2L directly behind a kernel of the pass
     MH_TRY(run_cols<TOP>(ctx, D->p2m, pool, pool, false, "dlp_fmm_contract", dep));
     MH_TRY(run_chain<TOP>(ctx, D->chain_up.get(), V->P, D->DM_off, D->DL_off, pool, true, "dlp_fmm_chain"));
     if (sizeof(TOP) == 4) MH_TRY(tc_split(ctx, D->tc, 0, D->vec32.p));   // multipoles final
-    // boxes whose V and X lists hold no dipoles get no M2L / P2L task: their locals are zeroed
-    // here, since the downward chain adds into the leaves' locals
-    MH_CUDA(ctx, cudaMemsetAsync(pool + D->DL_off, 0, (D->DU_off - D->DL_off) * sizeof(TOP), ctx->stream));
-    MH_TRY(run(D->m2l.get()));
+    if constexpr (sizeof(TOP) == 8)
+        MH_TRY(run_orbits(ctx, &D->m2l64, pool, pool, D->temp.p, "dlp_fmm_contract", behind));
+    else
+        MH_TRY(run_phase_on<TOP>(ctx, ops, D->d_op_off.p, D->d_op_C.p, pool, D->vec.p, D->temp.p, D->m2l.get(),
+                                 "dlp_fmm_contract", &D->tc, behind));
     MH_TRY(run_cols<TOP>(ctx, D->p2l, pool, pool, true, "dlp_fmm_contract"));
     MH_TRY(run_chain<TOP>(ctx, V->chain.get(), V->P, D->DM_off, D->DL_off, pool, false, "dlp_fmm_chain"));
     if (sizeof(TOP) == 4) MH_TRY(tc_split(ctx, D->tc, 1, D->vec32.p));   // locals final
@@ -2514,11 +2544,12 @@ mh_status volume_dipole_apply(mh_ctx* ctx, mh_tree* t, const double* w, const in
     const bool mixed = prec == MH_PREC_MIXED;
     if (!D->near_blocks) MH_CUDA(ctx, cudaMemsetAsync(D->vec.p + D->DU_off, 0, t->n_leaves * D->qq * 8, st));
     // strengths in dipole order, in the precision that the contractions and the near field read
-    const unsigned gw = (unsigned)mh_grid(D->nd, 256);
+    const int64_t nz = D->DU_off - D->DL_off;
+    const unsigned gw = (unsigned)mh_grid(std::max(D->nd, (nz + 3) / 4), 256);
     if (mixed)
-        k_dip_weights<float><<<gw, 256, 0, st>>>(w, perm, D->nd, D->vec32.p + D->W_off);
+        k_dip_weights<float><<<gw, 256, 0, st>>>(w, perm, D->nd, D->vec32.p + D->W_off, D->vec32.p + D->DL_off, nz);
     else
-        k_dip_weights<double><<<gw, 256, 0, st>>>(w, perm, D->nd, D->vec.p + D->W_off);
+        k_dip_weights<double><<<gw, 256, 0, st>>>(w, perm, D->nd, D->vec.p + D->W_off, D->vec.p + D->DL_off, nz);
     MH_LAUNCHED(ctx);
     // The near field reads the weights and adds into U^h only; the passes read the weights and
     // touch only the expansions until their output phase adds the far field to U^h.  Without
@@ -2605,11 +2636,18 @@ void bie_row(double* row, int p, const double* v, double th) {
     }
 }
 
-__global__ void k_bie_gather_w(const double* __restrict__ w, const int32_t* __restrict__ perm, int64_t n,
-                               double* __restrict__ ws) {
+// Dipole strengths sigma |y'| h in sorted order, and zeros in the locals (as k_dip_weights).
+__global__ void k_bie_weights(const double* __restrict__ sigma, const double* __restrict__ geo,
+                              const int32_t* __restrict__ curve_of, const int32_t* __restrict__ nn,
+                              const int32_t* __restrict__ perm, int64_t n, double* __restrict__ ws,
+                              double* __restrict__ zero, int64_t n_zero) {
     mh_dep_wait();
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) ws[i] = w[perm[i]];
+    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+    if (j < n) {
+        const int32_t i = perm[j];
+        ws[j] = sigma[i] * geo[8 * (int64_t)i + 6] * (2.0 * MH_PI / nn[curve_of[i]]);
+    }
+    for (int64_t e = j; e < n_zero; e += stride) zero[e] = 0.0;
 }
 
 }  // namespace
@@ -2745,23 +2783,24 @@ bool volume_bie_ready(const mh_tree* t) {
     return V && V->bie;
 }
 
-// w: dipole strengths in node order (device); u: the trapezoid double layer at every node, in
-// node order (device), as defined above.  Runs on the context stream, with its own M2M / L2L
+// sigma: density in node order (device), geo / curve_of / nn: the boundary's node records; u: the trapezoid
+// double layer at every node, in node order (device), as defined above.  Runs on the context stream, with its own M2M / L2L
 // chain over the boxes that hold boundary nodes.
-mh_status volume_bie_apply(mh_ctx* ctx, mh_tree* t, const double* w, double* u) {
+mh_status volume_bie_apply(mh_ctx* ctx, mh_tree* t, const double* sigma, const double* geo, const int32_t* curve_of,
+                           const int32_t* nn, double* u) {
     VolData* V = static_cast<VolData*>(t->vol);
     if (!V || !V->bie) return mh_fail(ctx, MH_ERR_INVALID_ARG, "on-surface multipole pass not set up");
     BieData* B = V->bie.get();
     if (B->nd == 0) return MH_OK;
     prof_scope ps(ctx, "bie_fmm", B->flops, 0.0);
     cudaStream_t st = ctx->stream;
-    const unsigned g = (unsigned)mh_grid(B->nd, 256);
-    (void)mh_launch_dep(st, k_bie_gather_w, dim3(g), dim3(256), 0, w, B->perm.p, B->nd, B->vec.p + B->W_off);
+    const int64_t nz = B->vec_len - B->DL_off;
+    k_bie_weights<<<mh_grid(std::max(B->nd, (nz + 3) / 4), 256), 256, 0, st>>>(
+        sigma, geo, curve_of, nn, B->perm.p, B->nd, B->vec.p + B->W_off, B->vec.p + B->DL_off, nz);
     MH_LAUNCHED(ctx);
     MH_TRY(run_cols<double>(ctx, B->p2m, B->vec.p, B->vec.p, false, "bie_fmm_contract"));
     MH_TRY(run_chain<double>(ctx, B->chain.get(), V->P, B->DM_off, B->DL_off, B->vec.p, true, "bie_fmm_chain"));
-    MH_CUDA(ctx, cudaMemsetAsync(B->vec.p + B->DL_off, 0, (B->vec_len - B->DL_off) * 8, st));
-    MH_TRY(run_orbits(ctx, &B->m2l, B->vec.p, B->vec.p, B->temp.p, "bie_fmm_contract", false));
+    MH_TRY(run_orbits(ctx, &B->m2l, B->vec.p, B->vec.p, B->temp.p, "bie_fmm_contract", true));
     MH_TRY(run_cols<double>(ctx, B->p2l, B->vec.p, B->vec.p, true, "bie_fmm_contract"));
     MH_TRY(run_chain<double>(ctx, B->chain.get(), V->P, B->DM_off, B->DL_off, B->vec.p, false, "bie_fmm_chain"));
     MH_TRY(run_cols<double>(ctx, B->out, B->vec.p, u, false, "bie_fmm_contract"));
