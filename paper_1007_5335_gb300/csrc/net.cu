@@ -13,6 +13,7 @@
 //   k_gemm<T, EPI>  tiled matrix product (64 x 64 tiles, 4 x 4 outputs per thread) with
 //                   bias / tanh / tanh-derivative epilogues: binary32 training passes and
 //                   the binary64 closed-form start
+//   k_grads         gradients of all layers' weights and biases
 //   k_chol, k_trinv_lower   one-block Cholesky and triangular inverse (CholeskyQR2 and
 //                   the ridge normal equations, sizes <= 1025)
 //   k_adam          Adam update (Kingma & Ba) with bias correction
@@ -41,7 +42,7 @@ struct mh_net {
     dbuf<float> xin, hA, hB, yout;
     dbuf<double> rbuf, ebuf, scal;   // scal: |r|, 1/(|r| g), <r,w>, <w,w>
     // training scratch
-    dbuf<float> G, Mo, Vo, best, xb, yb, yh, act[3], dzd, dzw1, dzw2;
+    dbuf<float> G, Mo, Vo, best, xb, yb, yh, act[3], dzd, dzw[3];
     dbuf<double> lpart;
     dbuf<float> gpart;               // partial tiles of split training products, and their counters
     dbuf<unsigned> gcnt;
@@ -53,6 +54,7 @@ namespace {
 constexpr int GEMM_T = 64;    // tile edge
 constexpr int GEMM_K = 16;    // k slab
 constexpr int GEMM_PARTS = 304;   // partial tiles of a split product (two blocks per SM)
+constexpr int GEMM_CNT = 2 * GEMM_PARTS;   // counters: tiles x (1 + groups of parts), at most 1 + one group a part
 
 enum { EPI_NONE = 0, EPI_BIAS = 1, EPI_BIAS_TANH = 2, EPI_TANH_BACK = 3 };
 
@@ -61,22 +63,24 @@ enum { EPI_NONE = 0, EPI_BIAS = 1, EPI_BIAS_TANH = 2, EPI_TANH_BACK = 3 };
 // The next slab is loaded into registers while the current one is multiplied (double-buffered
 // shared memory, one barrier a slab).  gridDim.z > 1 splits k between blocks: each writes its
 // partial tile, the last block of a tile to finish (counted per tile, reset by that block) adds
-// them in k order and applies the epilogue.  A minibatch of 64 has 4 tiles in most of its products
-// and chains of up to 192 slabs, so 4 of 152 SMs worked through ~2 us a slab: loss and gradient at
-// d = 3072, w = 256 took 788 us unsplit.
+// them in k order and applies the epilogue; more than 8 parts meet in two stages.  A minibatch of 64 has 4
+// tiles in most of its products and chains of up to 192 slabs, so 4 of 152 SMs worked through ~2 us a
+// slab: loss and gradient at 64 samples, d = 3072, w = 256 took 788 us unsplit, 178 us with one
+// block adding all 76 parts (20 us of it a product), gradients of weights and biases between the links and
+// copied inputs; 131 us with the gradients in one launch (k_grads), inputs read in place and 28 parts; 118 us
+// with 76 parts in two stages.
+// One block's share z of S of tile (i0, j0), number `tile` of `tiles`.
 template <typename T, int EPI>
-__global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, const T* __restrict__ A, int64_t sam, int64_t sak,
-                                              const T* __restrict__ B, int64_t sbk, int64_t sbn, T* __restrict__ C,
-                                              int64_t ldc, const T* __restrict__ bias, const T* __restrict__ aux,
-                                              T* part, unsigned* cnt) {
-    mh_dep_wait();
+__device__ __forceinline__ void gemm_tile(int i0, int j0, int tile, int tiles, int z, int S, int M, int N, int K,
+                                          const T* __restrict__ A, int64_t sam, int64_t sak, const T* __restrict__ B,
+                                          int64_t sbk, int64_t sbn, T* __restrict__ C, int64_t ldc,
+                                          const T* __restrict__ bias, const T* __restrict__ aux, T* part, unsigned* cnt) {
     __shared__ __align__(16) T As[2][GEMM_K][GEMM_T + 4];
     __shared__ __align__(16) T Bs[2][GEMM_K][GEMM_T + 4];
     __shared__ int last;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int i0 = blockIdx.y * GEMM_T, j0 = blockIdx.x * GEMM_T;
-    const int S = gridDim.z, slabs = (K + GEMM_K - 1) / GEMM_K;
-    const int s0 = (int)((int64_t)slabs * blockIdx.z / S), s1 = (int)((int64_t)slabs * (blockIdx.z + 1) / S);
+    const int slabs = (K + GEMM_K - 1) / GEMM_K;
+    const int s0 = (int)((int64_t)slabs * z / S), s1 = (int)((int64_t)slabs * (z + 1) / S);
     const bool ka = sak == 1, nb = sbn == 1;
     T ra[4], rb[4], acc[4][4];
 #pragma unroll
@@ -131,29 +135,53 @@ __global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, const T* __re
         __syncthreads();
     }
     if (S > 1) {
-        const int tile = blockIdx.y * gridDim.x + blockIdx.x, tiles = gridDim.x * gridDim.y;
-        T* mine = part + ((int64_t)blockIdx.z * tiles + tile) * (GEMM_T * GEMM_T) + tid;
+        auto put = [&](int slot) {
+            T* p = part + ((int64_t)slot * tiles + tile) * (GEMM_T * GEMM_T) + tid;
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
+            for (int e = 0; e < 16; ++e) p[256 * e] = acc[e >> 2][e & 3];
+        };
+        // true in the last of n blocks to arrive (which resets the counter)
+        auto arrive = [&](unsigned* c, int n) {
+            __threadfence();
+            __syncthreads();
+            if (tid == 0) last = atomicAdd(c, 1u) == (unsigned)(n - 1);
+            __syncthreads();
+            if (!last) return false;
+            __threadfence();
+            if (tid == 0) *c = 0u;
+            return true;
+        };
+        // sum of n parts in order, up to 64 loads in flight a thread
+        auto gather = [&](int first, int n, int step) {
+            constexpr int U = sizeof(T) == 4 ? 4 : 1;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) mine[256 * (4 * r + c)] = acc[r][c];
-        __threadfence();
-        __syncthreads();
-        if (tid == 0) last = atomicAdd(cnt + tile, 1u) == (unsigned)(S - 1);
-        __syncthreads();
-        if (!last) return;
-        __threadfence();
-        if (tid == 0) cnt[tile] = 0u;
+            for (int e = 0; e < 16; ++e) acc[e >> 2][e & 3] = T(0);
+            for (int q0 = 0; q0 < n; q0 += U) {
+                T v[U][16];
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
+                for (int u = 0; u < U; ++u) {
+                    const T* p = part + ((int64_t)(first + (q0 + u) * step) * tiles + tile) * (GEMM_T * GEMM_T) + tid;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) acc[r][c] = T(0);
-        for (int z = 0; z < S; ++z) {
-            const T* p = part + ((int64_t)z * tiles + tile) * (GEMM_T * GEMM_T) + tid;
+                    for (int e = 0; e < 16; ++e) v[u][e] = q0 + u < n ? __ldcg(p + 256 * e) : T(0);
+                }
 #pragma unroll
-            for (int r = 0; r < 4; ++r)
+                for (int u = 0; u < U; ++u)
 #pragma unroll
-                for (int c = 0; c < 4; ++c) acc[r][c] += __ldcg(p + 256 * (4 * r + c));
+                    for (int e = 0; e < 16; ++e) acc[e >> 2][e & 3] += v[u][e];
+            }
+        };
+        // many parts meet in two stages of about sqrt(S): a part is 16 KB through the one SM that adds it
+        int gs = S;
+        if (S > 8)
+            for (gs = 3; gs * gs < S;) ++gs;
+        const int grp = z / gs, groups = (S + gs - 1) / gs;
+        put(z);
+        if (!arrive(cnt + (1 + grp) * tiles + tile, min(gs, S - grp * gs))) return;
+        gather(grp * gs, min(gs, S - grp * gs), 1);
+        if (groups > 1) {
+            put(grp * gs);
+            if (!arrive(cnt + tile, groups)) return;
+            gather(0, groups, gs);
         }
     }
 #pragma unroll
@@ -171,6 +199,17 @@ __global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, const T* __re
             }
             C[(int64_t)i * ldc + j] = v;
         }
+}
+
+template <typename T, int EPI>
+__global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, const T* __restrict__ A, int64_t sam, int64_t sak,
+                                              const T* __restrict__ B, int64_t sbk, int64_t sbn, T* __restrict__ C,
+                                              int64_t ldc, const T* __restrict__ bias, const T* __restrict__ aux,
+                                              T* part, unsigned* cnt) {
+    mh_dep_wait();
+    gemm_tile<T, EPI>(blockIdx.y * GEMM_T, blockIdx.x * GEMM_T, blockIdx.y * gridDim.x + blockIdx.x,
+                      gridDim.x * gridDim.y, blockIdx.z, gridDim.z, M, N, K, A, sam, sak, B, sbk, sbn, C, ldc, bias, aux,
+                      part, cnt);
 }
 
 // part, cnt (nullable): workspace of a split product (GEMM_PARTS tiles); k is split while the
@@ -483,10 +522,12 @@ __global__ void k_gather_rows(const float* __restrict__ X, const int32_t* __rest
     }
 }
 
-// dz = (yh - t) * inv; per-block partial sums of (yh - t)^2 (binary64) into part.
+// dz = (yh - t) * inv; per-block partial sums of (yh - t)^2 (binary64) into part, added by the last block to
+// finish (cnt, reset by it): out = scale * sum.
 __global__ void k_loss_dz(const float* __restrict__ yh, const float* __restrict__ t, int64_t n, float inv,
-                          float* __restrict__ dz, double* __restrict__ part) {
+                          float* __restrict__ dz, double* part, unsigned* cnt, double scale, double* out) {
     mh_dep_wait();
+    __shared__ int last;
     double s = 0.0;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
         const float df = yh[e] - t[e];
@@ -494,7 +535,21 @@ __global__ void k_loss_dz(const float* __restrict__ yh, const float* __restrict_
         s = fma((double)df, (double)df, s);
     }
     s = block_sum_d(s);
-    if (threadIdx.x == 0) part[blockIdx.x] = s;
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = s;
+        __threadfence();
+        last = atomicAdd(cnt, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    s = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) s += __ldcg(part + i);
+    s = block_sum_d(s);
+    if (threadIdx.x == 0) {
+        out[0] = s * scale;
+        *cnt = 0u;
+    }
 }
 
 __global__ void k_sum_parts(const double* __restrict__ part, int n, double scale, double* out) {
@@ -505,22 +560,49 @@ __global__ void k_sum_parts(const double* __restrict__ part, int n, double scale
     if (threadIdx.x == 0) out[0] = s * scale;
 }
 
-// out[j] = sum_i z[i][j] in binary64: 32 columns x 8 row shares per block, the shares added in order
-// (a thread per column took 15 us at 64 rows: a chain of binary64 additions).
-__global__ void __launch_bounds__(256) k_colsum(const float* __restrict__ z, int64_t rows, int64_t cols,
-                                                float* __restrict__ out) {
+// Gradients of a layer's weights (dz^T a: M x N, sums over the rows) and biases (column sums of dz).
+struct grad_layer {
+    const float *dz, *a;   // rows x M, rows x N
+    float *gW, *gb;
+    int M, N;
+    int tile0, col0;       // first tile of the weights, first block of the biases
+};
+
+struct grad_layers {
+    grad_layer l[4];
+    int tiles;             // of all weights; the blocks behind them sum columns
+};
+
+// All layers' gradients in one launch, once every dz is there: products of the minibatch's length (64: 4 slabs) that
+// fill the chip together but not one by one, and nothing of the backward chain waits for them.
+// Columns are summed in binary64: 32 columns x 8 row shares per block, the shares added in order (a thread per
+// column took 15 us at 64 rows: a chain of binary64 additions).
+__global__ void __launch_bounds__(256) k_grads(const grad_layers L, int rows, float* part, unsigned* cnt) {
     mh_dep_wait();
+    int b = blockIdx.x;
+    if (b < L.tiles) {
+        const int k = (b >= L.l[1].tile0) + (b >= L.l[2].tile0) + (b >= L.l[3].tile0);
+        const grad_layer g = L.l[k];
+        const int tx = (g.N + GEMM_T - 1) / GEMM_T, t = b - g.tile0;
+        gemm_tile<float, EPI_NONE>(t / tx * GEMM_T, t % tx * GEMM_T, b, L.tiles, blockIdx.z, gridDim.z, g.M, g.N, rows, g.dz, 1,
+                                   g.M, g.a, g.N, 1, g.gW, g.N, nullptr, nullptr, part, cnt);
+        return;
+    }
+    if (blockIdx.z) return;
+    b -= L.tiles;
+    const int k = (b >= L.l[1].col0) + (b >= L.l[2].col0) + (b >= L.l[3].col0);
+    const grad_layer g = L.l[k];
     __shared__ double sh[8][33];
-    const int c = threadIdx.x & 31, g = threadIdx.x >> 5;
-    const int64_t j = blockIdx.x * (int64_t)32 + c;
+    const int c = threadIdx.x & 31, q0 = threadIdx.x >> 5;
+    const int64_t j = (int64_t)(b - g.col0) * 32 + c;
     double s = 0.0;
-    if (j < cols)
-        for (int64_t i = g; i < rows; i += 8) s += z[i * cols + j];
-    sh[g][c] = s;
+    if (j < g.M)
+        for (int64_t i = q0; i < rows; i += 8) s += g.dz[i * g.M + j];
+    sh[q0][c] = s;
     __syncthreads();
-    if (g != 0 || j >= cols) return;
+    if (q0 != 0 || j >= g.M) return;
     for (int q = 1; q < 8; ++q) s += sh[q][c];
-    out[j] = (float)s;
+    g.gb[j] = (float)s;
 }
 
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
@@ -697,8 +779,8 @@ mh_status check_net(mh_ctx* ctx, const mh_net* net) {
 mh_status ensure_rows(mh_ctx* ctx, mh_net* net, int64_t rows) {
     if (!net->gcnt.p) {
         MH_ALLOC(ctx, net->gpart, (int64_t)GEMM_PARTS * GEMM_T * GEMM_T);
-        MH_ALLOC(ctx, net->gcnt, GEMM_PARTS);
-        MH_CUDA(ctx, cudaMemsetAsync(net->gcnt.p, 0, GEMM_PARTS * sizeof(unsigned), ctx->stream));
+        MH_ALLOC(ctx, net->gcnt, GEMM_CNT + 1);   // tiles of a product and their groups of parts; blocks of the loss
+        MH_CUDA(ctx, cudaMemsetAsync(net->gcnt.p, 0, (GEMM_CNT + 1) * sizeof(unsigned), ctx->stream));
     }
     if (rows <= net->cap_rows) return MH_OK;
     MH_ALLOC(ctx, net->xb, rows * net->d);
@@ -706,19 +788,18 @@ mh_status ensure_rows(mh_ctx* ctx, mh_net* net, int64_t rows) {
     MH_ALLOC(ctx, net->yh, rows * net->d);
     MH_ALLOC(ctx, net->dzd, rows * net->d);
     for (int i = 0; i < 3; ++i) MH_ALLOC(ctx, net->act[i], rows * net->w);
-    MH_ALLOC(ctx, net->dzw1, rows * net->w);
-    MH_ALLOC(ctx, net->dzw2, rows * net->w);
+    for (int i = 0; i < 3; ++i) MH_ALLOC(ctx, net->dzw[i], rows * net->w);
     net->cap_rows = rows;
     return MH_OK;
 }
 
-// Training-kernel forward of `rows` inputs in net->xb; output in net->yh.
-mh_status train_forward(mh_ctx* ctx, mh_net* net, int64_t rows) {
+// Training-kernel forward of `rows` inputs x; output in net->yh.
+mh_status train_forward(mh_ctx* ctx, mh_net* net, const float* x, int64_t rows) {
     cudaStream_t st = ctx->stream;
     const float* P = net->P.p;
     const int w = net->w;
     const int64_t d = net->d;
-    const float* in = net->xb.p;
+    const float* in = x;
     int64_t ld_in = d;
     for (int l = 0; l < 3; ++l) {
         gemm<float, EPI_BIAS_TANH>(st, (int)rows, w, net->lin[l], in, ld_in, 1, P + net->oW[l], 1, net->lin[l],
@@ -733,53 +814,51 @@ mh_status train_forward(mh_ctx* ctx, mh_net* net, int64_t rows) {
     return MH_OK;
 }
 
-// Loss of net->yh against net->yb over rows x d; dz (nullable) receives dL/dyh.  Result on device in out.
-mh_status train_loss(mh_ctx* ctx, mh_net* net, int64_t rows, float* dz, double* out) {
+// Loss of net->yh against y over rows x d; dz (nullable) receives dL/dyh.  Result on device in out.
+mh_status train_loss(mh_ctx* ctx, mh_net* net, const float* y, int64_t rows, float* dz, double* out) {
     const int64_t n = rows * net->d;
     const int nb = ew_grid(n);
     if ((int64_t)net->lpart.n < nb) MH_ALLOC(ctx, net->lpart, 152 * 8);
-    (void)mh_launch_dep(ctx->stream, k_loss_dz, dim3(nb), dim3(256), 0, net->yh.p, net->yb.p, n,
-                        (float)(1.0 / (double)n), dz, net->lpart.p);
-    MH_LAUNCHED(ctx);
-    (void)mh_launch_dep(ctx->stream, k_sum_parts, dim3(1), dim3(1024), 0, net->lpart.p, nb, 0.5 / (double)n, out);
+    (void)mh_launch_dep(ctx->stream, k_loss_dz, dim3(nb), dim3(256), 0, net->yh.p, y, n, (float)(1.0 / (double)n), dz,
+                        net->lpart.p, net->gcnt.p + GEMM_CNT, 0.5 / (double)n, out);
     MH_LAUNCHED(ctx);
     return MH_OK;
 }
 
-// Backward pass from dz = dL/dyh (net->dzd) into the gradient buffer g.
-mh_status train_backward(mh_ctx* ctx, mh_net* net, int64_t rows, float* g) {
+// Backward pass of inputs x from dz = dL/dyh (net->dzd) into the gradient buffer g.
+mh_status train_backward(mh_ctx* ctx, mh_net* net, const float* x, int64_t rows, float* g) {
     cudaStream_t st = ctx->stream;
     const float* P = net->P.p;
-    const int w = net->w;
-    const int64_t d = net->d;
-    const int R = (int)rows;
-    // layer 4
-    gemm<float, EPI_NONE>(st, (int)d, w, R, net->dzd.p, 1, d, net->act[2].p, w, 1, g + net->oW[3], w,
-                          (const float*)nullptr, (const float*)nullptr, net->gpart.p, net->gcnt.p);
-    MH_LAUNCHED(ctx);
-    (void)mh_launch_dep(st, k_colsum, dim3(mh_grid(d, 32)), dim3(256), 0, net->dzd.p, rows, d, g + net->ob[3]);
-    MH_LAUNCHED(ctx);
-    gemm<float, EPI_TANH_BACK>(st, R, w, (int)d, net->dzd.p, d, 1, P + net->oW[3], w, 1, net->dzw1.p, w,
-                               (const float*)nullptr, (const float*)net->act[2].p, net->gpart.p, net->gcnt.p);
-    MH_LAUNCHED(ctx);
-    float* dz = net->dzw1.p;
-    float* dn = net->dzw2.p;
+    const int w = net->w, R = (int)rows;
+    // dz of layers 2, 1, 0
     for (int l = 2; l >= 0; --l) {
-        const float* a_in = l > 0 ? net->act[l - 1].p : net->xb.p;
-        const int64_t ld_in = l > 0 ? w : d;
-        gemm<float, EPI_NONE>(st, w, net->lin[l], R, dz, 1, w, a_in, ld_in, 1, g + net->oW[l], net->lin[l],
-                              (const float*)nullptr, (const float*)nullptr, net->gpart.p, net->gcnt.p);
+        const float* dz = l == 2 ? net->dzd.p : net->dzw[l + 1].p;
+        const int out = l == 2 ? (int)net->d : w;   // of layer l + 1
+        gemm<float, EPI_TANH_BACK>(st, R, w, out, dz, out, 1, P + net->oW[l + 1], w, 1, net->dzw[l].p, w,
+                                   (const float*)nullptr, (const float*)net->act[l].p, net->gpart.p, net->gcnt.p);
         MH_LAUNCHED(ctx);
-        (void)mh_launch_dep(st, k_colsum, dim3(mh_grid(w, 32)), dim3(256), 0, dz, rows, (int64_t)w, g + net->ob[l]);
-        MH_LAUNCHED(ctx);
-        if (l > 0) {
-            gemm<float, EPI_TANH_BACK>(st, R, w, w, dz, w, 1, P + net->oW[l], w, 1, dn, w,
-                                       (const float*)nullptr, (const float*)net->act[l - 1].p, net->gpart.p,
-                                       net->gcnt.p);
-            MH_LAUNCHED(ctx);
-            std::swap(dz, dn);
-        }
     }
+    grad_layers L;
+    int tiles = 0, cols = 0;
+    for (int l = 0; l < 4; ++l) {
+        grad_layer& k = L.l[l];
+        k.dz = l == 3 ? net->dzd.p : net->dzw[l].p;
+        k.a = l == 0 ? x : net->act[l - 1].p;
+        k.gW = g + net->oW[l];
+        k.gb = g + net->ob[l];
+        k.M = l == 3 ? (int)net->d : w;
+        k.N = (int)net->lin[l];
+        k.tile0 = tiles;
+        k.col0 = cols;
+        tiles += ((k.M + GEMM_T - 1) / GEMM_T) * ((k.N + GEMM_T - 1) / GEMM_T);
+        cols += (k.M + 31) / 32;
+    }
+    L.tiles = tiles;
+    const int slabs = (R + GEMM_K - 1) / GEMM_K;
+    const int S = tiles <= GEMM_PARTS / 2 ? std::max(1, std::min(GEMM_PARTS / tiles, slabs / 2)) : 1;
+    (void)mh_launch_dep(st, k_grads, dim3((unsigned)(tiles + cols), 1, (unsigned)S), dim3(256), 0, L, R, net->gpart.p,
+                        net->gcnt.p);
+    MH_LAUNCHED(ctx);
     return MH_OK;
 }
 
@@ -1129,11 +1208,15 @@ extern "C" mh_status mh_net_loss_grad(mh_ctx* ctx, mh_net* net, const float* X_d
     if (n < 1) return mh_fail(ctx, MH_ERR_INVALID_ARG, "n must be positive");
     cudaStream_t st = ctx->stream;
     MH_TRY(ensure_rows(ctx, net, n));
-    MH_CUDA(ctx, cudaMemcpyAsync(net->xb.p, X_dev, n * net->d * 4, cudaMemcpyDeviceToDevice, st));
-    MH_CUDA(ctx, cudaMemcpyAsync(net->yb.p, T_dev, n * net->d * 4, cudaMemcpyDeviceToDevice, st));
-    MH_TRY(train_forward(ctx, net, n));
-    MH_TRY(train_loss(ctx, net, n, net->dzd.p, net->scal.p + 4));
-    if (grad_dev) MH_TRY(train_backward(ctx, net, n, grad_dev));
+    // the inputs are read where they are, unless the gradient is to be written over them
+    const float* x = X_dev;
+    if (grad_dev && X_dev < grad_dev + net->n_params && grad_dev < X_dev + n * net->d) {
+        MH_CUDA(ctx, cudaMemcpyAsync(net->xb.p, X_dev, n * net->d * 4, cudaMemcpyDeviceToDevice, st));
+        x = net->xb.p;
+    }
+    MH_TRY(train_forward(ctx, net, x, n));
+    MH_TRY(train_loss(ctx, net, T_dev, n, net->dzd.p, net->scal.p + 4));
+    if (grad_dev) MH_TRY(train_backward(ctx, net, x, n, grad_dev));
     if (loss_host) {
         MH_CUDA(ctx, cudaMemcpyAsync(loss_host, net->scal.p + 4, 8, cudaMemcpyDeviceToHost, st));
     }
@@ -1152,7 +1235,7 @@ extern "C" mh_status mh_net_forward(mh_ctx* ctx, mh_net* net, const float* X_dev
     if (training_kernels) {
         MH_TRY(ensure_rows(ctx, net, n));
         MH_CUDA(ctx, cudaMemcpyAsync(net->xb.p, X_dev, n * d * 4, cudaMemcpyDeviceToDevice, st));
-        MH_TRY(train_forward(ctx, net, n));
+        MH_TRY(train_forward(ctx, net, net->xb.p, n));
         MH_CUDA(ctx, cudaMemcpyAsync(Y_dev, net->yh.p, n * d * 4, cudaMemcpyDeviceToDevice, st));
     } else {
         for (int64_t r = 0; r < n; ++r) MH_TRY(infer_one(ctx, net, arith, X_dev + r * d, Y_dev + r * d));
@@ -1187,8 +1270,8 @@ extern "C" mh_status mh_net_train(mh_ctx* ctx, mh_net* net, const float* X_dev, 
         MH_LAUNCHED(ctx);
         k_gather_rows<<<ew_grid(n_val * d), 256, 0, st>>>(Yv_dev, nullptr, n_val, d, sy, net->yb.p);
         MH_LAUNCHED(ctx);
-        MH_TRY(train_forward(ctx, net, n_val));
-        MH_TRY(train_loss(ctx, net, n_val, nullptr, net->scal.p + 5));
+        MH_TRY(train_forward(ctx, net, net->xb.p, n_val));
+        MH_TRY(train_loss(ctx, net, net->yb.p, n_val, nullptr, net->scal.p + 5));
         MH_CUDA(ctx, cudaMemcpyAsync(out, net->scal.p + 5, 8, cudaMemcpyDeviceToHost, st));
         MH_CUDA(ctx, cudaStreamSynchronize(st));
         return MH_OK;
@@ -1206,9 +1289,9 @@ extern "C" mh_status mh_net_train(mh_ctx* ctx, mh_net* net, const float* X_dev, 
         MH_LAUNCHED(ctx);
         k_gather_rows<<<ew_grid((int64_t)batch * d), 256, 0, st>>>(Y_dev, idx, batch, d, sy, net->yb.p);
         MH_LAUNCHED(ctx);
-        MH_TRY(train_forward(ctx, net, batch));
-        MH_TRY(train_loss(ctx, net, batch, net->dzd.p, net->scal.p + 4));
-        MH_TRY(train_backward(ctx, net, batch, net->G.p));
+        MH_TRY(train_forward(ctx, net, net->xb.p, batch));
+        MH_TRY(train_loss(ctx, net, net->yb.p, batch, net->dzd.p, net->scal.p + 4));
+        MH_TRY(train_backward(ctx, net, net->xb.p, batch, net->G.p));
         const float bc1 = (float)(1.0 - std::pow(0.9, t)), bc2 = (float)(1.0 - std::pow(0.999, t));
         k_adam<<<ew_grid(np), 256, 0, st>>>(net->P.p, net->G.p, net->Mo.p, net->Vo.p, np, (float)lr, b1, b2, 1e-8f,
                                             bc1, bc2);
