@@ -1617,7 +1617,8 @@ __global__ void __launch_bounds__(BS) k_dlp_coarse(const double* __restrict__ xy
                                                    int64_t nt, const double* __restrict__ geo,
                                                    const double* __restrict__ sigma,
                                                    const int32_t* __restrict__ curve_of, const int32_t* __restrict__ nn,
-                                                   int64_t ns, mh_pair_tab tab, double pref, double* out) {
+                                                   int64_t ns, int64_t per, mh_pair_tab tab, double pref,
+                                                   double* out) {
     mh_dep_wait();
     __shared__ double2 sp[BS], sn[BS];
     __shared__ int sk[BS];
@@ -1626,11 +1627,10 @@ __global__ void __launch_bounds__(BS) k_dlp_coarse(const double* __restrict__ xy
     const double px = active ? xy[2 * t] : 0.0, py = active ? xy[2 * t + 1] : 0.0;
     const uint32_t mask = active ? fine[t] : 0xffffffffu;
     double acc = 0.0;
-    const int64_t ntile = (ns + BS - 1) / BS, per = (ntile + gridDim.y - 1) / gridDim.y;
-    const int64_t sbeg = blockIdx.y * per * BS, send = min(ns, (blockIdx.y + 1) * per * BS);
+    const int64_t sbeg = blockIdx.y * per, send = min(ns, sbeg + per);
     for (int64_t s0 = sbeg; s0 < send; s0 += BS) {
         const int64_t s = s0 + threadIdx.x;
-        if (s < ns) {
+        if (s < send) {
             const double* g = geo + 8 * s;
             const int k = curve_of[s];
             const double wh = sigma[s] * (2.0 * MH_PI / nn[k]);   // n |y'| = (y2', -y1')
@@ -1639,7 +1639,7 @@ __global__ void __launch_bounds__(BS) k_dlp_coarse(const double* __restrict__ xy
             sk[threadIdx.x] = k;
         }
         __syncthreads();
-        const int cnt = (ns - s0) < BS ? (int)(ns - s0) : BS;
+        const int cnt = (int)min((int64_t)BS, send - s0);
         if (active) {
             for (int i = 0; i < cnt; ++i) {
                 if ((mask >> sk[i]) & 1u) continue;
@@ -3047,7 +3047,12 @@ static mh_status coarse_sums(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targ
     cudaStream_t st = ctx->stream;
     const double pref = -1.0 / (2.0 * MH_PI * alpha * alpha) / (alpha * alpha);
     const int64_t nblk = (count + MH_TILE - 1) / MH_TILE, ntile = (b->n + MH_TILE - 1) / MH_TILE;
-    const int nsplit = (int)std::max<int64_t>(1, std::min<int64_t>(ntile, (152 * 8) / nblk));
+    // Shares of the sources, 8 blocks an SM: whole tiles in binary32 (culled by tile), in binary64 any multiple of 16 (with
+    // whole tiles 512 nodes were 8 blocks, 90 us: that step 348 -> 296 us, 2000 targets at 6144 nodes 1064 -> 1004 us)
+    const bool f64 = prec != MH_PREC_MIXED;
+    int nsplit = (int)std::max<int64_t>(1, std::min<int64_t>(f64 ? (b->n + 15) / 16 : ntile, (152 * 8) / nblk));
+    const int64_t per = ((b->n + nsplit - 1) / nsplit + 15) / 16 * 16;
+    if (f64) nsplit = (int)((b->n + per - 1) / per);
     if (nsplit > 1 && (int64_t)tg->part.n < nsplit * count) MH_ALLOC(ctx, tg->part, nsplit * count);
     const dim3 grid((unsigned)nblk, (unsigned)nsplit);
     double* out = nsplit > 1 ? tg->part.p : tg->ext.p + i0;
@@ -3061,10 +3066,10 @@ static mh_status coarse_sums(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targ
         const auto kern = k_dlp_coarse<MH_TILE>;
         if (dep)
             (void)mh_launch_dep(st, kern, grid, dim3(MH_TILE), 0, tg->xy.p + 2 * i0, tg->fine.p + i0, count, b->geo.p,
-                                sigma, b->d_curve_of.p, b->d_nn.p, b->n, tab, pref, out);
+                                sigma, b->d_curve_of.p, b->d_nn.p, b->n, per, tab, pref, out);
         else
             kern<<<grid, MH_TILE, 0, st>>>(tg->xy.p + 2 * i0, tg->fine.p + i0, count, b->geo.p, sigma, b->d_curve_of.p,
-                                           b->d_nn.p, b->n, tab, pref, out);
+                                           b->d_nn.p, b->n, per, tab, pref, out);
     }
     MH_LAUNCHED(ctx);
     if (nsplit > 1) {
