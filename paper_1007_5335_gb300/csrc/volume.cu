@@ -13,10 +13,12 @@
 // form of length 2p+1 ([a_0, a_1, b_1, ..., a_p, b_p], M_{-n} = conj(M_n) for a real B).
 //
 // Every pass is a batch of small dense contractions "y_dst += T_op x_src" with the
-// operator T_op chosen by (level, relative configuration).  Tasks are sorted by operator;
-// a block stages one operator and up to 64 source vectors in shared memory and writes
-// its products to a task-indexed buffer, and a segmented reduction sums the products of
-// each destination in a fixed order (deterministic, no atomics).  The near tables form their
+// operator T_op chosen by (level, relative configuration).  Tasks are sorted by operator; a block
+// takes one operator and some of its source vectors and writes the products to a task-indexed
+// buffer, and a segmented reduction sums the products of each destination in a fixed order
+// (deterministic, no atomics).  Binary32: on the tensor cores (contract_tc.cu), or k_apply without them.
+// Binary64: mirror-image sources share a product (orbit.cuh).  Operators of one source vector of their own (dipoles,
+// boundary nodes): k_cols.  M2M and L2L: one launch per tree level.  The near tables form their
 // own phase, which needs only the node values: it runs beside the multipole passes on a
 // second stream and writes U first; the output phase then adds the far field.
 #include <algorithm>
