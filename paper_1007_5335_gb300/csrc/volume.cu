@@ -1088,7 +1088,7 @@ struct VolData {
     std::unique_ptr<BieData> bie;        // on-surface double layer (matrix-free BIE operator)
     int P = 0, qq = 0;
     int64_t B_off = 0, U_off = 0, M_off = 0, L_off = 0, vec_len = 0;
-    dbuf<double> ops64, vec, temp;
+    dbuf<double> vec, temp;
     dbuf<float> ops32, vec32;            // vec32: binary32 mirror of vec (node values, expansions)
     dbuf<int64_t> d_op_off;
     dbuf<int32_t> d_op_C;
@@ -1809,10 +1809,14 @@ mh_status volume_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, VolData* V)
     }
     for (auto& tk : t_near) tk.op = first_near_op + (-1 - tk.op);
     const int64_t total = near_base + (int64_t)nnear * qq * qq;
-    MH_ALLOC(ctx, V->ops64, total);
     cudaStream_t st = ctx->stream;
-    if (near_base) MH_CUDA(ctx, cudaMemcpyAsync(V->ops64.p, pool.data.data(), near_base * 8, cudaMemcpyHostToDevice, st));
+    // every operator in binary64 on the host: source of the binary32 copy, of the tensor-core images and of the
+    // operators in class order
+    std::vector<double> all(pool.data);
+    all.resize(total);
     if (nnear) {
+        dbuf<double> tables;
+        MH_ALLOC(ctx, tables, total - near_base);
         dbuf<NearCfg> dcfg;
         dbuf<double> dxi, dgx, dgw;
         MH_ALLOC(ctx, dcfg, nnear);
@@ -1824,16 +1828,12 @@ mh_status volume_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, VolData* V)
         MH_CUDA(ctx, cudaMemcpyAsync(dgx.p, g16x.data(), NGLN * 8, cudaMemcpyHostToDevice, st));
         MH_CUDA(ctx, cudaMemcpyAsync(dgw.p, g16w.data(), NGLN * 8, cudaMemcpyHostToDevice, st));
         k_near_tables<<<(unsigned)(nnear * qq), 256, 0, st>>>(dcfg.p, q, dxi.p, dgx.p, dgw.p, k, pref,
-                                                              V->ops64.p + near_base);
+                                                              tables.p);
         MH_LAUNCHED(ctx);
+        MH_CUDA(ctx, cudaMemcpyAsync(all.data() + near_base, tables.p, (total - near_base) * 8, cudaMemcpyDeviceToHost, st));
         MH_CUDA(ctx, cudaStreamSynchronize(st));
     }
     MH_ALLOC(ctx, V->ops32, total);
-    // every operator in binary64 on the host (the near tables were formed on the device): source
-    // of the binary32 copy and of the tensor-core images
-    std::vector<double> all(total);
-    MH_CUDA(ctx, cudaMemcpyAsync(all.data(), V->ops64.p, total * 8, cudaMemcpyDeviceToHost, st));
-    MH_CUDA(ctx, cudaStreamSynchronize(st));
     {
         // binary32 copy of every operator (mixed precision)
         std::vector<float> f(all.begin(), all.end());
@@ -1893,8 +1893,6 @@ mh_status volume_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, VolData* V)
     MH_CUDA(ctx, cudaMemsetAsync(V->vec.p, 0, V->vec_len * 8, st));
     MH_CUDA(ctx, cudaMemsetAsync(V->vec32.p, 0, (V->vec_len + TC_POOL_PAD) * 4, st));
     // shared-memory opt-in for the contraction kernel
-    int maxs = 0;
-    for (auto* ph : {V->p2m.get(), V->m2l.get(), V->out.get(), V->near.get()}) maxs = std::max(maxs, ph->smem);
     MH_CUDA(ctx, cudaFuncSetAttribute(k_apply<double, double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       160 * 1024));
     MH_CUDA(ctx, cudaFuncSetAttribute(k_apply<float, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024));
@@ -2456,9 +2454,11 @@ mh_status volume_dipole_setup(mh_ctx* ctx, mh_tree* t, double alpha, int p, cons
     // upload the operator pool (volume translation operators + dipole blocks)
     cudaStream_t st = ctx->stream;
     const int64_t total = (int64_t)pool.data.size();
-    MH_ALLOC(ctx, D->ops64, total);
     MH_ALLOC(ctx, D->ops32, total);
-    MH_CUDA(ctx, cudaMemcpyAsync(D->ops64.p, pool.data.data(), total * 8, cudaMemcpyHostToDevice, st));
+    if (near_blocks) {   // the output phase in binary64 (else by orbits)
+        MH_ALLOC(ctx, D->ops64, total);
+        MH_CUDA(ctx, cudaMemcpyAsync(D->ops64.p, pool.data.data(), total * 8, cudaMemcpyHostToDevice, st));
+    }
     {
         std::vector<float> f(pool.data.begin(), pool.data.end());
         MH_CUDA(ctx, cudaMemcpyAsync(D->ops32.p, f.data(), total * 4, cudaMemcpyHostToDevice, st));
