@@ -3039,6 +3039,23 @@ static mh_status pair_table(mh_ctx* ctx, mh_boundary* b, double alpha) {
     return MH_OK;
 }
 
+// Shares of the sources of a trapezoid sum over nblk blocks of targets, 8 blocks an SM: whole tiles in
+// binary32 (culled by tile), in binary64 any multiple of 16 (with whole tiles 512 nodes were 8 blocks, 90 us:
+// that step 348 -> 296 us, 2000 targets at 6144 nodes 1064 -> 1004 us).
+struct coarse_shares {
+    int n;         // shares
+    int64_t per;   // sources of a share (binary64)
+};
+
+static coarse_shares coarse_split(int64_t ns, int64_t nblk, bool f64) {
+    const int64_t units = f64 ? (ns + 15) / 16 : (ns + MH_TILE - 1) / MH_TILE;
+    coarse_shares s;
+    s.n = (int)std::max<int64_t>(1, std::min<int64_t>(units, (152 * 8) / nblk));
+    s.per = ((ns + s.n - 1) / s.n + 15) / 16 * 16;
+    if (f64) s.n = (int)((ns + s.per - 1) / s.per);
+    return s;
+}
+
 // Trapezoid sums at the points [i0, i0 + count) of the extended target set into tg->ext (mixed
 // precision: b->w32 holds this density's weights).  The sources are split over the grid so that
 // about 8 blocks per SM run whatever the number of targets, the partial sums added in a fixed order.
@@ -3046,14 +3063,15 @@ static mh_status coarse_sums(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targ
                              const double* sigma, mh_precision prec, bool dep) {
     cudaStream_t st = ctx->stream;
     const double pref = -1.0 / (2.0 * MH_PI * alpha * alpha) / (alpha * alpha);
-    const int64_t nblk = (count + MH_TILE - 1) / MH_TILE, ntile = (b->n + MH_TILE - 1) / MH_TILE;
-    // Shares of the sources, 8 blocks an SM: whole tiles in binary32 (culled by tile), in binary64 any multiple of 16 (with
-    // whole tiles 512 nodes were 8 blocks, 90 us: that step 348 -> 296 us, 2000 targets at 6144 nodes 1064 -> 1004 us)
     const bool f64 = prec != MH_PREC_MIXED;
-    int nsplit = (int)std::max<int64_t>(1, std::min<int64_t>(f64 ? (b->n + 15) / 16 : ntile, (152 * 8) / nblk));
-    const int64_t per = ((b->n + nsplit - 1) / nsplit + 15) / 16 * 16;
-    if (f64) nsplit = (int)((b->n + per - 1) / per);
-    if (nsplit > 1 && (int64_t)tg->part.n < nsplit * count) MH_ALLOC(ctx, tg->part, nsplit * count);
+    const int64_t nblk = (count + MH_TILE - 1) / MH_TILE;
+    const coarse_shares sh = coarse_split(b->n, nblk, f64);
+    const int nsplit = sh.n;
+    const int64_t per = sh.per;
+    // Room for either precision's shares at the first call: a recorded graph of one precision holds the
+    // buffer, so a step of the other one must not replace it.
+    const int most = std::max(nsplit, coarse_split(b->n, nblk, !f64).n);
+    if (most > 1) MH_RESERVE(ctx, tg->part, most * count);
     const dim3 grid((unsigned)nblk, (unsigned)nsplit);
     double* out = nsplit > 1 ? tg->part.p : tg->ext.p + i0;
     if (prec == MH_PREC_MIXED)
