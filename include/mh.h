@@ -182,7 +182,10 @@ mh_status mh_volume_potential(mh_ctx* ctx, mh_tree* tree, double alpha, int p, c
  *   n_targets < 0 is MH_ERR_INVALID_ARG.
  * A boundary switched to the matrix-free operator (mh_problem_matrix_free) forms A sigma that
  * way, in binary64 whatever prec says; alpha must then be the problem's (else
- * MH_ERR_INVALID_ARG). */
+ * MH_ERR_INVALID_ARG).
+ * Threads: with the dense operator for alpha assembled by an earlier call, binary64 calls with
+ * targets only read the boundary (their buffers belong to the context), so host threads with a
+ * context each may make them on one boundary at the same time. */
 mh_status mh_double_layer_apply(mh_ctx* ctx, mh_boundary* bnd, double alpha, const double* sigma_dev,
                                 const double* targets_dev, int64_t n_targets, double* out_dev,
                                 mh_precision prec);

@@ -19,7 +19,6 @@ namespace {
 
 constexpr int UPSAMPLE = 16;        // fine grid for targets within 10 h_s of a curve
 constexpr int FINE_TG = 4;          // auxiliary targets per block of the binary32 upsampled rule
-constexpr int64_t DLP_KEEP = 1 << 16;   // largest target set whose buffers a boundary keeps (some 50 MB)
 constexpr double NEAR_NODE = 12.0;  // project on the curve when the nearest node is within 12 h*
 constexpr double NEAR_FINE = 10.0;  // d < 10 h_s: upsampled rule
 constexpr double NEAR_LINE = 0.25;  // d < h_s/4: interpolation along the normal
@@ -3027,14 +3026,22 @@ static mh_status prep_mixed(mh_ctx* ctx, mh_boundary* b) {
     return MH_OK;
 }
 
-// The binary64 pair table of the boundary for alpha (recorded graphs hold it: a rebuild counts as
-// a new operator generation, and the eager step before a recording makes it).
-static mh_status pair_table(mh_ctx* ctx, mh_boundary* b, double alpha) {
-    if (b->ptab_alpha == alpha) return MH_OK;
-    if (!b->ptab.p) MH_ALLOC(ctx, b->ptab, PT_WORDS * PT_BINS);
-    k_pair_table<<<(PT_BINS + 127) / 128, 128, 0, ctx->stream>>>(mh_pair_tab_make(nullptr, alpha), alpha, b->ptab.p);
+// The binary64 pair table for alpha in t.
+static mh_status pair_table(mh_ctx* ctx, pair_tab_buf& t, double alpha) {
+    if (t.alpha == alpha) return MH_OK;
+    MH_RESERVE(ctx, t.c, PT_WORDS * PT_BINS);
+    t.alpha = -1.0;
+    k_pair_table<<<(PT_BINS + 127) / 128, 128, 0, ctx->stream>>>(mh_pair_tab_make(nullptr, alpha), alpha, t.c.p);
     MH_LAUNCHED(ctx);
-    b->ptab_alpha = alpha;
+    t.alpha = alpha;
+    return MH_OK;
+}
+
+// The same for the boundary's own table: recorded graphs hold it, so a rebuild counts as a new operator
+// generation, and the eager step before a recording makes it.
+static mh_status step_pair_table(mh_ctx* ctx, mh_boundary* b, double alpha) {
+    if (b->ptab.alpha == alpha) return MH_OK;
+    MH_TRY(pair_table(ctx, b->ptab, alpha));
     b->op.gen += 1;
     return MH_OK;
 }
@@ -3059,8 +3066,9 @@ static coarse_shares coarse_split(int64_t ns, int64_t nblk, bool f64) {
 // Trapezoid sums at the points [i0, i0 + count) of the extended target set into tg->ext (mixed
 // precision: b->w32 holds this density's weights).  The sources are split over the grid so that
 // about 8 blocks per SM run whatever the number of targets, the partial sums added in a fixed order.
+// ptab: the pair table for alpha (binary64).
 static mh_status coarse_sums(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* tg, int64_t i0, int64_t count,
-                             const double* sigma, mh_precision prec, bool dep) {
+                             const double* sigma, mh_precision prec, const pair_tab_buf& ptab, bool dep) {
     cudaStream_t st = ctx->stream;
     const double pref = -1.0 / (2.0 * MH_PI * alpha * alpha) / (alpha * alpha);
     const bool f64 = prec != MH_PREC_MIXED;
@@ -3079,8 +3087,7 @@ static mh_status coarse_sums(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targ
                             b->src32.p, b->w32.p, b->d_curve_of.p, b->tile_c.p, b->tile_r.p, b->n,
                             mh_dl32_make(alpha, MH_DL_CUT32), pref, out);
     else {
-        MH_TRY(pair_table(ctx, b, alpha));
-        const mh_pair_tab tab = mh_pair_tab_make(b->ptab.p, alpha);
+        const mh_pair_tab tab = mh_pair_tab_make(ptab.c.p, alpha);
         const auto kern = k_dlp_coarse<MH_TILE>;
         if (dep)
             (void)mh_launch_dep(st, kern, grid, dim3(MH_TILE), 0, tg->xy.p + 2 * i0, tg->fine.p + i0, count, b->geo.p,
@@ -3100,7 +3107,7 @@ static mh_status coarse_sums(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targ
 
 // Upsampled sums of the set's groups, added to tg->ext; weights b->wf32 (mixed) or wf64.
 static mh_status fine_sums(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* tg, const double* wf64,
-                           mh_precision prec) {
+                           mh_precision prec, const pair_tab_buf& ptab) {
     cudaStream_t st = ctx->stream;
     const double pref = -1.0 / (2.0 * MH_PI * alpha * alpha) / (alpha * alpha);
     const unsigned grid = (unsigned)(tg->n_groups * tg->fine_slices);
@@ -3109,20 +3116,20 @@ static mh_status fine_sums(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_target
                             tg->grp_curve.p, tg->grp_pair.p, tg->fine_slices, b->fine32.p, b->wf32.p, b->d_fine_off.p,
                             b->d_fchunk_off.p, b->fchunk_cf.p, b->fchunk_r.p, mh_dl32_make(alpha, MH_DL_CUT32),
                             (float)(MH_DL_CUT32 * alpha), pref, tg->grp_part.p, tg->grp_cnt.p, tg->ext.p);
-    else {
-        MH_TRY(pair_table(ctx, b, alpha));
+    else
         (void)mh_launch_dep(st, k_dlp_fine64_grp<FINE_TG>, dim3(grid), dim3(256), 0, tg->xy.p, tg->pair_tgt.p,
                             tg->grp_curve.p, tg->grp_pair.p, tg->fine_slices, b->fine_geo.p, wf64, b->d_fine_off.p,
-                            mh_pair_tab_make(b->ptab.p, alpha), pref, tg->grp_part.p, tg->grp_cnt.p, tg->ext.p);
-    }
+                            mh_pair_tab_make(ptab.c.p, alpha), pref, tg->grp_part.p, tg->grp_cnt.p, tg->ext.p);
     MH_LAUNCHED(ctx);
     return MH_OK;
 }
 
-mh_status dlp_evaluate(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* tg, const double* sigma,
-                       double* out, mh_precision prec) {
+// U^h at the targets classified in E->tg.
+static mh_status dlp_evaluate(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_eval* E, const double* sigma, double* out,
+                              mh_precision prec) {
     cudaStream_t st = ctx->stream;
     MH_TRY(bie_assemble(ctx, b, alpha));
+    dlp_targets* tg = &E->tg;
     dbuf<double>& ext = tg->ext;
     dbuf<double>& asig = tg->asig;
     prof_scope ps_all(ctx, "dlp_evaluate");
@@ -3131,14 +3138,15 @@ mh_status dlp_evaluate(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* t
         k_weights32<<<mh_grid(b->n, 256), 256, 0, st>>>(sigma, b->geo.p, b->d_curve_of.p, b->d_nn.p, b->n, b->w32.p);
         MH_LAUNCHED(ctx);
     }
+    if (prec != MH_PREC_MIXED) MH_TRY(pair_table(ctx, E->ptab, alpha));
     if (tg->n_ext) {
         prof_scope ps(ctx, "dlp_coarse", DL_FLOPS * tg->n_ext * b->n, 24.0 * (tg->n_ext + b->n));
-        MH_TRY(coarse_sums(ctx, b, alpha, tg, 0, tg->n_ext, sigma, prec, true));
+        MH_TRY(coarse_sums(ctx, b, alpha, tg, 0, tg->n_ext, sigma, prec, E->ptab, true));
     }
     if (tg->n_pairs) {
-        MH_TRY(dlp_fine_weights(ctx, b, sigma, prec, true));
+        MH_TRY(dlp_fine_weights(ctx, b, sigma, prec, E->fine, true));
         prof_scope ps(ctx, "dlp_fine", DL_FLOPS * (tg->fine_nodes_main + tg->fine_nodes_aux), 24.0 * b->n_fine);
-        MH_TRY(fine_sums(ctx, b, alpha, tg, b->wf64.p, prec));
+        MH_TRY(fine_sums(ctx, b, alpha, tg, E->fine.wf.p, prec, E->ptab));
     }
     if (tg->n_line) {
         MH_TRY(bie_apply(ctx, b, sigma, asig.p, MH_PREC_FP64));
@@ -3157,39 +3165,37 @@ __global__ void k_f2d(const float* __restrict__ a, double* __restrict__ b, int64
 }
 
 // Density times |y'| h_f on the 16x fine grid from the density's Fourier coefficients sc
-// (binary64): into wf32 (mixed) or wf64 (binary64).
-static mh_status fine_density(mh_ctx* ctx, mh_boundary* b, const double* sc, mh_precision prec, float* wf32,
-                              double* wf64) {
+// (binary64, ws.sc): into b->wf32 (mixed) or ws.wf (binary64).
+static mh_status fine_density(mh_ctx* ctx, mh_boundary* b, mh_precision prec, fine_ws& ws) {
     cudaStream_t st = ctx->stream;
     const int64_t nmodes = b->n / 2 + b->n_curves;
     const int max_n = *std::max_element(b->n_nodes.begin(), b->n_nodes.end());
     const dim3 grid((unsigned)((max_n + 15) / 16), (unsigned)b->n_curves);
     if (prec == MH_PREC_MIXED) {
         if (!b->fcp32.p) MH_ALLOC(ctx, b->fcp32, nmodes * UPSAMPLE);
-        k_fine_coef<float2><<<mh_grid(nmodes * UPSAMPLE, 256), 256, 0, st>>>(sc, b->d_nn.p, b->d_off.p, b->n_curves,
+        k_fine_coef<float2><<<mh_grid(nmodes * UPSAMPLE, 256), 256, 0, st>>>(ws.sc.p, b->d_nn.p, b->d_off.p, b->n_curves,
                                                                              nmodes, b->fcp32.p);
         MH_LAUNCHED(ctx);
         k_fine_density_s<float, float2><<<grid, 256, max_n * sizeof(float2), st>>>(
-            b->fcp32.p, b->tw32.p, b->fine_geo.p, b->d_nn.p, b->d_off.p, b->d_fine_off.p, wf32);
+            b->fcp32.p, b->tw32.p, b->fine_geo.p, b->d_nn.p, b->d_off.p, b->d_fine_off.p, b->wf32.p);
     } else {
-        if (!b->fcp64.p) MH_ALLOC(ctx, b->fcp64, nmodes * UPSAMPLE);
-        k_fine_coef<double2><<<mh_grid(nmodes * UPSAMPLE, 256), 256, 0, st>>>(sc, b->d_nn.p, b->d_off.p, b->n_curves,
-                                                                              nmodes, b->fcp64.p);
+        MH_RESERVE(ctx, ws.cp, nmodes * UPSAMPLE);
+        k_fine_coef<double2><<<mh_grid(nmodes * UPSAMPLE, 256), 256, 0, st>>>(ws.sc.p, b->d_nn.p, b->d_off.p, b->n_curves,
+                                                                              nmodes, ws.cp.p);
         MH_LAUNCHED(ctx);
         k_fine_density_s<double, double2><<<grid, 256, max_n * sizeof(double2), st>>>(
-            b->fcp64.p, b->tw.p, b->fine_geo.p, b->d_nn.p, b->d_off.p, b->d_fine_off.p, wf64);
+            ws.cp.p, b->tw.p, b->fine_geo.p, b->d_nn.p, b->d_off.p, b->d_fine_off.p, ws.wf.p);
     }
     MH_LAUNCHED(ctx);
     return MH_OK;
 }
 
-mh_status dlp_fine_weights(mh_ctx* ctx, mh_boundary* b, const double* sigma, mh_precision prec, bool spectrum64) {
+mh_status dlp_fine_weights(mh_ctx* ctx, mh_boundary* b, const double* sigma, mh_precision prec, fine_ws& ws,
+                           bool spectrum64) {
     cudaStream_t st = ctx->stream;
     const int64_t nmodes = b->n / 2 + b->n_curves;
-    if (!b->sc64.p) {
-        MH_ALLOC(ctx, b->sc64, 2 * nmodes);
-        MH_ALLOC(ctx, b->wf64, b->n_fine);
-    }
+    MH_RESERVE(ctx, ws.sc, 2 * nmodes);
+    MH_RESERVE(ctx, ws.wf, b->n_fine);
     const bool mixed = prec == MH_PREC_MIXED;
     if (mixed) MH_TRY(prep_mixed(ctx, b));
     const int max_n = *std::max_element(b->n_nodes.begin(), b->n_nodes.end());
@@ -3199,11 +3205,11 @@ mh_status dlp_fine_weights(mh_ctx* ctx, mh_boundary* b, const double* sigma, mh_
         const dim3 grid(UPSAMPLE, (unsigned)b->n_curves);
         if (mixed && !spectrum64)
             (void)mh_launch_dep(st, k_fine_weights_fft<float, float2>, grid, dim3(256), 2 * max_n * sizeof(float2), sigma,
-                                b->tw32.p, b->fine_geo.p, b->d_nn.p, b->d_off.p, b->d_fine_off.p, b->wf32.p, b->wf64.p);
+                                b->tw32.p, b->fine_geo.p, b->d_nn.p, b->d_off.p, b->d_fine_off.p, b->wf32.p, ws.wf.p);
         else
             (void)mh_launch_dep(st, k_fine_weights_fft<double, double2>, grid, dim3(256), 2 * max_n * sizeof(double2),
                                 sigma, b->tw.p, b->fine_geo.p, b->d_nn.p, b->d_off.p, b->d_fine_off.p,
-                                mixed ? b->wf32.p : nullptr, b->wf64.p);
+                                mixed ? b->wf32.p : nullptr, ws.wf.p);
         MH_LAUNCHED(ctx);
         return MH_OK;
     }
@@ -3211,15 +3217,15 @@ mh_status dlp_fine_weights(mh_ctx* ctx, mh_boundary* b, const double* sigma, mh_
         k_to_float_vec<<<mh_grid(b->n, 256), 256, 0, st>>>(sigma, b->x32.p, b->n);
         MH_LAUNCHED(ctx);
         k_fourier_scalar32<<<(unsigned)nmodes, 128, 0, st>>>(b->x32.p, b->d_nn.p, b->d_off.p, b->tw32.p, b->n_curves,
-                                                             nmodes, b->sc64.p);
+                                                             nmodes, ws.sc.p);
     } else {
         k_fourier_scalar<<<(unsigned)nmodes, 128, 0, st>>>(sigma, b->d_nn.p, b->d_off.p, b->tw.p, b->n_curves,
-                                                           nmodes, b->sc64.p);
+                                                           nmodes, ws.sc.p);
     }
     MH_LAUNCHED(ctx);
-    MH_TRY(fine_density(ctx, b, b->sc64.p, prec, b->wf32.p, b->wf64.p));
+    MH_TRY(fine_density(ctx, b, prec, ws));
     if (mixed) {
-        k_f2d<<<mh_grid(b->n_fine, 256), 256, 0, st>>>(b->wf32.p, b->wf64.p, b->n_fine);
+        k_f2d<<<mh_grid(b->n_fine, 256), 256, 0, st>>>(b->wf32.p, ws.wf.p, b->n_fine);
         MH_LAUNCHED(ctx);
     }
     return MH_OK;
@@ -3237,10 +3243,11 @@ mh_status dlp_aux_sums(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* t
         MH_LAUNCHED(ctx);
     }
     // binary64: the first launch here, behind the side stream's event wait
-    MH_TRY(coarse_sums(ctx, b, alpha, tg, n, naux, sigma, prec, prec == MH_PREC_MIXED));
+    if (prec != MH_PREC_MIXED) MH_TRY(step_pair_table(ctx, b, alpha));
+    MH_TRY(coarse_sums(ctx, b, alpha, tg, n, naux, sigma, prec, b->ptab, prec == MH_PREC_MIXED));
     if (tg->n_groups) {
         prof_scope ps(ctx, "dlp_fine", DL_FLOPS * tg->fine_nodes_aux, 24.0 * b->n_fine);
-        MH_TRY(fine_sums(ctx, b, alpha, tg, b->wf64.p, prec));
+        MH_TRY(fine_sums(ctx, b, alpha, tg, b->fine.wf.p, prec, b->ptab));
     }
     return MH_OK;
 }
@@ -3268,13 +3275,11 @@ extern "C" mh_status mh_double_layer_apply(mh_ctx* ctx, mh_boundary* b, double a
     }
     if (n_targets < 0) return mh_fail(ctx, MH_ERR_INVALID_ARG, "n_targets < 0");
     if (n_targets == 0) return MH_OK;   // no targets: nothing to evaluate, out_dev untouched
-    // the target set's buffers stay with the boundary for the next call (some twenty allocations and
-    // frees cost ~0.3 ms), unless this call was a large one
-    if (!b->eval) b->eval.reset(new dlp_targets());
-    mh_status s = dlp_classify(ctx, b, targets_dev, n_targets, b->eval.get(), true);
-    if (s == MH_OK) s = dlp_evaluate(ctx, b, alpha, b->eval.get(), sigma_dev, out_dev, prec);
+    if (!ctx->eval) ctx->eval.reset(new dlp_eval());
+    mh_status s = dlp_classify(ctx, b, targets_dev, n_targets, &ctx->eval->tg, true);
+    if (s == MH_OK) s = dlp_evaluate(ctx, b, alpha, ctx->eval.get(), sigma_dev, out_dev, prec);
     if (s == MH_OK) MH_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    if (s != MH_OK || n_targets > DLP_KEEP) b->eval.reset();
+    if (s != MH_OK || ctx->eval->bytes() > DLP_KEEP) ctx->eval.reset();
     return s;
 }
 

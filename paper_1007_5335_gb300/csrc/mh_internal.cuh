@@ -24,6 +24,8 @@ struct prof_region {
     double flops = 0.0, bytes = 0.0;   // algorithmic work of the timed launches
 };
 
+struct dlp_eval;
+
 struct mh_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -34,6 +36,7 @@ struct mh_ctx {
     bool tensor_cores = true; // binary32 contractions on the tensor cores (mh_set_tensor_cores)
     int64_t loop_nodes = 0;   // graph WHILE nodes recorded (their body kernels: loop_kernels each)
     std::map<std::string, prof_region> prof;
+    std::unique_ptr<dlp_eval> eval;   // what mh_double_layer_apply at targets writes (below)
     ~mh_ctx();
 };
 
@@ -105,6 +108,11 @@ struct dbuf {
     }
     cudaError_t reserve(size_t count) { return count <= n ? cudaSuccess : alloc(count); }
 };
+
+template <class... B>
+inline size_t mh_bytes(const B&... b) {
+    return (size_t(0) + ... + (b.n * sizeof(*b.p)));
+}
 
 #define MH_RESERVE(ctx, buf, count) MH_CUDA(ctx, (buf).reserve(count))
 #define MH_ALLOC(ctx, buf, count) MH_CUDA(ctx, (buf).alloc(count))
@@ -311,7 +319,37 @@ struct dlp_targets {
     dbuf<unsigned> grp_cnt;
     // evaluation workspaces (allocated once by dlp_classify)
     dbuf<double> ext, asig, part;
+    size_t bytes() const {
+        return mh_bytes(xy, fine0, lcurve, ldata, fine, region, line_tgt, line_curve, line_data, line_l, line_w, line_woff,
+                        pair_tgt, pair_curve, grp_curve, grp_pair, grp_part, grp_cnt, ext, asig, part);
+    }
 };
+
+// A binary64 pair table (pair64.cuh) and the alpha it holds.
+struct pair_tab_buf {
+    dbuf<double2> c;
+    double alpha = -1.0;
+};
+
+// A density on its way to the 16x grid: Fourier coefficients, those of the sub-offsets (curves that are
+// not transformed by FFT), and the density times |y'| h_f there, in binary64.
+struct fine_ws {
+    dbuf<double> sc, wf;
+    dbuf<double2> cp;
+    size_t bytes() const { return mh_bytes(sc, wf, cp); }
+};
+
+// Everything that a binary64 mh_double_layer_apply at targets writes belongs to the context, so that contexts
+// on several host threads may evaluate on one boundary: the boundary is only read there (its operator for
+// alpha assembled before).  Kept for the next call (some twenty allocations and frees cost ~0.3 ms) up
+// to DLP_KEEP bytes: the interpolation weights alone are N_k doubles for every target within h_s/4.
+struct dlp_eval {
+    dlp_targets tg;
+    pair_tab_buf ptab;
+    fine_ws fine;
+    size_t bytes() const { return tg.bytes() + fine.bytes() + mh_bytes(ptab.c); }
+};
+constexpr size_t DLP_KEEP = 64 << 20;
 
 struct mh_boundary {
     int n_curves = 0;
@@ -347,9 +385,8 @@ struct mh_boundary {
     dbuf<float4> fchunk_cf;              // fine chunk centres as float-float (x_hi, x_lo, y_hi, y_lo)
     dbuf<float> fchunk_r;                // fine chunk radii
     dbuf<float> w32, wf32, x32;          // per call: weights, fine weights, GEMV input
-    dbuf<double> sc64, wf64;             // per call: density Fourier coefficients, fine weights
-    dbuf<double2> ptab;                  // binary64 pair table (pair64.cuh) for ptab_alpha
-    double ptab_alpha = -1.0;
+    fine_ws fine;                        // per step: the density on the 16x grid
+    pair_tab_buf ptab;                   // of the auxiliary sums of a step
     // matrix-free operator: the trapezoid sum by the on-surface multipole pass of a tree that
     // holds every node, the Alpert correction by binary64 chirp transforms per curve
     bool mfree = false;
@@ -361,14 +398,12 @@ struct mh_boundary {
     dbuf<int64_t> mf_moff;               // per curve: offset of its M_k-entry blocks (twiddles at moff/2)
     dbuf<int32_t> mf_M;                  // per curve: transform length M_k (power of two >= 2 N_k - 1)
     int mf_mmax = 0;
-    std::unique_ptr<dlp_targets> eval;   // buffers of mh_double_layer_apply's last target set
     dbuf<double2> mf_spec;               // per call: spectra c_m, m <= N_k/2
     dbuf<double> mf_S;                   // per call: [2 l][n] interpolated density at the Alpert nodes
     dbuf<double> mf_u;                   // per call: multipole-pass output
     SideStream mf_side;                  // the Alpert transforms run there beside the multipole pass
     dbuf<double> warm_dir, warm_w, warm_scal;   // warm-start direction, its image, scalars
     dbuf<float2> fcp32;                  // fine-grid coefficients by sub-offset (binary32)
-    dbuf<double2> fcp64;                 // (binary64)
 };
 
 #define MH_TILE 128
@@ -453,11 +488,9 @@ mh_status bie_apply64_gated(mh_ctx* ctx, mh_boundary* b, const double* x, double
 const double* gmres_final_residual(mh_boundary* b);
 // Everything a sync-free solve in precision prec needs (binary32 operator copy).
 mh_status bie_prepare(mh_ctx* ctx, mh_boundary* b, mh_precision prec);
-// all_groups: the upsampled rule will run at every pair (dlp_evaluate), not at the auxiliary ones only.
+// all_groups: the upsampled rule will run at every pair (mh_double_layer_apply), not at the auxiliary ones only.
 mh_status dlp_classify(mh_ctx* ctx, mh_boundary* b, const double* xy_dev, int64_t n, dlp_targets* tg,
                        bool all_groups = false);
-mh_status dlp_evaluate(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* tg,
-                       const double* sigma, double* out, mh_precision prec);
 // Sums at the auxiliary points of the normal-line rule into tg->ext (they need sigma and its fine
 // weights only, so they may run beside the pass that evaluates the other targets).
 mh_status dlp_aux_sums(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* tg, const double* sigma,
@@ -466,9 +499,9 @@ mh_status dlp_aux_sums(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* t
 // with A sigma = rhs - r.
 mh_status dlp_line_finish(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_targets* tg, const double* rhs,
                           const double* r, const double* base, const int32_t* idx, double* out);
-// Density on the 16x fine grid times |y'| h_f (binary64 in b->wf64; binary32 also in b->wf32
+// Density on the 16x fine grid times |y'| h_f (binary64 in ws.wf; binary32 also in b->wf32
 // when prec is mixed); spectrum64: mixed weights rounded from a binary64 spectrum, not a binary32 one.
-mh_status dlp_fine_weights(mh_ctx* ctx, mh_boundary* b, const double* sigma, mh_precision prec,
+mh_status dlp_fine_weights(mh_ctx* ctx, mh_boundary* b, const double* sigma, mh_precision prec, fine_ws& ws,
                            bool spectrum64 = false);
 // r0 (nullable): the binary64 residual rhs - A x of the initial guess, computed by the caller.
 mh_status gmres_run(mh_ctx* ctx, mh_boundary* b, const double* rhs, double* x, double tol, int max_iter,

@@ -396,7 +396,7 @@ static mh_status step_solve(mh_ctx* ctx, ProblemImpl* P, const double* f_next_de
     }
     if (s != MH_OK) return s;
     // U^h: trapezoid sum by the multipole method at every node, then the near-boundary rules
-    MH_TRY(dlp_fine_weights(ctx, b, sigma_dev, prec));
+    MH_TRY(dlp_fine_weights(ctx, b, sigma_dev, prec, b->fine));
     // the sums at the auxiliary points of the normal-line rule need only sigma and the fine
     // weights: without region timers they run on a second stream beside the multipole pass
     const bool aux_fork = !ctx->profiling && P->aux.s && P->tg.n_ext > P->tg.n;
@@ -409,7 +409,7 @@ static mh_status step_solve(mh_ctx* ctx, ProblemImpl* P, const double* f_next_de
     MH_TRY(sa);
     if (aux_fork) MH_TRY(P->aux.end(ctx));
     const double* du = nullptr;
-    MH_TRY(volume_dipole_apply(ctx, t, b->wf64.p, P->perm.p, prec, &du));
+    MH_TRY(volume_dipole_apply(ctx, t, b->fine.wf.p, P->perm.p, prec, &du));
     if (aux_fork) MH_CUDA(ctx, cudaStreamWaitEvent(st, P->aux.join, 0));
     k_combine<<<mh_grid(n, 256), 256, 0, st>>>(P->Up.p, du, P->region.p, P->d_ext_const.p, P->ext_mode, n, u_next_dev);
     MH_LAUNCHED(ctx);
