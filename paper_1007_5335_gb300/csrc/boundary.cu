@@ -2580,8 +2580,8 @@ static mh_status wait_progress(mh_ctx* ctx, const int* counter, int value) {
 // what the host has seen, and a step queued past the end of the process returns at once.  The
 // host follows through pinned memory instead of a copy and a synchronisation per look (~10 us of
 // idle GPU each: a solve at 6144 nodes of 13 steps in two sweeps took 705 us with those looks).
-mh_status gmres_run(mh_ctx* ctx, mh_boundary* bd, const double* b, double* x, double tol, int max_iter,
-                    mh_precision prec, mh_gmres_info* info, const double* r0) {
+static mh_status gmres_interactive(mh_ctx* ctx, mh_boundary* bd, const double* b, double* x, double tol, int max_iter,
+                                   mh_precision prec, mh_gmres_info* info, const double* r0) {
     prof_scope ps_all(ctx, "gmres");
     const int64_t n = bd->n;
     if (max_iter < 1 || max_iter > 1000) return mh_fail(ctx, MH_ERR_INVALID_ARG, "max_iter must be in 1..1000");
@@ -2596,9 +2596,11 @@ mh_status gmres_run(mh_ctx* ctx, mh_boundary* bd, const double* b, double* x, do
     const bool split = !bd->mfree && resid_ff(bd, mixed);
     gmres_dev* gs = ws.gs.p;
     gmres_k::progress* P = static_cast<gmres_k::progress*>(ws.prog);
-    // the counters run on from solve to solve (an earlier solve has nothing left that writes them)
-    const int steps0 = P->steps >> 1;
-    int begins = P->begins;
+    // an earlier solve has nothing left that writes the counters: its last word was its final sweep start
+    // (gmres_run waits for the stream where a solve ends in any other way)
+    __atomic_store_n(&P->steps, 0, __ATOMIC_RELEASE);
+    __atomic_store_n(&P->begins, 0, __ATOMIC_RELEASE);
+    int begins = 0;
     mh_gmres_info inf{0, 0, 0.0, 0, 0.0};
     // binary64: one sweep to the tolerance, then the true residual.  Mixed: sweeps of the
     // binary32-operator process inside binary64 iterative refinement.
@@ -2613,9 +2615,8 @@ mh_status gmres_run(mh_ctx* ctx, mh_boundary* bd, const double* b, double* x, do
         a.final_check = sweep >= (mixed ? 12 : 1) || inf.iterations >= max_iter;
         a.prog = P;
         a.seq = ++begins;
-        a.total0 = steps0;
         MH_TRY(sweep_begin(ctx, ws, a));
-        const int left = max_iter - inf.iterations, base = steps0 + inf.iterations;
+        const int left = max_iter - inf.iterations, base = inf.iterations;
         int queued = 0, seen = 0, seen_prev = 0;
         double res_prev = 0.0;
         // steps queued beyond the last one seen: two for the dense operator (a step past the end costs
@@ -2669,10 +2670,8 @@ mh_status gmres_run(mh_ctx* ctx, mh_boundary* bd, const double* b, double* x, do
             if (P->bn != 0.0) inf.initial_rel_residual = P->rn / P->bn;
             first = false;
         }
-        if (!std::isfinite(P->rn) || (P->started && !std::isfinite(P->res))) {
-            MH_CUDA(ctx, cudaStreamSynchronize(st));
+        if (!std::isfinite(P->rn) || (P->started && !std::isfinite(P->res)))
             return mh_fail(ctx, MH_ERR_NUMERIC, "GMRES residual is not finite");
-        }
         if (!P->started) {
             if (!P->done && supplied && P->rn <= tol * P->bn) {   // the caller's residual is within the tolerance: compute it
                 supplied = false;
@@ -2693,6 +2692,14 @@ mh_status gmres_run(mh_ctx* ctx, mh_boundary* bd, const double* b, double* x, do
         return mh_fail(ctx, MH_ERR_NOT_CONVERGED, "GMRES stopped after %d iterations at relative residual %.3e",
                        inf.iterations, inf.rel_residual);
     return MH_OK;
+}
+
+mh_status gmres_run(mh_ctx* ctx, mh_boundary* bd, const double* b, double* x, double tol, int max_iter,
+                    mh_precision prec, mh_gmres_info* info, const double* r0) {
+    const mh_status s = gmres_interactive(ctx, bd, b, x, tol, max_iter, prec, info, r0);
+    // a solve that broke off may have steps in flight that still write the counters
+    if (s != MH_OK && s != MH_ERR_NOT_CONVERGED) (void)cudaStreamSynchronize(ctx->stream);
+    return s;
 }
 
 // ---------------- sync-free GMRES (fixed schedule, device flags) ----------------

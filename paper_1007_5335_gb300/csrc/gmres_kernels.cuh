@@ -48,12 +48,13 @@ __device__ __forceinline__ double tree_sum(double v, int m) {
 __host__ __device__ inline int64_t gm_rows(int64_t n, int blocks) { return ((n + blocks - 1) / blocks + 31) / 32 * 32; }
 
 // What the interactive solver sees of a solve in progress: pinned host memory that the kernels
-// write (fields first, then the counter they are published by) and the host polls.
+// write (fields first, then the counter they are published by) and the host polls.  Both counters start
+// at 0 in every solve, so they stay as small as max_iter however long the boundary lives.
 struct progress {
     double rn, bn, res;     // ||r||, ||b|| of the last sweep start; residual estimate of the last step
-    int begins;             // sweep starts so far ...
+    int begins;             // sweep starts of this solve so far ...
     int started, done;      // ... and what the last one decided
-    int steps;              // 2 x Arnoldi steps so far (all sweeps and solves) + 1 if the last one ended its process
+    int steps;              // 2 x Arnoldi steps of this solve so far (all sweeps) + 1 if the last one ended its process
 };
 
 // Start of a sweep: r = b - ax (ax given) or r = r0 (r0 given, may alias r), its norm rn and, in
@@ -75,7 +76,7 @@ struct begin_args {
     int mixed, may_accept, final_check, recheck, first, loop_set;
     cudaGraphConditionalHandle loop;
     progress* prog;
-    int seq, total0;   // (prog) the start's number, steps counted before this solve
+    int seq;   // (prog) the start's number
 };
 
 __global__ void __launch_bounds__(GM_T) k_sweep_begin(begin_args a) {
@@ -120,8 +121,7 @@ __global__ void __launch_bounds__(GM_T) k_sweep_begin(begin_args a) {
     const bool lead = rank == 0 && threadIdx.x == 0;
     bool start = rn > 0.0, conv = false;
     if (lead && a.first) {
-        a.gs->done = a.gs->converged = a.gs->sweeps = a.gs->k = 0;
-        a.gs->total = a.total0;
+        a.gs->done = a.gs->converged = a.gs->sweeps = a.gs->k = a.gs->total = 0;
     }
     if (bn == 0.0) {
         for (int64_t e = e0 + threadIdx.x; e < e1; e += GM_T) a.x[e] = a.r[e] = 0.0;   // b = 0: x = 0, residual 0
