@@ -1185,14 +1185,17 @@ __global__ void k_scale_into(const double* __restrict__ r, const double* __restr
 // ---------------- classification of off-surface targets ----------------
 
 // Binary32 copy of the nodes for the classification: position relative to the origin (the mean node)
-// and normal times |y'| h.
+// and normal times |y'| h, both in units of 1/scale (the power of two at the nodes' extent, so that squares
+// neither overflow nor vanish in binary32 whatever the size of the domain).
 __global__ void k_cls32(const double* __restrict__ geo, const int32_t* __restrict__ curve_of,
-                        const int32_t* __restrict__ nn, int64_t n, double ox, double oy, float4* __restrict__ out) {
+                        const int32_t* __restrict__ nn, int64_t n, double ox, double oy, double scale,
+                        float4* __restrict__ out) {
     const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (j >= n) return;
     const double* g = geo + 8 * j;
-    const double h = 2.0 * MH_PI / nn[curve_of[j]];
-    out[j] = make_float4((float)(g[0] - ox), (float)(g[1] - oy), (float)(g[3] * h), (float)(-g[2] * h));
+    const double h = 2.0 * MH_PI / nn[curve_of[j]] * scale;
+    out[j] = make_float4((float)((g[0] - ox) * scale), (float)((g[1] - oy) * scale), (float)(g[3] * h),
+                         (float)(-g[2] * h));
 }
 
 // One warp per target.  For every curve: nearest node (smallest index on ties); if it is
@@ -1202,12 +1205,14 @@ __global__ void k_cls32(const double* __restrict__ geo, const int32_t* __restric
 // The scans over all nodes run in binary32 (the binary64 pipe has 1/64 of that rate): one finds
 // the smallest distance, a second one re-measures in binary64 every node whose binary32 distance
 // is within its rounding of it, so the nearest node is the binary64 one; the double layer, near
-// 0 or +-1 at these distances, is formed in binary64 only when it is not near either.  Newton's
+// 0 or +-1 at these distances, is formed in binary64 only when it is not near either, or when the target is
+// so near the curve (a very small one) that the binary32 positions do not resolve it: with positions off by
+// up to slack the sum is off by about slack / distance.  Newton's
 // iteration stops with a step below 1e-9 that is also 1000 times smaller than the one before
 // (quadratic convergence: the next one is below the rounding of t).  2000 targets, 6 x 1024 nodes: 1303 us with binary64 scans and 30
 // steps of a sincos per mode.
 __global__ void k_classify(const double* __restrict__ pts, int64_t npts, const double* __restrict__ geo,
-                           const float4* __restrict__ geo32, double ox, double oy, float extent,
+                           const float4* __restrict__ geo32, double ox, double oy, double scale, float extent,
                            const double* __restrict__ coef, const int32_t* __restrict__ nn,
                            const int32_t* __restrict__ off, int ncurves, int32_t* region, uint32_t* fine,
                            int32_t* line_curve, double* line_data) {
@@ -1215,7 +1220,9 @@ __global__ void k_classify(const double* __restrict__ pts, int64_t npts, const d
     const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     if (t >= npts) return;
     const double px = pts[2 * t], py = pts[2 * t + 1];
-    const float fx = (float)(px - ox), fy = (float)(py - oy);
+    // targets beyond 1e15 extents keep their direction only: every node is measured again in binary64
+    const float fx = fmaxf(-1e15f, fminf((float)((px - ox) * scale), 1e15f));
+    const float fy = fmaxf(-1e15f, fminf((float)((py - oy) * scale), 1e15f));
     // rounding of a binary32 distance: coordinates, their differences, the square root
     const float slack = 1e-6f * fmaxf(extent, fmaxf(fabsf(fx), fabsf(fy)));
     int reg = -1;
@@ -1305,7 +1312,7 @@ __global__ void k_classify(const double* __restrict__ pts, int64_t npts, const d
         } else {
             double acc = wind;
             const float a = fabsf(wind);
-            if (!(a < 0.1f || fabsf(a - 1.f) < 0.1f)) {
+            if (!(a < 0.1f || fabsf(a - 1.f) < 0.1f) || d2min < 4096.f * slack * slack) {
                 acc = 0.0;
                 for (int i = lane; i < N; i += 32) {
                     const double* g = geo + 8 * (int64_t)(o + i);
@@ -2103,11 +2110,14 @@ extern "C" mh_status mh_boundary_create(mh_ctx* ctx, int n_curves, const int32_t
             }
         b->cls_ox = sum[0] / tot;
         b->cls_oy = sum[1] / tot;
-        b->cls_extent = (float)std::max(hi[0] - lo[0], hi[1] - lo[1]);
+        const double extent = std::max(hi[0] - lo[0], hi[1] - lo[1]);
+        if (extent > 0.0 && std::isfinite(extent))
+            b->cls_scale = std::ldexp(1.0, -std::max(-1000, std::min(std::ilogb(extent), 1000)));
+        b->cls_extent = (float)(extent * b->cls_scale);
     }
     BCHK(b->geo32.alloc(tot));
     k_cls32<<<mh_grid(tot, 128), 128, 0, st>>>(b->geo.p, b->d_curve_of.p, b->d_nn.p, tot, b->cls_ox, b->cls_oy,
-                                               b->geo32.p);
+                                               b->cls_scale, b->geo32.p);
     ctx->launches++;
     BCHK(b->tw.alloc(tot));
     BCHK(b->half.alloc(tot));
@@ -2882,7 +2892,7 @@ mh_status dlp_classify(mh_ctx* ctx, mh_boundary* b, const double* xy_dev, int64_
     MH_RESERVE(ctx, ldata, 4 * n);
     if (n > 0) {
         k_classify<<<mh_grid(n * 32, 256), 256, 0, st>>>(xy_dev, n, b->geo.p, b->geo32.p, b->cls_ox, b->cls_oy,
-                                                         b->cls_extent, b->coef.p, b->d_nn.p, b->d_off.p, b->n_curves,
+                                                         b->cls_scale, b->cls_extent, b->coef.p, b->d_nn.p, b->d_off.p, b->n_curves,
                                                          tg->region.p, fine0.p, lcurve.p, ldata.p);
         MH_LAUNCHED(ctx);
     }

@@ -360,9 +360,10 @@ struct mh_boundary {
     dbuf<int32_t> d_curve_of;            // curve index of every node
     dbuf<double> xy;                     // [n][2]
     dbuf<double> geo;                    // [n][8]: x y x' y' x'' y'' |y'| kdiag
-    dbuf<float4> geo32;                  // binary32 nodes for the classification: x, y from the origin, normal |y'| h
-    double cls_ox = 0, cls_oy = 0;       // the origin (mean node)
-    float cls_extent = 0;                // largest side of the nodes' bounding box
+    dbuf<float4> geo32;                  // binary32 nodes for the classification (k_cls32)
+    double cls_ox = 0, cls_oy = 0;       // their origin (mean node)
+    double cls_scale = 1.0;              // and scale: a power of two that takes the extent to [1, 2)
+    float cls_extent = 0;                // largest side of the nodes' bounding box, scaled
     dbuf<double> coef;                   // per curve Fourier coefficients: [off*2 ...] see boundary.cu
     dbuf<double2> tw, half;              // per node (cos, sin)(2 pi r / N) and (cos, sin)(pi r / N)
     // fine (16x) grid per curve: positions, normals, speed*h_fine
