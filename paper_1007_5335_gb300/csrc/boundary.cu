@@ -2394,12 +2394,12 @@ static mh_status gemv_cpa_prepare(mh_ctx* ctx) {
     return MH_OK;
 }
 
-static void gemv64(cudaStream_t st, const double* A, const double* x, double* y, int64_t n, const int* gate) {
+static void gemv64(cudaStream_t st, const double* A, const double* x, double* y, int64_t n, const int* gate, bool dep) {
     if ((n & 1) == 0)
-        (void)mh_launch_dep(st, k_gemv64s<GEMV_SPLIT>, dim3((unsigned)((n + 8 / GEMV_SPLIT - 1) / (8 / GEMV_SPLIT))),
-                            dim3(256), 0, A, x, y, n, gate);
+        (void)mh_launch(st, dep, k_gemv64s<GEMV_SPLIT>, dim3((unsigned)((n + 8 / GEMV_SPLIT - 1) / (8 / GEMV_SPLIT))),
+                        dim3(256), 0, A, x, y, n, gate);
     else
-        (void)mh_launch_dep(st, k_gemv64, dim3(gemv_blocks(n)), dim3(256), 0, A, x, y, n, gate);
+        (void)mh_launch(st, dep, k_gemv64, dim3(gemv_blocks(n)), dim3(256), 0, A, x, y, n, gate);
 }
 
 // Product with the binary64 operator for a residual: in mixed precision a float-float product
@@ -2409,21 +2409,22 @@ static void gemv64(cudaStream_t st, const double* A, const double* x, double* y,
 // the two are separate so that a timed region can hold the GEMV alone.
 static bool resid_ff(const mh_boundary* b, bool mixed) { return mixed && (b->op.A16lo.p || b->op.A32lo.p); }
 
-static void resid_split(cudaStream_t st, mh_boundary* b, const double* x) {
-    (void)mh_launch_dep(st, k_split_vec, dim3(mh_grid(b->n, 256)), dim3(256), 0, x, b->xhi32.p, b->xlo32.p, b->n);
+static void resid_split(cudaStream_t st, mh_boundary* b, const double* x, bool dep) {
+    (void)mh_launch(st, dep, k_split_vec, dim3(mh_grid(b->n, 256)), dim3(256), 0, x, b->xhi32.p, b->xlo32.p, b->n);
 }
 
-static void resid_gemv(cudaStream_t st, mh_boundary* b, const double* x, double* y, const int* gate, bool mixed) {
+static void resid_gemv(cudaStream_t st, mh_boundary* b, const double* x, double* y, const int* gate, bool mixed,
+                       bool dep) {
     const int64_t n = b->n;
     const unsigned grid = (unsigned)((n + 8 / GEMV_SPLIT - 1) / (8 / GEMV_SPLIT));
     if (mixed && b->op.A16lo.p)
-        (void)mh_launch_dep(st, k_gemv_cph<GEMV_SPLIT>, dim3(grid), dim3(256), GH_SMEM, b->op.A32.p, b->op.A16lo.p,
-                            b->xhi32.p, b->xlo32.p, y, n, gate);
+        (void)mh_launch(st, dep, k_gemv_cph<GEMV_SPLIT>, dim3(grid), dim3(256), GH_SMEM, b->op.A32.p, b->op.A16lo.p,
+                        b->xhi32.p, b->xlo32.p, y, n, gate);
     else if (mixed && b->op.A32lo.p)
-        (void)mh_launch_dep(st, k_gemv_cpa<GEMV_SPLIT, 2>, dim3(grid), dim3(256), GC_SMEM2, b->op.A32.p, b->op.A32lo.p,
-                            b->xhi32.p, b->xlo32.p, y, n, gate);
+        (void)mh_launch(st, dep, k_gemv_cpa<GEMV_SPLIT, 2>, dim3(grid), dim3(256), GC_SMEM2, b->op.A32.p, b->op.A32lo.p,
+                        b->xhi32.p, b->xlo32.p, y, n, gate);
     else
-        gemv64(st, b->op.A64.p, x, y, n, gate);
+        gemv64(st, b->op.A64.p, x, y, n, gate, dep);
 }
 
 static const char* resid_region(mh_boundary* b, bool mixed, const int* gate) {
@@ -2438,18 +2439,19 @@ static double resid_bytes(mh_boundary* b, bool mixed) {
 }
 
 mh_status bie_apply64_gated(mh_ctx* ctx, mh_boundary* b, const double* x, double* y, const int* gate,
-                            mh_precision prec, bool x_split) {
+                            mh_precision prec, bool x_split, bool dep) {
     // the gate only skips work whose result the caller then ignores: the matrix-free form
     // always computes
     if (b->mfree) return bie_apply_mfree(ctx, b, x, y);
     MH_TRY(need_dense(ctx, b));
     const bool mixed = prec == MH_PREC_MIXED;
     if (resid_ff(b, mixed) && !x_split) {   // the split of x is not part of the timed GEMV region
-        resid_split(ctx->stream, b, x);
+        resid_split(ctx->stream, b, x, dep);
         MH_LAUNCHED(ctx);
+        dep = true;
     }
     prof_scope ps(ctx, resid_region(b, mixed, gate), 2.0 * b->n * b->n, resid_bytes(b, mixed));
-    resid_gemv(ctx->stream, b, x, y, gate, mixed);
+    resid_gemv(ctx->stream, b, x, y, gate, mixed, dep);
     MH_LAUNCHED(ctx);
     return MH_OK;
 }
@@ -2469,7 +2471,7 @@ mh_status bie_apply(mh_ctx* ctx, mh_boundary* b, const double* x, double* y, mh_
         gemv32(ctx->stream, b->op.A32.p, b->x32.p, y, b->n, nullptr);
     } else {
         prof_scope ps(ctx, "bie_gemv64", 2.0 * b->n * b->n, 8.0 * b->n * b->n + 16.0 * b->n);
-        gemv64(ctx->stream, b->op.A64.p, x, y, b->n, nullptr);
+        gemv64(ctx->stream, b->op.A64.p, x, y, b->n, nullptr, false);   // an entry point's first kernel
     }
     MH_LAUNCHED(ctx);
     return MH_OK;
@@ -2618,7 +2620,7 @@ static mh_status gmres_interactive(mh_ctx* ctx, mh_boundary* bd, const double* b
     for (int sweep = 0;;) {
         // binary64 residual of x; at the first sweep the caller's r0 (if given) stands in
         // for it, but convergence is only ever accepted on a residual computed here
-        if (!supplied) MH_TRY(bie_apply64_gated(ctx, bd, x, ws.w.p, nullptr, prec, split && sweep > 0));
+        if (!supplied) MH_TRY(bie_apply64_gated(ctx, bd, x, ws.w.p, nullptr, prec, split && sweep > 0, !first));
         gmres_k::begin_args a = begin_of(ws, b, supplied ? r0 : nullptr, x, n, max_iter + 2, mixed, tol, gs);
         a.first = first;
         a.recheck = supplied;
@@ -2655,7 +2657,7 @@ static mh_status gmres_interactive(mh_ctx* ctx, mh_boundary* bd, const double* b
                     if (mixed)
                         gemv32(st, bd->op.A32.p, ws.v32.p, ws.w.p, n, &gs->skip);
                     else
-                        gemv64(st, bd->op.A64.p, vk, ws.w.p, n, &gs->skip);
+                        gemv64(st, bd->op.A64.p, vk, ws.w.p, n, &gs->skip, true);
                     MH_LAUNCHED(ctx);
                 }
                 ++queued;
@@ -2829,10 +2831,10 @@ mh_status gmres_run_graph(mh_ctx* ctx, mh_boundary* bd, const double* b, double*
         const bool supplied = sw == 0 && r0;
         if (!supplied) {
             if (split && sw == 0) {
-                resid_split(st, bd, x);
+                resid_split(st, bd, x, true);
                 MH_LAUNCHED(ctx);
             }
-            resid_gemv(st, bd, x, ws.w.p, &gs->done, mixed);
+            resid_gemv(st, bd, x, ws.w.p, &gs->done, mixed, true);
             MH_LAUNCHED(ctx);
         }
         // while the stream is being captured (a batch graph), the Arnoldi process of a sweep is a
@@ -2859,7 +2861,7 @@ mh_status gmres_run_graph(mh_ctx* ctx, mh_boundary* bd, const double* b, double*
                 if (mixed)
                     gemv32(st, bd->op.A32.p, ws.v32.p, ws.w.p, n, &gs->skip);
                 else
-                    gemv64(st, bd->op.A64.p, ws.V.p + (int64_t)k * n, ws.w.p, n, &gs->skip);
+                    gemv64(st, bd->op.A64.p, ws.V.p + (int64_t)k * n, ws.w.p, n, &gs->skip, true);
                 MH_LAUNCHED(ctx);
                 MH_TRY(arnoldi_step(ctx, ws, n, k + 1, m + 1, mixed, gs, m));
             }

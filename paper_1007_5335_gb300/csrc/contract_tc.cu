@@ -727,10 +727,10 @@ mh_status tc_split_launch(mh_ctx* ctx, const float* src, int len, int64_t count,
 }
 
 mh_status tc_split_values(mh_ctx* ctx, const double* src, int len, int64_t count, int S, float* dst32, uint16_t* planes,
-                          int64_t plane, int64_t dst) {
+                          int64_t plane, int64_t dst, bool dep) {
     if (count <= 0) return MH_OK;
-    (void)mh_launch_dep(ctx->stream, k_split_values, dim3(mh_grid(count * S, 256)), dim3(256), 0, src, len, count, S, dst32,
-                        planes, plane, dst);
+    (void)mh_launch(ctx->stream, dep, k_split_values, dim3(mh_grid(count * S, 256)), dim3(256), 0, src, len, count, S, dst32,
+                    planes, plane, dst);
     MH_LAUNCHED(ctx);
     return MH_OK;
 }

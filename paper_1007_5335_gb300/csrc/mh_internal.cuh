@@ -125,7 +125,9 @@ inline size_t mh_bytes(const B&... b) {
 // and before any return, so it touches memory only when everything before it on the stream has
 // completed, and completes only after its predecessors; mh_launch_dep is used behind a kernel of
 // the same stream (a launch behind an event wait, a copy or a graph's conditional node is an ordinary
-// one).  Kernels that are launched either way call mh_dep_wait() too (no effect in an ordinary
+// one).  The first kernel of an entry point is an ordinary launch as well: the caller's last kernel need
+// not keep these rules (one that starts its dependents early and does not wait may end before its own
+// predecessors).  Kernels that are launched either way call mh_dep_wait() too (no effect in an ordinary
 // launch).  The wait comes before the trigger: at most one kernel waits behind the running one.
 __device__ __forceinline__ void mh_dep_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -133,7 +135,7 @@ __device__ __forceinline__ void mh_dep_wait() {
 }
 
 template <class... K, class... A>
-inline cudaError_t mh_launch_dep(cudaStream_t st, void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, A... args) {
+inline cudaError_t mh_launch(cudaStream_t st, bool dep, void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, A... args) {
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
@@ -143,8 +145,13 @@ inline cudaError_t mh_launch_dep(cudaStream_t st, void (*kernel)(K...), dim3 gri
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = dep ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<K>(args)...);
+}
+
+template <class... K, class... A>
+inline cudaError_t mh_launch_dep(cudaStream_t st, void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, A... args) {
+    return mh_launch(st, true, kernel, grid, block, smem, args...);
 }
 
 // ---- L2 residency hints ----
@@ -238,7 +245,7 @@ mh_status tc_split_launch(mh_ctx* ctx, const float* src, int len, int64_t count,
                           int64_t dst);
 // The same from binary64 vectors at src, which are also written to dst32 in binary32.
 mh_status tc_split_values(mh_ctx* ctx, const double* src, int len, int64_t count, int S, float* dst32, uint16_t* planes,
-                          int64_t plane, int64_t dst);
+                          int64_t plane, int64_t dst, bool dep);
 
 // Device-resident state of the sync-free GMRES (gmres_run_graph): every kernel of its fixed
 // schedule reads the flags at entry and returns at once when its work is not needed.
@@ -482,9 +489,10 @@ mh_status bie_apply(mh_ctx* ctx, mh_boundary* b, const double* x, double* y, mh_
 mh_status bie_mfree_setup(mh_ctx* ctx, mh_boundary* b, mh_tree* t, double alpha);
 mh_status bie_apply_mfree(mh_ctx* ctx, mh_boundary* b, const double* x, double* y);
 // y = A x in binary64, skipped when *gate != 0 (gate nullable).
-// Mixed precision: accurate to binary64 for residuals (float-float); x_split: b->xhi32, xlo32 hold x.
+// Mixed precision: accurate to binary64 for residuals (float-float); x_split: b->xhi32, xlo32 hold x;
+// dep: directly behind a kernel of the library (mh_launch_dep).
 mh_status bie_apply64_gated(mh_ctx* ctx, mh_boundary* b, const double* x, double* y, const int* gate,
-                            mh_precision prec, bool x_split = false);
+                            mh_precision prec, bool x_split = false, bool dep = true);
 // Where the last solve left the binary64 residual rhs - A x of its result.
 const double* gmres_final_residual(mh_boundary* b);
 // Everything a sync-free solve in precision prec needs (binary32 operator copy).
@@ -522,8 +530,9 @@ void mh_gauss_legendre(int n, double* x, double* w);
 const double* tree_gl_nodes(const mh_tree* t);
 
 // ---- volume.cu ----
+// dep: directly behind a kernel of the library.
 mh_status volume_apply(mh_ctx* ctx, mh_tree* t, double alpha, int p, const double* b, double* up,
-                       mh_precision prec);
+                       mh_precision prec, bool dep);
 void volume_free(mh_tree* t);
 // Threads per block of the binary32 near-field double-layer kernel (128, 256 or 512).
 mh_status volume_set_near_tile(mh_ctx* ctx, mh_tree* t, int threads);

@@ -213,18 +213,18 @@ __global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, const T* __re
 }
 
 // part, cnt (nullable): workspace of a split product (GEMM_PARTS tiles); k is split while the
-// tiles leave SMs without a block, down to two slabs a block.
+// tiles leave SMs without a block, down to two slabs a block.  dep: directly behind a kernel of the library.
 template <typename T, int EPI>
 void gemm(cudaStream_t st, int M, int N, int K, const T* A, int64_t sam, int64_t sak, const T* B, int64_t sbk,
           int64_t sbn, T* C, int64_t ldc, const T* bias = nullptr, const T* aux = nullptr, T* part = nullptr,
-          unsigned* cnt = nullptr) {
+          unsigned* cnt = nullptr, bool dep = true) {
     dim3 grid((unsigned)((N + GEMM_T - 1) / GEMM_T), (unsigned)((M + GEMM_T - 1) / GEMM_T));
     const int64_t tiles = (int64_t)grid.x * grid.y;
     const int slabs = (K + GEMM_K - 1) / GEMM_K;
     if (part && tiles <= GEMM_PARTS / 2)
         grid.z = (unsigned)std::max<int64_t>(1, std::min<int64_t>(GEMM_PARTS / tiles, slabs / 2));
-    (void)mh_launch_dep(st, k_gemm<T, EPI>, grid, dim3(256), 0, M, N, K, A, sam, sak, B, sbk, sbn, C, ldc, bias, aux,
-                        part, cnt);
+    (void)mh_launch(st, dep, k_gemm<T, EPI>, grid, dim3(256), 0, M, N, K, A, sam, sak, B, sbk, sbn, C, ldc, bias, aux,
+                    part, cnt);
 }
 
 __device__ __forceinline__ double warp_sum_d(double v) {
@@ -793,8 +793,8 @@ mh_status ensure_rows(mh_ctx* ctx, mh_net* net, int64_t rows) {
     return MH_OK;
 }
 
-// Training-kernel forward of `rows` inputs x; output in net->yh.
-mh_status train_forward(mh_ctx* ctx, mh_net* net, const float* x, int64_t rows) {
+// Training-kernel forward of `rows` inputs x; output in net->yh.  dep: directly behind a kernel of the library.
+mh_status train_forward(mh_ctx* ctx, mh_net* net, const float* x, int64_t rows, bool dep) {
     cudaStream_t st = ctx->stream;
     const float* P = net->P.p;
     const int w = net->w;
@@ -803,7 +803,8 @@ mh_status train_forward(mh_ctx* ctx, mh_net* net, const float* x, int64_t rows) 
     int64_t ld_in = d;
     for (int l = 0; l < 3; ++l) {
         gemm<float, EPI_BIAS_TANH>(st, (int)rows, w, net->lin[l], in, ld_in, 1, P + net->oW[l], 1, net->lin[l],
-                                   net->act[l].p, w, P + net->ob[l], (const float*)nullptr, net->gpart.p, net->gcnt.p);
+                                   net->act[l].p, w, P + net->ob[l], (const float*)nullptr, net->gpart.p, net->gcnt.p,
+                                   dep || l > 0);
         MH_LAUNCHED(ctx);
         in = net->act[l].p;
         ld_in = w;
@@ -1214,7 +1215,7 @@ extern "C" mh_status mh_net_loss_grad(mh_ctx* ctx, mh_net* net, const float* X_d
         MH_CUDA(ctx, cudaMemcpyAsync(net->xb.p, X_dev, n * net->d * 4, cudaMemcpyDeviceToDevice, st));
         x = net->xb.p;
     }
-    MH_TRY(train_forward(ctx, net, x, n));
+    MH_TRY(train_forward(ctx, net, x, n, false));
     MH_TRY(train_loss(ctx, net, T_dev, n, net->dzd.p, net->scal.p + 4));
     if (grad_dev) MH_TRY(train_backward(ctx, net, x, n, grad_dev));
     if (loss_host) {
@@ -1235,7 +1236,7 @@ extern "C" mh_status mh_net_forward(mh_ctx* ctx, mh_net* net, const float* X_dev
     if (training_kernels) {
         MH_TRY(ensure_rows(ctx, net, n));
         MH_CUDA(ctx, cudaMemcpyAsync(net->xb.p, X_dev, n * d * 4, cudaMemcpyDeviceToDevice, st));
-        MH_TRY(train_forward(ctx, net, net->xb.p, n));
+        MH_TRY(train_forward(ctx, net, net->xb.p, n, false));
         MH_CUDA(ctx, cudaMemcpyAsync(Y_dev, net->yh.p, n * d * 4, cudaMemcpyDeviceToDevice, st));
     } else {
         for (int64_t r = 0; r < n; ++r) MH_TRY(infer_one(ctx, net, arith, X_dev + r * d, Y_dev + r * d));
@@ -1270,7 +1271,7 @@ extern "C" mh_status mh_net_train(mh_ctx* ctx, mh_net* net, const float* X_dev, 
         MH_LAUNCHED(ctx);
         k_gather_rows<<<ew_grid(n_val * d), 256, 0, st>>>(Yv_dev, nullptr, n_val, d, sy, net->yb.p);
         MH_LAUNCHED(ctx);
-        MH_TRY(train_forward(ctx, net, net->xb.p, n_val));
+        MH_TRY(train_forward(ctx, net, net->xb.p, n_val, true));
         MH_TRY(train_loss(ctx, net, net->yb.p, n_val, nullptr, net->scal.p + 5));
         MH_CUDA(ctx, cudaMemcpyAsync(out, net->scal.p + 5, 8, cudaMemcpyDeviceToHost, st));
         MH_CUDA(ctx, cudaStreamSynchronize(st));
@@ -1289,7 +1290,7 @@ extern "C" mh_status mh_net_train(mh_ctx* ctx, mh_net* net, const float* X_dev, 
         MH_LAUNCHED(ctx);
         k_gather_rows<<<ew_grid((int64_t)batch * d), 256, 0, st>>>(Y_dev, idx, batch, d, sy, net->yb.p);
         MH_LAUNCHED(ctx);
-        MH_TRY(train_forward(ctx, net, net->xb.p, batch));
+        MH_TRY(train_forward(ctx, net, net->xb.p, batch, true));
         MH_TRY(train_loss(ctx, net, net->yb.p, batch, net->dzd.p, net->scal.p + 4));
         MH_TRY(train_backward(ctx, net, net->xb.p, batch, net->G.p));
         const float bc1 = (float)(1.0 - std::pow(0.9, t)), bc2 = (float)(1.0 - std::pow(0.999, t));
@@ -1338,7 +1339,7 @@ mh_status warm_start_run(mh_ctx* ctx, mh_boundary* b, double alpha, mh_net* net,
     }
     prof_scope ps(ctx, "warm_start");
     if (!r_ready) {
-        MH_TRY(bie_apply64_gated(ctx, b, sigma, r0, nullptr, prec));
+        MH_TRY(bie_apply64_gated(ctx, b, sigma, r0, nullptr, prec, false, false));
         k_resid<<<mh_grid(n, 256), 256, 0, st>>>(rhs, r0, n);
         MH_LAUNCHED(ctx);
     }

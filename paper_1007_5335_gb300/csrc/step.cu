@@ -237,7 +237,7 @@ extern "C" mh_status mh_problem_create(mh_ctx* ctx, mh_tree* tree, mh_boundary* 
     // operators: boundary (alpha) and volume (alpha, p) -- built once here
     MH_TRY(bie_assemble(ctx, bnd, P->alpha));
     MH_CUDA(ctx, cudaMemsetAsync(P->B.p, 0, n * 8, st));
-    MH_TRY(volume_apply(ctx, tree, P->alpha, p, P->B.p, P->Up.p, MH_PREC_FP64));
+    MH_TRY(volume_apply(ctx, tree, P->alpha, p, P->B.p, P->Up.p, MH_PREC_FP64, false));
     MH_CUDA(ctx, cudaStreamSynchronize(st));
     *out = P.release();
     return MH_OK;
@@ -347,7 +347,7 @@ static mh_status step_solve(mh_ctx* ctx, ProblemImpl* P, const double* f_next_de
     mh_tree* t = P->tree;
     mh_boundary* b = P->bnd;
     const int64_t n = t->n_nodes, ng = b->n;
-    MH_TRY(volume_apply(ctx, t, P->alpha, P->p, P->B.p, P->Up.p, prec));
+    MH_TRY(volume_apply(ctx, t, P->alpha, P->p, P->B.p, P->Up.p, prec, true));
     // rhs = -2 alpha^2 (f - U^p) on Gamma
     MH_TRY(tree_interpolate(ctx, t, P->Up.p, b->xy.p, P->bnd_leaf.p, ng, f_next_dev, -2.0 * P->alpha * P->alpha, P->rhs.p));
     mh_gmres_info gi{};

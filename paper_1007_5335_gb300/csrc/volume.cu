@@ -2876,7 +2876,7 @@ static mh_status volume_run(mh_ctx* ctx, mh_tree* t, VolData* V, double* up) {
 }
 
 mh_status volume_apply(mh_ctx* ctx, mh_tree* t, double alpha, int p, const double* b, double* up,
-                       mh_precision prec) {
+                       mh_precision prec, bool dep) {
     MH_TRY(volume_ensure(ctx, t, alpha, p));
     VolData* V = static_cast<VolData*>(t->vol);
     const int64_t nn = t->n_nodes;
@@ -2885,7 +2885,8 @@ mh_status volume_apply(mh_ctx* ctx, mh_tree* t, double alpha, int p, const doubl
         // node values in binary32 once: every contraction then gathers binary32
         if (V->tc.ready && ctx->tensor_cores && !V->tc.ranges.empty()) {
             const TcImages::Range& r = V->tc.ranges[0];
-            MH_TRY(tc_split_values(ctx, b, r.len, r.count, r.S, V->vec32.p + V->B_off, V->tc.planes.p, V->tc.plane, r.dst));
+            MH_TRY(tc_split_values(ctx, b, r.len, r.count, r.S, V->vec32.p + V->B_off, V->tc.planes.p, V->tc.plane, r.dst,
+                                   dep));
         } else {
             k_d2f<<<mh_grid(nn, 256), 256, 0, ctx->stream>>>(b, V->vec32.p + V->B_off, nn);
             MH_LAUNCHED(ctx);
@@ -2925,6 +2926,6 @@ extern "C" mh_status mh_volume_potential(mh_ctx* ctx, mh_tree* t, double alpha, 
     if (!ctx || !t || !b_dev || !up_dev) return mh_fail(ctx, MH_ERR_INVALID_ARG, "null argument");
     if (!(alpha > 0)) return mh_fail(ctx, MH_ERR_INVALID_ARG, "alpha must be positive");
     if (p < 1 || p > 40) return mh_fail(ctx, MH_ERR_INVALID_ARG, "p must be in 1..40");
-    MH_TRY(volume_apply(ctx, t, alpha, p, b_dev, up_dev, prec));
+    MH_TRY(volume_apply(ctx, t, alpha, p, b_dev, up_dev, prec, false));
     return mh_tree_check(ctx, t);
 }
