@@ -293,7 +293,7 @@ __global__ void k_split_lo16(const double* __restrict__ a, const float* __restri
 }
 
 // x = xh + xl with xh = x rounded to binary32
-__global__ void k_split_vec(const double* __restrict__ x, float* __restrict__ xh, float* __restrict__ xl, int64_t n) {
+__global__ void k_split_vec(const double* x, float* __restrict__ xh, float* __restrict__ xl, int64_t n) {
     mh_dep_wait();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i < n) {
@@ -304,8 +304,8 @@ __global__ void k_split_vec(const double* __restrict__ x, float* __restrict__ xh
 }
 
 // y = A x, one warp per row, 16-byte loads (N_Gamma is even, so rows stay aligned).
-__global__ void k_gemv64(const double* __restrict__ A, const double* __restrict__ x, double* __restrict__ y,
-                         int64_t n, const int* __restrict__ gate = nullptr) {
+__global__ void k_gemv64(const double* __restrict__ A, const double* x, double* __restrict__ y,
+                         int64_t n, const int* gate = nullptr) {
     mh_dep_wait();
     if (gate && *gate) return;
     const int lane = threadIdx.x & 31;
@@ -316,7 +316,7 @@ __global__ void k_gemv64(const double* __restrict__ A, const double* __restrict_
         double acc = 0.0;
         for (int64_t c = lane; c < n / 2; c += 32) {
             double2 av = __ldcs(a + c);
-            double2 xx = __ldg(xv + c);
+            double2 xx = xv[c];
             acc = fma(av.x, xx.x, acc);
             acc = fma(av.y, xx.y, acc);
         }
@@ -329,8 +329,8 @@ __global__ void k_gemv64(const double* __restrict__ A, const double* __restrict_
 // from binary64 run on the slow FP64 pipe of this part and must stay out of the loop).
 // One warp per row; four independent loads in flight per lane (16-byte loads when the
 // row length is a multiple of 4, 8-byte loads otherwise).
-__global__ void k_gemv32(const float* __restrict__ A, const float* __restrict__ x, double* __restrict__ y,
-                         int64_t n, const int* __restrict__ gate = nullptr) {
+__global__ void k_gemv32(const float* __restrict__ A, const float* x, double* __restrict__ y,
+                         int64_t n, const int* gate = nullptr) {
     mh_dep_wait();
     if (gate && *gate) return;
     const int lane = threadIdx.x & 31;
@@ -346,22 +346,21 @@ __global__ void k_gemv32(const float* __restrict__ A, const float* __restrict__ 
             for (; c + 96 < n4; c += 128) {
                 const float4 a0 = __ldcs(a4 + c), a1 = __ldcs(a4 + c + 32), a2 = __ldcs(a4 + c + 64),
                              a3 = __ldcs(a4 + c + 96);
-                const float4 x0 = __ldg(x4 + c), x1 = __ldg(x4 + c + 32), x2 = __ldg(x4 + c + 64),
-                             x3 = __ldg(x4 + c + 96);
+                const float4 x0 = x4[c], x1 = x4[c + 32], x2 = x4[c + 64], x3 = x4[c + 96];
                 f0 = fmaf(a0.x, x0.x, fmaf(a0.y, x0.y, fmaf(a0.z, x0.z, fmaf(a0.w, x0.w, f0))));
                 f1 = fmaf(a1.x, x1.x, fmaf(a1.y, x1.y, fmaf(a1.z, x1.z, fmaf(a1.w, x1.w, f1))));
                 f2 = fmaf(a2.x, x2.x, fmaf(a2.y, x2.y, fmaf(a2.z, x2.z, fmaf(a2.w, x2.w, f2))));
                 f3 = fmaf(a3.x, x3.x, fmaf(a3.y, x3.y, fmaf(a3.z, x3.z, fmaf(a3.w, x3.w, f3))));
             }
             for (; c < n4; c += 32) {
-                const float4 av = __ldcs(a4 + c), xv = __ldg(x4 + c);
+                const float4 av = __ldcs(a4 + c), xv = x4[c];
                 f0 = fmaf(av.x, xv.x, fmaf(av.y, xv.y, fmaf(av.z, xv.z, fmaf(av.w, xv.w, f0))));
             }
         } else {
             const float2* a2p = reinterpret_cast<const float2*>(a);
             const float2* x2p = reinterpret_cast<const float2*>(x);
             for (int64_t c = lane; c < n / 2; c += 32) {
-                const float2 av = __ldcs(a2p + c), xv = __ldg(x2p + c);
+                const float2 av = __ldcs(a2p + c), xv = x2p[c];
                 f0 = fmaf(av.x, xv.x, fmaf(av.y, xv.y, f0));
             }
         }
@@ -373,49 +372,56 @@ __global__ void k_gemv32(const float* __restrict__ A, const float* __restrict__ 
 }
 
 // Row-split GEMVs: SPLIT warps share a row (contiguous segments in 16-byte units, combined in
-// a fixed order through shared memory).  Blocks of 8 / SPLIT rows keep the hardware's dynamic
-// block scheduling fine-grained, so no SM is left with a whole extra block of rows at the end
-// of the sweep over the operator.  n must be a multiple of 4 (binary32) or 2 (binary64).
+// a fixed order through shared memory).  Turns of 8 / SPLIT rows keep the end of the sweep over the
+// operator even: a block a turn in binary64 and float-float, resident blocks that take turns in
+// binary32.  n must be a multiple of 4 (binary32) or 2 (binary64).
 template <int SPLIT>
-__global__ void __launch_bounds__(256) k_gemv32s(const float* __restrict__ A, const float* __restrict__ x,
-                                                 double* __restrict__ y, int64_t n, const int* __restrict__ gate) {
+__global__ void __launch_bounds__(256) k_gemv32s(const float* __restrict__ A, const float* x, double* __restrict__ y,
+                                                 int64_t n, const int* gate) {
     mh_dep_wait();
     if (gate && *gate) return;
     __shared__ float part[8];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t row = (int64_t)blockIdx.x * (8 / SPLIT) + warp / SPLIT;
     const int q = warp % SPLIT;
-    float f0 = 0.f, f1 = 0.f, f2 = 0.f, f3 = 0.f;
-    if (row < n) {
-        const uint64_t pol = mh_l2_policy((row + 1) * n * 4 <= MH_L2_KEEP);
-        const int64_t n4 = n >> 2;
-        const int64_t c0 = q * n4 / SPLIT, c1 = (q + 1) * n4 / SPLIT;
-        const float4* a4 = reinterpret_cast<const float4*>(A + row * n);
-        const float4* x4 = reinterpret_cast<const float4*>(x);
-        int64_t c = c0 + lane;
-        for (; c + 96 < c1; c += 128) {
-            const float4 a0 = mh_ld_hint(a4 + c, pol), a1 = mh_ld_hint(a4 + c + 32, pol),
-                         a2 = mh_ld_hint(a4 + c + 64, pol), a3 = mh_ld_hint(a4 + c + 96, pol);
-            const float4 x0 = __ldg(x4 + c), x1 = __ldg(x4 + c + 32), x2 = __ldg(x4 + c + 64), x3 = __ldg(x4 + c + 96);
-            f0 = fmaf(a0.x, x0.x, fmaf(a0.y, x0.y, fmaf(a0.z, x0.z, fmaf(a0.w, x0.w, f0))));
-            f1 = fmaf(a1.x, x1.x, fmaf(a1.y, x1.y, fmaf(a1.z, x1.z, fmaf(a1.w, x1.w, f1))));
-            f2 = fmaf(a2.x, x2.x, fmaf(a2.y, x2.y, fmaf(a2.z, x2.z, fmaf(a2.w, x2.w, f2))));
-            f3 = fmaf(a3.x, x3.x, fmaf(a3.y, x3.y, fmaf(a3.z, x3.z, fmaf(a3.w, x3.w, f3))));
+    const int64_t n4 = n >> 2;
+    const int c0 = (int)(q * n4 / SPLIT), c1 = (int)((q + 1) * n4 / SPLIT);
+    const float4* x4 = reinterpret_cast<const float4*>(x);
+    // A block's wait drops what L1 holds, so x is read from L2 again by every block: the resident blocks
+    // (6 an SM at 40 registers) take the rows in turn, and the operator does not go through L1.  Mixed solve at 6144
+    // nodes: 611 us with a block for every two rows, 599 so.
+    for (int64_t r0 = (int64_t)blockIdx.x * (8 / SPLIT); r0 < n; r0 += (int64_t)gridDim.x * (8 / SPLIT)) {
+        const int64_t row = r0 + warp / SPLIT;
+        float f0 = 0.f, f1 = 0.f, f2 = 0.f, f3 = 0.f;
+        if (row < n) {
+            const uint64_t pol = mh_l2_policy((row + 1) * n * 4 <= MH_L2_KEEP);
+            const float4* a4 = reinterpret_cast<const float4*>(A + row * n);
+            int c = c0 + lane;
+#pragma unroll 1
+            for (; c + 96 < c1; c += 128) {
+                const float4 a0 = mh_ld_hint(a4 + c, pol), a1 = mh_ld_hint(a4 + c + 32, pol),
+                             a2 = mh_ld_hint(a4 + c + 64, pol), a3 = mh_ld_hint(a4 + c + 96, pol);
+                const float4 x0 = x4[c], x1 = x4[c + 32], x2 = x4[c + 64], x3 = x4[c + 96];
+                f0 = fmaf(a0.x, x0.x, fmaf(a0.y, x0.y, fmaf(a0.z, x0.z, fmaf(a0.w, x0.w, f0))));
+                f1 = fmaf(a1.x, x1.x, fmaf(a1.y, x1.y, fmaf(a1.z, x1.z, fmaf(a1.w, x1.w, f1))));
+                f2 = fmaf(a2.x, x2.x, fmaf(a2.y, x2.y, fmaf(a2.z, x2.z, fmaf(a2.w, x2.w, f2))));
+                f3 = fmaf(a3.x, x3.x, fmaf(a3.y, x3.y, fmaf(a3.z, x3.z, fmaf(a3.w, x3.w, f3))));
+            }
+            for (; c < c1; c += 32) {
+                const float4 av = mh_ld_hint(a4 + c, pol), xv = x4[c];
+                f0 = fmaf(av.x, xv.x, fmaf(av.y, xv.y, fmaf(av.z, xv.z, fmaf(av.w, xv.w, f0))));
+            }
         }
-        for (; c < c1; c += 32) {
-            const float4 av = mh_ld_hint(a4 + c, pol), xv = __ldg(x4 + c);
-            f0 = fmaf(av.x, xv.x, fmaf(av.y, xv.y, fmaf(av.z, xv.z, fmaf(av.w, xv.w, f0))));
-        }
-    }
-    float f = (f0 + f1) + (f2 + f3);
+        float f = (f0 + f1) + (f2 + f3);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
-    if (lane == 0) part[warp] = f;
-    __syncthreads();
-    if (q == 0 && lane == 0 && row < n) {
-        float t = part[warp];
-        for (int k = 1; k < SPLIT; ++k) t += part[warp + k];
-        y[row] = (double)t;
+        for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+        if (lane == 0) part[warp] = f;
+        __syncthreads();
+        if (q == 0 && lane == 0 && row < n) {
+            float t = part[warp];
+            for (int k = 1; k < SPLIT; ++k) t += part[warp + k];
+            y[row] = (double)t;
+        }
+        __syncthreads();
     }
 }
 
@@ -454,8 +460,8 @@ __device__ __forceinline__ void cp_async_wait_all() {
 
 template <int SPLIT, int M>
 __global__ void __launch_bounds__(256) k_gemv_cpa(const float* __restrict__ A, const float* __restrict__ Al,
-                                                  const float* __restrict__ xh, const float* __restrict__ xl,
-                                                  double* __restrict__ y, int64_t n, const int* __restrict__ gate) {
+                                                  const float* xh, const float* xl,
+                                                  double* __restrict__ y, int64_t n, const int* gate) {
     mh_dep_wait();
     if (gate && *gate) return;
     extern __shared__ __align__(16) float4 gc_stage[];   // [warp][M][GC_PIECE * 32]
@@ -488,7 +494,7 @@ __global__ void __launch_bounds__(256) k_gemv_cpa(const float* __restrict__ A, c
                 const int64_t c = p0 + lane + 32 * u;
                 if (c < c1) {
                     const float4 av = st[lane + 32 * u];
-                    const float4 uv = __ldg(xh4 + c);
+                    const float4 uv = xh4[c];
                     if (M == 1) {
                         hi = fmaf(av.x, uv.x, hi);
                         hi = fmaf(av.y, uv.y, hi);
@@ -496,7 +502,7 @@ __global__ void __launch_bounds__(256) k_gemv_cpa(const float* __restrict__ A, c
                         hi = fmaf(av.w, uv.w, hi);
                     } else {
                         const float4 bv = st[GC_PIECE * 32 + lane + 32 * u];
-                        const float4 vv = __ldg(xl4 + c);
+                        const float4 vv = xl4[c];
                         ff_acc(hi, lo, av.x, bv.x, uv.x, vv.x);
                         ff_acc(hi, lo, av.y, bv.y, uv.y, vv.y);
                         ff_acc(hi, lo, av.z, bv.z, uv.z, vv.z);
@@ -546,8 +552,8 @@ constexpr int GH_PIECE = 2;   // 16-byte groups of binary16 per lane per piece: 
 
 template <int SPLIT>
 __global__ void __launch_bounds__(256, 4) k_gemv_cph(const float* __restrict__ A, const uint16_t* __restrict__ Ah,
-                                                  const float* __restrict__ xh, const float* __restrict__ xl,
-                                                  double* __restrict__ y, int64_t n, const int* __restrict__ gate) {
+                                                  const float* xh, const float* xl,
+                                                  double* __restrict__ y, int64_t n, const int* gate) {
     mh_dep_wait();
     if (gate && *gate) return;
     extern __shared__ __align__(16) float4 gc_stage[];   // [warp][3 GH_PIECE * 32]
@@ -585,8 +591,8 @@ __global__ void __launch_bounds__(256, 4) k_gemv_cph(const float* __restrict__ A
             for (int v = 0; v < 2 * GH_PIECE; ++v) {
                 const int j = lane + 32 * v;
                 if (2 * p0 + j < 2 * c1) {
-                    xu[v] = __ldg(xh4 + 2 * p0 + j);
-                    xv[v] = __ldg(xl4 + 2 * p0 + j);
+                    xu[v] = xh4[2 * p0 + j];
+                    xv[v] = xl4[2 * p0 + j];
                 }
             }
             cp_async_wait_all();
@@ -629,8 +635,8 @@ __global__ void __launch_bounds__(256, 4) k_gemv_cph(const float* __restrict__ A
 }
 
 template <int SPLIT>
-__global__ void __launch_bounds__(256) k_gemv64s(const double* __restrict__ A, const double* __restrict__ x,
-                                                 double* __restrict__ y, int64_t n, const int* __restrict__ gate) {
+__global__ void __launch_bounds__(256) k_gemv64s(const double* __restrict__ A, const double* x,
+                                                 double* __restrict__ y, int64_t n, const int* gate) {
     mh_dep_wait();
     if (gate && *gate) return;
     __shared__ double part[8];
@@ -646,12 +652,12 @@ __global__ void __launch_bounds__(256) k_gemv64s(const double* __restrict__ A, c
         int64_t c = c0 + lane;
         for (; c + 32 < c1; c += 64) {
             const double2 u = __ldcs(a + c), v = __ldcs(a + c + 32);
-            const double2 xu = __ldg(xv + c), xw = __ldg(xv + c + 32);
+            const double2 xu = xv[c], xw = xv[c + 32];
             a0 = fma(u.x, xu.x, fma(u.y, xu.y, a0));
             a1 = fma(v.x, xw.x, fma(v.y, xw.y, a1));
         }
         for (; c < c1; c += 32) {
-            const double2 u = __ldcs(a + c), xu = __ldg(xv + c);
+            const double2 u = __ldcs(a + c), xu = xv[c];
             a0 = fma(u.x, xu.x, fma(u.y, xu.y, a0));
         }
     }
@@ -745,7 +751,7 @@ __global__ void k_prep_fine32(const double* __restrict__ fg, const int64_t* __re
     }
 }
 
-__global__ void k_weights32(const double* __restrict__ sigma, const double* __restrict__ geo,
+__global__ void k_weights32(const double* sigma, const double* __restrict__ geo,
                             const int32_t* __restrict__ curve_of, const int32_t* __restrict__ nn, int64_t n, float* w) {
     mh_dep_wait();
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -764,7 +770,7 @@ __global__ void k_weights32(const double* __restrict__ sigma, const double* __re
 // test (mh_dl32_pair_far; pairs beyond the cut come out below the rounding of the sum).
 __global__ void __launch_bounds__(MH_TILE) k_dlp_coarse32(const double* __restrict__ xy,
                                                           const uint32_t* __restrict__ fine, int64_t nt,
-                                                          const float4* __restrict__ src, const float* __restrict__ w,
+                                                          const float4* __restrict__ src, const float* w,
                                                           const int32_t* __restrict__ curve_of,
                                                           const double2* __restrict__ tc, const float* __restrict__ tr,
                                                           int64_t ns, mh_dl32 c32, double pref, double* out) {
@@ -904,7 +910,7 @@ __device__ __forceinline__ void fine_chunk(const float4* __restrict__ fine32, co
 template <int TG>
 __global__ void __launch_bounds__(256) k_dlp_fine32_grp(
     const double* __restrict__ xy, const int32_t* __restrict__ pair_tgt, const int32_t* __restrict__ grp_curve,
-    const int32_t* __restrict__ grp_pair, int slices, const float4* __restrict__ fine32, const float* __restrict__ wf,
+    const int32_t* __restrict__ grp_pair, int slices, const float4* __restrict__ fine32, const float* wf,
     const int64_t* __restrict__ foff, const int64_t* __restrict__ coff, const float4* __restrict__ ccf,
     const float* __restrict__ crad, mh_dl32 c32, float cut_r, double pref, double* part, unsigned* cnt,
     double* out) {
@@ -1009,7 +1015,7 @@ __global__ void __launch_bounds__(256) k_dlp_fine32_grp(
 template <int TG>
 __global__ void __launch_bounds__(256) k_dlp_fine64_grp(
     const double* __restrict__ xy, const int32_t* __restrict__ pair_tgt, const int32_t* __restrict__ grp_curve,
-    const int32_t* __restrict__ grp_pair, int slices, const double* __restrict__ fg, const double* __restrict__ wf,
+    const int32_t* __restrict__ grp_pair, int slices, const double* __restrict__ fg, const double* wf,
     const int64_t* __restrict__ foff, mh_pair_tab tab, double pref, double* part, unsigned* cnt, double* out) {
     mh_dep_wait();
     __shared__ double red[8][TG];
@@ -1540,7 +1546,7 @@ __device__ __forceinline__ void sincospi_t(float x, float* s, float* c) { sincos
 __device__ __forceinline__ void sincospi_t(double x, double* s, double* c) { sincospi(x, s, c); }
 
 template <typename T, typename T2>
-__global__ void __launch_bounds__(256) k_fine_weights_fft(const double* __restrict__ sigma, const T2* __restrict__ tw,
+__global__ void __launch_bounds__(256) k_fine_weights_fft(const double* sigma, const T2* __restrict__ tw,
                                                           const double* __restrict__ fg, const int32_t* __restrict__ nn,
                                                           const int32_t* __restrict__ off,
                                                           const int64_t* __restrict__ foff, float* __restrict__ wf,
@@ -1621,7 +1627,7 @@ __global__ void __launch_bounds__(256) k_fine_weights_fft(const double* __restri
 template <int BS>
 __global__ void __launch_bounds__(BS) k_dlp_coarse(const double* __restrict__ xy, const uint32_t* __restrict__ fine,
                                                    int64_t nt, const double* __restrict__ geo,
-                                                   const double* __restrict__ sigma,
+                                                   const double* sigma,
                                                    const int32_t* __restrict__ curve_of, const int32_t* __restrict__ nn,
                                                    int64_t ns, int64_t per, mh_pair_tab tab, double pref,
                                                    double* out) {
@@ -2376,7 +2382,8 @@ constexpr size_t GH_SMEM = 8 * 3 * GH_PIECE * 32 * sizeof(float4);    // 24 KB
 // computes, and small pieces leave room for 8 blocks per SM, so some compute while others load).
 static void gemv32(cudaStream_t st, const float* A, const float* x, double* y, int64_t n, const int* gate) {
     if ((n & 3) == 0)
-        (void)mh_launch_dep(st, k_gemv32s<GEMV_SPLIT>, dim3((unsigned)((n + 8 / GEMV_SPLIT - 1) / (8 / GEMV_SPLIT))),
+        (void)mh_launch_dep(st, k_gemv32s<GEMV_SPLIT>,
+                            dim3((unsigned)std::min<int64_t>(152 * 6, (n + 8 / GEMV_SPLIT - 1) / (8 / GEMV_SPLIT))),
                             dim3(256), 0, A, x, y, n, gate);
     else
         (void)mh_launch_dep(st, k_gemv32, dim3(gemv_blocks(n)), dim3(256), 0, A, x, y, n, gate);

@@ -302,7 +302,7 @@ template <typename TD>
 __global__ void __launch_bounds__(TC_THREADS, 1) k_contract_tc(
     const __nv_bfloat16* __restrict__ img, const int64_t* __restrict__ img_off_op, const int32_t* __restrict__ kpad_op,
     const int32_t* __restrict__ chunk_op, const int32_t* __restrict__ chunk_t0, int n_chunks,
-    const uint16_t* __restrict__ spl, int64_t plane, const int64_t* __restrict__ tc_src, int R, int npad, int kmax,
+    const uint16_t* spl, int64_t plane, const int64_t* __restrict__ tc_src, int R, int npad, int kmax,
     int nst, float* __restrict__ temp, const int64_t* __restrict__ task_dst, int accumulate, TD* dst, int* err) {
     mh_dep_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -240,7 +240,7 @@ __device__ __forceinline__ void sum_dots(const double* part, int C, int cap, int
 }
 
 // ws -= sum_i h_i V_i on the slice (threads t of nt).
-__device__ __forceinline__ void subtract(const double* __restrict__ V, int64_t n, int64_t e0, int cnt, double* ws,
+__device__ __forceinline__ void subtract(const double* V, int64_t n, int64_t e0, int cnt, double* ws,
                                          const double* h, int k1, int t, int nt) {
     for (int e = t; e < cnt; e += nt) {
         const double* v = V + e0 + e;
@@ -390,8 +390,8 @@ __global__ void __launch_bounds__(GM_T) k_arnoldi(step_args a) {
 // R in shared memory.
 constexpr int GE_REG = 32;
 
-__global__ void __launch_bounds__(256) k_sweep_end(const double* __restrict__ V, const double* __restrict__ H, int ldh,
-                                                   const double* __restrict__ g, const gmres_dev* gs, int64_t n,
+__global__ void __launch_bounds__(256) k_sweep_end(const double* V, const double* H, int ldh,
+                                                   const double* g, const gmres_dev* gs, int64_t n,
                                                    double* x, float* __restrict__ xh, float* __restrict__ xl) {
     mh_dep_wait();
     if (gs->done) return;

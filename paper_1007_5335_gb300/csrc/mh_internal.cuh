@@ -129,6 +129,9 @@ inline size_t mh_bytes(const B&... b) {
 // not keep these rules (one that starts its dependents early and does not wait may end before its own
 // predecessors).  Kernels that are launched either way call mh_dep_wait() too (no effect in an ordinary
 // launch).  The wait comes before the trigger: at most one kernel waits behind the running one.
+// What a kernel of the stream may have written is read by plain loads: no const __restrict__, no __ldg.  The
+// read-only path asks for data that is constant over the kernel's whole life, and a dependent kernel is
+// already resident while its predecessor writes; set-up data alone is read that way.
 __device__ __forceinline__ void mh_dep_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -170,7 +173,7 @@ __device__ __forceinline__ uint64_t mh_l2_policy(bool keep) {
 }
 __device__ __forceinline__ float4 mh_ld_hint(const float4* p, uint64_t policy) {
     float4 v;
-    asm volatile("ld.global.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
+    asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
                  : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
                  : "l"(p), "l"(policy));
     return v;

@@ -72,9 +72,9 @@ enum { EPI_NONE = 0, EPI_BIAS = 1, EPI_BIAS_TANH = 2, EPI_TANH_BACK = 3 };
 // One block's share z of S of tile (i0, j0), number `tile` of `tiles`.
 template <typename T, int EPI>
 __device__ __forceinline__ void gemm_tile(int i0, int j0, int tile, int tiles, int z, int S, int M, int N, int K,
-                                          const T* __restrict__ A, int64_t sam, int64_t sak, const T* __restrict__ B,
+                                          const T* A, int64_t sam, int64_t sak, const T* B,
                                           int64_t sbk, int64_t sbn, T* __restrict__ C, int64_t ldc,
-                                          const T* __restrict__ bias, const T* __restrict__ aux, T* part, unsigned* cnt) {
+                                          const T* __restrict__ bias, const T* aux, T* part, unsigned* cnt) {
     __shared__ __align__(16) T As[2][GEMM_K][GEMM_T + 4];
     __shared__ __align__(16) T Bs[2][GEMM_K][GEMM_T + 4];
     __shared__ int last;
@@ -202,9 +202,9 @@ __device__ __forceinline__ void gemm_tile(int i0, int j0, int tile, int tiles, i
 }
 
 template <typename T, int EPI>
-__global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, const T* __restrict__ A, int64_t sam, int64_t sak,
-                                              const T* __restrict__ B, int64_t sbk, int64_t sbn, T* __restrict__ C,
-                                              int64_t ldc, const T* __restrict__ bias, const T* __restrict__ aux,
+__global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, const T* A, int64_t sam, int64_t sak,
+                                              const T* B, int64_t sbk, int64_t sbn, T* __restrict__ C,
+                                              int64_t ldc, const T* __restrict__ bias, const T* aux,
                                               T* part, unsigned* cnt) {
     mh_dep_wait();
     gemm_tile<T, EPI>(blockIdx.y * GEMM_T, blockIdx.x * GEMM_T, blockIdx.y * gridDim.x + blockIdx.x,
@@ -524,7 +524,7 @@ __global__ void k_gather_rows(const float* __restrict__ X, const int32_t* __rest
 
 // dz = (yh - t) * inv; per-block partial sums of (yh - t)^2 (binary64) into part, added by the last block to
 // finish (cnt, reset by it): out = scale * sum.
-__global__ void k_loss_dz(const float* __restrict__ yh, const float* __restrict__ t, int64_t n, float inv,
+__global__ void k_loss_dz(const float* yh, const float* __restrict__ t, int64_t n, float inv,
                           float* __restrict__ dz, double* part, unsigned* cnt, double scale, double* out) {
     mh_dep_wait();
     __shared__ int last;
@@ -552,7 +552,7 @@ __global__ void k_loss_dz(const float* __restrict__ yh, const float* __restrict_
     }
 }
 
-__global__ void k_sum_parts(const double* __restrict__ part, int n, double scale, double* out) {
+__global__ void k_sum_parts(const double* part, int n, double scale, double* out) {
     mh_dep_wait();
     double s = 0.0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) s += part[i];

@@ -503,7 +503,7 @@ constexpr int CHAIN_SMEM_MAX = 64 * 1024;   // p = 40 (P = 81) in binary64 takes
 // (TwoSum: the sum of the products with binary64-like accuracy and no binary64 instruction per
 // product), converted once per output.
 template <typename TT, typename TD>
-__global__ void k_reduce(const TT* __restrict__ temp, int R, const int64_t* __restrict__ dst_off,
+__global__ void k_reduce(const TT* temp, int R, const int64_t* __restrict__ dst_off,
                          const int32_t* __restrict__ dst_ptr, const int32_t* __restrict__ dst_task, int64_t n_dst,
                          int accumulate, TD* dst) {
     mh_dep_wait();
@@ -1973,7 +1973,7 @@ __device__ __forceinline__ void near_finish(double acc, bool act, int qq, int i,
 __global__ void __launch_bounds__(NEAR_T) k_dip_near64(
     const double* __restrict__ nodes, const NearChunk* __restrict__ chunks, const int2* __restrict__ leaf_red,
     const int32_t* __restrict__ flat_idx, const double2* __restrict__ dxy, const double2* __restrict__ dnrm,
-    const double* __restrict__ w, int qq, mh_pair_tab tab, double pref, double* part, unsigned* cnt,
+    const double* w, int qq, mh_pair_tab tab, double pref, double* part, unsigned* cnt,
     double* out) {
     mh_dep_wait();
     __shared__ double2 sp[NEAR_T], sn[NEAR_T];
@@ -2012,7 +2012,7 @@ template <int NT>
 __global__ void __launch_bounds__(NT) k_dip_near32(
     const double* __restrict__ nodes, const NearChunk* __restrict__ chunks, const int2* __restrict__ leaf_red,
     const double2* __restrict__ leaf_c, const int32_t* __restrict__ flat_idx, const float4* __restrict__ flat32,
-    const float* __restrict__ w, int qq, mh_dl32 c32, double pref, double* part, unsigned* cnt, double* out) {
+    const float* w, int qq, mh_dl32 c32, double pref, double* part, unsigned* cnt, double* out) {
     mh_dep_wait();
     __shared__ float4 s4[NT];
     const NearChunk ch = chunks[blockIdx.x];
@@ -2058,7 +2058,7 @@ __global__ void __launch_bounds__(NT) k_dip_near32(
 // zero: the locals of the pass (boxes whose V and X lists hold no dipoles get no M2L / P2L task, and the
 // downward chain adds into the leaves' locals).
 template <typename T>
-__global__ void k_dip_weights(const double* __restrict__ w, const int32_t* __restrict__ perm, int64_t n, T* ws, T* zero,
+__global__ void k_dip_weights(const double* w, const int32_t* __restrict__ perm, int64_t n, T* ws, T* zero,
                               int64_t n_zero) {
     mh_dep_wait();
     const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
@@ -2639,7 +2639,7 @@ void bie_row(double* row, int p, const double* v, double th) {
 }
 
 // Dipole strengths sigma |y'| h in sorted order, and zeros in the locals (as k_dip_weights).
-__global__ void k_bie_weights(const double* __restrict__ sigma, const double* __restrict__ geo,
+__global__ void k_bie_weights(const double* sigma, const double* __restrict__ geo,
                               const int32_t* __restrict__ curve_of, const int32_t* __restrict__ nn,
                               const int32_t* __restrict__ perm, int64_t n, double* __restrict__ ws,
                               double* __restrict__ zero, int64_t n_zero) {
