@@ -101,10 +101,14 @@ struct dbuf {
     }
     cudaError_t alloc(size_t count) {
         release();
-        n = count;
         if (count == 0) return cudaSuccess;
         g_mh_alloc_calls.fetch_add(1, std::memory_order_relaxed);
-        return cudaMalloc((void**)&p, count * sizeof(T));
+        const cudaError_t e = cudaMalloc((void**)&p, count * sizeof(T));
+        if (e == cudaSuccess)
+            n = count;   // a failed allocation leaves no room: the next reserve tries again
+        else
+            p = nullptr;
+        return e;
     }
     cudaError_t reserve(size_t count) { return count <= n ? cudaSuccess : alloc(count); }
 };
