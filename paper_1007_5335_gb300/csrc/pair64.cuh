@@ -43,18 +43,32 @@ struct mh_pair_tab {
     double inv_alpha = 0.0;
 };
 
+// Outside 1e-150 < alpha < 1e150 or so the octaves leave the range of binary64 exponents: the table stays
+// unused (hi0 above every number), every pair within the cut takes K1 directly.
 inline mh_pair_tab mh_pair_tab_make(const double2* c, double alpha) {
     mh_pair_tab T;
     T.c = c;
-    const int e0 = std::ilogb(alpha * alpha) - 14;   // first octave: [2^e0, 2^(e0+1))
-    T.hi0 = (e0 + 1023) << 20;
-    T.hi1 = (e0 + PT_OCT + 1023) << 20;
-    const double cut = 2025.0 * alpha * alpha;
+    const double a2 = alpha * alpha, cut = std::fmin(2025.0 * a2, 1.7976931348623157e308);
+    const bool ok = a2 >= 2.2250738585072014e-308 && a2 <= 1.7976931348623157e308;
+    const int e0 = (ok ? std::ilogb(a2) : 0) - 14 + 1023;   // biased exponent of the first octave
+    if (ok && e0 >= 1 && e0 + PT_OCT + PT_OCT_FAR <= 2046) {
+        T.hi0 = e0 << 20;
+        T.hi1 = (e0 + PT_OCT) << 20;
+    } else {
+        T.hi0 = T.hi1 = 0x7fffffff;
+    }
     uint64_t bits;
     std::memcpy(&bits, &cut, 8);
     T.hi_cut = (int)(bits >> 32);
     T.inv_alpha = 1.0 / alpha;
     return T;
+}
+
+// Bin of a number with the high word hi, hi0 <= hi <= hi_cut.
+__host__ __device__ __forceinline__ int mh_pair_bin(int hi, const mh_pair_tab& T) {
+    const bool far = hi >= T.hi1;
+    const int bits = far ? PT_BITS_FAR : PT_BITS;
+    return ((hi - (far ? T.hi1 : T.hi0)) >> (20 - bits)) + (far ? PT_OCT << PT_BITS : 0);
 }
 
 // K1(z)/z for rho below the table (r < alpha/128; rho = 0 gives 0: the offset is 0 there).
@@ -71,7 +85,7 @@ __device__ __forceinline__ double mh_pair_f(double rho, const mh_pair_tab& T) {
     if (hi < T.hi0) return mh_pair_near(rho, T.inv_alpha);
     const bool far = hi >= T.hi1;
     const int bits = far ? PT_BITS_FAR : PT_BITS;
-    const int bin = ((hi - (far ? T.hi1 : T.hi0)) >> (20 - bits)) + (far ? PT_OCT << PT_BITS : 0);
+    const int bin = mh_pair_bin(hi, T);
     const double2* c = T.c + PT_WORDS * bin;
     const double2 a = __ldg(c), b = __ldg(c + 1);
     const float4 q = __ldg(reinterpret_cast<const float4*>(c + 2));
@@ -88,7 +102,7 @@ __device__ __forceinline__ double mh_pair_f(double rho, const mh_pair_tab& T) {
 // Table entries for one alpha: a thread per bin, K_n by the (stable) forward recurrence.
 static __global__ void k_pair_table(mh_pair_tab T, double alpha, double2* __restrict__ out) {
     const int bin = blockIdx.x * blockDim.x + threadIdx.x;
-    if (bin >= PT_BINS) return;
+    if (bin >= PT_BINS || T.hi0 == 0x7fffffff) return;
     const bool far = bin >= (PT_OCT << PT_BITS);
     const int sh = far ? 20 - PT_BITS_FAR : 20 - PT_BITS;
     const int i = far ? bin - (PT_OCT << PT_BITS) : bin;
