@@ -575,7 +575,7 @@ struct ColSum {
 // dst[row[o R + r]] (row < 0: none).  The operator is set-up data: its first columns are loaded before the
 // wait for the vector, the next ones while a batch is summed.
 template <typename T>
-__global__ void __launch_bounds__(256) k_cols(const T* __restrict__ ops, const int32_t* __restrict__ src,
+__global__ void __launch_bounds__(256) k_cols(const T* __restrict__ ops, const uint32_t* __restrict__ src,
                                               const ColChunk* __restrict__ chunks, const int2* __restrict__ out_red,
                                               const int64_t* __restrict__ at, const int32_t* __restrict__ row, int R,
                                               const T* vec, T* part, unsigned* cnt, int accumulate, T* dst) {
@@ -587,7 +587,7 @@ __global__ void __launch_bounds__(256) k_cols(const T* __restrict__ ops, const i
     int64_t c = ch.c0 + g;
     const int64_t end = g < G ? ch.c1 : 0;
     T a[U];
-    int32_t at_x[U];
+    uint32_t at_x[U];
 #pragma unroll
     for (int u = 0; u < U; ++u)
         if (c + u * G < end) {
@@ -652,7 +652,9 @@ __global__ void __launch_bounds__(256) k_cols(const T* __restrict__ ops, const i
 struct ColBuild {
     int R = 0;
     std::vector<double> a;
-    std::vector<int32_t> src, row;
+    std::vector<uint32_t> src;   // offsets into the pass's vector (below 2^32: 34 GB of it; build_cols checks)
+    std::vector<int32_t> row;
+    int64_t last = 0;            // largest offset
     std::vector<int64_t> at, first{0};
     explicit ColBuild(int rows) : R(rows) {}
     void open(int64_t dst) { at.push_back(dst); }
@@ -660,8 +662,9 @@ struct ColBuild {
     void add(int nc, const std::vector<double>& m, int64_t src0) {
         for (int c = 0; c < nc; ++c) {
             for (int r = 0; r < R; ++r) a.push_back(m[(size_t)r * nc + c]);
-            src.push_back((int32_t)(src0 + c));
+            src.push_back((uint32_t)(src0 + c));
         }
+        last = std::max(last, src0 + nc - 1);
     }
     void close() { first.push_back((int64_t)src.size()); }
 };
@@ -673,7 +676,8 @@ struct ColSet {
     double flops = 0, bytes = 0;
     dbuf<double> ops64, part;   // part: sized in binary64 words, room for either type
     dbuf<float> ops32;
-    dbuf<int32_t> src, row;
+    dbuf<uint32_t> src;
+    dbuf<int32_t> row;
     dbuf<ColChunk> chunks;
     dbuf<int2> out_red;
     dbuf<int64_t> at;
@@ -684,6 +688,8 @@ mh_status build_cols(mh_ctx* ctx, const ColBuild& b, bool both, ColSet* S) {
     S->R = b.R;
     S->n = (int64_t)b.first.size() - 1;
     if (S->n == 0) return MH_OK;
+    if (b.last > (int64_t)UINT32_MAX)
+        return mh_fail(ctx, MH_ERR_INVALID_ARG, "the tree has too many boxes for the column form of its outputs");
     std::vector<ColChunk> ch;
     std::vector<int2> red(S->n, make_int2(0, 1));
     int32_t slots = 0;

@@ -1,5 +1,5 @@
 """Index arithmetic of the kernels at the ends of its range, on the host (compiled with the library's own
-headers): the bin of a pair for any alpha."""
+headers): the bin of a pair for any alpha, and the offsets of single columns in a vector beyond 2^31 entries."""
 import ctypes
 import os
 
@@ -29,6 +29,17 @@ extern "C" int bins(double alpha, int* lo, int* hi) {
 }
 """
 
+COLUMNS = r"""
+#include "volume.cu"
+extern "C" long column_offset(long at) {
+    ColBuild b(1);
+    b.open(0);
+    b.add(1, {1.0}, at);
+    b.close();
+    return b.last > (long)UINT32_MAX ? -1 : (long)b.src[0];
+}
+"""
+
 
 def test_pair_bins_stay_inside_the_table():
     lib = compile_cuda(PAIRS)
@@ -46,3 +57,11 @@ def test_pair_bins_stay_inside_the_table():
     lo, hi = ctypes.c_int(), ctypes.c_int()
     assert lib.bins(float("inf"), ctypes.byref(lo), ctypes.byref(hi)) < 0
     assert used > 60
+
+
+def test_column_offsets_beyond_two_to_the_31():
+    lib = compile_cuda(COLUMNS)
+    lib.column_offset.argtypes, lib.column_offset.restype = [ctypes.c_long], ctypes.c_long
+    for at in (0, 2 ** 31 - 1, 2 ** 31, 3_000_000_000, 2 ** 32 - 1):
+        assert lib.column_offset(at) == at
+    assert lib.column_offset(2 ** 32) == -1
