@@ -9,15 +9,24 @@
 // bin holds the 7 Taylor coefficients about its centre,
 //   d^j/drho^j f = (-1/(2 alpha^2))^j K_{1+j}(z) / z^{1+j}
 // (the derivative rule of z^{-n} K_n(z)).
-//   bins     128 an octave from rho = 2^-14 alpha^2 for 20 octaves (|t/rho| <= 1/256: the eighth
-//            term is below 256^-7 = 1.4e-17 of f), 512 an octave for the six above, where f falls
-//            like e^{-z} (z = 45: (z/2048)^7/7! = 4e-16); octaves start at a power of two, so
-//            the two ranges reach past 2025 alpha^2 = (45 alpha)^2 whatever alpha is.
+//   bins     128 an octave from rho = 2^-14 alpha^2 for 20 octaves (to z = 5.7 .. 8; |t/rho| <= 1/256 with t the
+//            distance from the centre), 512 an octave for the six above, where f falls like e^{-z}
+//            (1/1024); octaves start at a power of two, so the two ranges reach past 2025 alpha^2 =
+//            (45 alpha)^2 whatever alpha is.
+//   eighth   the first term left out, relative to f: at most 1.4e-17 for z <= 0.5, 4.2e-16 at z = 5.7, 1e-15 at
+//            the cut, at the edges of a bin at the start of its octave; a 128th of that half way to the centre.
 //   lookup   the bin is the top bits of rho's binary64 pattern; the bits below them, shifted up, are
 //            the place in the bin, tau in [-1/2, 1/2) in units of its width (integer pipe, and one
 //            subtraction).
-//   terms    tau^0..3 in binary64; tau^4..6 together are below 256^-4 = 2.4e-10 of f, so their factor
-//            of tau^4 is formed in binary32 (1.4e-17 of f) and widened by its bits.
+//   terms    tau^0..3 in binary64; tau^4..6 together are at most 2.4e-10 of f for z <= 0.1, 4e-9 at z = 5.7 and
+//            1.3e-8 at the cut (bin edges again), so their factor of tau^4 is formed in binary32 (1.4e-17,
+//            2.4e-16, 8e-16 of f) and widened by its bits.
+//   entries  the value at a centre carries the rounding of z = sqrt(rho)/alpha, z eps of e^{-z}, unless it is
+//            corrected to first order (k_pair_table).
+// Error of f against 30 digits, 30,000 distances over the whole range at alpha^2 = 1e-3, 2^-10 and 0.03 (rms /
+// largest): table 1.2e-16 / 4.6e-16 for z < 1, 2.2e-16 / 8.4e-16 for 1 < z < 2, 1.5e-16 / 6.5e-16 above; K1 and
+// its factors per pair 1.1 to 1.5e-16 / 5.6e-16, 2.6e-16 / 9.1e-16, and 2.9e-16 / 1.1e-15 (z < 5) rising to
+// 2.3e-15 / 7.1e-15 (z > 20); seven binary64 coefficients the table's to three digits.
 // 48 bytes per bin (four doubles, three floats, padding), three 16-byte loads from L1.
 // A pair then takes 12 binary64 instructions: offsets 2, rho 2, tau 1, Horner 4, dot product 2,
 // accumulate 1, and no comparison, conversion, square root or division.
@@ -110,10 +119,13 @@ static __global__ void k_pair_table(mh_pair_tab T, double alpha, double2* __rest
     const double lo = __hiloint2double(first, 0), width = 2.0 * (__hiloint2double(first + (1 << (sh - 1)), 0) - lo);
     const double rho = lo + 0.5 * width;
     const double z = sqrt(rho) / alpha, d = -0.5 * width / (alpha * alpha);
+    // dz = sqrt(rho)/alpha - z: K1 falls like e^{-z}, so the rounding of z alone is z eps of an entry
+    const double p = z * alpha, pe = fma(z, alpha, -p), q = p * p, qe = fma(p, p, -q);
+    const double dz = (((rho - q) - qe) - 2.0 * p * pe) / (2.0 * p * alpha);
     double km = mh_k0(z), k = mh_k1(z), scale = 1.0 / z, c[7];
     for (int j = 0; j < 7; ++j) {   // c_j = (-width/(2 alpha^2))^j / j! K_{1+j}(z) / z^{1+j}
-        c[j] = scale * k;
         const double kn = km + (2.0 * (j + 1) / z) * k;
+        c[j] = j == 0 ? (k - dz * kn) / z : scale * k;   // (K1/z)' = -K2/z
         km = k;
         k = kn;
         scale *= d / (z * (j + 1));
