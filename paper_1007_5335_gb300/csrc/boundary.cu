@@ -2466,7 +2466,7 @@ mh_status bie_apply64_gated(mh_ctx* ctx, mh_boundary* b, const double* x, double
 const double* gmres_final_residual(mh_boundary* b) { return b->ws.r.p; }
 
 
-mh_status bie_apply(mh_ctx* ctx, mh_boundary* b, const double* x, double* y, mh_precision prec) {
+mh_status bie_apply(mh_ctx* ctx, mh_boundary* b, const double* x, double* y, mh_precision prec, bool dep) {
     if (b->mfree) return bie_apply_mfree(ctx, b, x, y);
     MH_TRY(need_dense(ctx, b));
     if (prec == MH_PREC_MIXED) {
@@ -2478,7 +2478,7 @@ mh_status bie_apply(mh_ctx* ctx, mh_boundary* b, const double* x, double* y, mh_
         gemv32(ctx->stream, b->op.A32.p, b->x32.p, y, b->n, nullptr);
     } else {
         prof_scope ps(ctx, "bie_gemv64", 2.0 * b->n * b->n, 8.0 * b->n * b->n + 16.0 * b->n);
-        gemv64(ctx->stream, b->op.A64.p, x, y, b->n, nullptr, false);   // an entry point's first kernel
+        gemv64(ctx->stream, b->op.A64.p, x, y, b->n, nullptr, dep);
     }
     MH_LAUNCHED(ctx);
     return MH_OK;
@@ -3175,7 +3175,7 @@ static mh_status dlp_evaluate(mh_ctx* ctx, mh_boundary* b, double alpha, dlp_eva
         MH_TRY(fine_sums(ctx, b, alpha, tg, E->fine.wf.p, prec, E->ptab));
     }
     if (tg->n_line) {
-        MH_TRY(bie_apply(ctx, b, sigma, asig.p, MH_PREC_FP64));
+        MH_TRY(bie_apply(ctx, b, sigma, asig.p, MH_PREC_FP64, true));
         (void)mh_launch_dep(st, k_dlp_line, dim3(mh_grid(tg->n_line * 32, 256)), dim3(256), 0, tg->line_tgt.p,
                             tg->line_curve.p, tg->line_l.p, tg->n_line, asig.p, nullptr, b->d_nn.p, b->d_off.p,
                             tg->line_w.p, tg->line_woff.p, tg->n, -0.5 / (alpha * alpha), ext.p, nullptr, nullptr, ext.p);

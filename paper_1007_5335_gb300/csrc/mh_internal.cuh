@@ -490,7 +490,8 @@ mh_status warm_start_prepare(mh_ctx* ctx, mh_boundary* b);
 
 // ---- boundary.cu ----
 mh_status bie_assemble(mh_ctx* ctx, mh_boundary* b, double alpha);
-mh_status bie_apply(mh_ctx* ctx, mh_boundary* b, const double* x, double* y, mh_precision prec);
+mh_status bie_apply(mh_ctx* ctx, mh_boundary* b, const double* x, double* y, mh_precision prec,
+                    bool dep = false);
 // Matrix-free operator: set-up after volume_bie_setup on tree t (releases the dense forms; every
 // later operator product of b goes through it), and one product y = A x (binary64).
 mh_status bie_mfree_setup(mh_ctx* ctx, mh_boundary* b, mh_tree* t, double alpha);
