@@ -710,11 +710,11 @@ __global__ void k_prep_src32(const double* __restrict__ geo, int64_t n, float4* 
 }
 
 // Fine nodes relative to chunk centres: chunks of MH_TILE fine nodes inside each curve.
-// Per fine chunk: offsets of its nodes from the chunk centre (binary32), the centre in
-// binary64 and as float-float pairs (x_hi, x_lo, y_hi, y_lo), and the chunk radius.
+// Per fine chunk: offsets of its nodes from the chunk centre (binary32), the centre as
+// float-float pairs (x_hi, x_lo, y_hi, y_lo), and the chunk radius.
 __global__ void k_prep_fine32(const double* __restrict__ fg, const int64_t* __restrict__ foff,
-                              const int64_t* __restrict__ coff, int ncurves, float4* out, double2* cc,
-                              float4* ccf, float* crad) {
+                              const int64_t* __restrict__ coff, int ncurves, float4* out, float4* ccf,
+                              float* crad) {
     const int64_t chunk = blockIdx.x;
     int k = 0;
     while (k + 1 < ncurves && chunk >= coff[k + 1]) ++k;
@@ -729,7 +729,6 @@ __global__ void k_prep_fine32(const double* __restrict__ fg, const int64_t* __re
         }
         cx = ax / cnt;
         cy = ay / cnt;
-        cc[chunk] = make_double2(cx, cy);
     }
     __syncthreads();
     float r2max = 0.f;
@@ -2983,7 +2982,6 @@ mh_status dlp_classify(mh_ctx* ctx, mh_boundary* b, const double* xy_dev, int64_
     MH_RESERVE(ctx, tg->line_curve, tg->n_line);
     MH_RESERVE(ctx, tg->line_data, 4 * tg->n_line);
     MH_RESERVE(ctx, tg->pair_tgt, tg->n_pairs);
-    MH_RESERVE(ctx, tg->pair_curve, tg->n_pairs);
     if (n > 0) MH_CUDA(ctx, cudaMemcpyAsync(tg->xy.p, xy_dev, 2 * n * 8, cudaMemcpyDeviceToDevice, st));
     if (tg->n_ext) MH_CUDA(ctx, cudaMemcpyAsync(tg->fine.p, fext.data(), tg->n_ext * 4, cudaMemcpyHostToDevice, st));
     if (tg->n_line) {
@@ -3006,10 +3004,8 @@ mh_status dlp_classify(mh_ctx* ctx, mh_boundary* b, const double* xy_dev, int64_
                                                                       tg->line_woff.p, tg->line_w.p, tg->line_l.p);
         MH_LAUNCHED(ctx);
     }
-    if (tg->n_pairs) {
+    if (tg->n_pairs)
         MH_CUDA(ctx, cudaMemcpyAsync(tg->pair_tgt.p, pt.data(), tg->n_pairs * 4, cudaMemcpyHostToDevice, st));
-        MH_CUDA(ctx, cudaMemcpyAsync(tg->pair_curve.p, pc.data(), tg->n_pairs * 4, cudaMemcpyHostToDevice, st));
-    }
     MH_RESERVE(ctx, tg->ext, std::max<int64_t>(tg->n_ext, 1));
     MH_RESERVE(ctx, tg->asig, b->n);
     MH_CUDA(ctx, cudaStreamSynchronize(st));
@@ -3033,7 +3029,6 @@ static mh_status prep_mixed(mh_ctx* ctx, mh_boundary* b) {
     b->n_fchunks = b->fchunk_off[b->n_curves];
     MH_ALLOC(ctx, b->d_fchunk_off, b->n_curves + 1);
     MH_ALLOC(ctx, b->fine32, b->n_fine);
-    MH_ALLOC(ctx, b->fchunk_c, b->n_fchunks);
     MH_ALLOC(ctx, b->wf32, b->n_fine);
     MH_CUDA(ctx, cudaMemcpyAsync(b->d_fchunk_off.p, b->fchunk_off.data(), (b->n_curves + 1) * 8,
                                  cudaMemcpyHostToDevice, st));
@@ -3045,8 +3040,8 @@ static mh_status prep_mixed(mh_ctx* ctx, mh_boundary* b) {
                                                             reinterpret_cast<float*>(b->tw32.p), 2 * b->n);
     MH_LAUNCHED(ctx);
     k_prep_fine32<<<(unsigned)b->n_fchunks, 128, 0, st>>>(b->fine_geo.p, b->d_fine_off.p, b->d_fchunk_off.p,
-                                                          b->n_curves, b->fine32.p, b->fchunk_c.p,
-                                                          b->fchunk_cf.p, b->fchunk_r.p);
+                                                          b->n_curves, b->fine32.p, b->fchunk_cf.p,
+                                                          b->fchunk_r.p);
     MH_LAUNCHED(ctx);
     MH_CUDA(ctx, cudaStreamSynchronize(st));
     return MH_OK;

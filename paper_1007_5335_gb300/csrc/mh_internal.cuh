@@ -321,7 +321,7 @@ struct dlp_targets {
     // fine pairs (ext target, curve)
     int64_t n_pairs = 0, n_pairs_main = 0;   // pairs of user targets come first
     double fine_nodes_main = 0, fine_nodes_aux = 0;   // work counts
-    dbuf<int32_t> pair_tgt, pair_curve;
+    dbuf<int32_t> pair_tgt;
     // upsampled rule at the auxiliary points (at every pair of a set classified with all_groups):
     // groups of FINE_TG pairs on one curve (grp_pair, -1 padded), each group's fine nodes in
     // fine_slices slices, one block per (group, slice); partial sums per (group, slice, pair) in
@@ -335,7 +335,7 @@ struct dlp_targets {
     dbuf<double> ext, asig, part;
     size_t bytes() const {
         return mh_bytes(xy, fine0, lcurve, ldata, fine, region, line_tgt, line_curve, line_data, line_l, line_w, line_woff,
-                        pair_tgt, pair_curve, grp_curve, grp_pair, grp_part, grp_cnt, ext, asig, part);
+                        pair_tgt, grp_curve, grp_pair, grp_part, grp_cnt, ext, asig, part);
     }
 };
 
@@ -393,7 +393,7 @@ struct mh_boundary {
     std::vector<int64_t> fchunk_off;     // per curve first chunk
     dbuf<int64_t> d_fchunk_off;
     dbuf<float4> src32, fine32;          // (dx, dy, nx, ny)
-    dbuf<double2> tile_c, fchunk_c;
+    dbuf<double2> tile_c;
     dbuf<float> tile_r;                  // per source tile: largest distance of a node from its centre
     dbuf<float2> tw32;                   // binary32 copy of the twiddles e^{2 pi i r / N_k}
     dbuf<float> xhi32, xlo32;            // float-float split of the input of a residual product
