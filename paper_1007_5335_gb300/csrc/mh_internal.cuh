@@ -125,9 +125,10 @@ inline size_t mh_bytes(const B&... b) {
 // A kernel launched right behind another one on a stream costs about 2.2 us of drain and launch
 // latency (0.9 us inside a graph); with programmatic dependent launch it is on the SMs and waiting
 // when its predecessor ends (0.6 us; 16 blocks of 512 threads, chains of 500 launches).  The
-// rules here: a kernel launched by mh_launch_dep calls mh_dep_wait() first thing, in every thread
-// and before any return, so it touches memory only when everything before it on the stream has
-// completed, and completes only after its predecessors; mh_launch_dep is used behind a kernel of
+// rules here: a kernel launched by mh_launch_dep calls mh_dep_wait() in every thread and before any
+// return, with nothing before it but loads of set-up data (operators, weights of the geometry), so it touches
+// what the stream writes only when everything before it has completed, and completes only after its
+// predecessors; mh_launch_dep is used behind a kernel of
 // the same stream (a launch behind an event wait, a copy or a graph's conditional node is an ordinary
 // one).  The first kernel of an entry point is an ordinary launch as well: the caller's last kernel need
 // not keep these rules (one that starts its dependents early and does not wait may end before its own
@@ -166,7 +167,10 @@ inline cudaError_t mh_launch_dep(cudaStream_t st, void (*kernel)(K...), dim3 gri
 // L2, so in plain order every step streams all of it from HBM.  The first MH_L2_KEEP bytes are read
 // with an evict-last hint and stay for the next step, the rest with evict-first.  k_gemv32s in a
 // chain, 6144 nodes: 24.2 us without, 20.4 with 40 MB kept, 19.0 (64), 17.5 (80), 17.0 (88), 18.2
-// (96), 23.5 (112): 72 MB leaves the rest of the step its share.
+// (96), 23.5 (112): 72 MB leaves the rest of the step its share.  The share is one boundary's: in a batch
+// of large problems the kept parts exceed the L2 together and give nothing.  Mixed batch steps from a zero
+// density, with 72 / 24 / 0 MB kept: one problem of 7168 nodes 1290 / 1320 / 1360 us, two (7168, 8192)
+// 2190 / 2040 / 2100, four (7168 to 9216) 4070 / 4015 / 4000.
 constexpr int64_t MH_L2_KEEP = 72 << 20;
 
 __device__ __forceinline__ uint64_t mh_l2_policy(bool keep) {

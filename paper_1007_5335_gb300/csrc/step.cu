@@ -392,7 +392,9 @@ static mh_status step_solve(mh_ctx* ctx, ProblemImpl* P, const double* f_next_de
         info->gmres_iterations = gi.iterations;
         info->gmres_rel_residual = gi.rel_residual;
         info->initial_rel_residual = gi.initial_rel_residual;
-        info->warm_c = have_c ? *P->c_host : 0.0;   // gmres_run synchronised the stream
+        // c_host's copy stands before the solve on the stream, and the solve has ended: gmres_run has seen its last
+        // residual, published by a kernel behind the copy (or has waited for the stream)
+        info->warm_c = have_c ? *P->c_host : 0.0;
     }
     if (s != MH_OK) return s;
     // U^h: trapezoid sum by the multipole method at every node, then the near-boundary rules

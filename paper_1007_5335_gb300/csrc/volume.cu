@@ -295,7 +295,7 @@ __global__ void k_apply(const TOP* __restrict__ ops, const int64_t* __restrict__
     TOP* sX = sA + R * lda;
     const TOP* A = ops + op_off[op];
     if (nt == 1) {
-        // a single source vector (operators owned by one leaf: dipole P2M / P2L): a GEMV that
+        // a single source vector (operators owned by one leaf: dense near blocks of dipoles): a GEMV that
         // reads every operator row once, coalesced, straight from global memory
         const int64_t s0 = task_src[t0];
         for (int e = threadIdx.x; e < C; e += blockDim.x) sA[e] = src[s0 + e];
@@ -2540,8 +2540,8 @@ static mh_status dipole_out(mh_ctx* ctx, mh_tree* t, VolData* V, DipData* D, con
                              D->temp.p, D->out.get(), "dlp_fmm_contract", &D->tc);
 }
 
-// w_sorted: dipole strengths in the leaf-sorted order given to volume_dipole_setup.
-// Returns a device pointer to U^h at every volume node (leaf-major), valid until the next call.
+// Dipole j of the leaf-sorted order given to volume_dipole_setup has the strength w[perm[j]].
+// *u: device pointer to U^h at every volume node (leaf-major), valid until the next call.
 mh_status volume_dipole_apply(mh_ctx* ctx, mh_tree* t, const double* w, const int32_t* perm, mh_precision prec,
                               const double** u) {
     VolData* V = static_cast<VolData*>(t->vol);
