@@ -25,6 +25,15 @@ extern "C" int set_cycle(mh_boundary* b, long n, long m) {
     k_cycle<<<(unsigned)((n + 255) / 256), 256>>>(b->op.A64.p, n, m);
     return (int)cudaDeviceSynchronize();
 }
+extern "C" int set_matrix(mh_boundary* b, const double* a, long n) {
+    if (b->n != n || (long)b->op.A64.n < n * n) return -1;
+    return (int)cudaMemcpy(b->op.A64.p, a, n * n * 8, cudaMemcpyHostToDevice);
+}
+extern "C" int set_cluster(mh_boundary* b, int blocks) {
+    const int had = b->ws.cluster;
+    b->ws.cluster = blocks;
+    return had;
+}
 extern "C" void set_steps(mh_boundary* b, int v) { static_cast<gmres_k::progress*>(b->ws.prog)->steps = v; }
 """
 
@@ -36,6 +45,8 @@ def native():
     lib = compile_cuda(SOURCE)
     lib.set_cycle.argtypes = [ctypes.c_void_p, ctypes.c_long, ctypes.c_long]
     lib.set_steps.argtypes = [ctypes.c_void_p, ctypes.c_int]
+    lib.set_matrix.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_long]
+    lib.set_cluster.argtypes = [ctypes.c_void_p, ctypes.c_int]
     return lib
 
 
@@ -86,3 +97,38 @@ def test_cyclic_shift(native, n, cycle):
     ref = torch.zeros_like(x)
     ref[cycle - 1] = 1.0                                           # A e_{m-1} = e_0
     assert (x - ref).abs().max().item() <= 1e-12
+
+
+def _general(native, n, seed, cluster=None):
+    """A solve with a full operator (standard normal entries / sqrt(n) + 1.2 I: eigenvalues in a disc that nearly
+    reaches 0, so GMRES takes many steps) against the direct one: ||x - ref|| <= tol ||b|| ||A^-1||, plus the
+    direct solve's own rounding."""
+    import torch
+    alpha = 0.3
+    mh, ctx, bnd = _boundary(n, alpha)
+    rng = np.random.default_rng(seed)
+    A = np.ascontiguousarray(rng.standard_normal((n, n)) / np.sqrt(n) + 1.2 * np.eye(n))
+    rhs = rng.standard_normal(n)
+    torch.cuda.synchronize()
+    assert native.set_matrix(bnd.h, A.ctypes.data, n) == 0
+    x = torch.zeros(n, dtype=torch.float64, device="cuda:0")
+    b = torch.tensor(rhs, device="cuda:0")
+    if cluster:
+        mh.mh_gmres_solve(ctx, bnd, alpha, b, x, tol=0.5, max_iter=1000)   # makes the workspace
+        assert native.set_cluster(bnd.h, cluster) in (8, 16)
+        x.zero_()
+    info = mh.mh_gmres_solve(ctx, bnd, alpha, b, x, tol=1e-11, max_iter=1000, prec=mh.MH_PREC_FP64)
+    ref = np.linalg.solve(A, rhs)
+    inv = np.linalg.norm(np.linalg.inv(A), 2)
+    bound = 1e-11 * np.linalg.norm(rhs) * inv + n * 2.3e-16 * np.linalg.cond(A) * np.linalg.norm(ref)
+    assert np.linalg.norm(x.cpu().numpy() - ref) <= bound
+    return info
+
+
+@pytest.mark.parametrize("n", [40, 130, 600])
+def test_long_triangular_solve(native, n):
+    assert _general(native, n, n).iterations > 32
+
+
+def test_cluster_of_eight_on_a_long_boundary(native):
+    assert _general(native, 1100, 1, cluster=8).iterations > 32
